@@ -83,9 +83,12 @@ typedef enum {
     GDWS_OPT_DW_MATH = 4,  /* bf16 fused path, where the GDW stage runs: 1 = on the ALUs (fp32
                               multiply-adds); 2 = on the tensor cores as k*k block-sparse
                               products per 16-channel window (fp32 accumulation), for stride 1
-                              or 2 and k <= 5, else GDWS_ERR_UNSUPPORTED; 0 (default) = the library
-                              chooses (see gdws_plan_gdw_stage).  Both give the same result
-                              up to summation order                                         */
+                              or 2 and k <= 5, else GDWS_ERR_UNSUPPORTED; 3 = nowhere: the two
+                              stages are folded into one k x k convolution when the weights are
+                              packed (see gdws_forward), for the same layers with at most 64 MB
+                              of folded filters; 0 (default) = the library chooses by estimated
+                              time for each input size (see gdws_plan_form).  1 and 2 give the
+                              same result up to summation order; 3 rounds elsewhere (gdws_forward) */
     GDWS_OPT_OUT_DTYPE = 5 /* bf16 plans: 0 (default) = y has the dtype of x; 1 = y is fp32
                               (GDWS_F32, NHWC): bias and ReLU are applied to the fp32 sums of
                               the PW stage and stored without the rounding to bf16.  Every
@@ -110,7 +113,7 @@ typedef enum {
  * Host work: offsets off_c, the intermediate-channel -> input-channel table, the
  * padding of G to the tensor-core chunk, output-patch choice.  If a CUDA device is
  * current, the plan also allocates its device tables and packed-weight buffers
- * (O(G*(k*k+D)) bytes) on it; with no device the plan is still valid for the
+ * (O(G*(k*k+D)) bytes, and 2*C*k*k*D for the folded form where it is covered) on it; with no device the plan is still valid for the
  * host-side queries below and allocates at the first device call.
  * Errors: GDWS_ERR_INVALID_ARG, GDWS_ERR_ALLOC, GDWS_ERR_CUDA.
  */
@@ -152,12 +155,19 @@ GDWS_API int gdws_out_dim(int in, int k, int stride, int pad);
 /*
  * gdws_plan_gdw_stage -- where the fused bf16 kernel of this plan runs the GDW stage (Section 3.1,
  * Definition) with the current GDWS_OPT_DW_MATH: *stage = 1 (ALUs) or 2 (tensor cores).  With the option
- * at 0 the choice follows the measured cost of the two kernels: the tensor-core form costs k*k products
+ * at 0 (where the folded form is not taken, see gdws_plan_form) the choice follows the measured cost of the two kernels: the tensor-core form costs k*k products
  * per window of 16 input channels whatever their g_c, the ALU form costs in proportion to sum g_c; the
  * tensor cores are taken for k = 3 or 5, stride 1 (with at most 256 output channels) or 2, and an average
  * g_c of at least 4 (at least 2.7 with at most 128 output channels).  Host only; errors: GDWS_ERR_INVALID_ARG.
  */
 GDWS_API gdws_status_t gdws_plan_gdw_stage(const gdws_plan_t *plan, int *stage);
+
+/*
+ * gdws_plan_form -- the kernel a fused bf16 forward of n x C x h x w takes with the plan's current options: *form = 1 or 2
+ * (two stages, the GDW stage on the ALUs or on the tensor cores, as gdws_plan_gdw_stage) or 3 (one k x k convolution with
+ * folded filters).  Host only; errors: GDWS_ERR_INVALID_ARG.
+ */
+GDWS_API gdws_status_t gdws_plan_form(gdws_plan_t *plan, int n, int h, int w, int *form);
 
 /*
  * gdws_pack_weights -- convert one weight set to the kernels' internal form
@@ -190,8 +200,11 @@ GDWS_API gdws_status_t gdws_set_workspace(gdws_plan_t *plan, void *workspace, si
  *          them on `stream` first (F32 plans read them in place).
  *   y      DEVICE tensor, same dtype and layout as x, y->n == x->n, y->c == D,
  *          y->h/w == H'/W'.
- * Accumulation is fp32 on both paths; the bf16 path rounds the intermediate z to bf16
- * before the tensor-core contraction and y to bf16 on store.
+ * Accumulation is fp32 on both paths.  A bf16 forward rounds to bf16 once between the two linear maps and y on
+ * store: the two-stage kernels round the intermediate z, the folded one the filters
+ * W[d,c] = sum_j P[d,off_c+j] K[off_c+j] (Property 1 and 2), which are formed in fp32.  The errors have the same bound,
+ * 2^-9 sum |P| |K| |x| per output; which is smaller depends on the data (z where filters cancel a large constant part of x,
+ * W where pointwise weights cancel).  GDWS_OPT_DW_MATH = 1 or 2 keeps to the first for every size.
  * Device memory is never allocated here.  Errors: GDWS_ERR_INVALID_ARG (shape, dtype,
  * alignment, NULL), GDWS_ERR_UNSUPPORTED, GDWS_ERR_WORKSPACE (unfused path without a large
  * enough workspace), GDWS_ERR_ARCH, GDWS_ERR_CUDA (launch failure, reported synchronously).

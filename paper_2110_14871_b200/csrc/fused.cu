@@ -944,8 +944,13 @@ static gdws_status_t run_tiled(gdws_plan_s *p, const gdws_tensor_t *x, void *out
 
 gdws_status_t bf16_fused(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t *y, cudaStream_t st)
 {
-    // GDWS_OPT_DW_MATH: 1 = GDW stage on the ALUs, 2 = on the tensor cores, 0 = whichever measured faster for this kind of layer
-    if (gdw_stage_of(p) == 2) {
+    // GDWS_OPT_DW_MATH: 1 = GDW stage on the ALUs, 2 = on the tensor cores, 3 = folded, 0 = whichever measured faster for this kind of layer
+    const int form = bf16_form_of(p, x->n, x->h, x->w, y->dtype == GDWS_F32);
+    if (form == 3) {
+        const gdws_status_t rc = bf16_folded(p, x, y, st);
+        if (rc != GDWS_ERR_UNSUPPORTED || p->opt_dw_math == 3) return rc;
+    }
+    if (form == 2 || (form == 3 && gdw_stage_of(p) == 2)) {
         const gdws_status_t rc = bf16_fused_tc(p, x, y, st);
         if (rc != GDWS_ERR_UNSUPPORTED || p->opt_dw_math == 2) return rc;     // chosen automatically but no tile fits: the ALU kernel
     }

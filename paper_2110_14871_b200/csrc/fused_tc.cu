@@ -33,6 +33,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <new>
 #include <vector>
 
 #include "sm100.cuh"
@@ -695,33 +696,6 @@ void tc_pack(gdws_plan_s *p, const void *dw_w, const void *pw_w, int is_bf16, cu
 // ------------------------------------------------------------------------------------------
 namespace {
 
-// Input row h = stride * ho + u - pad of filter row u (columns alike).  With stride 2 the input is read through four
-// dense views, one per parity of row and column (every other row, every other column): in the view of parity par
-// filter row u reads row ho + off of the view, which turns the strided access into a unit-stride one.
-struct TcTaps {
-    int par[5] = {}, off[5] = {};          // per filter row (the filter is square and padded alike: same for columns)
-    int omin[2] = {}, omax[2] = {};        // per parity: smallest and largest offset
-    bool used[2] = {};
-    int ext = 0;                           // halo of a copy: the largest omax - omin
-    int npar = 0;
-};
-
-TcTaps tc_taps(int k, int stride, int pad)
-{
-    TcTaps t;
-    for (int par = 0; par < 2; ++par) { t.omin[par] = 1 << 20; t.omax[par] = -(1 << 20); }
-    for (int u = 0; u < k; ++u) {
-        const int i = u - pad;
-        const int par = ((i % stride) + stride) % stride;
-        t.par[u] = par; t.off[u] = (i - par) / stride;
-        t.used[par] = true;
-        t.omin[par] = std::min(t.omin[par], t.off[u]); t.omax[par] = std::max(t.omax[par], t.off[u]);
-    }
-    for (int par = 0; par < 2; ++par)
-        if (t.used[par]) { t.ext = std::max(t.ext, t.omax[par] - t.omin[par]); ++t.npar; }
-    return t;
-}
-
 struct TcGeom {
     int layout = 0;              // 1: boxes with halo rows (one image per tile; one box per parity pair), 2: one copy per
                                  // filter row and column parity, 3: one copy per tap (maps at most 4 wide)
@@ -837,24 +811,33 @@ void tc_choose_order(const std::vector<TcChunk> &chunks, int nz, int nw, std::ve
 
 }  // namespace
 
-gdws_status_t bf16_fused_tc(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t *y, cudaStream_t st)
+namespace {
+
+struct TcLaunch {
+    LaunchKey key;
+    TcParams P;
+    TcGeom g;
+    void (*kernel)(TcParams) = nullptr;
+    int grid = 0;
+    size_t smem = 0;
+    const void *x = nullptr, *y = nullptr;       // the addresses the tensor maps were encoded for
+};
+
+// Everything about a launch but the addresses of x and y.
+gdws_status_t tc_prepare(gdws_plan_s *p, int n, int Ho, int Wo, bool out_f32, TcLaunch *L)
 {
-    if (!p->tc_ok) return fail(GDWS_ERR_UNSUPPORTED, "tensor-core GDW path: layer not covered (stride 1 or 2, k <= 5, C and D multiples of 8)");
     const int nchunks = (int)p->tc_chunks.size();
     if (nchunks > kTcMaxChunks) return fail(GDWS_ERR_UNSUPPORTED, "tensor-core GDW path: %d chunks (at most %d)", nchunks, kTcMaxChunks);
     if (p->sm_count <= 0) {
         cudaError_t e = cudaDeviceGetAttribute(&p->sm_count, cudaDevAttrMultiProcessorCount, p->device);
         if (e != cudaSuccess) return cuda_fail(e, "cudaDeviceGetAttribute(MultiProcessorCount)");
     }
-    const int Ho = y->h, Wo = y->w, k = p->k;
-    TcGeom g;
-    if (!tc_geometry(p, x->n, Ho, Wo, &g)) return fail(GDWS_ERR_UNSUPPORTED, "tensor-core GDW path: no tile");
+    const int k = p->k;
+    TcGeom &g = L->g;
+    if (!tc_geometry(p, n, Ho, Wo, &g)) return fail(GDWS_ERR_UNSUPPORTED, "tensor-core GDW path: no tile");
     const int64_t nitems = g.tiles() * p->tc_nparts;
     if (nitems > 0x7fffffffLL) return fail(GDWS_ERR_UNSUPPORTED, "too many tiles");
-    tensor_map_encode_fn encode = encode_fn();
-    if (!encode) return fail(GDWS_ERR_CUDA, "cuTensorMapEncodeTiled is not available from this driver");
-
-    TcParams P;
+    TcParams &P = L->P;
     memset(&P, 0, sizeof(P));
     const int Dloc = p->tc_dloc, m = p->tc_maxslabs;
     // a B operand plane holds one 32-byte row per intermediate channel of the layer's largest chunk
@@ -862,7 +845,7 @@ gdws_status_t bf16_fused_tc(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_
     P.wslab_bytes = (uint32_t)Dloc * 32u;
     P.xslot_bytes = (uint32_t)((g.xbox + 255) / 256 * 256);
     // Shared memory: output staging (optional) | B operand buffers | z slabs | weight slabs | input boxes | tables
-    const bool can_stage = y->dtype != GDWS_F32 && p->D % 64 == 0 && Dloc % 64 == 0 && ((uintptr_t)y->ptr & 15) == 0 && nitems > p->sm_count;
+    const bool can_stage = !out_f32 && p->D % 64 == 0 && Dloc % 64 == 0 && nitems > p->sm_count;
     const size_t tables = (size_t)nchunks * sizeof(TcChunk) + (size_t)p->tc_nparts * Dloc * 4 + kTcMaxNB * 256 + 256;
     double best_score = -1;
     int b_ost = 0, b_nx = 0, b_nb = 0, b_nz = 0, b_nw = 0;
@@ -885,21 +868,15 @@ gdws_status_t bf16_fused_tc(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_
     if (best_score < 0) return fail(GDWS_ERR_UNSUPPORTED, "tensor-core GDW path: shared memory does not fit this layer");
     P.ostage = b_ost ? 16384 : 0; P.nx = b_nx; P.nb = b_nb; P.nz = b_nz; P.nw = b_nw;
     {
-        if (p->tc_lay_nz != P.nz || p->tc_lay_nw != P.nw || (int)p->tc_lay_order.size() != nchunks) {
-            std::vector<int> order, slabs, zpos, zdep, wpos, wdep;
-            tc_choose_order(p->tc_chunks, P.nz, P.nw, &order);
-            for (int i : order) slabs.push_back(p->tc_chunks[i].npad / 16);
-            if (!tc_ring_places(slabs, P.nz, &zpos, &zdep) || !tc_ring_places(slabs, P.nw, &wpos, &wdep))
-                return fail(GDWS_ERR_UNSUPPORTED, "tensor-core GDW path: a chunk does not fit the slab rings");
-            p->tc_lay_order.resize(nchunks); p->tc_lay_ring.resize(nchunks);
-            for (int q = 0; q < nchunks; ++q) {
-                p->tc_lay_order[q] = (uint8_t)order[q];
-                p->tc_lay_ring[q] = (uint32_t)zpos[q] | ((uint32_t)wpos[q] << 8) | ((uint32_t)zdep[q] << 16) | ((uint32_t)wdep[q] << 19);
-            }
-            p->tc_lay_nz = P.nz; p->tc_lay_nw = P.nw;
+        std::vector<int> order, slabs, zpos, zdep, wpos, wdep;
+        tc_choose_order(p->tc_chunks, P.nz, P.nw, &order);
+        for (int i : order) slabs.push_back(p->tc_chunks[i].npad / 16);
+        if (!tc_ring_places(slabs, P.nz, &zpos, &zdep) || !tc_ring_places(slabs, P.nw, &wpos, &wdep))
+            return fail(GDWS_ERR_UNSUPPORTED, "tensor-core GDW path: a chunk does not fit the slab rings");
+        for (int q = 0; q < nchunks; ++q) {
+            P.order[q] = (uint8_t)order[q];
+            P.ring[q] = (uint32_t)zpos[q] | ((uint32_t)wpos[q] << 8) | ((uint32_t)zdep[q] << 16) | ((uint32_t)wdep[q] << 19);
         }
-        memcpy(P.order, p->tc_lay_order.data(), (size_t)nchunks);
-        memcpy(P.ring, p->tc_lay_ring.data(), (size_t)nchunks * 4);
     }
     P.off_b = (uint32_t)P.ostage;
     P.off_z = P.off_b + (uint32_t)P.nb * P.bbuf_bytes;
@@ -912,35 +889,6 @@ gdws_status_t bf16_fused_tc(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_
 
     const int sd = p->stride;
     const TcTaps taps = tc_taps(k, sd, p->pad);
-    for (int hp = 0; hp < sd; ++hp)
-        for (int wp = 0; wp < sd; ++wp) {
-            if (!taps.used[hp] || !taps.used[wp]) continue;
-            // x as a rank-4 tensor, innermost first: channels, width, height, batch; a box holds 16 channels (32 bytes) per
-            // pixel.  With stride 2: the rows of parity hp and the columns of parity wp only.
-            const int Wp = (x->w - wp + sd - 1) / sd, Hp = (x->h - hp + sd - 1) / sd;
-            if (Wp <= 0 || Hp <= 0) return fail(GDWS_ERR_UNSUPPORTED, "tensor-core GDW path: input too small for stride %d", sd);
-            const cuuint64_t dims[4] = {(cuuint64_t)p->C, (cuuint64_t)Wp, (cuuint64_t)Hp, (cuuint64_t)x->n};
-            const cuuint64_t strides[3] = {(cuuint64_t)sd * p->C * 2, (cuuint64_t)sd * x->w * p->C * 2, (cuuint64_t)x->h * x->w * p->C * 2};
-            const cuuint32_t box[4] = {16, (cuuint32_t)g.IW, (cuuint32_t)g.IH, (cuuint32_t)g.TN};
-            const cuuint32_t estr[4] = {1, 1, 1, 1};
-            void *base = (uint8_t *)x->ptr + ((size_t)hp * x->w + wp) * p->C * 2;
-            const CUresult r = encode(&P.tmap_xp[hp * 2 + wp], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, base, dims, strides, box, estr,
-                                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B,
-                                      CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-            if (r != CUDA_SUCCESS) return fail(GDWS_ERR_CUDA, "cuTensorMapEncodeTiled (x) failed with code %d", (int)r);
-        }
-    if (P.ostage) {
-        const cuuint64_t dims[4] = {(cuuint64_t)p->D, (cuuint64_t)Wo, (cuuint64_t)Ho, (cuuint64_t)x->n};
-        const cuuint64_t strides[3] = {(cuuint64_t)p->D * 2, (cuuint64_t)Wo * p->D * 2, (cuuint64_t)Ho * Wo * p->D * 2};
-        const cuuint32_t box[4] = {64, (cuuint32_t)g.PW, (cuuint32_t)g.PH, (cuuint32_t)g.TN};
-        const cuuint32_t estr[4] = {1, 1, 1, 1};
-        const CUresult r = encode(&P.tmap_y, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, y->ptr, dims, strides, box, estr,
-                                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                                  CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-        if (r != CUDA_SUCCESS) return fail(GDWS_ERR_CUDA, "cuTensorMapEncodeTiled (y) failed with code %d", (int)r);
-    } else {
-        P.tmap_y = P.tmap_xp[taps.used[0] ? 0 : 3];
-    }
     // Where each copy of the box goes, and where the A operand of tap (u, v) starts.
     const uint32_t px = 32;      // bytes of one staged pixel (16 channels)
     int nl = 0;
@@ -991,10 +939,10 @@ gdws_status_t bf16_fused_tc(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_
     P.nloads = nl;
     // bytes that arrive per box: every copy delivers its full box (positions outside the image are zero-filled)
     P.xbox_bytes = nl * g.TN * g.IH * g.IW * 32;
-    P.y = (uint16_t *)y->ptr; P.filt = p->d_tc_filt; P.pw = p->d_tc_pw; P.bias = p->d_bias; P.chunks = p->d_tc_chunks;
+    P.filt = p->d_tc_filt; P.pw = p->d_tc_pw; P.bias = p->d_bias; P.chunks = p->d_tc_chunks;
     P.status = p->d_status;
-    P.N = x->n; P.Ho = Ho; P.Wo = Wo; P.D = p->D; P.Dloc = Dloc; P.Dpad_tot = p->tc_nparts * Dloc; P.nparts = p->tc_nparts;
-    P.nchunks = nchunks; P.pad = p->pad; P.relu = (p->opt_relu ? kOutRelu : 0) | (y->dtype == GDWS_F32 ? kOutF32 : 0);
+    P.N = n; P.Ho = Ho; P.Wo = Wo; P.D = p->D; P.Dloc = Dloc; P.Dpad_tot = p->tc_nparts * Dloc; P.nparts = p->tc_nparts;
+    P.nchunks = nchunks; P.pad = p->pad; P.relu = (p->opt_relu ? kOutRelu : 0) | (out_f32 ? kOutF32 : 0);
     P.TN = g.TN; P.PH = g.PH; P.PW = g.PW; P.tiles_h = g.tiles_h; P.tiles_w = g.tiles_w; P.nitems = (int)nitems;
     P.nacc = Dloc <= 128 ? 2 : 1;
     P.rec_hw = p->tc_rec_hw; P.nslabs_total = p->tc_nslabs;
@@ -1009,30 +957,90 @@ gdws_status_t bf16_fused_tc(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_
     };
     magic(p->tc_nparts, P.dv_parts); magic(g.tiles_h * g.tiles_w, P.dv_thw); magic(g.tiles_w, P.dv_tw);
 
-    const int grid = (int)(nitems < p->sm_count ? nitems : p->sm_count);
-    cudaError_t e = cudaSuccess;
-#define GDWS_TC_LAUNCH(KK)                                                                                              \
-    do {                                                                                                                \
-        static bool attr_set[64] = {};                                                                                  \
-        if (!attr_set[p->device & 63]) {                                                                                \
-            e = cudaFuncSetAttribute(fused_tc_kernel<KK>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);       \
-            if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(fused_tc_kernel)");                         \
-            attr_set[p->device & 63] = true;                                                                            \
-        }                                                                                                               \
-        e = launch_overlapped(fused_tc_kernel<KK>, (unsigned)grid, kTcThreads, smem, st, P);                              \
-        if (e != cudaSuccess) return cuda_fail(e, "fused_tc_kernel launch");                                            \
-    } while (0)
+    L->grid = (int)(nitems < p->sm_count ? nitems : p->sm_count);
+    L->smem = smem;
     switch (k) {
-    case 1: GDWS_TC_LAUNCH(1); break;
-    case 2: GDWS_TC_LAUNCH(2); break;
-    case 3: GDWS_TC_LAUNCH(3); break;
-    case 4: GDWS_TC_LAUNCH(4); break;
-    case 5: GDWS_TC_LAUNCH(5); break;
+    case 1: L->kernel = fused_tc_kernel<1>; break;
+    case 2: L->kernel = fused_tc_kernel<2>; break;
+    case 3: L->kernel = fused_tc_kernel<3>; break;
+    case 4: L->kernel = fused_tc_kernel<4>; break;
+    case 5: L->kernel = fused_tc_kernel<5>; break;
     default: return fail(GDWS_ERR_UNSUPPORTED, "tensor-core GDW path: k=%d", k);
     }
-#undef GDWS_TC_LAUNCH
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_fail(e, "fused_tc_kernel launch");
+    static bool attr_set[64][6] = {};
+    if (!attr_set[p->device & 63][k]) {
+        cudaError_t e = cudaFuncSetAttribute(L->kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+        if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(fused_tc_kernel)");
+        attr_set[p->device & 63][k] = true;
+    }
+    return GDWS_OK;
+}
+
+// x as a rank-4 tensor, innermost first: channels, width, height, batch; a box holds 16 channels (32 bytes) per
+// pixel.  With stride 2: one map per parity, the rows of parity hp and the columns of parity wp only.
+gdws_status_t tc_map_x(const gdws_plan_s *p, const gdws_tensor_t *x, TcLaunch *L)
+{
+    tensor_map_encode_fn encode = encode_fn();
+    if (!encode) return fail(GDWS_ERR_CUDA, "cuTensorMapEncodeTiled is not available from this driver");
+    const int sd = p->stride;
+    const TcTaps taps = tc_taps(p->k, sd, p->pad);
+    for (int hp = 0; hp < sd; ++hp)
+        for (int wp = 0; wp < sd; ++wp) {
+            if (!taps.used[hp] || !taps.used[wp]) continue;
+            const int Wp = (x->w - wp + sd - 1) / sd, Hp = (x->h - hp + sd - 1) / sd;
+            if (Wp <= 0 || Hp <= 0) return fail(GDWS_ERR_UNSUPPORTED, "tensor-core GDW path: input too small for stride %d", sd);
+            const cuuint64_t dims[4] = {(cuuint64_t)p->C, (cuuint64_t)Wp, (cuuint64_t)Hp, (cuuint64_t)x->n};
+            const cuuint64_t strides[3] = {(cuuint64_t)sd * p->C * 2, (cuuint64_t)sd * x->w * p->C * 2, (cuuint64_t)x->h * x->w * p->C * 2};
+            const cuuint32_t box[4] = {16, (cuuint32_t)L->g.IW, (cuuint32_t)L->g.IH, (cuuint32_t)L->g.TN};
+            const cuuint32_t estr[4] = {1, 1, 1, 1};
+            void *base = (uint8_t *)x->ptr + ((size_t)hp * x->w + wp) * p->C * 2;
+            const CUresult r = encode(&L->P.tmap_xp[hp * 2 + wp], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, base, dims, strides, box, estr,
+                                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B,
+                                      CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+            if (r != CUDA_SUCCESS) return fail(GDWS_ERR_CUDA, "cuTensorMapEncodeTiled (x) failed with code %d", (int)r);
+        }
+    L->x = x->ptr;
+    return GDWS_OK;
+}
+
+gdws_status_t tc_map_y(const gdws_plan_s *p, const gdws_tensor_t *y, TcLaunch *L)
+{
+    L->P.y = (uint16_t *)y->ptr;
+    if (L->P.ostage) {
+        const cuuint64_t dims[4] = {(cuuint64_t)p->D, (cuuint64_t)y->w, (cuuint64_t)y->h, (cuuint64_t)y->n};
+        const cuuint64_t strides[3] = {(cuuint64_t)p->D * 2, (cuuint64_t)y->w * p->D * 2, (cuuint64_t)y->h * y->w * p->D * 2};
+        const cuuint32_t box[4] = {64, (cuuint32_t)L->g.PW, (cuuint32_t)L->g.PH, (cuuint32_t)L->g.TN};
+        const cuuint32_t estr[4] = {1, 1, 1, 1};
+        const CUresult r = encode_fn()(&L->P.tmap_y, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, y->ptr, dims, strides, box, estr,
+                                       CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                                       CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+        if (r != CUDA_SUCCESS) return fail(GDWS_ERR_CUDA, "cuTensorMapEncodeTiled (y) failed with code %d", (int)r);
+    }
+    L->y = y->ptr;
+    return GDWS_OK;
+}
+
+}  // namespace
+
+gdws_status_t bf16_fused_tc(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t *y, cudaStream_t st)
+{
+    if (!p->tc_ok) return fail(GDWS_ERR_UNSUPPORTED, "tensor-core GDW path: layer not covered (stride 1 or 2, k <= 5, C and D multiples of 8)");
+    const bool out_f32 = y->dtype == GDWS_F32;
+    const LaunchKey key = {x->n, x->h, x->w, (p->opt_relu ? 1 : 0) | (out_f32 ? 2 : 0)};
+    gdws_status_t rc;
+    TcLaunch *L = LaunchCache<TcLaunch>::find(p->launch_cache[1], key);
+    if (!L) {
+        std::unique_ptr<TcLaunch> e(new (std::nothrow) TcLaunch);
+        if (!e) return fail(GDWS_ERR_ALLOC, "out of host memory");
+        e->key = key;
+        rc = tc_prepare(p, x->n, y->h, y->w, out_f32, e.get());
+        if (rc != GDWS_OK) return rc;
+        L = LaunchCache<TcLaunch>::add(p->launch_cache[1], std::move(e));
+    }
+    if (L->x != x->ptr && (rc = tc_map_x(p, x, L)) != GDWS_OK) return rc;
+    if (L->y != y->ptr && (rc = tc_map_y(p, y, L)) != GDWS_OK) return rc;
+    const cudaError_t e = launch_overlapped(L->kernel, (unsigned)L->grid, kTcThreads, L->smem, st, L->P);
+    if (e != cudaSuccess) { cudaGetLastError(); return cuda_fail(e, "fused_tc_kernel launch"); }
     p->launches++;
     return GDWS_OK;
 }

@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+#include <memory>
 #include <string>
 #include <utility>
 #include <vector>
@@ -81,15 +83,14 @@ struct gdws_plan_s {
     // Tensor-core GDW path (fused_tc.cu): chunk list, output-channel split, packed sizes.
     bool tc_ok = false;              // the layer is one the path covers (stride 1, k <= 5, ...)
     std::vector<gdws::TcChunk> tc_chunks;
-    // last layout of the tensor-core path's slab rings (chunk order within a work item, places and waits), kept per
-    // ring sizes: working it out tries a few dozen orders
-    int tc_lay_nz = 0, tc_lay_nw = 0;
-    std::vector<uint8_t> tc_lay_order;
-    std::vector<uint32_t> tc_lay_ring;
     int tc_nslabs = 0;               // sum of npad / 16 over the chunks
     int tc_maxslabs = 0;             // largest npad / 16 of one chunk
     int tc_nparts = 1, tc_dloc = 0;  // blocks per tile along D, output channels per block (multiple of 16, <= 256)
     int tc_rec_hw = 0;               // 16-bit words per filter record (channel slot, then k*k taps; multiple of 8)
+
+    // Folded path (fold.cu): the layer as one k x k convolution.
+    bool fold_ok = false;            // the layer is one the path covers
+    int fold_nwin = 0, fold_dp = 0;  // windows of 64 input channels; output channels rounded up to 32
 
     int opt_path = GDWS_PATH_AUTO;
     int opt_relu = 0;
@@ -112,6 +113,7 @@ struct gdws_plan_s {
     gdws::TcChunk *d_tc_chunks = nullptr;
     uint16_t *d_tc_filt = nullptr; // [tc_nslabs * 16][tc_rec_hw]: per intermediate slot, channel index inside the window and the taps (bf16)
     uint16_t *d_tc_pw = nullptr;   // [tc_nparts][tc_nslabs][2][tc_dloc][8] bf16: pointwise weights, one K = 16 operand slab per 16 slots
+    uint16_t *d_fold = nullptr;    // [fold_nwin][k*k][fold_dp][64] bf16: folded filters
     int *d_status = nullptr;       // device status word
     bool packed = false;
 
@@ -120,6 +122,10 @@ struct gdws_plan_s {
 
     void *stage_x = nullptr, *stage_y = nullptr;  // gdws_forward_host staging
     size_t stage_x_bytes = 0, stage_y_bytes = 0;
+
+    // Prepared launches of the three fused bf16 kernels and the choice between them (LaunchCache below; each file knows its
+    // own types).
+    std::shared_ptr<void> launch_cache[4];
 
     int64_t launches = 0;
 };
@@ -146,6 +152,37 @@ inline cudaError_t launch_overlapped(void (*kernel)(KArgs...), unsigned grid, un
     cfg.attrs = attr; cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
+// What a launch needs besides the tensors' addresses depends on the input size and a few options only: tile shape, work
+// split, shared-memory layout, kernel.  Working it out takes longer than a small layer runs, so a plan keeps the last few;
+// a call with the same key encodes tensor maps anew only for the addresses that differ from the last call's.
+struct LaunchKey {
+    int n, h, w, flags;          // input extents; flags: relu, output type, forced options
+    bool operator==(const LaunchKey &o) const { return n == o.n && h == o.h && w == o.w && flags == o.flags; }
+};
+template <class Entry> struct LaunchCache {
+    static constexpr size_t kKeep = 8;
+    std::vector<std::unique_ptr<Entry>> entries;      // the most recently used one last
+    // The entry of `key`, or null.
+    static Entry *find(std::shared_ptr<void> &slot, const LaunchKey &key)
+    {
+        if (!slot) return nullptr;
+        auto &v = static_cast<LaunchCache *>(slot.get())->entries;
+        for (size_t i = v.size(); i-- > 0;)
+            if (v[i]->key == key) {
+                if (i + 1 != v.size()) std::rotate(v.begin() + i, v.begin() + i + 1, v.end());
+                return v.back().get();
+            }
+        return nullptr;
+    }
+    static Entry *add(std::shared_ptr<void> &slot, std::unique_ptr<Entry> e)
+    {
+        if (!slot) slot = std::shared_ptr<void>(new LaunchCache, [](void *c) { delete static_cast<LaunchCache *>(c); });
+        auto &v = static_cast<LaunchCache *>(slot.get())->entries;
+        if (v.size() >= kKeep) v.erase(v.begin());
+        v.push_back(std::move(e));
+        return v.back().get();
+    }
+};
 // x and y of a forward call against the plan: pointers, alignment, extents, dtype/layout pair, no overlap
 gdws_status_t check_pair(const gdws_plan_s *p, const gdws_tensor_t *x, const gdws_tensor_t *y);
 // static_ws.cu: looks up (once per device, the device being current) the address of the built-in scratch array
@@ -160,7 +197,7 @@ inline size_t dtype_size(gdws_dtype_t d) { return d == GDWS_F32 ? 4 : 2; }
 // row), and beyond 256 output channels the tensor-core kernel computes the GDW stage once per 256 of them.
 inline int gdw_stage_of(const gdws_plan_s *p)
 {
-    if (p->opt_dw_math == 1 || p->opt_dw_math == 2) return p->opt_dw_math;
+    if (p->opt_dw_math != 0) return p->opt_dw_math;
     if (!(p->tc_ok && (p->k == 3 || p->k == 5) && p->stride <= 2)) return 1;
     if (p->stride == 1 && p->Dpad > 256) return 1;     // measured equal or slower there; with stride 2 faster at D = 512 too
     // average multiplier of at least 4, or of at least 2.7 when the PW products are small (at most 128 output channels)
@@ -189,5 +226,37 @@ gdws_status_t bf16_depthwise_tiled(gdws_plan_s *p, const gdws_tensor_t *x, void 
 // fused_tc.cu
 void tc_pack(gdws_plan_s *p, const void *dw_w, const void *pw_w, int is_bf16, cudaStream_t s);
 gdws_status_t bf16_fused_tc(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t *y, cudaStream_t s);
+
+// fold.cu
+void fold_pack(gdws_plan_s *p, const void *dw_w, const void *pw_w, int is_bf16, cudaStream_t s);
+gdws_status_t bf16_folded(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t *y, cudaStream_t s);
+int bf16_form_of(gdws_plan_s *p, int n, int h, int w, bool out_f32);   // 1 / 2: two stages, GDW on the ALUs / the tensor cores; 3: folded
+
+// Input row h = stride * ho + u - pad of filter row u (columns alike).  With stride 2 the input is read through four
+// dense views, one per parity of row and column (every other row, every other column): in the view of parity par
+// filter row u reads row ho + off of the view, which turns the strided access into a unit-stride one.
+struct TcTaps {
+    int par[5] = {}, off[5] = {};          // per filter row (the filter is square and padded alike: same for columns)
+    int omin[2] = {}, omax[2] = {};        // per parity: smallest and largest offset
+    bool used[2] = {};
+    int ext = 0;                           // halo of a copy: the largest omax - omin
+    int npar = 0;
+};
+
+inline TcTaps tc_taps(int k, int stride, int pad)
+{
+    TcTaps t;
+    for (int par = 0; par < 2; ++par) { t.omin[par] = 1 << 20; t.omax[par] = -(1 << 20); }
+    for (int u = 0; u < k; ++u) {
+        const int i = u - pad;
+        const int par = ((i % stride) + stride) % stride;
+        t.par[u] = par; t.off[u] = (i - par) / stride;
+        t.used[par] = true;
+        t.omin[par] = std::min(t.omin[par], t.off[u]); t.omax[par] = std::max(t.omax[par], t.off[u]);
+    }
+    for (int par = 0; par < 2; ++par)
+        if (t.used[par]) { t.ext = std::max(t.ext, t.omax[par] - t.omin[par]); ++t.npar; }
+    return t;
+}
 
 }  // namespace gdws

@@ -68,6 +68,7 @@ static void free_device(gdws_plan_s *p)
     release(p->d_tc_chunks);
     release(p->d_tc_filt);
     release(p->d_tc_pw);
+    release(p->d_fold);
     release(p->stage_x);
     release(p->stage_y);
     p->stage_x_bytes = 0;
@@ -108,6 +109,7 @@ gdws_status_t ensure_device(gdws_plan_s *p)
         GDWS_TRY_ALLOC(p->d_tc_filt, sizeof(uint16_t) * (size_t)p->tc_nslabs * 16 * p->tc_rec_hw);
         GDWS_TRY_ALLOC(p->d_tc_pw, sizeof(uint16_t) * (size_t)p->tc_nparts * p->tc_nslabs * 16 * p->tc_dloc);
     }
+    if (p->fold_ok) GDWS_TRY_ALLOC(p->d_fold, sizeof(uint16_t) * (size_t)p->fold_nwin * k2 * p->fold_dp * 64);
 #undef GDWS_TRY_ALLOC
     p->device = dev;
     if (cudaDeviceGetAttribute(&p->sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) p->sm_count = 0;
@@ -378,6 +380,10 @@ gdws_status_t gdws_plan(int C, int D, int k, int stride, int pad, const int32_t 
         delete p;
         return fail(GDWS_ERR_ALLOC, "gdws_plan: out of host memory");
     }
+    p->fold_nwin = (C + 63) / 64;
+    p->fold_dp = round_up(D, 32);
+    // the folded filters (2 C k^2 D bytes) have to be worth their memory; 64 MB hold 1024 x 1024 channels of 5 x 5 filters
+    p->fold_ok = stride <= 2 && k <= 5 && C % 8 == 0 && D % 8 == 0 && (size_t)p->fold_nwin * k * k * p->fold_dp * 128 <= ((size_t)64 << 20);
     int ndev = 0;
     if (cudaGetDeviceCount(&ndev) == cudaSuccess && ndev > 0) {
         gdws_status_t st = ensure_device(p);
@@ -412,7 +418,7 @@ gdws_status_t gdws_plan_set_option(gdws_plan_t *p, int key, int value)
         if (value != 0 && value != 1) return fail(GDWS_ERR_INVALID_ARG, "a_layout must be 0 or 1");
         p->opt_a_layout = value; return GDWS_OK;
     case GDWS_OPT_DW_MATH:
-        if (value < 0 || value > 2) return fail(GDWS_ERR_INVALID_ARG, "dw_math must be 0, 1 or 2");
+        if (value < 0 || value > 3) return fail(GDWS_ERR_INVALID_ARG, "dw_math must be 0, 1, 2 or 3");
         p->opt_dw_math = value; return GDWS_OK;
     case GDWS_OPT_OUT_DTYPE:
         if (value != 0 && value != 1) return fail(GDWS_ERR_INVALID_ARG, "out_dtype must be 0 (as x) or 1 (fp32)");
@@ -479,6 +485,15 @@ gdws_status_t gdws_plan_gdw_stage(const gdws_plan_t *p, int *stage)
 {
     if (!p || !stage) return fail(GDWS_ERR_INVALID_ARG, "gdws_plan_gdw_stage: NULL argument");
     *stage = gdw_stage_of(p);
+    return GDWS_OK;
+}
+
+gdws_status_t gdws_plan_form(gdws_plan_t *p, int n, int h, int w, int *form)
+{
+    if (!p || !form) return fail(GDWS_ERR_INVALID_ARG, "gdws_plan_form: NULL argument");
+    if (n < 1 || gdws_out_dim(h, p->k, p->stride, p->pad) < 1 || gdws_out_dim(w, p->k, p->stride, p->pad) < 1)
+        return fail(GDWS_ERR_INVALID_ARG, "gdws_plan_form: no output for n=%d h=%d w=%d", n, h, w);
+    *form = bf16_form_of(p, n, h, w, p->opt_out_f32 != 0);
     return GDWS_OK;
 }
 

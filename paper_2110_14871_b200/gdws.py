@@ -28,7 +28,7 @@ EXPORTS = [
     "gdws_out_dim", "gdws_pack_weights", "gdws_workspace_bytes", "gdws_set_workspace", "gdws_forward",
     "gdws_depthwise", "gdws_pointwise", "gdws_forward_host", "gdws_status", "gdws_launch_count",
     "gdws_last_error", "gdws_version", "gdws_destroy", "gdws_forward_static", "gdws_static_scratch_bytes",
-    "gdws_measure_fma_rate", "gdws_measure_code_size", "gdws_selftest_wait", "gdws_plan_gdw_stage",
+    "gdws_measure_fma_rate", "gdws_measure_code_size", "gdws_selftest_wait", "gdws_plan_gdw_stage", "gdws_plan_form",
 ]
 
 
@@ -74,6 +74,8 @@ def lib() -> ctypes.CDLL:
     L.gdws_plan_tile.restype = ci
     L.gdws_plan_gdw_stage.argtypes = [vp, pint]
     L.gdws_plan_gdw_stage.restype = ci
+    L.gdws_plan_form.argtypes = [vp, ci, ci, ci, pint]
+    L.gdws_plan_form.restype = ci
     L.gdws_out_dim.argtypes = [ci, ci, ci, ci]
     L.gdws_out_dim.restype = ci
     L.gdws_pack_weights.argtypes = [vp, vp, vp, vp, ci, vp]
@@ -246,6 +248,12 @@ class Plan:
         st = ctypes.c_int()
         _check(lib().gdws_plan_gdw_stage(self._h, ctypes.byref(st)))
         return st.value
+
+    def form(self, n: int, h: int, w: int) -> int:
+        """gdws_plan_form: 1 / 2 = two stages (GDW stage on the ALUs / the tensor cores), 3 = folded filters."""
+        form = ctypes.c_int()
+        _check(lib().gdws_plan_form(self._h, n, h, w, ctypes.byref(form)))
+        return form.value
 
     def workspace_bytes(self, dtype: int, n: int, h: int, w: int) -> int:
         return int(lib().gdws_workspace_bytes(self._h, dtype, n, h, w))
