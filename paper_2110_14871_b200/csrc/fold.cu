@@ -675,8 +675,11 @@ gdws_status_t fold_prepare(gdws_plan_s *p, int n, int Ho, int Wo, bool out_f32, 
     const bool can_stay = units >= 2 && units <= kFoldMaxB && (g.nparts == 1 || nitems <= nclusters);
     const bool several = P.nboxes > 1;       // boxes per window: more in flight to cover their latency
     const double products = k * k * (p->C / 16.0) * fold_mma_cycles(g.Npart), epilogue = 1400.0 * nblk;
-    const int groups = epilogue > 1.4 * products ? 4 : (epilogue > 0.7 * products ? 2 : 1);
-    if (can_stay) placed = place(true, groups, several ? 4 : 3, kFoldMaxA, 0) || place(true, std::min(groups, 2), several ? 3 : 2, kFoldMaxA, 0) || place(true, 1, several ? 3 : 2, kFoldMaxA, 0);
+    // Filters that stay leave memory for staging: four groups where an item's epilogue is not well below its products
+    // (64 -> 64 channels at 32 x 32: 53 us with two groups, 38 with four).  A ring of filters needs it more.
+    const int stay_groups = epilogue > 0.75 * products ? 4 : (epilogue > 0.35 * products ? 2 : 1);
+    const int groups = epilogue > 1.4 * products ? 4 : (epilogue > 0.8 * products ? 2 : 1);
+    for (int gr = stay_groups; can_stay && gr >= 1 && !placed; gr >>= 1) placed = place(true, gr, several ? (gr == 4 ? 4 : 3) : (gr == 4 ? 3 : 2), kFoldMaxA, 0);
     // ring: three units of filters (one being read, two on their way), then boxes, then more of both
     if (!placed) placed = place(false, groups, several ? 4 : 3, several ? 4 : 3, 4) || place(false, groups, 3, 3, 3) || place(false, std::min(groups, 2), 2, 3, 3) || place(false, 1, 2, 3, 3) ||
                           place(false, 1, 2, 3, 2);
