@@ -1,89 +1,8 @@
-// bf16 NHWC kernels for sm_100a: weight packing, the unfused GDW kernel and the pointwise
+// bf16 NHWC kernels for sm_100a: the unfused GDW kernel and the pointwise
 // 1x1 convolution as a tcgen05/TMEM GEMM.
 #include "sm100.cuh"
 
 namespace gdws {
-
-// ------------------------------------------------------------------------------------------
-// Weight packing
-// ------------------------------------------------------------------------------------------
-__device__ __forceinline__ float load_weight(const void *w, size_t idx, int is_bf16)
-{
-    return is_bf16 ? bf16_bits_to_float(((const uint16_t *)w)[idx]) : ((const float *)w)[idx];
-}
-
-// pw_w[D][G] -> one operand image per 64-wide K chunk: rows d (zero rows up to Dpad), 64 bf16
-// of K per 128-byte row, 128-byte swizzle; columns beyond G are zero.
-__global__ void pack_pw_kernel(const void *__restrict__ pw, int is_bf16, int D, int Dpad, int G, int nchunks,
-                               uint16_t *__restrict__ img)
-{
-    const long long total = (long long)nchunks * Dpad * kChunk;
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
-         t += (long long)gridDim.x * blockDim.x) {
-        const int kk = (int)(t % kChunk);
-        const long long r = t / kChunk;
-        const int d = (int)(r % Dpad);
-        const int q = (int)(r / Dpad);
-        const int i = q * kChunk + kk;
-        float v = 0.f;
-        if (d < D && i < G) v = load_weight(pw, (size_t)d * G + i, is_bf16);
-        const uint32_t off = (uint32_t)(d >> 3) * 1024u + (uint32_t)(d & 7) * 128u +
-                             (uint32_t)(((kk >> 3) ^ (d & 7)) << 4) + (uint32_t)(kk & 7) * 2u;
-        img[(size_t)q * Dpad * kChunk + (off >> 1)] = float_to_bf16_bits(v);
-    }
-}
-
-// dw_w[G][k][k] -> (1) fp32 taps [Gpad][k*k] (zero rows for the padding) for the unfused kernel,
-// (2) [Gpad][wstride] words for the fused kernel: the taps, then the index of the channel inside the
-// input box staged for its K chunk (chan[i] - first channel of that box).
-__global__ void pack_dw_kernel(const void *__restrict__ dw, int is_bf16, int G, int Gpad, int k2, int wstride,
-                               const int32_t *__restrict__ chan, const int32_t *__restrict__ chunk_meta,
-                               float *__restrict__ out, uint32_t *__restrict__ outp)
-{
-    const int total = Gpad * wstride;
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
-        const int i = t / wstride, j = t - i * wstride;
-        uint32_t word = 0;
-        if (j < k2) {
-            float v = 0.f;
-            if (i < G) v = load_weight(dw, (size_t)i * k2 + j, is_bf16);
-            v = bf16_bits_to_float(float_to_bf16_bits(v));
-            out[(size_t)i * k2 + j] = v;
-            word = __float_as_uint(v);
-        } else if (j == k2 && i < G) {
-            word = (uint32_t)(chan[i] - chunk_meta[4 * (i / kChunk) + 2]);
-        }
-        outp[t] = word;
-    }
-}
-
-__global__ void pack_bias_kernel(const float *__restrict__ bias, int D, int Dpad, float *__restrict__ out)
-{
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < Dpad) out[t] = (bias && t < D) ? bias[t] : 0.f;
-}
-
-gdws_status_t bf16_pack(gdws_plan_s *p, const void *dw_w, const void *pw_w, const float *bias, gdws_dtype_t dtype,
-                        cudaStream_t st)
-{
-    const int is_bf16 = dtype == GDWS_BF16;
-    const int k2 = p->k * p->k;
-    const long long tot_pw = (long long)p->nchunks * p->Dpad * kChunk;
-    int blocks = (int)((tot_pw + 255) / 256);
-    if (blocks > sm_count_of(p) * 8) blocks = sm_count_of(p) * 8;
-    pack_pw_kernel<<<blocks, 256, 0, st>>>(pw_w, is_bf16, p->D, p->Dpad, p->G, p->nchunks, p->d_pw_img);
-    int blocks2 = (p->Gpad * p->wstride + 255) / 256;
-    pack_dw_kernel<<<blocks2, 256, 0, st>>>(dw_w, is_bf16, p->G, p->Gpad, k2, p->wstride, p->d_chan, p->d_chunk_meta,
-                                            p->d_dw, p->d_dwpack);
-    pack_bias_kernel<<<(p->Dpad + 255) / 256, 256, 0, st>>>(bias, p->D, p->Dpad, p->d_bias);
-    p->launches += 3;
-    tc_pack(p, dw_w, pw_w, is_bf16, st);
-    fold_pack(p, dw_w, pw_w, is_bf16, st);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_fail(e, "weight pack launch");
-    p->packed = true;
-    return GDWS_OK;
-}
 
 // ------------------------------------------------------------------------------------------
 // Unfused GDW kernel: z[pixel][Gpad] (bf16), one thread per pixel and group of 8 intermediate

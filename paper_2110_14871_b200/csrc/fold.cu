@@ -436,54 +436,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kFoldThreads, 1) fol
 }
 
 // ------------------------------------------------------------------------------------------
-// Filter folding: W[d,c,tap] = sum_j P[d, off_c+j] K[off_c+j, tap] in fp32, rounded to bf16 once.
-// ------------------------------------------------------------------------------------------
-// out rows are (window of 64 input channels, tap, output channel), 64 input channels each; rows d >= D and channels
-// >= C are zero.  A block takes one window and 16 output channels: thread = one channel x 4 output channels, up to 9
-// taps at a time in registers, so a filter tap read once serves 4 output channels.
-constexpr int kFoldPackD = 16, kFoldPackTaps = 9;
-
-__global__ void __launch_bounds__(256) fold_pack_kernel(const void *__restrict__ dw, const void *__restrict__ pw, int is_bf16, int C, int D, int Dp,
-                                                        int G, int k2, const int32_t *__restrict__ off, uint16_t *__restrict__ out)
-{
-    const int c = (int)blockIdx.x * 64 + (threadIdx.x & 63);
-    const int d0 = (int)blockIdx.y * kFoldPackD + (threadIdx.x >> 6) * 4;
-    const int i0 = c < C ? off[c] : 0, i1 = c < C ? off[c + 1] : 0;
-    auto weight = [&](const void *w, size_t idx) {       // the two-stage kernels use the weights rounded to bf16 as well
-        return is_bf16 ? bf16_bits_to_float(((const uint16_t *)w)[idx]) : bf16_bits_to_float(float_to_bf16_bits(((const float *)w)[idx]));
-    };
-    for (int t0 = 0; t0 < k2; t0 += kFoldPackTaps) {
-        float acc[4][kFoldPackTaps] = {};
-        for (int i = i0; i < i1; ++i) {
-            float p[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) p[e] = d0 + e < D ? weight(pw, (size_t)(d0 + e) * G + i) : 0.f;
-#pragma unroll
-            for (int t = 0; t < kFoldPackTaps; ++t) {
-                const float v = t0 + t < k2 ? weight(dw, (size_t)i * k2 + t0 + t) : 0.f;
-#pragma unroll
-                for (int e = 0; e < 4; ++e) acc[e][t] = fmaf(p[e], v, acc[e][t]);
-            }
-        }
-#pragma unroll
-        for (int t = 0; t < kFoldPackTaps; ++t)
-            if (t0 + t < k2)
-#pragma unroll
-                for (int e = 0; e < 4; ++e)
-                    if (d0 + e < Dp)
-                        out[(((size_t)blockIdx.x * k2 + t0 + t) * Dp + d0 + e) * 64 + (threadIdx.x & 63)] = float_to_bf16_bits(acc[e][t]);
-    }
-}
-
-void fold_pack(gdws_plan_s *p, const void *dw_w, const void *pw_w, int is_bf16, cudaStream_t st)
-{
-    if (!p->fold_ok) return;
-    fold_pack_kernel<<<dim3((unsigned)p->fold_nwin, (unsigned)((p->fold_dp + kFoldPackD - 1) / kFoldPackD)), 256, 0, st>>>(
-        dw_w, pw_w, is_bf16, p->C, p->D, p->fold_dp, p->G, p->k * p->k, p->d_off, p->d_fold);
-    p->launches++;
-}
-
-// ------------------------------------------------------------------------------------------
 // Host side
 // ------------------------------------------------------------------------------------------
 namespace {

@@ -28,6 +28,10 @@
 //     optional ReLU, round to bf16 and store y.
 // Every wait is bounded; a wait that runs out raises a block-wide abort flag that turns all later
 // waits into no-ops, so the block still reaches its teardown, frees TMEM and ends.
+#include <string.h>
+
+#include <new>
+
 #include "sm100.cuh"
 
 namespace gdws {
@@ -806,43 +810,54 @@ __global__ void __launch_bounds__(kFusedThreads, 1) fused_bf16_kernel(const __gr
 // ------------------------------------------------------------------------------------------
 // Host side
 // ------------------------------------------------------------------------------------------
+typedef void (*FusedKernel)(FusedParams);
+
 template <int K, int MODE, int S, int PS, int VAR>
-static gdws_status_t launch_one(const FusedParams &P, int device, int grid, size_t smem, cudaStream_t st)
+static gdws_status_t kernel_one(int device, FusedKernel *out)
 {
-    cudaError_t e = cudaSuccess;
     static bool attr_set[64] = {};
     if (!attr_set[device & 63]) {   // once per device: allow the full dynamic shared memory
-        e = cudaFuncSetAttribute(fused_bf16_kernel<K, MODE, S, PS, VAR>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+        const cudaError_t e = cudaFuncSetAttribute(fused_bf16_kernel<K, MODE, S, PS, VAR>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
         if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(fused_bf16_kernel)");
         attr_set[device & 63] = true;
     }
-    e = launch_overlapped(fused_bf16_kernel<K, MODE, S, PS, VAR>, (unsigned)grid, kFusedThreads, smem, st, P);
-    return e == cudaSuccess ? GDWS_OK : cuda_fail(e, "fused_bf16_kernel launch");
+    *out = fused_bf16_kernel<K, MODE, S, PS, VAR>;
+    return GDWS_OK;
 }
 
 template <int K, int MODE, int S, int PS>
-static gdws_status_t launch_fused(const FusedParams &P, int device, int grid, size_t smem, cudaStream_t st)
+static gdws_status_t kernel_fused(const FusedParams &P, int device, FusedKernel *out)
 {
-    if (P.zout) return launch_one<K, MODE, S, PS, 1>(P, device, grid, smem, st);
+    if (P.zout) return kernel_one<K, MODE, S, PS, 1>(device, out);
     if (P.nsplit > 1) {
-        if constexpr (K == 3 && MODE != 0) return launch_one<K, MODE, S, PS, 2>(P, device, grid, smem, st);
+        if constexpr (K == 3 && MODE != 0) return kernel_one<K, MODE, S, PS, 2>(device, out);
         else return fail(GDWS_ERR_UNSUPPORTED, "several blocks per tile: no such kernel for k=%d", K);
     }
-    return launch_one<K, MODE, S, PS, 0>(P, device, grid, smem, st);
+    return kernel_one<K, MODE, S, PS, 0>(device, out);
 }
 
 template <int K, int MODE, int S>
-static gdws_status_t launch_fast(const FusedParams &P, int device, int grid, size_t smem, cudaStream_t st)
+static gdws_status_t kernel_fast(const FusedParams &P, int device, FusedKernel *out)
 {
     switch (P.ps) {
-    case 64: return launch_fused<K, MODE, S, 64>(P, device, grid, smem, st);
-    case 128: return launch_fused<K, MODE, S, 128>(P, device, grid, smem, st);
-    case 256: return launch_fused<K, MODE, S, 256>(P, device, grid, smem, st);
+    case 64: return kernel_fused<K, MODE, S, 64>(P, device, out);
+    case 128: return kernel_fused<K, MODE, S, 128>(P, device, out);
+    case 256: return kernel_fused<K, MODE, S, 256>(P, device, out);
     default: return fail(GDWS_ERR_UNSUPPORTED, "staged pixel size %d", P.ps);
     }
 }
 
-static gdws_status_t run_tiled(gdws_plan_s *p, const gdws_tensor_t *x, void *out, int Ho, int Wo, bool zout, bool out_f32, cudaStream_t st)
+struct AluLaunch {
+    LaunchKey key;
+    FusedParams P;
+    Tile t;
+    FusedKernel kernel = nullptr;
+    int grid = 0;
+    const void *x = nullptr, *out = nullptr;      // the addresses the tensor maps were encoded for
+};
+
+// Everything about a launch but the addresses of the tensors.
+static gdws_status_t alu_prepare(gdws_plan_s *p, int n, int h, int w, int Ho, int Wo, bool zout, bool out_f32, AluLaunch *L)
 {
     if (!zout && p->Dpad > 512) return fail(GDWS_ERR_UNSUPPORTED, "bf16 fused kernel supports D <= 512 (got %d)", p->D);
     if (p->D % 8 || p->C % 8)
@@ -851,49 +866,22 @@ static gdws_status_t run_tiled(gdws_plan_s *p, const gdws_tensor_t *x, void *out
         cudaError_t e = cudaDeviceGetAttribute(&p->sm_count, cudaDevAttrMultiProcessorCount, p->device);
         if (e != cudaSuccess) return cuda_fail(e, "cudaDeviceGetAttribute(MultiProcessorCount)");
     }
-    Tile t;
-    if (!choose_tile(p, x->n, x->h, x->w, &t))
+    Tile &t = L->t;
+    if (!choose_tile(p, n, h, w, &t))
         return fail(GDWS_ERR_UNSUPPORTED, "no fused tile fits this shape in shared memory");
     if (t.tiles() > 0x7fffffffLL) return fail(GDWS_ERR_UNSUPPORTED, "too many tiles");
-    tensor_map_encode_fn encode = encode_fn();
-    if (!encode) return fail(GDWS_ERR_CUDA, "cuTensorMapEncodeTiled is not available from this driver");
-    FusedParams P;
-    {
-        // x as a rank-4 tensor, innermost first: channels, width, height, batch
-        const cuuint64_t dims[4] = {(cuuint64_t)p->C, (cuuint64_t)x->w, (cuuint64_t)x->h, (cuuint64_t)x->n};
-        const cuuint64_t strides[3] = {(cuuint64_t)p->C * 2, (cuuint64_t)x->w * p->C * 2,
-                                       (cuuint64_t)x->h * x->w * p->C * 2};
-        const cuuint32_t box[4] = {(cuuint32_t)t.cbox, (cuuint32_t)t.IW, (cuuint32_t)t.IH, (cuuint32_t)t.TN};
-        const cuuint32_t estr[4] = {1, 1, 1, 1};
-        const CUresult r = encode(&P.tmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, x->ptr, dims, strides, box, estr,
-                                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                                  CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-        if (r != CUDA_SUCCESS) return fail(GDWS_ERR_CUDA, "cuTensorMapEncodeTiled failed with code %d", (int)r);
-    }
+    FusedParams &P = L->P;
+    memset(&P, 0, sizeof(P));
     // The staged epilogue pays when it overlaps the next tile's main loop; a block with a single tile would
     // only wait for its one staging buffer between the column blocks.
-    const bool tma_out = !zout && !out_f32 && t.ostage && (reinterpret_cast<uintptr_t>(out) & 15) == 0 && t.tiles() > p->sm_count;
-    if (tma_out) {
-        // y as a rank-4 tensor, innermost first: channels, width, height, batch
-        const cuuint64_t dims[4] = {(cuuint64_t)p->D, (cuuint64_t)Wo, (cuuint64_t)Ho, (cuuint64_t)x->n};
-        const cuuint64_t strides[3] = {(cuuint64_t)p->D * 2, (cuuint64_t)Wo * p->D * 2, (cuuint64_t)Ho * Wo * p->D * 2};
-        const cuuint32_t box[4] = {64, (cuuint32_t)t.PW, (cuuint32_t)t.PH, (cuuint32_t)t.TN};
-        const cuuint32_t estr[4] = {1, 1, 1, 1};
-        const CUresult r = encode(&P.tmap_y, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, out, dims, strides, box, estr,
-                                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                                  CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-        if (r != CUDA_SUCCESS) return fail(GDWS_ERR_CUDA, "cuTensorMapEncodeTiled (y) failed with code %d", (int)r);
-    } else {
-        P.tmap_y = P.tmap;
-    }
-    P.y = (uint16_t *)out;
+    const bool tma_out = !zout && !out_f32 && t.ostage && t.tiles() > p->sm_count;
     P.dwpack = p->d_dwpack; P.pw_img = p->d_pw_img; P.bias = p->d_bias;
     P.chunk_meta = reinterpret_cast<const int4 *>(p->d_chunk_meta); P.status = p->d_status;
     // Few tiles and many output channels: two blocks per tile, each with half of the channels (and of the weight stream).
     const int nsplit = (!zout && t.fast && p->k == 3 && p->Dpad == p->D && p->D >= 256 && p->D % 32 == 0 && 2 * t.tiles() <= p->sm_count) ? 2 : 1;
     const int Dloc = p->Dpad / nsplit;
     P.nsplit = nsplit; P.Dtot = zout ? p->Gpad : p->D; P.Dpad_tot = p->Dpad;
-    P.N = x->n; P.H = x->h; P.W = x->w; P.C = p->C; P.Ho = Ho; P.Wo = Wo; P.D = zout ? p->Gpad : (nsplit > 1 ? Dloc : p->D); P.Dpad = Dloc;
+    P.N = n; P.H = h; P.W = w; P.C = p->C; P.Ho = Ho; P.Wo = Wo; P.D = zout ? p->Gpad : (nsplit > 1 ? Dloc : p->D); P.Dpad = Dloc;
     P.G = p->G; P.nchunks = p->nchunks; P.stride = p->stride; P.pad = p->pad;
     P.relu = (p->opt_relu ? kOutRelu : 0) | (out_f32 ? kOutF32 : 0);
     P.TN = t.TN; P.PH = t.PH; P.PW = t.PW; P.tiles_h = t.tiles_h; P.tiles_w = t.tiles_w; P.ntiles = (int)t.tiles();
@@ -916,30 +904,85 @@ static gdws_status_t run_tiled(gdws_plan_s *p, const gdws_tensor_t *x, void *out
     P.nacc = P.acc_cols <= 256 ? 2 : 1;
     P.a_kmajor = zout ? 1 : p->opt_a_layout;
     P.zout = zout ? 1 : 0;
-    const size_t smem = t.smem;     // one block per SM (register file), so the TMEM columns are never oversubscribed
-    const int grid = nsplit > 1 ? P.ntiles * nsplit : (P.ntiles < p->sm_count ? P.ntiles : p->sm_count);
+    // one block per SM (register file), so the TMEM columns are never oversubscribed
+    L->grid = nsplit > 1 ? P.ntiles * nsplit : (P.ntiles < p->sm_count ? P.ntiles : p->sm_count);
     const int dev = p->device;
-    gdws_status_t rc;
-    if (t.fast == 1 && p->k == 3 && p->stride == 1) rc = launch_fast<3, 1, 1>(P, dev, grid, smem, st);
-    else if (t.fast == 1 && p->k == 3 && p->stride == 2) rc = launch_fast<3, 1, 2>(P, dev, grid, smem, st);
-    else if (t.fast == 1 && p->k == 5 && p->stride == 1) rc = launch_fast<5, 1, 1>(P, dev, grid, smem, st);
-    else if (t.fast == 1 && p->k == 5 && p->stride == 2) rc = launch_fast<5, 1, 2>(P, dev, grid, smem, st);
-    else if (t.fast == 2 && p->stride == 1) rc = launch_fast<3, 2, 1>(P, dev, grid, smem, st);
-    else if (t.fast == 2 && p->stride == 2) rc = launch_fast<3, 2, 2>(P, dev, grid, smem, st);
+    if (t.fast == 1 && p->k == 3 && p->stride == 1) return kernel_fast<3, 1, 1>(P, dev, &L->kernel);
+    else if (t.fast == 1 && p->k == 3 && p->stride == 2) return kernel_fast<3, 1, 2>(P, dev, &L->kernel);
+    else if (t.fast == 1 && p->k == 5 && p->stride == 1) return kernel_fast<5, 1, 1>(P, dev, &L->kernel);
+    else if (t.fast == 1 && p->k == 5 && p->stride == 2) return kernel_fast<5, 1, 2>(P, dev, &L->kernel);
+    else if (t.fast == 2 && p->stride == 1) return kernel_fast<3, 2, 1>(P, dev, &L->kernel);
+    else if (t.fast == 2 && p->stride == 2) return kernel_fast<3, 2, 2>(P, dev, &L->kernel);
     else {
         switch (p->k) {
-        case 1: rc = launch_fused<1, 0, 1, 0>(P, dev, grid, smem, st); break;
-        case 2: rc = launch_fused<2, 0, 1, 0>(P, dev, grid, smem, st); break;
-        case 3: rc = launch_fused<3, 0, 1, 0>(P, dev, grid, smem, st); break;
-        case 4: rc = launch_fused<4, 0, 1, 0>(P, dev, grid, smem, st); break;
-        case 5: rc = launch_fused<5, 0, 1, 0>(P, dev, grid, smem, st); break;
-        case 6: rc = launch_fused<6, 0, 1, 0>(P, dev, grid, smem, st); break;
-        case 7: rc = launch_fused<7, 0, 1, 0>(P, dev, grid, smem, st); break;
+        case 1: return kernel_fused<1, 0, 1, 0>(P, dev, &L->kernel);
+        case 2: return kernel_fused<2, 0, 1, 0>(P, dev, &L->kernel);
+        case 3: return kernel_fused<3, 0, 1, 0>(P, dev, &L->kernel);
+        case 4: return kernel_fused<4, 0, 1, 0>(P, dev, &L->kernel);
+        case 5: return kernel_fused<5, 0, 1, 0>(P, dev, &L->kernel);
+        case 6: return kernel_fused<6, 0, 1, 0>(P, dev, &L->kernel);
+        case 7: return kernel_fused<7, 0, 1, 0>(P, dev, &L->kernel);
         default: return fail(GDWS_ERR_UNSUPPORTED, "k=%d", p->k);
         }
     }
-    if (rc == GDWS_OK) p->launches++;
-    return rc;
+}
+
+// x as a rank-4 tensor, innermost first: channels, width, height, batch
+static gdws_status_t alu_map_x(const gdws_plan_s *p, const gdws_tensor_t *x, AluLaunch *L)
+{
+    tensor_map_encode_fn encode = encode_fn();
+    if (!encode) return fail(GDWS_ERR_CUDA, "cuTensorMapEncodeTiled is not available from this driver");
+    const Tile &t = L->t;
+    const cuuint64_t dims[4] = {(cuuint64_t)p->C, (cuuint64_t)x->w, (cuuint64_t)x->h, (cuuint64_t)x->n};
+    const cuuint64_t strides[3] = {(cuuint64_t)p->C * 2, (cuuint64_t)x->w * p->C * 2, (cuuint64_t)x->h * x->w * p->C * 2};
+    const cuuint32_t box[4] = {(cuuint32_t)t.cbox, (cuuint32_t)t.IW, (cuuint32_t)t.IH, (cuuint32_t)t.TN};
+    const cuuint32_t estr[4] = {1, 1, 1, 1};
+    const CUresult r = encode(&L->P.tmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, x->ptr, dims, strides, box, estr,
+                              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                              CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) return fail(GDWS_ERR_CUDA, "cuTensorMapEncodeTiled failed with code %d", (int)r);
+    L->x = x->ptr;
+    return GDWS_OK;
+}
+
+// y as a rank-4 tensor, innermost first: channels, width, height, batch (where the epilogue stores by TMA)
+static gdws_status_t alu_map_y(const gdws_plan_s *p, void *out, int n, int Ho, int Wo, AluLaunch *L)
+{
+    L->P.y = (uint16_t *)out;
+    if (L->P.ostage) {
+        const Tile &t = L->t;
+        const cuuint64_t dims[4] = {(cuuint64_t)p->D, (cuuint64_t)Wo, (cuuint64_t)Ho, (cuuint64_t)n};
+        const cuuint64_t strides[3] = {(cuuint64_t)p->D * 2, (cuuint64_t)Wo * p->D * 2, (cuuint64_t)Ho * Wo * p->D * 2};
+        const cuuint32_t box[4] = {64, (cuuint32_t)t.PW, (cuuint32_t)t.PH, (cuuint32_t)t.TN};
+        const cuuint32_t estr[4] = {1, 1, 1, 1};
+        const CUresult r = encode_fn()(&L->P.tmap_y, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, out, dims, strides, box, estr,
+                                       CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                                       CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+        if (r != CUDA_SUCCESS) return fail(GDWS_ERR_CUDA, "cuTensorMapEncodeTiled (y) failed with code %d", (int)r);
+    }
+    L->out = out;
+    return GDWS_OK;
+}
+
+static gdws_status_t run_tiled(gdws_plan_s *p, const gdws_tensor_t *x, void *out, int Ho, int Wo, bool zout, bool out_f32, cudaStream_t st)
+{
+    const LaunchKey key = {x->n, x->h, x->w, (p->opt_relu ? 1 : 0) | (out_f32 ? 2 : 0) | (zout ? 4 : 0) | (p->opt_a_layout ? 8 : 0) | (p->opt_tile << 4)};
+    gdws_status_t rc;
+    AluLaunch *L = LaunchCache<AluLaunch>::find(p->launch_cache[0], key);
+    if (!L) {
+        std::unique_ptr<AluLaunch> e(new (std::nothrow) AluLaunch);
+        if (!e) return fail(GDWS_ERR_ALLOC, "out of host memory");
+        e->key = key;
+        rc = alu_prepare(p, x->n, x->h, x->w, Ho, Wo, zout, out_f32, e.get());
+        if (rc != GDWS_OK) return rc;
+        L = LaunchCache<AluLaunch>::add(p->launch_cache[0], std::move(e));
+    }
+    if (L->x != x->ptr && (rc = alu_map_x(p, x, L)) != GDWS_OK) return rc;
+    if (L->out != out && (rc = alu_map_y(p, out, x->n, Ho, Wo, L)) != GDWS_OK) return rc;
+    const cudaError_t e = launch_overlapped(L->kernel, (unsigned)L->grid, kFusedThreads, L->t.smem, st, L->P);
+    if (e != cudaSuccess) { cudaGetLastError(); return cuda_fail(e, "fused_bf16_kernel launch"); }
+    p->launches++;
+    return GDWS_OK;
 }
 
 gdws_status_t bf16_fused(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t *y, cudaStream_t st)

@@ -638,60 +638,6 @@ __global__ void __launch_bounds__(kTcThreads, 1) fused_tc_kernel(const __grid_co
 }
 
 // ------------------------------------------------------------------------------------------
-// Weight packing
-// ------------------------------------------------------------------------------------------
-__device__ __forceinline__ float tc_load_weight(const void *w, size_t idx, int is_bf16)
-{
-    return is_bf16 ? bf16_bits_to_float(((const uint16_t *)w)[idx]) : ((const float *)w)[idx];
-}
-
-// dw_w[G][k][k] -> one record per intermediate slot: the slot's channel inside its 16-channel window
-// (0xFFFF for the padding slots of a chunk), then the k*k taps as bf16.
-__global__ void tc_pack_filt_kernel(const void *__restrict__ dw, int is_bf16, int k2, int rec_hw, const TcChunk *__restrict__ chunks,
-                                    const int32_t *__restrict__ chan, uint16_t *__restrict__ out)
-{
-    const TcChunk ch = chunks[blockIdx.x];
-    for (int e = threadIdx.x; e < ch.npad * rec_hw; e += blockDim.x) {
-        const int t = e / rec_hw, h = e - t * rec_hw;
-        uint16_t val = 0;
-        if (h == 0) val = t < ch.n ? (uint16_t)(chan[ch.i0 + t] - ch.cbase) : (uint16_t)0xFFFFu;
-        else if (h <= k2 && t < ch.n) val = float_to_bf16_bits(tc_load_weight(dw, (size_t)(ch.i0 + t) * k2 + (h - 1), is_bf16));
-        out[((size_t)ch.slab0 * 16 + t) * rec_hw + h] = val;
-    }
-}
-
-// pw_w[D][G] -> [part][slab][output channel][16] bf16: per 16 intermediate slots one K-major operand slab of the
-// pointwise product, 32 bytes per output channel, 32-byte swizzle.
-__global__ void tc_pack_pw_kernel(const void *__restrict__ pw, int is_bf16, int D, int G, int Dloc, int nslabs,
-                                  const TcChunk *__restrict__ chunks, uint16_t *__restrict__ out)
-{
-    const TcChunk ch = chunks[blockIdx.x];
-    const int part = blockIdx.y;
-    const int per_slab = 16 * Dloc;
-    for (int e = threadIdx.x; e < (ch.npad >> 4) * per_slab; e += blockDim.x) {
-        const int s = e / per_slab;
-        int rem = e - s * per_slab;
-        const int dl = rem >> 4, kk = rem & 15;
-        const int t = s * 16 + kk, d = part * Dloc + dl;
-        float val = 0.f;
-        if (t < ch.n && d < D) val = tc_load_weight(pw, (size_t)d * G + ch.i0 + t, is_bf16);
-        // row dl of the slab: 32 bytes, its two 16-byte halves swapped in rows 4..7 of every 8 (32-byte swizzle)
-        out[((size_t)part * nslabs + ch.slab0 + s) * per_slab + dl * 16 + ((((kk >> 3) ^ ((dl >> 2) & 1))) << 3) + (kk & 7)] =
-            float_to_bf16_bits(val);
-    }
-}
-
-void tc_pack(gdws_plan_s *p, const void *dw_w, const void *pw_w, int is_bf16, cudaStream_t st)
-{
-    if (!p->tc_ok) return;
-    const int nch = (int)p->tc_chunks.size();
-    tc_pack_filt_kernel<<<nch, 256, 0, st>>>(dw_w, is_bf16, p->k * p->k, p->tc_rec_hw, p->d_tc_chunks, p->d_chan, p->d_tc_filt);
-    tc_pack_pw_kernel<<<dim3(nch, p->tc_nparts), 256, 0, st>>>(pw_w, is_bf16, p->D, p->G, p->tc_dloc, p->tc_nslabs, p->d_tc_chunks,
-                                                            p->d_tc_pw);
-    p->launches += 2;
-}
-
-// ------------------------------------------------------------------------------------------
 // Host side
 // ------------------------------------------------------------------------------------------
 namespace {

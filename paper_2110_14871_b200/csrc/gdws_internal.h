@@ -99,7 +99,8 @@ struct gdws_plan_s {
     int opt_dw_math = 0;
     int opt_out_f32 = 0;           // bf16 plans: y is fp32
 
-    // device side (allocated by ensure_device)
+    // device side: one allocation (ensure_device), the pointers below lie in it
+    void *d_arena = nullptr;
     int device = -1;
     int sm_count = 0;              // SMs of the plan's device (grid size of the persistent kernel)
     bool arch_ok = false;          // the plan's device was checked to be compute capability 10.x
@@ -215,20 +216,20 @@ gdws_status_t f32_pointwise(gdws_plan_s *p, const float *z, const float *pw_w, c
 gdws_status_t f32_fused(gdws_plan_s *p, const gdws_tensor_t *x, const float *dw_w, const float *pw_w,
                         const float *bias, gdws_tensor_t *y, cudaStream_t s);
 
-// bf16.cu
+// pack.cu
 gdws_status_t bf16_pack(gdws_plan_s *p, const void *dw_w, const void *pw_w, const float *bias,
                         gdws_dtype_t dtype, cudaStream_t s);
+
+// bf16.cu
 gdws_status_t bf16_depthwise(gdws_plan_s *p, const gdws_tensor_t *x, void *z, cudaStream_t s);
 gdws_status_t bf16_pointwise(gdws_plan_s *p, const void *z, gdws_tensor_t *y, cudaStream_t s);
 gdws_status_t bf16_fused(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t *y, cudaStream_t s);
 gdws_status_t bf16_depthwise_tiled(gdws_plan_s *p, const gdws_tensor_t *x, void *z, cudaStream_t s);
 
 // fused_tc.cu
-void tc_pack(gdws_plan_s *p, const void *dw_w, const void *pw_w, int is_bf16, cudaStream_t s);
 gdws_status_t bf16_fused_tc(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t *y, cudaStream_t s);
 
 // fold.cu
-void fold_pack(gdws_plan_s *p, const void *dw_w, const void *pw_w, int is_bf16, cudaStream_t s);
 gdws_status_t bf16_folded(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t *y, cudaStream_t s);
 int bf16_form_of(gdws_plan_s *p, int n, int h, int w, bool out_f32);   // 1 / 2: two stages, GDW on the ALUs / the tensor cores; 3: folded
 

@@ -57,18 +57,14 @@ static void free_device(gdws_plan_s *p)
     cudaDeviceSynchronize();
     // every pointer is cleared as it is freed: a plan that outlives a failed set-up is set up again from scratch
     auto release = [](auto *&ptr) { cudaFree(ptr); ptr = nullptr; };
-    release(p->d_off);
-    release(p->d_chan);
-    release(p->d_chunk_meta);
-    release(p->d_dw);
-    release(p->d_dwpack);
-    release(p->d_pw_img);
-    release(p->d_bias);
-    release(p->d_status);
-    release(p->d_tc_chunks);
-    release(p->d_tc_filt);
-    release(p->d_tc_pw);
-    release(p->d_fold);
+    release(p->d_arena);
+    p->d_off = p->d_chan = p->d_chunk_meta = nullptr;
+    p->d_dw = p->d_bias = nullptr;
+    p->d_dwpack = nullptr;
+    p->d_pw_img = p->d_tc_filt = p->d_tc_pw = p->d_fold = nullptr;
+    p->d_tc_chunks = nullptr;
+    p->d_status = nullptr;
+    for (auto &c : p->launch_cache) c.reset();     // prepared launches hold the pointers
     release(p->stage_x);
     release(p->stage_y);
     p->stage_x_bytes = 0;
@@ -85,42 +81,49 @@ gdws_status_t ensure_device(gdws_plan_s *p)
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return cuda_fail(e, "cudaGetDevice");
     const size_t k2 = (size_t)p->k * p->k;
-    const size_t img = (size_t)p->nchunks * p->Dpad * kChunk * sizeof(uint16_t);
-#define GDWS_TRY_ALLOC(ptr, bytes)                                                   \
-    do {                                                                             \
-        e = cudaMalloc((void **)&(ptr), (bytes));                                    \
-        if (e != cudaSuccess) {                                                      \
-            p->device = dev;                                                         \
-            free_device(p);                                                          \
-            cudaGetLastError();                                                      \
-            return fail(GDWS_ERR_ALLOC, "cudaMalloc(%zu) failed: %s", (size_t)(bytes), cudaGetErrorString(e)); \
-        }                                                                            \
-    } while (0)
-    GDWS_TRY_ALLOC(p->d_off, sizeof(int32_t) * (p->C + 1));
-    GDWS_TRY_ALLOC(p->d_chan, sizeof(int32_t) * p->Gpad);
-    GDWS_TRY_ALLOC(p->d_chunk_meta, sizeof(int32_t) * 4 * p->nchunks);
-    GDWS_TRY_ALLOC(p->d_dw, sizeof(float) * p->Gpad * k2);
-    GDWS_TRY_ALLOC(p->d_dwpack, sizeof(uint32_t) * p->Gpad * p->wstride);
-    GDWS_TRY_ALLOC(p->d_pw_img, img);
-    GDWS_TRY_ALLOC(p->d_bias, sizeof(float) * p->Dpad);
-    GDWS_TRY_ALLOC(p->d_status, sizeof(int));
-    if (p->tc_ok) {
-        GDWS_TRY_ALLOC(p->d_tc_chunks, sizeof(TcChunk) * p->tc_chunks.size());
-        GDWS_TRY_ALLOC(p->d_tc_filt, sizeof(uint16_t) * (size_t)p->tc_nslabs * 16 * p->tc_rec_hw);
-        GDWS_TRY_ALLOC(p->d_tc_pw, sizeof(uint16_t) * (size_t)p->tc_nparts * p->tc_nslabs * 16 * p->tc_dloc);
+    // One allocation and one upload: the tables the host fills first (with the zeroed bias and status word), then what
+    // gdws_pack_weights fills.  (A dozen allocations, copies and memsets took most of a plan's set-up time.)
+    size_t bytes = 0;
+    std::vector<std::pair<void **, size_t>> places;
+    auto place = [&](auto *&ptr, size_t n) {
+        places.emplace_back((void **)&ptr, bytes);
+        bytes += (n + 255) / 256 * 256;
+    };
+    std::vector<uint8_t> tables;
+    try {
+        place(p->d_off, sizeof(int32_t) * (p->C + 1));
+        place(p->d_chan, sizeof(int32_t) * p->Gpad);
+        place(p->d_chunk_meta, sizeof(int32_t) * 4 * p->nchunks);
+        if (p->tc_ok) place(p->d_tc_chunks, sizeof(TcChunk) * p->tc_chunks.size());
+        place(p->d_bias, sizeof(float) * p->Dpad);
+        place(p->d_status, sizeof(int));
+        tables.assign(bytes, 0);
+        auto fill = [&](size_t i, const void *src, size_t n) { memcpy(tables.data() + places[i].second, src, n); };
+        fill(0, p->off.data(), sizeof(int32_t) * (p->C + 1));
+        fill(1, p->chan.data(), sizeof(int32_t) * p->Gpad);
+        fill(2, p->chunk_meta.data(), sizeof(int32_t) * 4 * p->nchunks);
+        if (p->tc_ok) fill(3, p->tc_chunks.data(), sizeof(TcChunk) * p->tc_chunks.size());
+        place(p->d_dw, sizeof(float) * p->Gpad * k2);
+        place(p->d_dwpack, sizeof(uint32_t) * p->Gpad * p->wstride);
+        place(p->d_pw_img, (size_t)p->nchunks * p->Dpad * kChunk * sizeof(uint16_t));
+        if (p->tc_ok) {
+            place(p->d_tc_filt, sizeof(uint16_t) * (size_t)p->tc_nslabs * 16 * p->tc_rec_hw);
+            place(p->d_tc_pw, sizeof(uint16_t) * (size_t)p->tc_nparts * p->tc_nslabs * 16 * p->tc_dloc);
+        }
+        if (p->fold_ok) place(p->d_fold, sizeof(uint16_t) * (size_t)p->fold_nwin * k2 * p->fold_dp * 64);
+    } catch (...) {
+        return fail(GDWS_ERR_ALLOC, "out of host memory");
     }
-    if (p->fold_ok) GDWS_TRY_ALLOC(p->d_fold, sizeof(uint16_t) * (size_t)p->fold_nwin * k2 * p->fold_dp * 64);
-#undef GDWS_TRY_ALLOC
+    e = cudaMalloc(&p->d_arena, bytes);
+    if (e != cudaSuccess) {
+        p->d_arena = nullptr;
+        cudaGetLastError();
+        return fail(GDWS_ERR_ALLOC, "cudaMalloc(%zu) failed: %s", bytes, cudaGetErrorString(e));
+    }
+    for (auto &pl : places) *pl.first = (uint8_t *)p->d_arena + pl.second;
     p->device = dev;
     if (cudaDeviceGetAttribute(&p->sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) p->sm_count = 0;
-    e = cudaMemcpy(p->d_off, p->off.data(), sizeof(int32_t) * (p->C + 1), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(p->d_chan, p->chan.data(), sizeof(int32_t) * p->Gpad, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess)
-        e = cudaMemcpy(p->d_chunk_meta, p->chunk_meta.data(), sizeof(int32_t) * 4 * p->nchunks, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && p->tc_ok)
-        e = cudaMemcpy(p->d_tc_chunks, p->tc_chunks.data(), sizeof(TcChunk) * p->tc_chunks.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemset(p->d_status, 0, sizeof(int));
-    if (e == cudaSuccess) e = cudaMemset(p->d_bias, 0, sizeof(float) * p->Dpad);
+    e = cudaMemcpy(p->d_arena, tables.data(), tables.size(), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
         free_device(p);
         return cuda_fail(e, "plan table upload");
