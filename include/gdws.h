@@ -228,8 +228,10 @@ GDWS_API gdws_status_t gdws_pointwise(gdws_plan_t *plan, const void *z, const vo
 
 /*
  * gdws_forward_host -- the same forward with HOST activations: copies x_host to the
- * device, runs gdws_forward with the packed weights, copies y back, all on `stream`,
- * then waits for the stream.  x_host / y_host: HOST, same dtype/layout rules as
+ * device, runs gdws_forward with the packed weights, copies y back, after what is on `stream`,
+ * and waits for it all.  Large pinned batches go through in pieces of whole images whose copies
+ * overlap with each other's forward (on two streams of the plan beside `stream`); the kernel
+ * is then the one that fits a piece (gdws_plan_form).  x_host / y_host: HOST, same dtype/layout rules as
  * gdws_forward (pinned memory makes the copies asynchronous with respect to the host).
  * The plan keeps device staging buffers that grow (cudaMalloc) when a call needs more
  * than any earlier one; weights must have been packed (bf16) or be passed (f32).

@@ -17,6 +17,7 @@ namespace gdws {
 constexpr int kChunk = 64;          // intermediate channels per tensor-core K chunk (one 128-byte swizzle row of bf16)
 constexpr int kTileRows = 128;      // output pixels per tensor-core tile (UMMA M)
 constexpr int kMaxK = 7;
+constexpr int kHostPieces = 8;      // pieces that gdws_forward_host overlaps
 constexpr int kMaxSmem = 225 * 1024;      // dynamic shared memory a block may ask for (227 KB minus static use)
 
 // Bits of the device status word.
@@ -123,6 +124,8 @@ struct gdws_plan_s {
 
     void *stage_x = nullptr, *stage_y = nullptr;  // gdws_forward_host staging
     size_t stage_x_bytes = 0, stage_y_bytes = 0;
+    cudaStream_t copy_in = nullptr, copy_out = nullptr;        // its copies, where they overlap (created by the first such call)
+    cudaEvent_t copy_events[2 * gdws::kHostPieces + 1] = {};   // per piece: copied in, computed; then: where the call began
 
     // Prepared launches of the three fused bf16 kernels and the choice between them (LaunchCache below; each file knows its
     // own types).
@@ -138,6 +141,7 @@ gdws_status_t fail(gdws_status_t st, const char *fmt, ...);
 gdws_status_t cuda_fail(cudaError_t e, const char *what);
 gdws_status_t ensure_device(gdws_plan_s *p);   // allocate device tables on the current device
 gdws_status_t check_arch();
+void free_host_pipeline(gdws_plan_s *p);       // streams and events of gdws_forward_host
 
 // Launch with programmatic stream serialisation: the kernel may be scheduled while the kernel before it in the stream
 // is still running (once all blocks of that one have executed griddepcontrol.launch_dependents, which the library's

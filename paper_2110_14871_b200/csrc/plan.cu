@@ -48,6 +48,17 @@ gdws_status_t check_arch()
     return GDWS_OK;
 }
 
+void free_host_pipeline(gdws_plan_s *p)
+{
+    if (p->copy_in) cudaStreamDestroy(p->copy_in);
+    if (p->copy_out) cudaStreamDestroy(p->copy_out);
+    p->copy_in = p->copy_out = nullptr;
+    for (cudaEvent_t &ev : p->copy_events) {
+        if (ev) cudaEventDestroy(ev);
+        ev = nullptr;
+    }
+}
+
 static void free_device(gdws_plan_s *p)
 {
     if (p->device < 0) return;
@@ -65,6 +76,7 @@ static void free_device(gdws_plan_s *p)
     p->d_tc_chunks = nullptr;
     p->d_status = nullptr;
     for (auto &c : p->launch_cache) c.reset();     // prepared launches hold the pointers
+    free_host_pipeline(p);
     release(p->stage_x);
     release(p->stage_y);
     p->stage_x_bytes = 0;

@@ -10,6 +10,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 from typing import Optional, Sequence, Tuple
 
 import numpy as np
@@ -44,6 +45,9 @@ class Tensor(ctypes.Structure):
                 ("n", ctypes.c_int), ("c", ctypes.c_int), ("h", ctypes.c_int), ("w", ctypes.c_int)]
 
 
+_PACK_TENSOR = struct.Struct("@P6i").pack_into      # the fields of gdws_tensor_t in one call
+assert struct.calcsize("@P6i") == ctypes.sizeof(Tensor)
+
 _lib = None
 
 
@@ -61,7 +65,6 @@ def lib() -> ctypes.CDLL:
     pi32 = ctypes.POINTER(ctypes.c_int32)
     pint = ctypes.POINTER(ctypes.c_int)
     pi64 = ctypes.POINTER(ctypes.c_int64)
-    pt = ctypes.POINTER(Tensor)
     L.gdws_plan.argtypes = [ci, ci, ci, ci, ci, pi32, ctypes.POINTER(vp)]
     L.gdws_plan.restype = ci
     L.gdws_plan_set_option.argtypes = [vp, ci, ci]
@@ -84,15 +87,15 @@ def lib() -> ctypes.CDLL:
     L.gdws_workspace_bytes.restype = ctypes.c_size_t
     L.gdws_set_workspace.argtypes = [vp, vp, ctypes.c_size_t]
     L.gdws_set_workspace.restype = ci
-    L.gdws_forward.argtypes = [vp, pt, vp, vp, vp, pt, vp]
+    L.gdws_forward.argtypes = [vp] * 7
     L.gdws_forward.restype = ci
-    L.gdws_depthwise.argtypes = [vp, pt, vp, vp, vp]
+    L.gdws_depthwise.argtypes = [vp] * 5
     L.gdws_depthwise.restype = ci
-    L.gdws_pointwise.argtypes = [vp, vp, vp, vp, pt, vp]
+    L.gdws_pointwise.argtypes = [vp] * 6
     L.gdws_pointwise.restype = ci
-    L.gdws_forward_host.argtypes = [vp, pt, vp, vp, vp, pt, vp]
+    L.gdws_forward_host.argtypes = [vp] * 7
     L.gdws_forward_host.restype = ci
-    L.gdws_forward_static.argtypes = [vp, pt, vp, vp, vp, pt, vp]
+    L.gdws_forward_static.argtypes = [vp] * 7
     L.gdws_forward_static.restype = ci
     L.gdws_static_scratch_bytes.argtypes = []
     L.gdws_static_scratch_bytes.restype = ctypes.c_size_t
@@ -154,13 +157,19 @@ def _check(status: int) -> None:
         raise GdwsError(status, last_error())
 
 
+_dtypes = None      # torch dtype -> code
+_raw_stream = None  # once torch has initialised CUDA: its current stream of the current device, as an integer
+
+
 def _dtype_code(t) -> int:
-    import torch
-    if t.dtype == torch.float32:
-        return F32
-    if t.dtype == torch.bfloat16:
-        return BF16
-    raise TypeError(f"unsupported dtype {t.dtype}")
+    global _dtypes
+    if _dtypes is None:
+        import torch
+        _dtypes = {torch.float32: F32, torch.bfloat16: BF16}
+    code = _dtypes.get(t.dtype)
+    if code is None:
+        raise TypeError(f"unsupported dtype {t.dtype}")
+    return code
 
 
 def _ptr(t) -> Optional[int]:
@@ -168,27 +177,43 @@ def _ptr(t) -> Optional[int]:
 
 
 def _stream(stream) -> Optional[int]:
+    global _raw_stream
     if stream is None:
+        if _raw_stream is not None:
+            return _raw_stream()
         import torch
-        return torch.cuda.current_stream().cuda_stream if torch.cuda.is_available() else None
+        if not torch.cuda.is_available():
+            return None
+        raw, device = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+        if torch.cuda.is_initialized() and raw and device:
+            _raw_stream = lambda: raw(device())  # noqa: E731
+        return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
 
 
-def tensor_desc(t, layout: str) -> Tensor:
-    """gdws_tensor_t for a contiguous 4-D torch tensor stored in ``layout`` order."""
+_LAYOUTS = {"NCHW": NCHW, "NHWC": NHWC}
+
+
+def _fill_desc(d: Tensor, t, layout: str) -> None:
     if t.dim() != 4 or not t.is_contiguous():
         raise ValueError("expected a contiguous 4-D tensor")
-    if layout == "NCHW":
-        n, c, h, w = t.shape
-        code = NCHW
-    elif layout == "NHWC":
-        n, h, w, c = t.shape
-        code = NHWC
-    else:
+    code = _LAYOUTS.get(layout)
+    if code is None:
         raise ValueError(layout)
-    return Tensor(t.data_ptr(), _dtype_code(t), code, int(n), int(c), int(h), int(w))
+    if code == NCHW:
+        n, c, h, w = t.shape
+    else:
+        n, h, w, c = t.shape
+    _PACK_TENSOR(d, 0, t.data_ptr(), _dtype_code(t), code, n, c, h, w)
+
+
+def tensor_desc(t, layout: str) -> Tensor:
+    """gdws_tensor_t for a contiguous 4-D torch tensor stored in ``layout`` order."""
+    d = Tensor()
+    _fill_desc(d, t, layout)
+    return d
 
 
 class Plan:
@@ -204,7 +229,9 @@ class Plan:
         _check(st)
         self._h = handle
         self.C, self.D, self.k, self.stride, self.pad = C, D, k, stride, pad
-        self._keep = []
+        # descriptors of x and y, filled per call (a plan serves one host thread at a time)
+        self._xd, self._yd = Tensor(), Tensor()
+        self._xp, self._yp = ctypes.addressof(self._xd), ctypes.addressof(self._yd)
 
     # -- lifetime
     def destroy(self) -> None:
@@ -273,30 +300,32 @@ class Plan:
     def pack_weights(self, dw_w, pw_w, bias=None, stream=None) -> None:
         _check(lib().gdws_pack_weights(self._h, _ptr(dw_w), _ptr(pw_w), _ptr(bias), _dtype_code(dw_w), _stream(stream)))
 
+    def _call(self, fn, x, y, layout: str, dw_w, pw_w, bias, stream) -> None:
+        _fill_desc(self._xd, x, layout)
+        _fill_desc(self._yd, y, layout)
+        st = fn(self._h, self._xp, None if dw_w is None else dw_w.data_ptr(), None if pw_w is None else pw_w.data_ptr(),
+                None if bias is None else bias.data_ptr(), self._yp, _stream(stream))
+        if st:
+            raise GdwsError(st, last_error())
+
     def forward(self, x, y, layout: str, dw_w=None, pw_w=None, bias=None, stream=None) -> None:
-        xd, yd = tensor_desc(x, layout), tensor_desc(y, layout)
-        _check(lib().gdws_forward(self._h, ctypes.byref(xd), _ptr(dw_w), _ptr(pw_w), _ptr(bias), ctypes.byref(yd),
-                                  _stream(stream)))
+        self._call(_lib.gdws_forward, x, y, layout, dw_w, pw_w, bias, stream)
 
     def depthwise(self, x, z, layout: str, dw_w=None, stream=None) -> None:
-        xd = tensor_desc(x, layout)
-        _check(lib().gdws_depthwise(self._h, ctypes.byref(xd), _ptr(dw_w), z.data_ptr(), _stream(stream)))
+        _fill_desc(self._xd, x, layout)
+        _check(_lib.gdws_depthwise(self._h, self._xp, _ptr(dw_w), z.data_ptr(), _stream(stream)))
 
     def pointwise(self, z, y, layout: str, pw_w=None, bias=None, stream=None) -> None:
-        yd = tensor_desc(y, layout)
-        _check(lib().gdws_pointwise(self._h, z.data_ptr(), _ptr(pw_w), _ptr(bias), ctypes.byref(yd), _stream(stream)))
+        _fill_desc(self._yd, y, layout)
+        _check(_lib.gdws_pointwise(self._h, z.data_ptr(), _ptr(pw_w), _ptr(bias), self._yp, _stream(stream)))
 
     def forward_host(self, x_host, y_host, layout: str, dw_w=None, pw_w=None, bias=None, stream=None) -> None:
-        xd, yd = tensor_desc(x_host, layout), tensor_desc(y_host, layout)
-        _check(lib().gdws_forward_host(self._h, ctypes.byref(xd), _ptr(dw_w), _ptr(pw_w), _ptr(bias), ctypes.byref(yd),
-                                       _stream(stream)))
+        self._call(_lib.gdws_forward_host, x_host, y_host, layout, dw_w, pw_w, bias, stream)
 
     def forward_static(self, x, y, layout: str, dw_w=None, pw_w=None, bias=None, stream=None) -> None:
         """gdws_forward_static: the unfused forward with the intermediate in the library's built-in
         scratch array; for callers that must not allocate device memory."""
-        xd, yd = tensor_desc(x, layout), tensor_desc(y, layout)
-        _check(lib().gdws_forward_static(self._h, ctypes.byref(xd), _ptr(dw_w), _ptr(pw_w), _ptr(bias),
-                                         ctypes.byref(yd), _stream(stream)))
+        self._call(_lib.gdws_forward_static, x, y, layout, dw_w, pw_w, bias, stream)
 
     def status(self) -> None:
         _check(lib().gdws_status(self._h))

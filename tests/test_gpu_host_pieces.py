@@ -1,0 +1,37 @@
+"""gdws_forward_host with pinned batches large enough to go through in overlapping pieces: ragged piece sizes, images whose
+bytes are no multiple of 16, two calls in a row on the same buffers, weights passed with the call."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2110_14871_b200 import build as gbuild
+from paper_2110_14871_b200 import inputs as gi
+
+from util import TOL, make_plan, rel_err, run_oracle, small_spec, to_device
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    gbuild.build_library()
+
+
+@pytest.mark.parametrize("dtype,N,C,D,H,W", [("bf16", 61, 64, 64, 20, 20), ("bf16", 3, 128, 256, 40, 41), ("f32", 37, 13, 15, 31, 33)])
+def test_pieces_match_reference(dtype, N, C, D, H, W):
+    layout = "NHWC" if dtype == "bf16" else "NCHW"
+    spec = small_spec("t", N, C, D, H, W, 3, 1, 1, ("uniform", 1, 3), dtype, layout, seed=17)
+    data = gi.make_layer(spec)
+    ref, _ = run_oracle(data)
+    plan = make_plan(data)
+    dw, pw, b = to_device(data.dw_w, dtype), to_device(data.pw_w, dtype), torch.from_numpy(data.bias).cuda()
+    tdt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    x = torch.from_numpy(data.x).to(tdt).pin_memory()
+    y = torch.full(ref.shape, float("nan"), dtype=tdt).pin_memory()
+    for flip in (1.0, -1.0):                     # y is linear in x up to the bias: the second call sees other values
+        plan.forward_host(x if flip == 1.0 else (-x).pin_memory(), y, layout, dw, pw, b)
+        bias = data.bias.reshape((1, -1, 1, 1) if layout == "NCHW" else (1, 1, 1, -1)).astype(np.float64)
+        assert rel_err(y.float().numpy(), flip * (ref - bias) + bias) <= TOL[dtype]
+        y.fill_(float("nan"))
+    plan.status()
+    plan.destroy()
