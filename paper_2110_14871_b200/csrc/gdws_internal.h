@@ -17,7 +17,7 @@ namespace gdws {
 constexpr int kChunk = 64;          // intermediate channels per tensor-core K chunk (one 128-byte swizzle row of bf16)
 constexpr int kTileRows = 128;      // output pixels per tensor-core tile (UMMA M)
 constexpr int kMaxK = 7;
-constexpr int kHostPieces = 8;      // pieces that gdws_forward_host overlaps
+constexpr int kHostPieces = 5;      // pieces that gdws_forward_host overlaps
 constexpr int kMaxSmem = 225 * 1024;      // dynamic shared memory a block may ask for (227 KB minus static use)
 
 // Bits of the device status word.
@@ -102,6 +102,7 @@ struct gdws_plan_s {
 
     // device side: one allocation (ensure_device), the pointers below lie in it
     void *d_arena = nullptr;
+    size_t arena_bytes = 0;
     int device = -1;
     int sm_count = 0;              // SMs of the plan's device (grid size of the persistent kernel)
     bool arch_ok = false;          // the plan's device was checked to be compute capability 10.x
@@ -124,8 +125,6 @@ struct gdws_plan_s {
 
     void *stage_x = nullptr, *stage_y = nullptr;  // gdws_forward_host staging
     size_t stage_x_bytes = 0, stage_y_bytes = 0;
-    cudaStream_t copy_in = nullptr, copy_out = nullptr;        // its copies, where they overlap (created by the first such call)
-    cudaEvent_t copy_events[2 * gdws::kHostPieces + 1] = {};   // per piece: copied in, computed; then: where the call began
 
     // Prepared launches of the three fused bf16 kernels and the choice between them (LaunchCache below; each file knows its
     // own types).
@@ -141,7 +140,10 @@ gdws_status_t fail(gdws_status_t st, const char *fmt, ...);
 gdws_status_t cuda_fail(cudaError_t e, const char *what);
 gdws_status_t ensure_device(gdws_plan_s *p);   // allocate device tables on the current device
 gdws_status_t check_arch();
-void free_host_pipeline(gdws_plan_s *p);       // streams and events of gdws_forward_host
+// plan_mem.cu: memory of a plan's tables, on the current device
+cudaError_t plan_mem_alloc(int device, size_t bytes, void **out);
+void plan_mem_free(int device, void *ptr, size_t bytes);
+void plan_count(int device, int change);       // plans that hold memory of the device; the last one gives the shared things back
 
 // Launch with programmatic stream serialisation: the kernel may be scheduled while the kernel before it in the stream
 // is still running (once all blocks of that one have executed griddepcontrol.launch_dependents, which the library's
@@ -188,6 +190,15 @@ template <class Entry> struct LaunchCache {
         return v.back().get();
     }
 };
+// Two streams and the events that order the pieces of a gdws_forward_host call.  Creating them takes milliseconds: a call
+// borrows a set and gives it back (one more set per device for each call that runs at the same time, at most two kept).
+struct HostPipe {
+    int device = 0;
+    cudaStream_t in = nullptr, out = nullptr;
+    cudaEvent_t begin = nullptr, copied[kHostPieces] = {}, computed[kHostPieces] = {};
+};
+HostPipe *host_pipe_take(int device);       // null if it cannot be made; the device is current
+void host_pipe_give(HostPipe *p);           // its streams are idle
 // x and y of a forward call against the plan: pointers, alignment, extents, dtype/layout pair, no overlap
 gdws_status_t check_pair(const gdws_plan_s *p, const gdws_tensor_t *x, const gdws_tensor_t *y);
 // static_ws.cu: looks up (once per device, the device being current) the address of the built-in scratch array

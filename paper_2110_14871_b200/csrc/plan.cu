@@ -48,17 +48,6 @@ gdws_status_t check_arch()
     return GDWS_OK;
 }
 
-void free_host_pipeline(gdws_plan_s *p)
-{
-    if (p->copy_in) cudaStreamDestroy(p->copy_in);
-    if (p->copy_out) cudaStreamDestroy(p->copy_out);
-    p->copy_in = p->copy_out = nullptr;
-    for (cudaEvent_t &ev : p->copy_events) {
-        if (ev) cudaEventDestroy(ev);
-        ev = nullptr;
-    }
-}
-
 static void free_device(gdws_plan_s *p)
 {
     if (p->device < 0) return;
@@ -68,7 +57,8 @@ static void free_device(gdws_plan_s *p)
     cudaDeviceSynchronize();
     // every pointer is cleared as it is freed: a plan that outlives a failed set-up is set up again from scratch
     auto release = [](auto *&ptr) { cudaFree(ptr); ptr = nullptr; };
-    release(p->d_arena);
+    plan_mem_free(p->device, p->d_arena, p->arena_bytes);
+    p->d_arena = nullptr;
     p->d_off = p->d_chan = p->d_chunk_meta = nullptr;
     p->d_dw = p->d_bias = nullptr;
     p->d_dwpack = nullptr;
@@ -76,12 +66,12 @@ static void free_device(gdws_plan_s *p)
     p->d_tc_chunks = nullptr;
     p->d_status = nullptr;
     for (auto &c : p->launch_cache) c.reset();     // prepared launches hold the pointers
-    free_host_pipeline(p);
     release(p->stage_x);
     release(p->stage_y);
     p->stage_x_bytes = 0;
     p->stage_y_bytes = 0;
     p->packed = false;
+    plan_count(p->device, -1);
     cudaSetDevice(cur);
     p->device = -1;
 }
@@ -126,7 +116,8 @@ gdws_status_t ensure_device(gdws_plan_s *p)
     } catch (...) {
         return fail(GDWS_ERR_ALLOC, "out of host memory");
     }
-    e = cudaMalloc(&p->d_arena, bytes);
+    e = plan_mem_alloc(dev, bytes, &p->d_arena);
+    p->arena_bytes = bytes;
     if (e != cudaSuccess) {
         p->d_arena = nullptr;
         cudaGetLastError();
@@ -134,6 +125,7 @@ gdws_status_t ensure_device(gdws_plan_s *p)
     }
     for (auto &pl : places) *pl.first = (uint8_t *)p->d_arena + pl.second;
     p->device = dev;
+    plan_count(dev, 1);
     if (cudaDeviceGetAttribute(&p->sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) p->sm_count = 0;
     e = cudaMemcpy(p->d_arena, tables.data(), tables.size(), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {

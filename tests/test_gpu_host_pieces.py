@@ -17,7 +17,7 @@ def built():
     gbuild.build_library()
 
 
-@pytest.mark.parametrize("dtype,N,C,D,H,W", [("bf16", 61, 64, 64, 20, 20), ("bf16", 3, 128, 256, 40, 41), ("f32", 37, 13, 15, 31, 33)])
+@pytest.mark.parametrize("dtype,N,C,D,H,W", [("bf16", 61, 64, 64, 20, 20), ("bf16", 2, 128, 256, 80, 41), ("bf16", 90, 64, 64, 56, 54), ("f32", 53, 13, 15, 71, 63)])
 def test_pieces_match_reference(dtype, N, C, D, H, W):
     layout = "NHWC" if dtype == "bf16" else "NCHW"
     spec = small_spec("t", N, C, D, H, W, 3, 1, 1, ("uniform", 1, 3), dtype, layout, seed=17)
