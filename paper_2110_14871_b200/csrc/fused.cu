@@ -177,39 +177,41 @@ __device__ __forceinline__ void store_group(const FusedParams &P, uint32_t a_sta
 // chunk, so it is worked out once per kernel.  The thread owns up to four pixel groups (8 pixels each):
 // `in_off[m]` is where group m's input window starts inside a staged box (bytes, channel 0), `st_off[m]`
 // where its results go inside an operand stage, and bit m of `live` says whether the group has pixels.
-// In a pixel-contiguous stage a group's 8 results are one 16-byte piece at st_off[m]; in a channel-contiguous
-// stage (KMAJOR, the unfused GDW kernel) they are 8 two-byte elements in 8 consecutive 128-byte rows, each
-// in the 16-byte piece (kk/8) ^ (row & 7), and st_off[m] is the address of the first row's unswizzled piece 0.
+// In a pixel-contiguous stage a group's 8 results are one 16-byte piece at st_off[m].
 struct DwShare {
     uint32_t in_off[4];
     uint32_t st_off[4];
     uint32_t rowb;              // bytes per input row of the staged box
     uint32_t live;
-    uint32_t kg4;               // KMAJOR: 16 * (kk / 8)
 };
-template <bool KMAJOR>
-__device__ __forceinline__ uint32_t dw_st_off(int o, int kk)
+// The unfused GDW stage writes z itself: where the pixels of a thread's groups lie in z and which of them exist.
+// Neighbouring lanes own neighbouring channels, so a warp's two-byte stores of a pixel are 64 contiguous bytes.
+struct ZShare {
+    uint16_t *z;                // element of the thread's channel at the tile's first pixel of its first group
+    int gpad, Wo;
+    int rows, cols;             // rows / columns that exist, counted from there (0: none)
+};
+__device__ __forceinline__ void z_store8(uint16_t *z, int gpad, int ncols, const float (&v)[8])
 {
-    return KMAJOR ? (uint32_t)(o * 1024 + (kk & 7) * 2) : a_off_mn(o, kk);
-}
-template <bool KMAJOR>
-__device__ __forceinline__ void store_group_at(uint32_t addr, uint32_t kg4, const float (&v)[8])
-{
-    if (!KMAJOR) {
-        uint4 q;
-        q.x = pack_bf16x2(v[0], v[1]); q.y = pack_bf16x2(v[2], v[3]);
-        q.z = pack_bf16x2(v[4], v[5]); q.w = pack_bf16x2(v[6], v[7]);
-        sts128(addr, q);
-    } else {
 #pragma unroll
-        for (int e = 0; e < 8; ++e) sts16(addr + (uint32_t)(e * 128) + (kg4 ^ (uint32_t)(e << 4)), float_to_bf16_bits(v[e]));
+    for (int e = 0; e < 8; e += 2) {
+        const uint32_t w = pack_bf16x2(v[e], v[e + 1]);
+        if (e < ncols) z[(size_t)e * gpad] = (uint16_t)w;
+        if (e + 1 < ncols) z[(size_t)(e + 1) * gpad] = (uint16_t)(w >> 16);
     }
+}
+__device__ __forceinline__ void store_group_at(uint32_t addr, const float (&v)[8])
+{
+    uint4 q;
+    q.x = pack_bf16x2(v[0], v[1]); q.y = pack_bf16x2(v[2], v[3]);
+    q.z = pack_bf16x2(v[4], v[5]); q.w = pack_bf16x2(v[6], v[7]);
+    sts128(addr, q);
 }
 
 // ---- depthwise, k = 3 or 5, patches at least 8 wide: a thread computes 4 consecutive output rows of one
 // 8-pixel column group (its four pixel groups), reading each input row once and using it for up to K
 // output rows.
-template <int S, int PS, bool KMAJOR>
+template <int S, int PS>
 __device__ __forceinline__ DwShare dw_rows_share(const FusedParams &P, int kk, int run)
 {
     DwShare sh;
@@ -222,13 +224,12 @@ __device__ __forceinline__ DwShare dw_rows_share(const FusedParams &P, int kk, i
     sh.live = R0 < P.TN * P.PH ? 1u : 0u;
     sh.in_off[0] = (uint32_t)((tn * P.IH + ph0 * S) * P.IW + seg * 8 * S) * PS;
 #pragma unroll
-    for (int ro = 0; ro < 4; ++ro) sh.st_off[ro] = dw_st_off<KMAJOR>(o0 + ro * nseg, kk);
-    sh.kg4 = (uint32_t)(kk >> 3) << 4;
+    for (int ro = 0; ro < 4; ++ro) sh.st_off[ro] = a_off_mn(o0 + ro * nseg, kk);
     return sh;
 }
-template <int K, int S, int PS, bool KMAJOR>
+template <int K, int S, int PS, bool ZOUT>
 __device__ __forceinline__ void dw_rows(const DwShare &sh, uint32_t xs, int clb, const uint32_t (&w)[K * K], bool live_i,
-                                        uint32_t a_stage)
+                                        uint32_t a_stage, const ZShare &zs)
 {
     float acc[4][8];
     if (live_i && sh.live) {
@@ -262,11 +263,14 @@ __device__ __forceinline__ void dw_rows(const DwShare &sh, uint32_t xs, int clb,
             for (int e = 0; e < 8; ++e) acc[ro][e] = 0.f;
     }
 #pragma unroll
-    for (int ro = 0; ro < 4; ++ro) store_group_at<KMAJOR>(a_stage + sh.st_off[ro], sh.kg4, acc[ro]);
+    for (int ro = 0; ro < 4; ++ro) {
+        if (!ZOUT) store_group_at(a_stage + sh.st_off[ro], acc[ro]);
+        else if (ro < zs.rows) z_store8(zs.z + (size_t)ro * zs.Wo * zs.gpad, zs.gpad, zs.cols, acc[ro]);
+    }
 }
 
 // ---- depthwise, k = 3, 4-wide patches: a pixel group is 2 output rows x 4 columns of one image.
-template <int S, int PS, bool KMAJOR>
+template <int S, int PS>
 __device__ __forceinline__ DwShare dw_quads_share(const FusedParams &P, int kk, int run)
 {
     DwShare sh;
@@ -279,14 +283,13 @@ __device__ __forceinline__ DwShare dw_quads_share(const FusedParams &P, int kk, 
         const int tn = o / gpi, ph0 = (o - tn * gpi) * 2;
         if (tn < P.TN) sh.live |= 1u << m;
         sh.in_off[m] = (uint32_t)((tn * P.IH + ph0 * S) * P.IW) * PS;
-        sh.st_off[m] = dw_st_off<KMAJOR>(o, kk);
+        sh.st_off[m] = a_off_mn(o, kk);
     }
-    sh.kg4 = (uint32_t)(kk >> 3) << 4;
     return sh;
 }
-template <int S, int PS, bool KMAJOR>
+template <int S, int PS, bool ZOUT>
 __device__ __forceinline__ void dw_quads_k3(const DwShare &sh, uint32_t xs, int clb, const uint32_t (&w)[9], bool live_i,
-                                            uint32_t a_stage)
+                                            uint32_t a_stage, const FusedParams &P, uint16_t *z, int n0, int run, int ho0, int wo0)
 {
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
@@ -317,14 +320,26 @@ __device__ __forceinline__ void dw_quads_k3(const DwShare &sh, uint32_t xs, int 
 #pragma unroll
             for (int e = 0; e < 8; ++e) acc[e] = 0.f;
         }
-        store_group_at<KMAJOR>(a_stage + sh.st_off[m], sh.kg4, acc);
+        if (!ZOUT) {
+            store_group_at(a_stage + sh.st_off[m], acc);
+        } else {
+            const int gpi = P.PH >> 1, o = run * 4 + m, tn = o / gpi, ph0 = (o - tn * gpi) * 2;
+#pragma unroll
+            for (int ro = 0; ro < 2; ++ro)
+                if (((sh.live >> m) & 1u) && n0 + tn < P.N && ho0 + ph0 + ro < P.Ho) {
+                    uint16_t *zr = z + (((size_t)(n0 + tn) * P.Ho + ho0 + ph0 + ro) * P.Wo + wo0) * P.Dtot;
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        if (wo0 + e < P.Wo) zr[(size_t)e * P.Dtot] = float_to_bf16_bits(acc[ro * 4 + e]);
+                }
+        }
     }
 }
 
 // ---- depthwise, any k and stride: one pixel group at a time.
-template <int K>
+template <int K, bool ZOUT>
 __device__ __forceinline__ void dw_generic(const FusedParams &P, uint32_t xs, int clb, uint32_t wsm, int kk,
-                                           int run, bool live_i, uint32_t a_stage)
+                                           int run, bool live_i, uint32_t a_stage, uint16_t *z, int n0, int ho0, int wo0)
 {
     const int hw = P.PH * P.PW;
 #pragma unroll 1
@@ -353,7 +368,16 @@ __device__ __forceinline__ void dw_generic(const FusedParams &P, uint32_t xs, in
                 out[e] = acc;
             }
         }
-        store_group(P, a_stage, o, kk, out);
+        if (!ZOUT) {
+            store_group(P, a_stage, o, kk, out);
+        } else {
+#pragma unroll 1
+            for (int e = 0; e < 8; ++e) {
+                const int r = r0 + e, t2 = r / hw, rem = r - t2 * hw, ph = rem / P.PW, n = n0 + t2, ho = ho0 + ph, wo = wo0 + rem - ph * P.PW;
+                if (t2 < P.TN && n < P.N && ho < P.Ho && wo < P.Wo)
+                    z[(((size_t)n * P.Ho + ho) * P.Wo + wo) * P.Dtot] = float_to_bf16_bits(out[e]);
+            }
+        }
     }
 }
 
@@ -383,10 +407,10 @@ __device__ __forceinline__ void epilogue_row(const FusedParams &P, uint32_t t_ba
 
 // MODE: 0 generic, 1 row runs (k=3), 2 4-wide patches (k=3); S = stride and PS = bytes per staged
 // pixel for modes 1/2 (mode 0 reads both from the parameters).
-// ZOUT = true turns the kernel into the unfused GDW stage: the depthwise warps write channel-contiguous
-// stages and the four "epilogue" warps copy each finished stage to z[pixel][Gpad] in global memory
-// (16-byte stores, 128 contiguous bytes per pixel and chunk); no weights are streamed, no MMA is issued
-// and no TMEM is used.  P.y then points to z and P.D holds Gpad.
+// ZOUT = true turns the kernel into the unfused GDW stage: the depthwise warps write z[pixel][Gpad] in global memory from
+// their registers; no weights are streamed, no MMA is issued, no TMEM and no operand stages are used, and the control and
+// epilogue warps other than the input loader and the gate warp have nothing to do.  P.y then points to z and P.Dtot holds
+// Gpad.  (z through operand stages and a second set of warps: 58 us for 64 -> G = 189 channels, 64 x 56 x 56.)
 // VAR: 0 the fused kernel, 1 ZOUT, 2 the fused kernel with several blocks per tile (P.nsplit > 1).
 template <int K, int MODE, int S, int PS, int VAR>
 __global__ void __launch_bounds__(kFusedThreads, 1) fused_bf16_kernel(const __grid_constant__ FusedParams P)
@@ -408,7 +432,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) fused_bf16_kernel(const __gr
     (void)part; (void)bid; (void)nblocks
     uint8_t *base = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const uint32_t a_s = smem_u32(base);
-    const uint32_t o_s = a_s + (32768u << P.spg_shift);   // after the one or two operand stages per depthwise group: output staging
+    const uint32_t o_s = a_s + (ZOUT ? 0u : 32768u << P.spg_shift);   // after the one or two operand stages per depthwise group: output staging
     const uint32_t b_s = o_s + (uint32_t)P.ostage;
     const uint32_t x_s = b_s + (uint32_t)P.nsb * P.unit_bytes;
     const uint32_t bar_afree = smem_u32(&bars[0]);
@@ -432,7 +456,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) fused_bf16_kernel(const __gr
         const int i = tid - 32;
         if (i >= 0 && i < 8) {
             if (i < 4) {
-                mbar_init(bar_afree + 8 * i, ZOUT ? kEpiWarps : 1);
+                mbar_init(bar_afree + 8 * i, 1);
                 mbar_init(bar_open + 8 * i, 1);
             }
             if (i < 2) {
@@ -608,7 +632,9 @@ __global__ void __launch_bounds__(kFusedThreads, 1) fused_bf16_kernel(const __gr
             // is free again, then completes a phase of the group's "open" barrier (two per group, alternating).
             // Each depthwise warp checks that one barrier before a chunk, on its own: the warps of a group do
             // not wait for one another.  An "open" barrier is used again two chunks of the group later; by then
-            // the stage wait has shown that every warp of the group is past its earlier use.
+            // the stage wait has shown that every warp of the group is past its earlier use.  (ZOUT: the ring of filter
+            // blocks is exactly four long, so that this chunk's filters land only after the group released those of its
+            // chunk before last.)
             uint32_t wslot = 0, wpar = 0;
             uint32_t xs_cur = 0, xp_cur = 0, xs_next = 0, xp_next = 0;   // box slot and the parity of its "full" phase
             int gq = 0;
@@ -622,7 +648,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) fused_bf16_kernel(const __gr
                         if (++xs_next == (uint32_t)P.nslots) { xs_next = 0; xp_next ^= 1; }
                         mbar_wait_relaxed_call<kPollNs>(bar_xfull + 8 * xs_cur, xp_cur, &abort_flag, P.status, kStatusWaitOperand);
                     }
-                    if ((k >> P.spg_shift) >= 1) {
+                    if (!ZOUT && (k >> P.spg_shift) >= 1) {
                         const uint32_t sa = ((uint32_t)g << P.spg_shift) + ((uint32_t)k & ((1u << P.spg_shift) - 1u));
                         mbar_wait_relaxed_call<kPollNs>(bar_afree + 8 * sa, ((k >> P.spg_shift) - 1) & 1, &abort_flag, P.status, kStatusWaitStage);
                     }
@@ -642,8 +668,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) fused_bf16_kernel(const __gr
         const int tn = r / hw;
         const int rem = r - tn * hw;
         const int ph = rem / P.PW, pw_ = rem - (rem / P.PW) * P.PW;
-        int wq = 0;                                       // ZOUT: running index of the next finished chunk
-        for (int tl = 0; tl < my_tiles; ++tl) {
+        for (int tl = ZOUT ? my_tiles : 0; tl < my_tiles; ++tl) {
             int tile = bid + tl * nblocks;
             const int bn = fdiv31(tile, P.dv_thw);
             tile -= bn * tiles_hw;
@@ -651,24 +676,6 @@ __global__ void __launch_bounds__(kFusedThreads, 1) fused_bf16_kernel(const __gr
             const int n = bn * P.TN + tn, ho = bh * P.PH + ph, wo = bw * P.PW + pw_;
             const bool live = tn < P.TN && n < P.N && ho < P.Ho && wo < P.Wo;
             const size_t yrow = (((size_t)n * P.Ho + ho) * P.Wo + wo) * P.Dtot + part * P.Dpad;   // element index of the row's first channel
-            if (ZOUT) {
-                // this thread's pixel row of every finished stage goes to z (row r of the stage: 128 bytes, swizzled)
-                for (int q = 0; q < P.nchunks; ++q, ++wq) {
-                    named_bar_sync(kBarChunk0 + (wq & 3), kDwGroupWarps * 32 + kEpiWarps * 32);   // chunk wq is written
-                    const uint32_t sa = ((uint32_t)(wq & 1) << P.spg_shift) + ((uint32_t)(wq >> 1) & ((1u << P.spg_shift) - 1u));
-                    const uint32_t row_s = a_s + sa * 16384 + (uint32_t)r * 128;
-                    uint4 v[8];
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) v[c] = lds128(row_s + (uint32_t)((c ^ (r & 7)) << 4));
-                    warp_arrive(bar_afree + 8 * sa);
-                    if (live) {
-                        uint4 *dst = reinterpret_cast<uint4 *>(P.y + yrow + (size_t)q * kChunk);
-#pragma unroll
-                        for (int c = 0; c < 8; ++c) dst[c] = v[c];
-                    }
-                }
-                continue;
-            }
             const int buf = tl & (P.nacc - 1);            // one or two accumulators
             warp_wait(bar_accfull + 8 * buf, (tl >> (P.nacc - 1)) & 1, &abort_flag, P.status, kStatusWaitMma);
             tc_fence_after();
@@ -725,13 +732,15 @@ __global__ void __launch_bounds__(kFusedThreads, 1) fused_bf16_kernel(const __gr
         int wslot = g;
         while (wslot >= P.nwslots) wslot -= P.nwslots;
         DwShare share = {};
-        if (MODE == 1) share = dw_rows_share<S, PS, ZOUT>(P, il, run);
-        else if (MODE == 2) share = dw_quads_share<S, PS, ZOUT>(P, il, run);
+        if (MODE == 1) share = dw_rows_share<S, PS>(P, il, run);
+        else if (MODE == 2) share = dw_quads_share<S, PS>(P, il, run);
         // A depthwise warp checks one shared-memory barrier per chunk (the group's "open" barrier, kept by the
         // gate warp), and after the chunk's arithmetic its threads arrive, without waiting, at the chunk's
         // hand-over barrier, where the consumer waits.  A hand-over barrier is used again four chunks later, by the same group
         // and for the same stage (two chunks later with one stage per group); by then the gate warp has seen
         // that stage released, hence the consumer past the barrier.
+        int tl = 0;                                       // ZOUT: the chunk's tile
+        if (ZOUT) for (int j = g; j >= P.nchunks; j -= P.nchunks) ++tl;
         for (int gq = g, k = 0; gq < total_chunks; gq += 2, ++k) {
             const bool live_i = q * kChunk + il < P.G;
             const uint32_t sa = ((uint32_t)g << P.spg_shift) + ((uint32_t)k & ((1u << P.spg_shift) - 1u));   // this chunk's stage
@@ -757,10 +766,30 @@ __global__ void __launch_bounds__(kFusedThreads, 1) fused_bf16_kernel(const __gr
             } else {
                 clb = (int)lds32(wsm + (uint32_t)(K * K) * 4);
             }
-            if (MODE == 1) dw_rows<K, S, PS, ZOUT>(share, xs, clb, w, live_i, a_stage);
-            else if (MODE == 2) dw_quads_k3<S, PS, ZOUT>(share, xs, clb, reinterpret_cast<const uint32_t (&)[9]>(w), live_i, a_stage);
-            else dw_generic<K>(P, xs, clb, wsm, il, run, live_i, a_stage);
-            fence_proxy_async();      // every thread: its own writes become visible to the tensor-core proxy
+            int n0 = 0, ho0 = 0, wo0 = 0;
+            uint16_t *zc = nullptr;
+            ZShare zs = {};
+            if (ZOUT) {
+                GDWS_BLOCK_SHARE;
+                int tile = bid + tl * nblocks;
+                const int bn = fdiv31(tile, P.dv_thw);
+                tile -= bn * tiles_hw;
+                const int bh = fdiv31(tile, P.dv_tw);
+                n0 = bn * P.TN; ho0 = bh * P.PH; wo0 = (tile - bh * P.tiles_w) * P.PW;
+                zc = P.y + q * kChunk + il;
+                if (MODE == 1) {
+                    const int nseg = P.PW >> 3, seg = run % nseg, R0 = (run / nseg) * 4, tn = R0 / P.PH;
+                    const int n = n0 + tn, ho = ho0 + R0 - tn * P.PH, wo = wo0 + seg * 8;
+                    zs.gpad = P.Dtot; zs.Wo = P.Wo;
+                    zs.rows = share.live && n < P.N ? P.Ho - ho : 0;
+                    zs.cols = P.Wo - wo;
+                    zs.z = zc + (((size_t)n * P.Ho + ho) * P.Wo + wo) * P.Dtot;
+                }
+            }
+            if (MODE == 1) dw_rows<K, S, PS, ZOUT>(share, xs, clb, w, live_i, a_stage, zs);
+            else if (MODE == 2) dw_quads_k3<S, PS, ZOUT>(share, xs, clb, reinterpret_cast<const uint32_t (&)[9]>(w), live_i, a_stage, P, zc, n0, run, ho0, wo0);
+            else dw_generic<K, ZOUT>(P, xs, clb, wsm, il, run, live_i, a_stage, zc, n0, ho0, wo0);
+            if (!ZOUT) fence_proxy_async();      // every thread: its own writes become visible to the tensor-core proxy
             __syncwarp();
             if (lane == 0) {          // this warp is done with the chunk's filters and input box
                 const int flags = meta_tab[q].y;
@@ -769,9 +798,9 @@ __global__ void __launch_bounds__(kFusedThreads, 1) fused_bf16_kernel(const __gr
                 if (flags & 2) mbar_arrive(bar_xfree + 8 * xslot);
             }
             __syncwarp();
-            named_bar_arrive(kBarChunk0 + (gq & 3), kDwGroupWarps * 32 + (ZOUT ? kEpiWarps * 32 : 32));
+            if (!ZOUT) named_bar_arrive(kBarChunk0 + (gq & 3), kDwGroupWarps * 32 + 32);
             q += 2;
-            while (q >= P.nchunks) q -= P.nchunks;
+            while (q >= P.nchunks) { q -= P.nchunks; ++tl; }
             wslot += 2;
             while (wslot >= P.nwslots) wslot -= P.nwslots;
         }
@@ -893,6 +922,12 @@ static gdws_status_t alu_prepare(gdws_plan_s *p, int n, int h, int w, int Ho, in
             md[1] = (uint32_t)(31 + sh);
         };
         magic(t.tiles_h * t.tiles_w, P.dv_thw); magic(t.tiles_w, P.dv_tw);
+    }
+    if (zout) {      // no weight units and operand stages; exactly four filter blocks (see the gate warp)
+        t.nsb = 0; t.nwslots = 4;
+        t.smem = 1024 + (size_t)t.nslots * t.slot_bytes + (size_t)t.nwslots * kChunk * p->wstride * 4 + (size_t)p->nchunks * 16 + (size_t)Dloc * 4;
+        if (t.smem < (size_t)kMaxSmem / 2 + 2048) t.smem = (size_t)kMaxSmem / 2 + 2048;
+        if (t.smem > (size_t)kMaxSmem) return fail(GDWS_ERR_UNSUPPORTED, "no room for the filter ring");
     }
     P.IH = t.IH; P.IW = t.IW; P.ps = t.cbox * 2; P.nslots = t.nslots; P.nwslots = t.nwslots; P.nboxes = p->nboxes; P.nsb = t.nsb; P.wstride = p->wstride;
     P.spg_shift = t.spg == 2 ? 1 : 0;
