@@ -200,10 +200,17 @@ fused_f32_kernel(F32Shape s, const float *__restrict__ x, const float *__restric
                         tab[u * L + q0 + v] = n * s.xn + (hi + u) * s.xh + (wi + v) * s.xw;
         }
     }
-    constexpr int NI = NP / PT, PER = KC / NI;       // producer threads per pixel, each with PER consecutive channels of z
-    static_assert(NI * PT == NP && PER * NI == KC, "z phase covers the chunk");
+    constexpr int NI = NP / PT > 0 ? NP / PT : 1, PER = KC / NI;       // producer threads per pixel, each with PER consecutive channels of z
+    static_assert((NI * PT == NP || PT == 96) && PER * NI == KC, "z phase covers the chunk");
     const int zpx = pt % PT, zi = pt / PT;
     const int zq = p0 + zpx < npix ? zpx * s.stride + (wo0 + zpx) / s.Wo * ext : 0;
+    int zqs[PT >= 32 ? PT / 32 : 1];                 // the same per group of 32 pixels
+    if constexpr (PT >= 32)
+#pragma unroll
+        for (int g = 0; g < PT / 32; ++g) {
+            const int j = 32 * g + lane;
+            zqs[g] = p0 + j < npix ? j * s.stride + (wo0 + j) / s.Wo * ext : 0;
+        }
     const int nq = (s.G + KC - 1) / KC;
     asm volatile("griddepcontrol.wait;" ::: "memory");
     auto chan_of = [&](int q) { const int i = q * KC + lane; return lane < KC && i < s.G ? __ldg(chan + i) : -1; };
@@ -260,38 +267,68 @@ fused_f32_kernel(F32Shape s, const float *__restrict__ x, const float *__restric
         asm volatile("cp.async.commit_group;" ::: "memory");
         return m;
     };
+    // z of a chunk.  Tiles of 32 pixels and more: a warp takes PW consecutive channels and all PG groups of 32 pixels, lanes =
+    // pixels, so that a filter in registers serves PG pixels and a window all filters of its input channel (both come from
+    // shared memory, whose bandwidth the products need: 16 cycles of it per 16 cycles of multiply-adds).
     auto make_z = [&](int q, uint32_t m) {
-        float *dst = zb + (q & 1) * KC * ZS + zpx;
-        const float *xs = xb + (q & 1) * KC * kL + zq, *fs = fb + (q & 1) * KC * fp;
-        float xr[K ? K * K : 1];
-        int have = -1;
+        const float *fs = fb + (q & 1) * KC * fp;
+        if constexpr (PT >= 32 && K != 0 && K <= 3) {
+            constexpr int PG = PT / 32, PW = KC / WP > 0 ? KC / WP : 1;
+            static_assert(WP * PW == KC, "warps share the chunk");
+            const float *xs = xb + (q & 1) * KC * kL;
+            float *dst = zb + (q & 1) * KC * ZS + lane;
+            float acc[PW][PG];
+            float w[PW][f32_filt_pitch(K * K)];
+#pragma unroll
+            for (int j = 0; j < PW; ++j)
+#pragma unroll
+                for (int t = 0; t < f32_filt_pitch(K * K) / 4; ++t)
+                    *reinterpret_cast<float4 *>(&w[j][4 * t]) = *reinterpret_cast<const float4 *>(fs + (pwarp * PW + j) * fp + 4 * t);
+#pragma unroll
+            for (int g = 0; g < PG; ++g) {
+                float xr[K * K];
+#pragma unroll
+                for (int j = 0; j < PW; ++j) {
+                    const int kk = pwarp * PW + j;
+                    if (j == 0 || ((m >> kk) & 1u)) {      // the same for the whole warp
+                        const float *xc = xs + max(__popc(m & ((2u << kk) - 1u)) - 1, 0) * kL + zqs[g];
+#pragma unroll
+                        for (int u = 0; u < K; ++u)
+#pragma unroll
+                            for (int v = 0; v < K; ++v) xr[u * K + v] = xc[u * L + v];
+                    }
+                    float a = 0.f;
+#pragma unroll
+                    for (int t = 0; t < K * K; ++t) a = fmaf(w[j][t], xr[t], a);
+                    acc[j][g] = a;
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < PW; ++j)
+#pragma unroll
+                for (int g = 0; g < PG; ++g) dst[(pwarp * PW + j) * ZS + 32 * g] = acc[j][g];      // channels i >= G have zero filters
+            return;
+        } else {
+            if (pt >= NI * PT) return;
+            float *dst = zb + (q & 1) * KC * ZS + zpx;
+            const float *xs = xb + (q & 1) * KC * kL + zq;
 #pragma unroll (PER < 4 ? PER : 4)
-        for (int j = 0; j < PER; ++j) {
-            const int kk = zi * PER + j;
-            const int slot = max(__popc(m & ((2u << kk) - 1u)) - 1, 0);
-            const float *xc = xs + slot * kL, *ker = fs + kk * fp;
-            float acc = 0.f;
-            if constexpr (K != 0) {
-                if (slot != have) {
-                    have = slot;
+            for (int j = 0; j < PER; ++j) {
+                const int kk = zi * PER + j;
+                const int slot = max(__popc(m & ((2u << kk) - 1u)) - 1, 0);
+                const float *xc = xs + slot * kL, *ker = fs + kk * fp;
+                float acc = 0.f;
+                if constexpr (K != 0) {
 #pragma unroll
                     for (int u = 0; u < K; ++u)
 #pragma unroll
-                        for (int v = 0; v < K; ++v) xr[u * K + v] = xc[u * L + v];
+                        for (int v = 0; v < K; ++v) acc = fmaf(ker[u * K + v], xc[u * L + v], acc);
+                } else {
+                    for (int u = 0; u < k; ++u)
+                        for (int v = 0; v < k; ++v) acc = fmaf(ker[u * k + v], xc[u * L + v], acc);
                 }
-#pragma unroll
-                for (int t = 0; t < (K * K + 3) / 4; ++t) {
-                    const float4 w = *reinterpret_cast<const float4 *>(ker + 4 * t);
-                    acc = fmaf(w.x, xr[4 * t], acc);
-                    if (4 * t + 1 < K * K) acc = fmaf(w.y, xr[4 * t + 1 < K * K ? 4 * t + 1 : 0], acc);
-                    if (4 * t + 2 < K * K) acc = fmaf(w.z, xr[4 * t + 2 < K * K ? 4 * t + 2 : 0], acc);
-                    if (4 * t + 3 < K * K) acc = fmaf(w.w, xr[4 * t + 3 < K * K ? 4 * t + 3 : 0], acc);
-                }
-            } else {
-                for (int u = 0; u < k; ++u)
-                    for (int v = 0; v < k; ++v) acc = fmaf(ker[u * k + v], xc[u * L + v], acc);
+                dst[kk * ZS] = acc;
             }
-            dst[kk * ZS] = acc;          // channels i >= G have zero filters
         }
     };
 
@@ -517,7 +554,7 @@ gdws_status_t f32_launch_for(bool nhwc, const F32Shape &s, A... a)
 // Block tiles of fused_f32_kernel and the share of the multiply-add rate that a busy SM reaches with each (measured).
 struct F32Config { int pt, dt; double rate; };
 constexpr F32Config kF32Configs[] = {
-    {8, 16, 0.025}, {16, 32, 0.08}, {32, 32, 0.11}, {32, 64, 0.18}, {32, 128, 0.22}, {64, 128, 0.24}, {96, 128, 0.32}, {128, 128, 0.35},
+    {8, 16, 0.025}, {16, 32, 0.08}, {32, 32, 0.11}, {32, 64, 0.19}, {32, 128, 0.24}, {64, 128, 0.24}, {96, 128, 0.34}, {128, 128, 0.36},
 };
 
 // The tile whose busiest SM is done first: large tiles reuse more per load, small ones leave no SM idle.
@@ -555,12 +592,12 @@ gdws_status_t f32_fused(gdws_plan_s *p, const gdws_tensor_t *x, const float *dw_
     const gdws_plan_s *cp = p;
     switch (f32_config(p, (long long)s.N * s.Ho * s.Wo, s.Wo)) {
     case 0: rc = f32_launch_for<8, 16, 1, 1, 1, 128>(nhwc, s, cp, xp, dw_w, pw_w, bias, yp, st); break;
-    case 1: rc = f32_launch_for<16, 32, 2, 2, 1, 128>(nhwc, s, cp, xp, dw_w, pw_w, bias, yp, st); break;
-    case 2: rc = f32_launch_for<32, 32, 4, 2, 1, 128>(nhwc, s, cp, xp, dw_w, pw_w, bias, yp, st); break;
-    case 3: rc = f32_launch_for<32, 64, 4, 4, 1, 128>(nhwc, s, cp, xp, dw_w, pw_w, bias, yp, st); break;
-    case 4: rc = f32_launch_for<32, 128, 4, 8, 2, 128>(nhwc, s, cp, xp, dw_w, pw_w, bias, yp, st); break;
-    case 5: rc = f32_launch_for<64, 128, 8, 8, 2, 256>(nhwc, s, cp, xp, dw_w, pw_w, bias, yp, st); break;
-    case 6: rc = f32_launch_for<96, 128, 8, 8, 2, 192>(nhwc, s, cp, xp, dw_w, pw_w, bias, yp, st); break;
+    case 1: rc = f32_launch_for<16, 32, 2, 2, 1, 256>(nhwc, s, cp, xp, dw_w, pw_w, bias, yp, st); break;
+    case 2: rc = f32_launch_for<32, 32, 4, 2, 1, 256>(nhwc, s, cp, xp, dw_w, pw_w, bias, yp, st); break;
+    case 3: rc = f32_launch_for<32, 64, 4, 4, 1, 256>(nhwc, s, cp, xp, dw_w, pw_w, bias, yp, st); break;
+    case 4: rc = f32_launch_for<32, 128, 4, 8, 2, 256>(nhwc, s, cp, xp, dw_w, pw_w, bias, yp, st); break;
+    case 5: rc = f32_launch_for<64, 128, 8, 8, 1, 256>(nhwc, s, cp, xp, dw_w, pw_w, bias, yp, st); break;
+    case 6: rc = f32_launch_for<96, 128, 8, 8, 2, 256>(nhwc, s, cp, xp, dw_w, pw_w, bias, yp, st); break;
     case 7: rc = f32_launch_for<128, 128, 8, 8, 1, 256>(nhwc, s, cp, xp, dw_w, pw_w, bias, yp, st); break;
     default: return fail(GDWS_ERR_UNSUPPORTED, "too many pixels for the fp32 fused kernel");
     }
