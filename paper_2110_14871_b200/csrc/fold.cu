@@ -549,8 +549,9 @@ gdws_status_t fold_prepare(gdws_plan_s *p, int n, int Ho, int Wo, bool out_f32, 
     P.nacc = std::min(kFoldMaxAcc, 512 / P.acc_cols);
     while ((1 << P.nacc_shift) < P.nacc) ++P.nacc_shift;
     // Input boxes and product steps; run[s]: how many steps, from s on, read the same box (0 inside a run).  A box is one load;
-    // with one load per tap two of them, so that the taps can share a unit.
-    const int per_box = g.layout == 3 ? 2 : 1;
+    // with one load per tap two of them, so that the taps can share a unit, and with stride 2 the loads of both column
+    // parities: filter rows are then whole (k taps each, the unrolled kernels) where they would be 1, 2, 2 and 4 taps.
+    const int per_box = g.layout == 3 || sd == 2 ? 2 : 1;
     P.a_slot = P.a_load * (uint32_t)per_box;
     const TcTaps taps = tc_taps(k, sd, p->pad);
     int nl = 0, ns = 0, run[kFoldMaxSteps] = {}, run0 = 0;
