@@ -77,3 +77,15 @@ def test_folded_refuses_what_it_does_not_cover():
     with pytest.raises(gdws.GdwsError) as e:
         run_gpu(data, path=gdws.PATH_FUSED, dw_math=3)
     assert e.value.status == gdws.ERR_UNSUPPORTED
+
+
+def test_folded_filters_keep_their_sums_on_inputs_with_a_mean():
+    """Inputs of mean 4 and unit spread.  The nearest bf16 neighbour of every tap alone would let a filter's rounding errors
+    add up on the mean; with the taps' sums kept, the result is no worse than the two-stage kernels' (which round z).  Both
+    are compared with the reference in the 2-norm, where y's own rounding (2^-9 / sqrt(3) of each value) dominates."""
+    spec = small_spec("t", 3, 64, 64, 20, 20, 3, 1, 0, ("uniform", 3, 7), "bf16", "NHWC", seed=53)
+    data = gi.make_layer(spec)
+    data.x = gi.round_to_bf16(data.x + 4.0)
+    ref, _ = run_oracle(data)
+    err = {m: float(np.linalg.norm(run_gpu(data, path=gdws.PATH_FUSED, dw_math=m) - ref) / np.linalg.norm(ref)) for m in (1, 3)}
+    assert err[3] <= 1.1 * err[1], err
