@@ -443,7 +443,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) fused_bf16_kernel(const __gr
     const uint32_t bar_accfree = bar_accfull + 16;
     const uint32_t bar_wfull = bar_accfull + 32, bar_wfree = bar_wfull + 8 * kMaxSlots;
     const uint32_t bar_open = bar_wfree + 8 * kMaxSlots;       // a group's next chunk may start (two per group, alternating)
-    const uint32_t bar_drain = bar_open + 32;                  // the MMA warp's last commit, awaited before TMEM is freed
+    const uint32_t bar_drain = bar_open + 32;                  // the MMA warp's last commit, awaited by the last tile's epilogue helpers and before TMEM is freed
     const uint32_t wblock = (uint32_t)kChunk * P.wstride * 4;             // one chunk's filters
     const uint32_t w_s = x_s + (uint32_t)P.nslots * P.slot_bytes;         // ring of nwslots filter blocks
     int4 *meta_tab = reinterpret_cast<int4 *>(base + (w_s - a_s) + (size_t)P.nwslots * wblock);
@@ -564,7 +564,8 @@ __global__ void __launch_bounds__(kFusedThreads, 1) fused_bf16_kernel(const __gr
             // and gives back its shared memory (after an abort the waits above return at once, and products may have
             // been issued on operands that were not there: their results are undefined, but they too must have ended).
             // One more commit covers all earlier products; its wait is bounded and does not look at the abort flag.
-            if (lane == 0) {
+            // The depthwise warps wait for the same commit before they help with the last tile's epilogue.
+            if (elect_one()) {
                 umma_commit(bar_drain);
                 mbar_wait_drain(bar_drain, 0);
             }
@@ -825,7 +826,9 @@ __global__ void __launch_bounds__(kFusedThreads, 1) fused_bf16_kernel(const __gr
         const bool live = tn < P.TN && n < P.N && ho < P.Ho && wo < P.Wo;
         const size_t yrow = (((size_t)n * P.Ho + ho) * P.Wo + wo) * P.Dtot + part * P.Dpad;
         const int buf = tl & (P.nacc - 1);            // one or two accumulators
-        warp_wait(bar_accfull + 8 * buf, (tl >> (P.nacc - 1)) & 1, &abort_flag, P.status, kStatusWaitMma);
+        // Not the accumulator's "full" barrier: these warps have not waited for its earlier phases, and with at most four
+        // chunks per tile they can be done while a phase two back is the last complete one, which has the same parity.
+        warp_wait(bar_drain, 0, &abort_flag, P.status, kStatusWaitMma);
         tc_fence_after();
         const uint32_t t_base = tmem + ((uint32_t)(lg * 32) << 16) + (uint32_t)(buf * P.acc_cols);
         epilogue_row(P, t_base, bias_s, yrow, live, 1 + ((warp - kDwWarp0) >> 2), kTailShare);
