@@ -114,7 +114,10 @@ gdws_status_t forward_pieces(gdws_plan_s *p, HostPipe *pipe, const gdws_tensor_t
     if (e == cudaSuccess) e = cudaStreamWaitEvent(pipe->in, pipe->begin, 0);
     // the first and the last piece, whose copies nothing overlaps, half as large as the others
     int per = pieces == 2 ? (xh->n + 1) / 2 : (xh->n + pieces - 2) / (pieces - 1), first = pieces == 2 ? per : (per + 1) / 2;
-    if ((per * ximg) % 16 || (per * yimg) % 16) per = (per + 7) / 8 * 8, first = (first + 7) / 8 * 8;      // a piece starts on a 16-byte boundary (images are whole 2-byte elements)
+    int unit = 1;                // images that are whole 16-byte pieces of x and of y: every piece starts on such a boundary
+    while ((unit * ximg) % 16 || (unit * yimg) % 16) unit *= 2;
+    per = (per + unit - 1) / unit * unit;
+    first = (first + unit - 1) / unit * unit;
     for (int i = 0, n0 = 0, n = 0; n0 < xh->n && e == cudaSuccess; ++i, n0 += n) {
         n = std::min(i == 0 ? first : per, xh->n - n0);
         cudaEvent_t in = pipe->copied[i], done = pipe->computed[i];
