@@ -97,11 +97,13 @@ bool pinned(const void *ptr)
 // Pieces that gdws_forward_host takes a batch in: 1 (as a whole) for pageable memory, whose copies the host waits for
 // anyway, and for small ones.  A piece costs some 10 us, and of n pieces the first copy in and the last copy out overlap
 // nothing (measured, MB each way: 2.1 best with 2, 8.4 with 3, 33 with 5: 423 -> 292 us for 8.4).
-int host_pieces(const gdws_tensor_t *xh, const gdws_tensor_t *yh, size_t xb, size_t yb)
+int host_pieces(const gdws_plan_s *p, const gdws_tensor_t *xh, const gdws_tensor_t *yh, size_t xb, size_t yb)
 {
     const size_t mb = std::max(xb, yb) >> 20;
     const int n = std::min(xh->n, mb >= 28 ? kHostPieces : (mb >= 16 ? 4 : (mb >= 6 ? 3 : (mb >= 2 ? 2 : 1))));
     if (n < 2 || xh->n != yh->n || !pinned(xh->ptr) || !pinned(yh->ptr)) return 1;
+    // a workspace that does not hold the whole batch is refused where it is needed, even if it would hold a piece
+    if ((p->opt_path == GDWS_PATH_UNFUSED || (p->opt_path == GDWS_PATH_AUTO && p->ws)) && p->ws_bytes < gdws_workspace_bytes(p, xh->dtype, xh->n, xh->h, xh->w)) return 1;
     return n;
 }
 
@@ -265,7 +267,7 @@ gdws_status_t gdws_forward_host(gdws_plan_t *p, const gdws_tensor_t *xh, const v
     // Images are independent and contiguous: with both buffers pinned the batch goes through in pieces, so that a piece's
     // copy in, the forward of the one before and the copy out of an earlier one run at the same time (the link carries both
     // directions at once; 8.4 MB each way: 354 us one after the other, the link's time for one direction is 150).
-    const int pieces = host_pieces(xh, yh, xb, yb);
+    const int pieces = host_pieces(p, xh, yh, xb, yb);
     if (HostPipe *pipe = pieces > 1 ? host_pipe_take(p->device) : nullptr) {
         st = check_pair(p, &xd, &yd);
         if (st == GDWS_OK) st = forward_pieces(p, pipe, xh, &xd, dw_w, pw_w, bias, yh, &yd, pieces, cs);
