@@ -306,7 +306,7 @@ fused_f32_kernel(F32Shape s, const float *__restrict__ x, const float *__restric
 #pragma unroll
             for (int j = 0; j < PW; ++j)
 #pragma unroll
-                for (int g = 0; g < PG; ++g) dst[(pwarp * PW + j) * ZS + 32 * g] = acc[j][g];      // channels i >= G have zero filters
+                for (int g = 0; g < PG; ++g) dst[(pwarp * PW + j) * ZS + 32 * g] = q * KC + pwarp * PW + j < s.G ? acc[j][g] : 0.f;      // i >= G: not 0 * x, x may be infinite
             return;
         } else {
             if (pt >= NI * PT) return;
@@ -327,7 +327,7 @@ fused_f32_kernel(F32Shape s, const float *__restrict__ x, const float *__restric
                     for (int u = 0; u < k; ++u)
                         for (int v = 0; v < k; ++v) acc = fmaf(ker[u * k + v], xc[u * L + v], acc);
                 }
-                dst[kk * ZS] = acc;
+                dst[kk * ZS] = q * KC + kk < s.G ? acc : 0.f;
             }
         }
     };
