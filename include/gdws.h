@@ -88,7 +88,11 @@ typedef enum {
                               packed (see gdws_forward), for the same layers with at most 64 MB
                               of folded filters; 0 (default) = the library chooses by estimated
                               time for each input size (see gdws_plan_form).  1 and 2 give the
-                              same result up to summation order; 3 rounds elsewhere (gdws_forward) */
+                              same result up to summation order; 3 rounds elsewhere (gdws_forward).
+                              1 reads only channels with g_c > 0; 2 and 3 multiply the others (2:
+                              those that share a group of 16 with used ones) by zeros, so that an
+                              infinity or NaN in them reaches y.  0 takes 3 for layers with
+                              g_c = 0 only where no other kernel covers them (D > 512)      */
     GDWS_OPT_OUT_DTYPE = 5 /* bf16 plans: 0 (default) = y has the dtype of x; 1 = y is fp32
                               (GDWS_F32, NHWC): bias and ReLU are applied to the fp32 sums of
                               the PW stage and stored without the rounding to bf16.  Every

@@ -769,6 +769,9 @@ int bf16_form_of(gdws_plan_s *p, int n, int h, int w, bool out_f32)
 {
     const int stage = gdw_stage_of(p);
     if (p->opt_dw_math || !p->fold_ok || p->opt_tile || p->opt_a_layout) return stage;
+    // A channel with g_c = 0 is not part of the layer: the folded form would multiply it by zero filters, and an infinity or
+    // NaN in it would reach y.  (Beyond 512 output channels there is no ALU kernel to keep to.)
+    if (p->unused && !(stage == 1 && p->Dpad > 512)) return stage;
     const int Ho = gdws_out_dim(h, p->k, p->stride, p->pad), Wo = gdws_out_dim(w, p->k, p->stride, p->pad);
     if (n < 1 || Ho < 1 || Wo < 1) return stage;
     const LaunchKey key = {n, h, w, out_f32 ? 2 : 0};

@@ -69,6 +69,7 @@ struct gdws_plan_s {
     int G = 0, Gpad = 0, Dpad = 0, nchunks = 0;
     int wstride = 0;                 // 32-bit words per intermediate channel in d_dwpack (multiple of 4)
     std::vector<int32_t> g, off, chan;
+    bool unused = false;             // some g_c is 0
     std::vector<int32_t> chunk_c0;   // first input channel read by K chunk q (intermediate channels 64q..64q+63)
     std::vector<int32_t> chunk_c1;   // last input channel read by K chunk q
     int span_max = 0;                // widest channel range of one K chunk, counted from the chunk's first

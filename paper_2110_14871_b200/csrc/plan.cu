@@ -319,6 +319,7 @@ gdws_status_t gdws_plan(int C, int D, int k, int stride, int pad, const int32_t 
     for (int c = 0; c < C; ++c) {          // Property 2: rows of channel c start at off_c
         p->off[c] = acc;
         for (int j = 0; j < g[c]; ++j) p->chan[acc + j] = c;
+        p->unused = p->unused || g[c] == 0;
         acc += g[c];
     }
     p->off[C] = acc;

@@ -36,3 +36,12 @@ def test_option_overrides_the_estimates(dw_math):
     with pytest.raises(gdws.GdwsError):
         plan.form(0, 32, 32)
     plan.destroy()
+
+
+def test_unused_channels_keep_the_two_stages():
+    """g_c = 0: the folded form would multiply the channel by zero filters."""
+    g = np.full(64, 5, dtype=np.int32)
+    g[63] = 0
+    plan = gdws.Plan(64, 64, 3, 1, 1, g)
+    assert plan.form(512, 32, 32) == plan.gdw_stage() == 2
+    plan.destroy()

@@ -35,3 +35,16 @@ def test_f32_infinity_in_the_last_channel(N, C, D, H, W, k, layout):
     want[0, max(0, H // 2 + lo):H // 2 + s.pad + 1, max(0, W // 2 + lo):W // 2 + s.pad + 1] = True
     assert not np.isnan(y).any()
     assert np.array_equal(np.isposinf(y), np.broadcast_to(want[:, None], y.shape))
+
+
+@pytest.mark.parametrize("C,D,H,k,stride", [(24, 40, 20, 3, 1), (136, 72, 9, 3, 2), (64, 64, 16, 5, 1)])
+def test_bf16_unused_channel_is_not_read(C, D, H, k, stride):
+    """A channel with g_c = 0 is no part of the layer, whatever it holds: layers whose GDW stage runs on the ALUs by default."""
+    data = gi.make_layer(small_spec("t", 3, C, D, H, H + 1, k, stride, k // 2, ("const", 2), "bf16", "NHWC", seed=43))
+    data.g[5] = 0
+    G = int(data.g.sum())
+    data.dw_w, data.pw_w = data.dw_w[:G], np.ascontiguousarray(data.pw_w[:, :G])
+    want = run_gpu(data, path=gdws.PATH_FUSED)
+    for v in (np.inf, np.nan):
+        data.x[..., 5] = v
+        assert np.array_equal(run_gpu(data, path=gdws.PATH_FUSED), want) and np.isfinite(want).all()
