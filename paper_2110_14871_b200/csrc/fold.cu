@@ -776,13 +776,15 @@ int bf16_form_of(gdws_plan_s *p, int n, int h, int w, bool out_f32)
     if (n < 1 || Ho < 1 || Wo < 1) return stage;
     const LaunchKey key = {n, h, w, out_f32 ? 2 : 0};
     if (const FormChoice *c = LaunchCache<FormChoice>::find(p->launch_cache[3], key)) return c->form;
-    std::unique_ptr<FormChoice> c(new (std::nothrow) FormChoice);
     FoldGeom g;
     const bool fold = fold_geometry(p, n, Ho, Wo, out_f32, &g) && g.us < two_stage_us(p, n, h, w, Ho, Wo, stage);
-    if (!c) return fold ? 3 : stage;
-    c->key = key;
-    c->form = fold ? 3 : stage;
-    return LaunchCache<FormChoice>::add(p->launch_cache[3], std::move(c))->form;
+    const int form = fold ? 3 : stage;
+    if (std::unique_ptr<FormChoice> c{new (std::nothrow) FormChoice}) {
+        c->key = key;
+        c->form = form;
+        LaunchCache<FormChoice>::add(p->launch_cache[3], std::move(c));      // kept if there is memory for it
+    }
+    return form;
 }
 
 gdws_status_t bf16_folded(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t *y, cudaStream_t st)
@@ -799,6 +801,7 @@ gdws_status_t bf16_folded(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t 
         rc = fold_prepare(p, x->n, y->h, y->w, out_f32, e.get());
         if (rc != GDWS_OK) return rc;
         L = LaunchCache<FoldLaunch>::add(p->launch_cache[2], std::move(e));
+        if (!L) return fail(GDWS_ERR_ALLOC, "out of host memory");
     }
     if (L->x != x->ptr && (rc = fold_map_x(p, x, L)) != GDWS_OK) return rc;
     if (L->y != y->ptr && (rc = fold_map_y(p, y, L)) != GDWS_OK) return rc;

@@ -1014,6 +1014,7 @@ static gdws_status_t run_tiled(gdws_plan_s *p, const gdws_tensor_t *x, void *out
         rc = alu_prepare(p, x->n, x->h, x->w, Ho, Wo, zout, out_f32, e.get());
         if (rc != GDWS_OK) return rc;
         L = LaunchCache<AluLaunch>::add(p->launch_cache[0], std::move(e));
+        if (!L) return fail(GDWS_ERR_ALLOC, "out of host memory");
     }
     if (L->x != x->ptr && (rc = alu_map_x(p, x, L)) != GDWS_OK) return rc;
     if (L->out != out && (rc = alu_map_y(p, out, x->n, Ho, Wo, L)) != GDWS_OK) return rc;

@@ -815,10 +815,15 @@ gdws_status_t tc_prepare(gdws_plan_s *p, int n, int Ho, int Wo, bool out_f32, Tc
     P.ostage = b_ost ? 16384 : 0; P.nx = b_nx; P.nb = b_nb; P.nz = b_nz; P.nw = b_nw;
     {
         std::vector<int> order, slabs, zpos, zdep, wpos, wdep;
-        tc_choose_order(p->tc_chunks, P.nz, P.nw, &order);
-        for (int i : order) slabs.push_back(p->tc_chunks[i].npad / 16);
-        if (!tc_ring_places(slabs, P.nz, &zpos, &zdep) || !tc_ring_places(slabs, P.nw, &wpos, &wdep))
-            return fail(GDWS_ERR_UNSUPPORTED, "tensor-core GDW path: a chunk does not fit the slab rings");
+        bool fits = false;
+        try {
+            tc_choose_order(p->tc_chunks, P.nz, P.nw, &order);
+            for (int i : order) slabs.push_back(p->tc_chunks[i].npad / 16);
+            fits = tc_ring_places(slabs, P.nz, &zpos, &zdep) && tc_ring_places(slabs, P.nw, &wpos, &wdep);
+        } catch (const std::bad_alloc &) {
+            return fail(GDWS_ERR_ALLOC, "out of host memory");
+        }
+        if (!fits) return fail(GDWS_ERR_UNSUPPORTED, "tensor-core GDW path: a chunk does not fit the slab rings");
         for (int q = 0; q < nchunks; ++q) {
             P.order[q] = (uint8_t)order[q];
             P.ring[q] = (uint32_t)zpos[q] | ((uint32_t)wpos[q] << 8) | ((uint32_t)zdep[q] << 16) | ((uint32_t)wdep[q] << 19);
@@ -982,6 +987,7 @@ gdws_status_t bf16_fused_tc(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_
         rc = tc_prepare(p, x->n, y->h, y->w, out_f32, e.get());
         if (rc != GDWS_OK) return rc;
         L = LaunchCache<TcLaunch>::add(p->launch_cache[1], std::move(e));
+        if (!L) return fail(GDWS_ERR_ALLOC, "out of host memory");
     }
     if (L->x != x->ptr && (rc = tc_map_x(p, x, L)) != GDWS_OK) return rc;
     if (L->y != y->ptr && (rc = tc_map_y(p, y, L)) != GDWS_OK) return rc;

@@ -6,6 +6,7 @@
 
 #include <algorithm>
 #include <memory>
+#include <new>
 #include <string>
 #include <utility>
 #include <vector>
@@ -182,13 +183,19 @@ template <class Entry> struct LaunchCache {
             }
         return nullptr;
     }
+    // Keeps `e`; null without host memory for it (nothing is thrown across the C interface).
     static Entry *add(std::shared_ptr<void> &slot, std::unique_ptr<Entry> e)
     {
-        if (!slot) slot = std::shared_ptr<void>(new LaunchCache, [](void *c) { delete static_cast<LaunchCache *>(c); });
-        auto &v = static_cast<LaunchCache *>(slot.get())->entries;
-        if (v.size() >= kKeep) v.erase(v.begin());
-        v.push_back(std::move(e));
-        return v.back().get();
+        try {
+            if (!slot) slot = std::shared_ptr<void>(new LaunchCache, [](void *c) { delete static_cast<LaunchCache *>(c); });
+            auto &v = static_cast<LaunchCache *>(slot.get())->entries;
+            v.reserve(kKeep);
+            if (v.size() >= kKeep) v.erase(v.begin());
+            v.push_back(std::move(e));
+            return v.back().get();
+        } catch (const std::bad_alloc &) {
+            return nullptr;
+        }
     }
 };
 // Two streams and the events that order the pieces of a gdws_forward_host call.  Creating them takes milliseconds: a call
