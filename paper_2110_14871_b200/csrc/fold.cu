@@ -768,7 +768,10 @@ struct FormChoice {
 int bf16_form_of(gdws_plan_s *p, int n, int h, int w, bool out_f32)
 {
     const int stage = gdw_stage_of(p);
-    if (p->opt_dw_math || !p->fold_ok || p->opt_tile || p->opt_a_layout) return stage;
+    if (p->opt_dw_math) return p->opt_dw_math;
+    // one row or column and stride 2: the view of the odd ones is empty, and the kernels that read it refuse the input
+    if (p->stride == 2 && p->k <= 5 && (h < 2 || w < 2) && tc_taps(p->k, 2, p->pad).used[1]) return 1;
+    if (!p->fold_ok || p->opt_tile || p->opt_a_layout) return stage;
     // A channel with g_c = 0 is not part of the layer: the folded form would multiply it by zero filters, and an infinity or
     // NaN in it would reach y.  (Beyond 512 output channels there is no ALU kernel to keep to.)
     if (p->unused && !(stage == 1 && p->Dpad > 512)) return stage;

@@ -221,7 +221,7 @@ inline size_t dtype_size(gdws_dtype_t d) { return d == GDWS_F32 ? 4 : 2; }
 // row), and beyond 256 output channels the tensor-core kernel computes the GDW stage once per 256 of them.
 inline int gdw_stage_of(const gdws_plan_s *p)
 {
-    if (p->opt_dw_math != 0) return p->opt_dw_math;
+    if (p->opt_dw_math == 1 || p->opt_dw_math == 2) return p->opt_dw_math;
     if (!(p->tc_ok && (p->k == 3 || p->k == 5) && p->stride <= 2)) return 1;
     if (p->stride == 1 && p->Dpad > 256) return 1;     // measured equal or slower there; with stride 2 faster at D = 512 too
     // average multiplier of at least 4, or of at least 2.7 when the PW products are small (at most 128 output channels)

@@ -45,3 +45,19 @@ def test_unused_channels_keep_the_two_stages():
     plan = gdws.Plan(64, 64, 3, 1, 1, g)
     assert plan.form(512, 32, 32) == plan.gdw_stage() == 2
     plan.destroy()
+
+
+@pytest.mark.parametrize("H,W", [(1, 9), (9, 1), (1, 1)])
+@pytest.mark.parametrize("g", [2, 6])
+def test_stride_2_on_one_row_or_column_is_the_alu_kernel(g, H, W):
+    """The kernels that read one view per parity refuse an input without odd rows or columns."""
+    plan = _plan(64, 64, 3, 2, g)
+    assert plan.form(4, H, W) == 1 and plan.form(4, 9, 9) != 1
+    plan.destroy()
+
+
+def test_gdw_stage_is_one_of_the_two_stages():
+    for g, stage in ((2, 1), (6, 2)):
+        plan = _plan(64, 64, 3, 1, g, 3)
+        assert plan.gdw_stage() == stage and plan.form(4, 9, 9) == 3
+        plan.destroy()
