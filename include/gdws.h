@@ -86,7 +86,7 @@ typedef enum {
                               or 2 and k <= 5, else GDWS_ERR_UNSUPPORTED; 3 = nowhere: the two
                               stages are folded into one k x k convolution when the weights are
                               packed (see gdws_forward), for the same layers with at most 64 MB
-                              of folded filters; 0 (default) = the library chooses by estimated
+                              of folded filters a term; 0 (default) = the library chooses by estimated
                               time for each input size (see gdws_plan_form).  1 and 2 give the
                               same result up to summation order; 3 rounds elsewhere (gdws_forward).
                               1 reads only channels with g_c > 0; 2 and 3 multiply the others (2:
@@ -117,7 +117,7 @@ typedef enum {
  * Host work: offsets off_c, the intermediate-channel -> input-channel table, the
  * padding of G to the tensor-core chunk, output-patch choice.  If a CUDA device is
  * current, the plan also allocates its device tables and packed-weight buffers
- * (O(G*(k*k+D)) bytes, and 2*C*k*k*D for the folded form where it is covered) on it; with no device the plan is still valid for the
+ * (O(G*(k*k+D)) bytes, and 4*C*k*k*D for the folded form where it is covered) on it; with no device the plan is still valid for the
  * host-side queries below and allocates at the first device call.
  * Errors: GDWS_ERR_INVALID_ARG, GDWS_ERR_ALLOC, GDWS_ERR_CUDA.
  */
@@ -206,9 +206,12 @@ GDWS_API gdws_status_t gdws_set_workspace(gdws_plan_t *plan, void *workspace, si
  *          y->h/w == H'/W'.
  * Accumulation is fp32 on both paths.  A bf16 forward rounds to bf16 once between the two linear maps and y on
  * store: the two-stage kernels round the intermediate z, the folded one the filters
- * W[d,c] = sum_j P[d,off_c+j] K[off_c+j] (Property 1 and 2), which are formed in fp32.  The errors have the same bound,
- * 2^-9 sum |P| |K| |x| per output; which is smaller depends on the data (z where filters cancel a large constant part of x,
- * W where pointwise weights cancel).  GDWS_OPT_DW_MATH = 1 or 2 keeps to the first for every size.
+ * W[d,c] = sum_j P[d,off_c+j] K[off_c+j] (Property 1 and 2), which are formed in fp32.  Rounding to nearest errs by up to 2^-8 of
+ * a value, so before y's own rounding either form is within 2^-8 sum |P| |K| |x| per output.  On independent weights and inputs,
+ * with a mean or without, both have the same relative error (2.35e-3 of y in the 2-norm, y's rounding included).  Filters that
+ * pass less than half of their energy to a constant input (taps that sum to about zero) are folded into two bf16 terms, 2^-16
+ * instead of 2^-8, because z is small there and W is not; the forward then takes up to twice the products.  Products of weights
+ * have to stay in the range of fp32 where they are folded.  GDWS_OPT_DW_MATH = 1 or 2 keeps to the two stages for every size.
  * Device memory is never allocated here.  Errors: GDWS_ERR_INVALID_ARG (shape, dtype,
  * alignment, NULL), GDWS_ERR_UNSUPPORTED, GDWS_ERR_WORKSPACE (unfused path without a large
  * enough workspace), GDWS_ERR_ARCH, GDWS_ERR_CUDA (launch failure, reported synchronously).

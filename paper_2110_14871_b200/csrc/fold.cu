@@ -6,8 +6,8 @@
 //     y[pixel, d] = bias[d] + sum_{u,v,c} x[pixel shifted by (u,v), c] W[d,c,u,v]
 // as a tensor-core product with fp32 accumulators over k*k*C.  It takes C k^2 D multiply-adds per pixel where the two
 // stages take G (k^2 + D), but all of them run at full tensor-core rate: nothing is rounded, scattered or handed over
-// between two stages.  The one bf16 rounding between the stages moves from z to W (same size: measured 1.6e-3 of the
-// result either way).  bf16_form_of below decides per layer and input size.
+// between two stages.  The one bf16 rounding between the stages moves from z to W (measured 1.66e-3 of the result either
+// way, before y's own); where filters cut a constant input off W is taken in two terms (kFoldPass).  bf16_form_of below decides per layer and input size.
 //
 // What bounds it, and the layout that follows:
 //   * A operand (x): the input box of a tile is staged once per 64 input channels as [row][column][64 channels] (128 bytes
@@ -34,7 +34,7 @@
 
 namespace gdws {
 
-constexpr int kFoldAWarp = 2, kFoldBWarp = 4, kFoldTmemWarp = 6;     // two warps each for products, input boxes, filters
+constexpr int kFoldAWarp = 2, kFoldBWarp = 4, kFoldTmemWarp = 6, kFoldTermWarp = 7;     // two warps each for products, input boxes, filters
 constexpr int kFoldEpiWarp0 = 8, kFoldEpiGroups = 4;      // up to four groups of four epilogue warps
 constexpr int kFoldMaxSmem = 226 * 1024;                  // dynamic shared memory (227 KB less the barriers)
 constexpr int kFoldThreads = (kFoldEpiWarp0 + 4 * kFoldEpiGroups) * 32;
@@ -43,6 +43,15 @@ constexpr int kFoldMaxA = 8;             // input box slots
 constexpr int kFoldMaxB = 40;            // filter units in shared memory (one tap x 64 input channels each)
 constexpr uint32_t kFoldSw128 = 2u << 29;   // descriptor high word: layout type "128-byte swizzle"
 constexpr int kFoldMaxAcc = 8;           // accumulators in tensor memory
+// One term of the filters suffices if they pass this share of their energy to a constant input: sum over the filters of
+// (sum_t W)^2 against sum_t W^2.  The rounding errors of a filter's taps are independent, so on a mean m they add up to some
+// 2^-9.2 sqrt(sum_t W^2) m.  Where the filters let the mean through, y grows with it and the error is that of rounding z
+// (random filters, share 0.9 to 1.1: relative error of y 2.35e-3 in either form, whatever the mean); where they cut it off it is
+// all error.  Relative error of y for 128 -> 256 channels at a mean of 10 sigma, two stages | one term | two terms: share 0.46
+// 2.42e-3 | 3.09e-3 | 1.66e-3, share 0.28 2.25e-3 | 3.31e-3 | 1.62e-3, zero 2.41e-3 | 1.60e-2 | 1.66e-3 (at 100 sigma 1.57e-1 for
+// one term).  The second term costs 28 x 28 x 8 images of that layer 9.1 -> 12.0 us (two stages 16.7), 512 -> 512 channels 18.7 ->
+// 30.8 (44.7); random filters of 64 channels with g_c = 1 scatter by 0.18 around 1, so a line much nearer to 1 would catch them.
+constexpr float kFoldPass = 0.5f;
 // A unit is a run of product steps (taps) whose filters share one barrier: bits 0-7 its first step, 8-15 its steps,
 // then whether it is the first / last one that reads its input box.
 constexpr uint32_t kUnitFirst = 1u << 16, kUnitLast = 1u << 17, kUnitLastBox = 1u << 18;   // LastBox: the first unit of the window's last box
@@ -52,6 +61,8 @@ struct alignas(64) FoldParams {
     CUtensorMap tmap_w;          // folded filters as rows of 64 input channels, box (64, Npart / 2)
     CUtensorMap tmap_y;          // y as (D, Wo, Ho, N), box (128 bytes of channels, PW, PH, TN)
     const float *bias;
+    const float2 *sums;          // of the packing blocks (kFoldPass)
+    int nsums;
     int *status;
     int nwin, nk_last, nsteps, nunits, nboxes, mma_warps;
     uint32_t steps[kFoldMaxSteps];       // per product step of a window: A offset / 16, tap << 16
@@ -122,16 +133,82 @@ __device__ __forceinline__ void fold_issue(const FoldParams &P, int s0, int n, i
     }
 }
 
+// Whether the filters need their second term, by a whole warp: the packing blocks' sums, added in a fixed order.
+__device__ __forceinline__ bool fold_second_term(const FoldParams &P, int lane)
+{
+    float energy = 0.f, sum = 0.f;
+#pragma unroll 1
+    for (int b0 = 0; b0 < P.nsums; b0 += 256) {
+        float2 v[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int b = b0 + 32 * j + lane;
+            v[j] = b < P.nsums ? __ldcg(P.sums + b) : make_float2(0.f, 0.f);
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) { energy += v[j].x; sum += v[j].y; }
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) { energy += __shfl_xor_sync(0xffffffffu, energy, o); sum += __shfl_xor_sync(0xffffffffu, sum, o); }
+    return sum < kFoldPass * energy;
+}
+
+struct FoldBars { uint32_t afull, aempty, bfull, bempty, accfull, accfree; };
+
+// The rest of the products where the filters need their second term, by the thread that has issued item 0's first term: item 0's
+// windows once more, then the other items, twice through their windows each.  The filters pass through their ring, also where
+// there is room for all of one term.  (As a variant of the loops of the common case, with a flag in registers, it cost every
+// layer 2 to 4 %: what those loops compare with has to stay in the constant bank.)
+static __device__ __noinline__ void fold_second(const FoldParams *params, int my_items, uint32_t tmem, uint32_t a_s, uint32_t b_s, FoldBars bar, volatile int *abort_flag)
+{
+    const FoldParams &P = *params;
+    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(P.Npart >> 3) << 17) | (16u << 24);
+    const uint32_t a_hi = ((P.a_sbo >> 4) & 0x3FFFu) | (1u << 14) | kFoldSw128, b_hi = (1024u >> 4) | (1u << 14) | kFoldSw128;
+    const uint32_t a_lo0 = ((a_s & 0x3FFFFu) >> 4) | (1u << 16), b_lo0 = ((b_s & 0x3FFFFu) >> 4) | (1u << 16);
+    if (P.resident)              // item 0's first term did not release its filters
+        for (int u = 0; u < P.nb; ++u) umma_commit_pair(bar.bempty + 8 * (uint32_t)u);
+    // both rings as the first term leaves them
+    const int boxes = P.nwin * P.nboxes, units = P.nwin * P.nunits;
+    uint32_t aslot = (uint32_t)(boxes % P.na), apar = (uint32_t)(boxes / P.na) & 1u, bslot = (uint32_t)(units % P.nb), bpar = (uint32_t)(units / P.nb) & 1u;
+#pragma unroll 1
+    for (int it = 0; it < my_items; ++it) {
+        const int buf = it & (P.nacc - 1);
+        const uint32_t d = tmem + (uint32_t)(buf * P.acc_cols);
+        if (it >= P.nacc) fold_wait_cluster(bar.accfree + 8 * buf, (uint32_t)((it >> P.nacc_shift) - 1) & 1u, abort_flag, P.status, kStatusWaitStage);
+#pragma unroll 1
+        for (int w = it ? 0 : P.nwin; w < 2 * P.nwin; ++w) {
+            const int nk = w == P.nwin - 1 || w == 2 * P.nwin - 1 ? P.nk_last : 4;
+#pragma unroll 1
+            for (int u = 0; u < P.nunits; ++u) {
+                const uint32_t un = P.units[u];
+                if (un & kUnitFirst) mbar_wait_call(bar.afull + 8 * aslot, apar, abort_flag, P.status, kStatusWaitOperand);
+                mbar_wait_call(bar.bfull + 8 * bslot, bpar, abort_flag, P.status, kStatusWaitOperand);
+                tc_fence_after();
+                fold_issue<0, 0>(P, (int)(un & 0xFFu), (int)((un >> 8) & 0xFFu), nk, d, a_lo0 + aslot * (P.a_slot >> 4), a_hi, b_lo0 + bslot * (P.b_unit >> 4), b_hi, P.b_tap >> 4,
+                                 idesc, (uint32_t)(w | u));
+                umma_commit_pair(bar.bempty + 8 * bslot);
+                if (++bslot == (uint32_t)P.nb) { bslot = 0; bpar ^= 1u; }
+                if (un & kUnitLast) {
+                    umma_commit_pair(bar.aempty + 8 * aslot);
+                    if (++aslot == (uint32_t)P.na) { aslot = 0; apar ^= 1u; }
+                }
+            }
+        }
+        if (it != my_items - 1) umma_commit_pair(bar.accfull + 8 * buf);
+    }
+}
+
 // UNITS x STEPS: the window's units when they are all alike (unrolled: 3 x 3 taps or 9 x 1), 0: table driven.
 template <int UNITS, int STEPS>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kFoldThreads, 1) fold_kernel(const __grid_constant__ FoldParams P)
 {
     extern __shared__ uint8_t smem_raw[];
-    // afull[8] aempty[8] | bfull[40] bempty[40] | accfull[8] accfree[8] | turn[2] | drain
-    constexpr int kBars = 2 * kFoldMaxA + 2 * kFoldMaxB + 2 * kFoldMaxAcc + 3;
+    // afull[8] aempty[8] | bfull[40] bempty[40] | accfull[8] accfree[8] | turn[2] | drain | terms
+    constexpr int kBars = 2 * kFoldMaxA + 2 * kFoldMaxB + 2 * kFoldMaxAcc + 4;
     __shared__ __align__(8) uint64_t bars[kBars];
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
+    __shared__ int second_term;      // 1: the filters' second term is taken as well (bar_terms: it is known)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t rank = cluster_rank();
     volatile int *const vabort = &abort_flag;
@@ -141,15 +218,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kFoldThreads, 1) fol
     float *bias_sm = reinterpret_cast<float *>(base + P.off_bias);
     const uint32_t bar_afull = smem_u32(&bars[0]), bar_aempty = bar_afull + 8 * kFoldMaxA;
     const uint32_t bar_bfull = bar_aempty + 8 * kFoldMaxA, bar_bempty = bar_bfull + 8 * kFoldMaxB;
-    const uint32_t bar_accfull = bar_bempty + 8 * kFoldMaxB, bar_accfree = bar_accfull + 8 * kFoldMaxAcc, bar_turn = bar_accfree + 8 * kFoldMaxAcc, bar_drain = bar_turn + 16;
+    const uint32_t bar_accfull = bar_bempty + 8 * kFoldMaxB, bar_accfree = bar_accfull + 8 * kFoldMaxAcc, bar_turn = bar_accfree + 8 * kFoldMaxAcc, bar_drain = bar_turn + 16, bar_terms = bar_drain + 8;
 
-    if (tid == 0) abort_flag = 0;
+    if (tid == 0) abort_flag = second_term = 0;
     // Full barriers are used in the leader only (its own arrive with the bytes of both blocks); "free" barriers are
     // completed in both blocks by the leader's commits; accfree counts the epilogue warps of both blocks.
     if (tid < kBars) {
         static_assert(kBars <= kFoldThreads, "one barrier per thread");
         const int acc = tid - (2 * kFoldMaxA + 2 * kFoldMaxB);
-        mbar_init(bar_afull + 8 * (uint32_t)tid, acc >= kFoldMaxAcc && acc < 2 * kFoldMaxAcc ? 8u * (uint32_t)P.gb : (tid == kBars - 1 ? 2u : 1u));
+        mbar_init(bar_afull + 8 * (uint32_t)tid, acc >= kFoldMaxAcc && acc < 2 * kFoldMaxAcc ? 8u * (uint32_t)P.gb : (tid == kBars - 2 ? 2u : 1u));
         fence_mbar_init();
     }
     grid_launch_dependents();
@@ -172,6 +249,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kFoldThreads, 1) fol
     const int cluster = (int)blockIdx.x >> 1, nclusters = (int)gridDim.x >> 1;
     const int my_items = (P.nitems - cluster + nclusters - 1) / nclusters;
     const int nunits = UNITS ? UNITS : P.nunits;
+    // Whether an item takes the windows once more for the filters' second term.  All roles ask after the first item's first
+    // term, so that the sums are read beside the first copies and products.
+    auto two_terms = [&]() -> int {
+        fold_wait(bar_terms, 0, &abort_flag, P.status, kStatusWaitOperand);
+        return *(volatile int *)&second_term;
+    };
 
     if (warp < kFoldAWarp) {
         if (rank == 0 && elect_one()) {
@@ -202,8 +285,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kFoldThreads, 1) fol
             };
             const bool two = P.mma_warps == 2;
             if (warp == 1) skip_item();
+            int it = two || warp == 0 ? warp : my_items;
+            if (two && warp == 1 && two_terms()) it = my_items;      // fold_second takes all items
 #pragma unroll 1
-            for (int it = two || warp == 0 ? warp : my_items; it < my_items; it += P.mma_warps) {
+            for (; it < my_items; it += P.mma_warps) {
                 const int buf = it & (P.nacc - 1);
                 const uint32_t d = tmem + (uint32_t)(buf * P.acc_cols);
                 if (it >= P.nacc) {
@@ -238,6 +323,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kFoldThreads, 1) fol
                             if (++aslot == (uint32_t)P.na) { aslot = 0; a_lo = a_lo0; apar ^= 1u; }
                         }
                         if (w == P.nwin - 1 && u == nunits - 1) {
+                            if (it == 0 && two_terms()) {
+                                fold_second(&P, my_items, tmem, a_s, b_s, {bar_afull, bar_aempty, bar_bfull, bar_bempty, bar_accfull, bar_accfree}, &abort_flag);
+                                goto issued;
+                            }
                             if (it != my_items - 1) umma_commit_pair(bar_accfull + 8 * buf);
                             if (two) skip_item();
                         }
@@ -248,6 +337,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kFoldThreads, 1) fol
                     }
                 }
             }
+        issued:
             // Teardown: one more commit covers every product issued and every earlier commit's arrival in both blocks.
             umma_commit_pair(bar_drain);
         }
@@ -261,6 +351,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kFoldThreads, 1) fol
             uint32_t slot = (uint32_t)me, par = 1;           // na >= 2
             int n = 0;                                       // boxes up to here, both warps' together
             const uint32_t full0 = map_shared(bar_afull, 0);
+            int terms = 1;                                   // of the filters: the windows are taken once for each
             bool stop = false;
 #pragma unroll 1
             for (int it = 0; it < my_items && !stop; ++it) {
@@ -270,23 +361,27 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kFoldThreads, 1) fol
                 const int bh = fold_div(tile, P.dv_tw), bw = tile - bh * P.tiles_w;
                 const int n0 = bn * P.TN, h0 = bh * P.PH, w0 = bw * P.PW;
 #pragma unroll 1
-                for (int w = 0; w < P.nwin && !stop; ++w)
+                for (int t = 0; t < terms; ++t) {
 #pragma unroll 1
-                    for (int b = 0; b < P.nboxes; ++b, ++n) {
-                        if ((n & (step - 1)) != me) continue;
-                        if (n >= P.na) fold_wait(bar_aempty + 8 * slot, par, &abort_flag, P.status, kStatusWaitStage);
-                        if (*vabort) { stop = true; break; }
-                        const int l0 = (int)(P.boxes[b] & 0xFFu), nl = (int)(P.boxes[b] >> 8);
-                        if (rank == 0) mbar_expect_tx(bar_afull + 8 * slot, 2u * P.a_bytes * (uint32_t)nl);
+                    for (int w = 0; w < P.nwin && !stop; ++w)
 #pragma unroll 1
-                        for (int j = 0; j < nl; ++j) {
-                            const int l = l0 + j;
-                            tma_load_4d_pair(a_s + slot * P.a_slot + (uint32_t)j * P.a_load, &P.tmap_x[P.load_map[l]], w * 64, w0 + P.load_dw[l], h0 + P.load_dh[l],
-                                             n0, full0 + 8 * slot);
+                        for (int b = 0; b < P.nboxes; ++b, ++n) {
+                            if ((n & (step - 1)) != me) continue;
+                            if (n >= P.na) fold_wait(bar_aempty + 8 * slot, par, &abort_flag, P.status, kStatusWaitStage);
+                            if (*vabort) { stop = true; break; }
+                            const int l0 = (int)(P.boxes[b] & 0xFFu), nl = (int)(P.boxes[b] >> 8);
+                            if (rank == 0) mbar_expect_tx(bar_afull + 8 * slot, 2u * P.a_bytes * (uint32_t)nl);
+#pragma unroll 1
+                            for (int j = 0; j < nl; ++j) {
+                                const int l = l0 + j;
+                                tma_load_4d_pair(a_s + slot * P.a_slot + (uint32_t)j * P.a_load, &P.tmap_x[P.load_map[l]], w * 64, w0 + P.load_dw[l], h0 + P.load_dh[l],
+                                                 n0, full0 + 8 * slot);
+                            }
+                            slot += (uint32_t)step;
+                            if (slot >= (uint32_t)P.na) { slot -= (uint32_t)P.na; par ^= 1u; }
                         }
-                        slot += (uint32_t)step;
-                        if (slot >= (uint32_t)P.na) { slot -= (uint32_t)P.na; par ^= 1u; }
-                    }
+                    if (it + t == 0) terms += two_terms();
+                }
             }
             // Teardown: the last phase armed on each slot completes when both blocks' copies have landed (box j and those
             // of the same parity are this warp's; a warp that stopped early armed box n - 2 or n - 1 last).
@@ -301,35 +396,49 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kFoldThreads, 1) fol
             uint32_t slot = (uint32_t)me, par = 1;           // nb >= 2
             int n = 0;
             const uint32_t full0 = map_shared(bar_bfull, 0);
-            const int rounds = P.resident ? (my_items > 0 ? 1 : 0) : my_items;
+            int terms = 1;
             bool stop = false;
 #pragma unroll 1
-            for (int it = 0; it < rounds && !stop; ++it) {
+            for (int it = 0; it < my_items && !stop; ++it) {
                 const int item = cluster + it * nclusters;
                 const int part = item - fold_div(item, P.dv_parts) * P.nparts;
                 const int d0 = part * P.Npart + (int)rank * (P.Npart >> 1);
 #pragma unroll 1
-                for (int w = 0; w < P.nwin && !stop; ++w)
+                for (int t = 0; t < terms; ++t) {
+                    const int row0 = t * P.nwin * P.nsteps * P.Dp + d0;
 #pragma unroll 1
-                    for (int u = 0; u < nunits; ++u, ++n) {
-                        if ((n & (step - 1)) != me) continue;
-                        if (n >= P.nb) fold_wait(bar_bempty + 8 * slot, par, &abort_flag, P.status, kStatusWaitStage);
-                        if (*vabort) { stop = true; break; }
-                        const int s0 = (int)(P.units[u] & 0xFFu), ns = (int)((P.units[u] >> 8) & 0xFFu);
-                        if (rank == 0) mbar_expect_tx(bar_bfull + 8 * slot, 2u * P.b_tap * (uint32_t)ns);
+                    for (int w = 0; w < P.nwin && !stop; ++w)
 #pragma unroll 1
-                        for (int j = 0; j < ns; ++j) {
-                            const int tap = (int)((P.steps[s0 + j] >> 16) & 0xFFu);
-                            tma_load_2d_pair(b_s + slot * P.b_unit + (uint32_t)j * P.b_tap, &P.tmap_w, 0, (w * P.nsteps + tap) * P.Dp + d0, full0 + 8 * slot);
+                        for (int u = 0; u < nunits; ++u, ++n) {
+                            if ((n & (step - 1)) != me) continue;
+                            if (n >= P.nb) fold_wait(bar_bempty + 8 * slot, par, &abort_flag, P.status, kStatusWaitStage);
+                            if (*vabort) { stop = true; break; }
+                            const int s0 = (int)(P.units[u] & 0xFFu), ns = (int)((P.units[u] >> 8) & 0xFFu);
+                            if (rank == 0) mbar_expect_tx(bar_bfull + 8 * slot, 2u * P.b_tap * (uint32_t)ns);
+#pragma unroll 1
+                            for (int j = 0; j < ns; ++j) {
+                                const int tap = (int)((P.steps[s0 + j] >> 16) & 0xFFu);
+                                tma_load_2d_pair(b_s + slot * P.b_unit + (uint32_t)j * P.b_tap, &P.tmap_w, 0, (w * P.nsteps + tap) * P.Dp + row0, full0 + 8 * slot);
+                            }
+                            slot += (uint32_t)step;
+                            if (slot >= (uint32_t)P.nb) { slot -= (uint32_t)P.nb; par ^= 1u; }
                         }
-                        slot += (uint32_t)step;
-                        if (slot >= (uint32_t)P.nb) { slot -= (uint32_t)P.nb; par ^= 1u; }
-                    }
+                    if (it + t == 0) terms += two_terms();
+                }
+                if (P.resident && terms == 1) break;       // they stay
             }
             if (rank == 0)
                 for (int i = 0, j = n - 1; i < P.nb && j >= 0; ++i, --j)
                     if ((j & (step - 1)) == me) mbar_wait_drain(bar_bfull + 8 * (j % P.nb), (uint32_t)(j / P.nb) & 1u);
         }
+    } else if (warp == kFoldTermWarp) {
+        // ---------------- one term of the filters or two ----------------
+        const bool second = fold_second_term(P, lane);
+        if (lane == 0) {
+            second_term = second;
+            mbar_arrive(bar_terms);
+        }
+        __syncwarp();
     } else if (warp >= kFoldEpiWarp0) {
         // ---------------- epilogue: TMEM -> bias / ReLU -> y, 128 bytes of channels per pixel at a time ----------------
         // A block of rows (row r = pixel r of the tile) is staged with its 16-byte pieces swizzled by row, and stored by
@@ -537,7 +646,7 @@ gdws_status_t fold_prepare(gdws_plan_s *p, int n, int Ho, int Wo, bool out_f32, 
     P.D = p->D; P.Dp = p->fold_dp; P.Npart = g.Npart; P.nparts = g.nparts;
     P.relu = p->opt_relu; P.out_f32 = out_f32 ? 1 : 0;
     P.TN = g.TN; P.PH = g.PH; P.PW = g.PW; P.tiles_h = g.tiles_h; P.tiles_w = g.tiles_w; P.nitems = (int)nitems;
-    P.bias = p->d_bias; P.status = p->d_status;
+    P.bias = p->d_bias; P.status = p->d_status; P.sums = p->d_fold_sums; P.nsums = p->fold_nsums;
     P.a_bytes = (uint32_t)(g.TN * g.IH * g.IW * 128);
     P.a_load = (P.a_bytes + 1023u) / 1024u * 1024u;
     P.a_sbo = g.layout == 3 ? 1024u : (uint32_t)g.IW * 128u;
@@ -675,7 +784,7 @@ gdws_status_t fold_prepare(gdws_plan_s *p, int n, int Ho, int Wo, bool out_f32, 
     }
     tensor_map_encode_fn encode = encode_fn();
     if (!encode) return fail(GDWS_ERR_CUDA, "cuTensorMapEncodeTiled is not available from this driver");
-    const cuuint64_t dims[2] = {64, (cuuint64_t)P.nwin * P.nsteps * p->fold_dp};
+    const cuuint64_t dims[2] = {64, (cuuint64_t)2 * P.nwin * P.nsteps * p->fold_dp};
     const cuuint64_t strides[1] = {128};
     const cuuint32_t box[2] = {64, (cuuint32_t)g.Npart / 2}, estr[2] = {1, 1};
     const CUresult r = encode(&P.tmap_w, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, p->d_fold, dims, strides, box, estr,

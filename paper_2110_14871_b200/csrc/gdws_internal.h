@@ -94,6 +94,8 @@ struct gdws_plan_s {
     // Folded path (fold.cu): the layer as one k x k convolution.
     bool fold_ok = false;            // the layer is one the path covers
     int fold_nwin = 0, fold_dp = 0;  // windows of 64 input channels; output channels rounded up to 32
+    int fold_blocks = 0;             // packing blocks of the folded filters (windows x groups of kFoldPackD output channels)
+    int fold_sum_step = 1, fold_nsums = 0;   // every fold_sum_step-th group of a window writes its sums, fold_nsums in all
 
     int opt_path = GDWS_PATH_AUTO;
     int opt_relu = 0;
@@ -118,7 +120,8 @@ struct gdws_plan_s {
     gdws::TcChunk *d_tc_chunks = nullptr;
     uint16_t *d_tc_filt = nullptr; // [tc_nslabs * 16][tc_rec_hw]: per intermediate slot, channel index inside the window and the taps (bf16)
     uint16_t *d_tc_pw = nullptr;   // [tc_nparts][tc_nslabs][2][tc_dloc][8] bf16: pointwise weights, one K = 16 operand slab per 16 slots
-    uint16_t *d_fold = nullptr;    // [fold_nwin][k*k][fold_dp][64] bf16: folded filters
+    uint16_t *d_fold = nullptr;    // [2][fold_nwin][k*k][fold_dp][64] bf16: folded filters, then what their rounding left over
+    float2 *d_fold_sums = nullptr; // [fold_nsums]: sums that decide whether a forward takes both terms
     int *d_status = nullptr;       // device status word
     bool packed = false;
 
@@ -240,6 +243,7 @@ gdws_status_t f32_fused(gdws_plan_s *p, const gdws_tensor_t *x, const float *dw_
                         const float *bias, gdws_tensor_t *y, cudaStream_t s);
 
 // pack.cu
+constexpr int kFoldPackD = 4;      // output channels x 64 input channels per packing block
 gdws_status_t bf16_pack(gdws_plan_s *p, const void *dw_w, const void *pw_w, const float *bias,
                         gdws_dtype_t dtype, cudaStream_t s);
 

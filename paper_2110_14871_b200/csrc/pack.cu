@@ -8,7 +8,7 @@
 namespace gdws {
 
 constexpr int kPackThreads = 256, kPackPiece = 2048;     // elements of a block where the output is a flat array
-constexpr int kFoldPackPer = 1, kFoldPackD = 4 * kFoldPackPer, kFoldPackTaps = 9;
+constexpr int kFoldPackTaps = 9, kFoldPackBatch = 5;
 enum { kPackImg, kPackTaps, kPackBias, kPackFilt, kPackSlab, kPackFold, kPackParts };
 
 struct PackParams {
@@ -25,8 +25,9 @@ struct PackParams {
     const TcChunk *tc_chunks;
     int tc_nchunks, tc_nslabs, tc_dloc, tc_nparts, rec_hw;
     uint16_t *tc_filt, *tc_pw;
-    int fold_dblocks, fold_dp;
+    int fold_dblocks, fold_dp, fold_blocks, fold_sum_step;
     uint16_t *fold;
+    float2 *fold_sums;
 };
 
 __device__ __forceinline__ float load_weight(const void *w, size_t idx, int is_bf16)
@@ -112,74 +113,62 @@ __device__ void pack_slab(const PackParams &P, int idx)
     }
 }
 
-// Rounds a filter's taps to bf16, each to one of its two neighbours, so that the taps' sum keeps its value as far as the taps
-// with a fraction of at least kFlip of their spacing allow.  Activations have a mean: rounding every tap to its nearest
-// neighbour alone lets the errors of a filter add up on it.  (Relative error of y before its own rounding, 64 -> 64 channels:
-// inputs with a large mean 1.5e-3 -> 4e-4, half-rectified 1.64e-3 -> 1.5e-3, without a mean 1.66e-3 -> 1.8e-3.)
-constexpr float kFlip = 0.25f;
-template <int T> __device__ __forceinline__ void round_taps(float (&v)[T])
-{
-    float q[T], sum = 0.f;
-#pragma unroll
-    for (int t = 0; t < T; ++t) {
-        q[t] = bf16_bits_to_float(float_to_bf16_bits(v[t]));
-        sum += v[t] - q[t];
-    }
-#pragma unroll 1
-    for (int it = 0; it < 3; ++it) {
-        float best = fabsf(sum), step = 0.f;
-        int which = -1;
-#pragma unroll
-        for (int t = 0; t < T; ++t) {
-            const float e = v[t] - q[t];
-            const float u = __uint_as_float(__float_as_uint(v[t]) & 0x7F800000u) * 0.0078125f;     // spacing of bf16 values around v
-            const float left = fabsf(sum - copysignf(u, e));
-            if (e * sum > 0.f && fabsf(e) >= kFlip * u && left < best) { best = left; which = t; step = copysignf(u, e); }
-        }
-        if (which < 0) break;
-        sum -= step;
-#pragma unroll
-        for (int t = 0; t < T; ++t)
-            if (t == which) q[t] += step;
-    }
-#pragma unroll
-    for (int t = 0; t < T; ++t) v[t] = q[t];
-}
-
-// Folded filters: W[d,c,tap] = sum_j P[d, off_c+j] K[off_c+j, tap] in fp32, rounded to bf16 once (round_taps).  Rows are (window of 64
-// input channels, tap, output channel), 64 input channels each; rows d >= D and channels >= C are zero.  A block takes one
-// window and 4 output channels: thread = one channel x one output channel, up to 9 taps at a time in registers.  (Four
-// output channels per thread read a tap once for all four, but left a 72 -> 120 layer 16 blocks: 5 us slower.)
+// Folded filters: W[d,c,tap] = sum_j P[d, off_c+j] K[off_c+j, tap] in fp32, as two bf16 terms: W rounded to nearest, and what
+// that leaves over rounded to nearest.  Rows are (term, window of 64 input channels, tap, output channel), 64 input channels
+// each; rows d >= D and channels >= C are zero.  A block takes one window and 4 output channels: thread = one channel x one
+// output channel, up to 9 taps of 5 filters at a time in registers, their loads in flight together.  (Four output channels per
+// thread read a tap once for all four, but left a 72 -> 120 layer 16 blocks: 5 us slower.)
+// Beside them, per block (or every n-th): the sum of the squared taps and of the filters' squared tap sums, from which the
+// forward decides whether it takes the second term.
 __device__ void pack_fold(const PackParams &P, int idx)
 {
-    const int win = idx / P.fold_dblocks, cl = threadIdx.x & 63, c = win * 64 + cl;
-    const int d0 = (idx - win * P.fold_dblocks) * kFoldPackD + (threadIdx.x >> 6) * kFoldPackPer;
-    const int i0 = c < P.C ? P.off[c] : 0, i1 = c < P.C ? P.off[c + 1] : 0;
+    const int win = idx / P.fold_dblocks, group = idx - win * P.fold_dblocks, cl = threadIdx.x & 63, c = win * 64 + cl;
+    const int d = group * kFoldPackD + (threadIdx.x >> 6);
+    const int i0 = c < P.C ? P.off[c] : 0, i1 = c < P.C && d < P.D ? P.off[c + 1] : i0;
     auto weight = [&](const void *w, size_t i) {          // the two-stage kernels use the weights rounded to bf16 as well
         return P.is_bf16 ? bf16_bits_to_float(((const uint16_t *)w)[i]) : bf16_bits_to_float(float_to_bf16_bits(((const float *)w)[i]));
     };
+    const size_t term = (size_t)P.fold_dp * (P.fold_blocks / P.fold_dblocks) * P.k2 * 64;
+    float energy = 0.f, sum = 0.f;
     for (int t0 = 0; t0 < P.k2; t0 += kFoldPackTaps) {
-        float acc[kFoldPackPer][kFoldPackTaps] = {};
-#pragma unroll 4
-        for (int i = i0; i < i1; ++i) {
-            float p[kFoldPackPer];
+        float acc[kFoldPackTaps] = {};
+#pragma unroll 1
+        for (int i = i0; i < i1; i += kFoldPackBatch) {
+            float p[kFoldPackBatch], v[kFoldPackBatch][kFoldPackTaps];
 #pragma unroll
-            for (int e = 0; e < kFoldPackPer; ++e) p[e] = d0 + e < P.D ? weight(P.pw, (size_t)(d0 + e) * P.G + i) : 0.f;
+            for (int j = 0; j < kFoldPackBatch; ++j) {
+                p[j] = i + j < i1 ? weight(P.pw, (size_t)d * P.G + i + j) : 0.f;
 #pragma unroll
-            for (int t = 0; t < kFoldPackTaps; ++t) {
-                const float v = t0 + t < P.k2 ? weight(P.dw, (size_t)i * P.k2 + t0 + t) : 0.f;
-#pragma unroll
-                for (int e = 0; e < kFoldPackPer; ++e) acc[e][t] = fmaf(p[e], v, acc[e][t]);
+                for (int t = 0; t < kFoldPackTaps; ++t) v[j][t] = i + j < i1 && t0 + t < P.k2 ? weight(P.dw, (size_t)(i + j) * P.k2 + t0 + t) : 0.f;
             }
+#pragma unroll
+            for (int j = 0; j < kFoldPackBatch; ++j)
+#pragma unroll
+                for (int t = 0; t < kFoldPackTaps; ++t) acc[t] = fmaf(p[j], v[j][t], acc[t]);
         }
 #pragma unroll
-        for (int e = 0; e < kFoldPackPer; ++e) round_taps(acc[e]);      // taps beyond the filter are zeros and stay so
-#pragma unroll
         for (int t = 0; t < kFoldPackTaps; ++t)
-            if (t0 + t < P.k2)
+            if (t0 + t < P.k2) {
+                uint16_t *out = P.fold + (((size_t)win * P.k2 + t0 + t) * P.fold_dp + d) * 64 + cl;
+                const uint16_t hi = float_to_bf16_bits(acc[t]);
+                out[0] = hi;
+                out[term] = float_to_bf16_bits(acc[t] - bf16_bits_to_float(hi));
+                energy = fmaf(acc[t], acc[t], energy);
+                sum += acc[t];
+            }
+    }
+    if (group % P.fold_sum_step) return;
+    __shared__ float2 part[kPackThreads / 32];
+    float2 v = make_float2(energy, sum * sum);
 #pragma unroll
-                for (int e = 0; e < kFoldPackPer; ++e)
-                    if (d0 + e < P.fold_dp) P.fold[(((size_t)win * P.k2 + t0 + t) * P.fold_dp + d0 + e) * 64 + cl] = float_to_bf16_bits(acc[e][t]);
+    for (int o = 16; o; o >>= 1) { v.x += __shfl_xor_sync(0xffffffffu, v.x, o); v.y += __shfl_xor_sync(0xffffffffu, v.y, o); }
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        v = part[0];
+#pragma unroll
+        for (int w = 1; w < kPackThreads / 32; ++w) { v.x += part[w].x; v.y += part[w].y; }
+        P.fold_sums[win * ((P.fold_dblocks + P.fold_sum_step - 1) / P.fold_sum_step) + group / P.fold_sum_step] = v;
     }
 }
 
@@ -208,14 +197,15 @@ gdws_status_t bf16_pack(gdws_plan_s *p, const void *dw_w, const void *pw_w, cons
     P.pw_img = p->d_pw_img; P.taps = p->d_dw; P.dwpack = p->d_dwpack; P.bias_out = p->d_bias;
     P.tc_chunks = p->d_tc_chunks; P.tc_nchunks = (int)p->tc_chunks.size(); P.tc_nslabs = p->tc_nslabs; P.tc_dloc = p->tc_dloc;
     P.tc_nparts = p->tc_nparts; P.rec_hw = p->tc_rec_hw; P.tc_filt = p->d_tc_filt; P.tc_pw = p->d_tc_pw;
-    P.fold_dblocks = (p->fold_dp + kFoldPackD - 1) / kFoldPackD; P.fold_dp = p->fold_dp; P.fold = p->d_fold;
+    P.fold_dblocks = p->fold_dp / kFoldPackD; P.fold_dp = p->fold_dp; P.fold_blocks = p->fold_blocks; P.fold = p->d_fold;
+    P.fold_sum_step = p->fold_sum_step; P.fold_sums = p->d_fold_sums;
     const long long blocks[kPackParts] = {
         ((long long)p->nchunks * p->Dpad * kChunk + kPackPiece - 1) / kPackPiece,
         (p->Gpad * (long long)p->wstride + kPackPiece - 1) / kPackPiece,
         (p->Dpad + kPackThreads - 1) / kPackThreads,
         p->tc_ok ? (long long)p->tc_chunks.size() : 0,
         p->tc_ok ? (long long)p->tc_nslabs * p->tc_nparts : 0,
-        p->fold_ok ? (long long)p->fold_nwin * P.fold_dblocks : 0,
+        p->fold_ok ? (long long)p->fold_blocks : 0,
     };
     long long total = 0;
     for (int i = 0; i < kPackParts; ++i) {

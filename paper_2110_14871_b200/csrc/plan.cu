@@ -63,6 +63,7 @@ static void free_device(gdws_plan_s *p)
     p->d_dw = p->d_bias = nullptr;
     p->d_dwpack = nullptr;
     p->d_pw_img = p->d_tc_filt = p->d_tc_pw = p->d_fold = nullptr;
+    p->d_fold_sums = nullptr;
     p->d_tc_chunks = nullptr;
     p->d_status = nullptr;
     for (auto &c : p->launch_cache) c.reset();     // prepared launches hold the pointers
@@ -112,7 +113,10 @@ gdws_status_t ensure_device(gdws_plan_s *p)
             place(p->d_tc_filt, sizeof(uint16_t) * (size_t)p->tc_nslabs * 16 * p->tc_rec_hw);
             place(p->d_tc_pw, sizeof(uint16_t) * (size_t)p->tc_nparts * p->tc_nslabs * 16 * p->tc_dloc);
         }
-        if (p->fold_ok) place(p->d_fold, sizeof(uint16_t) * (size_t)p->fold_nwin * k2 * p->fold_dp * 64);
+        if (p->fold_ok) {
+            place(p->d_fold, 2 * sizeof(uint16_t) * (size_t)p->fold_nwin * k2 * p->fold_dp * 64);
+            place(p->d_fold_sums, sizeof(float2) * (size_t)p->fold_nsums);
+        }
     } catch (...) {
         return fail(GDWS_ERR_ALLOC, "out of host memory");
     }
@@ -390,7 +394,16 @@ gdws_status_t gdws_plan(int C, int D, int k, int stride, int pad, const int32_t 
     }
     p->fold_nwin = (C + 63) / 64;
     p->fold_dp = round_up(D, 32);
-    // the folded filters (2 C k^2 D bytes) have to be worth their memory; 64 MB hold 1024 x 1024 channels of 5 x 5 filters
+    {
+        // Sums for the choice between one and two terms: from every window, and from as many of its output channels as keep them
+        // at some 256, which a warp reads at once.  (What they look for is a matter of the depthwise filters, and those of a
+        // window go into all output channels.)
+        const int groups = p->fold_dp / kFoldPackD, most = std::max(1, 256 / p->fold_nwin);
+        p->fold_blocks = p->fold_nwin * groups;
+        p->fold_sum_step = (groups + most - 1) / most;
+        p->fold_nsums = p->fold_nwin * ((groups + p->fold_sum_step - 1) / p->fold_sum_step);
+    }
+    // the folded filters (2 C k^2 D bytes a term) have to be worth their memory; 64 MB hold 1024 x 1024 channels of 5 x 5 filters
     p->fold_ok = stride <= 2 && k <= 5 && C % 8 == 0 && D % 8 == 0 && (size_t)p->fold_nwin * k * k * p->fold_dp * 128 <= ((size_t)64 << 20);
     int ndev = 0;
     if (cudaGetDeviceCount(&ndev) == cudaSuccess && ndev > 0) {

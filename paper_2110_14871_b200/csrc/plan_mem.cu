@@ -16,7 +16,7 @@ namespace gdws {
 
 namespace {
 
-constexpr size_t kSlabBytes = (size_t)16 << 20, kPlanMemLargest = (size_t)8 << 20;
+constexpr size_t kSlabBytes = (size_t)32 << 20, kPlanMemLargest = (size_t)16 << 20;
 
 struct Slab {
     int device = 0;

@@ -1,6 +1,6 @@
 """The folded form of the bf16 forward (one k x k convolution with filters formed at pack time) against the CPU reference.
 The reference takes the two stages in fp64; the kernel rounds each folded filter tap to bf16 once (relative error up to
-2^-9) where the two-stage kernels round z, and both round y: the bound of the other bf16 kernels, 1e-2, applies."""
+2^-8) where the two-stage kernels round z, and both round y: the bound of the other bf16 kernels, 1e-2, applies."""
 import numpy as np
 import pytest
 import torch
@@ -80,9 +80,9 @@ def test_folded_refuses_what_it_does_not_cover():
 
 
 def test_folded_filters_keep_their_sums_on_inputs_with_a_mean():
-    """Inputs of mean 4 and unit spread.  The nearest bf16 neighbour of every tap alone would let a filter's rounding errors
-    add up on the mean; with the taps' sums kept, the result is no worse than the two-stage kernels' (which round z).  Both
-    are compared with the reference in the 2-norm, where y's own rounding (2^-9 / sqrt(3) of each value) dominates."""
+    """Inputs of mean 4 and unit spread, ordinary filters: what their taps' rounding adds on the mean is no more than what
+    rounding z adds in the two-stage kernels.  Both are compared with the reference in the 2-norm, where y's own rounding
+    (up to 2^-8 / sqrt(3) of each value) dominates."""
     spec = small_spec("t", 3, 64, 64, 20, 20, 3, 1, 0, ("uniform", 3, 7), "bf16", "NHWC", seed=53)
     data = gi.make_layer(spec)
     data.x = gi.round_to_bf16(data.x + 4.0)
