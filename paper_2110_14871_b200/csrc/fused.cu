@@ -337,9 +337,9 @@ __device__ __forceinline__ void dw_quads_k3(const DwShare &sh, uint32_t xs, int 
 }
 
 // ---- depthwise, any k and stride: one pixel group at a time.
-template <int K, bool ZOUT>
+template <int K>
 __device__ __forceinline__ void dw_generic(const FusedParams &P, uint32_t xs, int clb, uint32_t wsm, int kk,
-                                           int run, bool live_i, uint32_t a_stage, uint16_t *z, int n0, int ho0, int wo0)
+                                           int run, bool live_i, uint32_t a_stage)
 {
     const int hw = P.PH * P.PW;
 #pragma unroll 1
@@ -368,16 +368,7 @@ __device__ __forceinline__ void dw_generic(const FusedParams &P, uint32_t xs, in
                 out[e] = acc;
             }
         }
-        if (!ZOUT) {
-            store_group(P, a_stage, o, kk, out);
-        } else {
-#pragma unroll 1
-            for (int e = 0; e < 8; ++e) {
-                const int r = r0 + e, t2 = r / hw, rem = r - t2 * hw, ph = rem / P.PW, n = n0 + t2, ho = ho0 + ph, wo = wo0 + rem - ph * P.PW;
-                if (t2 < P.TN && n < P.N && ho < P.Ho && wo < P.Wo)
-                    z[(((size_t)n * P.Ho + ho) * P.Wo + wo) * P.Dtot] = float_to_bf16_bits(out[e]);
-            }
-        }
+        store_group(P, a_stage, o, kk, out);
     }
 }
 
@@ -407,15 +398,18 @@ __device__ __forceinline__ void epilogue_row(const FusedParams &P, uint32_t t_ba
 
 // MODE: 0 generic, 1 row runs (k=3), 2 4-wide patches (k=3); S = stride and PS = bytes per staged
 // pixel for modes 1/2 (mode 0 reads both from the parameters).
-// ZOUT = true turns the kernel into the unfused GDW stage: the depthwise warps write z[pixel][Gpad] in global memory from
-// their registers; no weights are streamed, no MMA is issued, no TMEM and no operand stages are used, and the control and
-// epilogue warps other than the input loader and the gate warp have nothing to do.  P.y then points to z and P.Dtot holds
-// Gpad.  (z through operand stages and a second set of warps: 58 us for 64 -> G = 189 channels, 64 x 56 x 56.)
+// ZOUT = true turns the kernel into the unfused GDW stage: z[pixel][Gpad] goes to global memory; no weights are streamed, no MMA
+// is issued and no TMEM is used.  P.y then points to z and P.Dtot holds Gpad.  In modes 1 and 2 (ZREG) the depthwise warps write
+// z from their registers, there are no operand stages, and the control and epilogue warps other than the input loader and the
+// gate warp have nothing to do (58 -> 47 us for 64 -> G = 189 channels, 64 x 56 x 56).  In mode 0 (ZSTAGE) they write
+// channel-contiguous stages, and the four epilogue warps copy each finished stage to z, 128 contiguous bytes per pixel and
+// chunk: a pixel's coordinates take divisions there, which cost more than the stages (496 channels, 76 x 58, stride 3: 116 us for
+// both stages of the layer, 264 with 2-byte stores from registers; 288 channels, k = 1, 16 x 24 x 20: 189 and 355).
 // VAR: 0 the fused kernel, 1 ZOUT, 2 the fused kernel with several blocks per tile (P.nsplit > 1).
 template <int K, int MODE, int S, int PS, int VAR>
 __global__ void __launch_bounds__(kFusedThreads, 1) fused_bf16_kernel(const __grid_constant__ FusedParams P)
 {
-    constexpr bool ZOUT = VAR == 1, SPLIT = VAR == 2;
+    constexpr bool ZOUT = VAR == 1, ZREG = ZOUT && MODE != 0, ZSTAGE = ZOUT && MODE == 0, SPLIT = VAR == 2;
     extern __shared__ uint8_t smem_raw[];
     // a_free[4] | b_full[8] b_free[8] | x_full[8] x_free[8] | acc_full[2] acc_free[2] | w_full[8] w_free[8] | open[4] | drain
     __shared__ __align__(8) uint64_t bars[4 + 2 * kMaxBUnits + 2 * kMaxSlots + 4 + 2 * kMaxSlots + 4 + 1];
@@ -432,7 +426,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) fused_bf16_kernel(const __gr
     (void)part; (void)bid; (void)nblocks
     uint8_t *base = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const uint32_t a_s = smem_u32(base);
-    const uint32_t o_s = a_s + (ZOUT ? 0u : 32768u << P.spg_shift);   // after the one or two operand stages per depthwise group: output staging
+    const uint32_t o_s = a_s + (ZREG ? 0u : 32768u << P.spg_shift);   // after the one or two operand stages per depthwise group: output staging
     const uint32_t b_s = o_s + (uint32_t)P.ostage;
     const uint32_t x_s = b_s + (uint32_t)P.nsb * P.unit_bytes;
     const uint32_t bar_afree = smem_u32(&bars[0]);
@@ -456,7 +450,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) fused_bf16_kernel(const __gr
         const int i = tid - 32;
         if (i >= 0 && i < 8) {
             if (i < 4) {
-                mbar_init(bar_afree + 8 * i, 1);
+                mbar_init(bar_afree + 8 * i, ZSTAGE ? kEpiWarps : 1);
                 mbar_init(bar_open + 8 * i, 1);
             }
             if (i < 2) {
@@ -633,7 +627,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) fused_bf16_kernel(const __gr
             // is free again, then completes a phase of the group's "open" barrier (two per group, alternating).
             // Each depthwise warp checks that one barrier before a chunk, on its own: the warps of a group do
             // not wait for one another.  An "open" barrier is used again two chunks of the group later; by then
-            // the stage wait has shown that every warp of the group is past its earlier use.  (ZOUT: the ring of filter
+            // the stage wait has shown that every warp of the group is past its earlier use.  (ZREG: the ring of filter
             // blocks is exactly four long, so that this chunk's filters land only after the group released those of its
             // chunk before last.)
             uint32_t wslot = 0, wpar = 0;
@@ -649,7 +643,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) fused_bf16_kernel(const __gr
                         if (++xs_next == (uint32_t)P.nslots) { xs_next = 0; xp_next ^= 1; }
                         mbar_wait_relaxed_call<kPollNs>(bar_xfull + 8 * xs_cur, xp_cur, &abort_flag, P.status, kStatusWaitOperand);
                     }
-                    if (!ZOUT && (k >> P.spg_shift) >= 1) {
+                    if (!ZREG && (k >> P.spg_shift) >= 1) {
                         const uint32_t sa = ((uint32_t)g << P.spg_shift) + ((uint32_t)k & ((1u << P.spg_shift) - 1u));
                         mbar_wait_relaxed_call<kPollNs>(bar_afree + 8 * sa, ((k >> P.spg_shift) - 1) & 1, &abort_flag, P.status, kStatusWaitStage);
                     }
@@ -669,7 +663,8 @@ __global__ void __launch_bounds__(kFusedThreads, 1) fused_bf16_kernel(const __gr
         const int tn = r / hw;
         const int rem = r - tn * hw;
         const int ph = rem / P.PW, pw_ = rem - (rem / P.PW) * P.PW;
-        for (int tl = ZOUT ? my_tiles : 0; tl < my_tiles; ++tl) {
+        int wq = 0;                                       // ZSTAGE: running index of the next finished chunk
+        for (int tl = ZREG ? my_tiles : 0; tl < my_tiles; ++tl) {
             int tile = bid + tl * nblocks;
             const int bn = fdiv31(tile, P.dv_thw);
             tile -= bn * tiles_hw;
@@ -677,6 +672,24 @@ __global__ void __launch_bounds__(kFusedThreads, 1) fused_bf16_kernel(const __gr
             const int n = bn * P.TN + tn, ho = bh * P.PH + ph, wo = bw * P.PW + pw_;
             const bool live = tn < P.TN && n < P.N && ho < P.Ho && wo < P.Wo;
             const size_t yrow = (((size_t)n * P.Ho + ho) * P.Wo + wo) * P.Dtot + part * P.Dpad;   // element index of the row's first channel
+            if (ZSTAGE) {
+                // this thread's pixel row of every finished stage goes to z (row r of the stage: 128 bytes, swizzled)
+                for (int q = 0; q < P.nchunks; ++q, ++wq) {
+                    named_bar_sync(kBarChunk0 + (wq & 3), kDwGroupWarps * 32 + kEpiWarps * 32);   // chunk wq is written
+                    const uint32_t sa = ((uint32_t)(wq & 1) << P.spg_shift) + ((uint32_t)(wq >> 1) & ((1u << P.spg_shift) - 1u));
+                    const uint32_t row_s = a_s + sa * 16384 + (uint32_t)r * 128;
+                    uint4 v[8];
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) v[c] = lds128(row_s + (uint32_t)((c ^ (r & 7)) << 4));
+                    warp_arrive(bar_afree + 8 * sa);
+                    if (live) {
+                        uint4 *dst = reinterpret_cast<uint4 *>(P.y + yrow + (size_t)q * kChunk);
+#pragma unroll
+                        for (int c = 0; c < 8; ++c) dst[c] = v[c];
+                    }
+                }
+                continue;
+            }
             const int buf = tl & (P.nacc - 1);            // one or two accumulators
             warp_wait(bar_accfull + 8 * buf, (tl >> (P.nacc - 1)) & 1, &abort_flag, P.status, kStatusWaitMma);
             tc_fence_after();
@@ -740,8 +753,8 @@ __global__ void __launch_bounds__(kFusedThreads, 1) fused_bf16_kernel(const __gr
         // hand-over barrier, where the consumer waits.  A hand-over barrier is used again four chunks later, by the same group
         // and for the same stage (two chunks later with one stage per group); by then the gate warp has seen
         // that stage released, hence the consumer past the barrier.
-        int tl = 0;                                       // ZOUT: the chunk's tile
-        if (ZOUT) for (int j = g; j >= P.nchunks; j -= P.nchunks) ++tl;
+        int tl = 0;                                       // ZREG: the chunk's tile
+        if (ZREG) for (int j = g; j >= P.nchunks; j -= P.nchunks) ++tl;
         for (int gq = g, k = 0; gq < total_chunks; gq += 2, ++k) {
             const bool live_i = q * kChunk + il < P.G;
             const uint32_t sa = ((uint32_t)g << P.spg_shift) + ((uint32_t)k & ((1u << P.spg_shift) - 1u));   // this chunk's stage
@@ -770,7 +783,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) fused_bf16_kernel(const __gr
             int n0 = 0, ho0 = 0, wo0 = 0;
             uint16_t *zc = nullptr;
             ZShare zs = {};
-            if (ZOUT) {
+            if (ZREG) {
                 GDWS_BLOCK_SHARE;
                 int tile = bid + tl * nblocks;
                 const int bn = fdiv31(tile, P.dv_thw);
@@ -789,7 +802,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) fused_bf16_kernel(const __gr
             }
             if (MODE == 1) dw_rows<K, S, PS, ZOUT>(share, xs, clb, w, live_i, a_stage, zs);
             else if (MODE == 2) dw_quads_k3<S, PS, ZOUT>(share, xs, clb, reinterpret_cast<const uint32_t (&)[9]>(w), live_i, a_stage, P, zc, n0, run, ho0, wo0);
-            else dw_generic<K, ZOUT>(P, xs, clb, wsm, il, run, live_i, a_stage, zc, n0, ho0, wo0);
+            else dw_generic<K>(P, xs, clb, wsm, il, run, live_i, a_stage);
             if (!ZOUT) fence_proxy_async();      // every thread: its own writes become visible to the tensor-core proxy
             __syncwarp();
             if (lane == 0) {          // this warp is done with the chunk's filters and input box
@@ -799,7 +812,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) fused_bf16_kernel(const __gr
                 if (flags & 2) mbar_arrive(bar_xfree + 8 * xslot);
             }
             __syncwarp();
-            if (!ZOUT) named_bar_arrive(kBarChunk0 + (gq & 3), kDwGroupWarps * 32 + 32);
+            if (!ZREG) named_bar_arrive(kBarChunk0 + (gq & 3), kDwGroupWarps * 32 + (ZSTAGE ? kEpiWarps * 32 : 32));
             q += 2;
             while (q >= P.nchunks) { q -= P.nchunks; ++tl; }
             wslot += 2;
@@ -926,7 +939,7 @@ static gdws_status_t alu_prepare(gdws_plan_s *p, int n, int h, int w, int Ho, in
         };
         magic(t.tiles_h * t.tiles_w, P.dv_thw); magic(t.tiles_w, P.dv_tw);
     }
-    if (zout) {      // no weight units and operand stages; exactly four filter blocks (see the gate warp)
+    if (zout && t.fast) {      // z from registers: no weight units and operand stages; exactly four filter blocks (see the gate warp)
         t.nsb = 0; t.nwslots = 4;
         t.smem = 1024 + (size_t)t.nslots * t.slot_bytes + (size_t)t.nwslots * kChunk * p->wstride * 4 + (size_t)p->nchunks * 16 + (size_t)Dloc * 4;
         if (t.smem < (size_t)kMaxSmem / 2 + 2048) t.smem = (size_t)kMaxSmem / 2 + 2048;
