@@ -94,17 +94,65 @@ bool pinned(const void *ptr)
     return a.type == cudaMemoryTypeHost;
 }
 
+// Images of a piece (all but the first one) and of the first: the first and the last piece, whose copies nothing overlaps, are
+// half as large as the others.
+void piece_sizes(int n, int pieces, size_t ximg, size_t yimg, int *per, int *first)
+{
+    *per = pieces == 2 ? (n + 1) / 2 : (n + pieces - 2) / (pieces - 1);
+    *first = pieces == 2 ? *per : (*per + 1) / 2;
+    int unit = 1;                // images that are whole 16-byte pieces of x and of y: every piece starts on such a boundary
+    while ((unit * ximg) % 16 || (unit * yimg) % 16) unit *= 2;
+    *per = (*per + unit - 1) / unit * unit;
+    *first = (*first + unit - 1) / unit * unit;
+}
+
+struct PieceChoice {
+    LaunchKey key;
+    int pieces = 1;
+};
+
 // Pieces that gdws_forward_host takes a batch in: 1 (as a whole) for pageable memory, whose copies the host waits for
 // anyway, and for small ones.  A piece costs some 10 us, and of n pieces the first copy in and the last copy out overlap
-// nothing (measured, MB each way: 2.1 best with 2, 8.4 with 3, 33 with 5: 423 -> 292 us for 8.4).
-int host_pieces(const gdws_plan_s *p, const gdws_tensor_t *xh, const gdws_tensor_t *yh, size_t xb, size_t yb)
+// nothing (measured, MB each way: 2.1 best with 2, 8.4 with 3, 33 with 5: 350 -> 290 us for 8.4).  Fewer where the estimated time
+// is a tenth shorter: a layer whose forward does not get shorter with fewer images takes that time once per piece (3 images of
+// 400 -> 400 channels, 7 x 7 filters, 38 tiles: 1340 us as a whole, 2609 in two pieces).
+int host_pieces(gdws_plan_s *p, const gdws_tensor_t *xh, const gdws_tensor_t *yh, size_t xb, size_t yb)
 {
     const size_t mb = std::max(xb, yb) >> 20;
-    const int n = std::min(xh->n, mb >= 28 ? kHostPieces : (mb >= 16 ? 4 : (mb >= 6 ? 3 : (mb >= 2 ? 2 : 1))));
-    if (n < 2 || xh->n != yh->n || !pinned(xh->ptr) || !pinned(yh->ptr)) return 1;
+    const int most = std::min(xh->n, mb >= 28 ? kHostPieces : (mb >= 16 ? 4 : (mb >= 6 ? 3 : (mb >= 2 ? 2 : 1))));
+    if (most < 2 || xh->n != yh->n || !pinned(xh->ptr) || !pinned(yh->ptr)) return 1;
     // a workspace that does not hold the whole batch is refused where it is needed, even if it would hold a piece
     if ((p->opt_path == GDWS_PATH_UNFUSED || (p->opt_path == GDWS_PATH_AUTO && p->ws)) && p->ws_bytes < gdws_workspace_bytes(p, xh->dtype, xh->n, xh->h, xh->w)) return 1;
-    return n;
+    const bool f32 = xh->dtype == GDWS_F32;
+    const LaunchKey key = {xh->n, xh->h, xh->w, (f32 ? 1 : 0) | (p->opt_out_f32 ? 2 : 0) | p->opt_path << 2 | p->opt_dw_math << 4};
+    if (const PieceChoice *c = LaunchCache<PieceChoice>::find(p->launch_cache[4], key)) return c->pieces;
+    auto forward_us = [&](int n) { return f32 ? f32_forward_us(p, n, xh->h, xh->w) : bf16_forward_us(p, n, xh->h, xh->w, p->opt_out_f32 != 0); };
+    const double ximg = (double)xb / xh->n, yimg = (double)yb / xh->n;
+    const double link = 18e-6, link_both = link + 4e-6 * std::min(ximg, yimg) / std::max(ximg, yimg);      // us per byte, one direction alone and with the other one busy
+    int best = 0;
+    double best_us = 0;
+    for (int pieces = most; pieces >= 1; --pieces) {
+        double in = 0, done = 0, out = 0;
+        if (pieces == 1) {
+            out = (xb + yb) * link + forward_us(xh->n);
+        } else {
+            int per, first;
+            piece_sizes(xh->n, pieces, xb / xh->n, yb / xh->n, &per, &first);
+            for (int i = 0, n0 = 0, n = 0; n0 < xh->n; ++i, n0 += n) {
+                n = std::min(i == 0 ? first : per, xh->n - n0);
+                in += n * ximg * link_both + 3.0;
+                done = std::max(in, done) + forward_us(n) + 2.0;
+                out = std::max(done, out) + n * yimg * link_both + 3.0;
+            }
+        }
+        if (!best || out < 0.9 * best_us) { best_us = out; best = pieces; }
+    }
+    if (std::unique_ptr<PieceChoice> c{new (std::nothrow) PieceChoice}) {
+        c->key = key;
+        c->pieces = best;
+        LaunchCache<PieceChoice>::add(p->launch_cache[4], std::move(c));
+    }
+    return best;
 }
 
 gdws_status_t forward_pieces(gdws_plan_s *p, HostPipe *pipe, const gdws_tensor_t *xh, const gdws_tensor_t *xd, const void *dw_w, const void *pw_w, const float *bias,
@@ -114,12 +162,8 @@ gdws_status_t forward_pieces(gdws_plan_s *p, HostPipe *pipe, const gdws_tensor_t
     // the copies start after what is on the caller's stream
     cudaError_t e = cudaEventRecord(pipe->begin, cs);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(pipe->in, pipe->begin, 0);
-    // the first and the last piece, whose copies nothing overlaps, half as large as the others
-    int per = pieces == 2 ? (xh->n + 1) / 2 : (xh->n + pieces - 2) / (pieces - 1), first = pieces == 2 ? per : (per + 1) / 2;
-    int unit = 1;                // images that are whole 16-byte pieces of x and of y: every piece starts on such a boundary
-    while ((unit * ximg) % 16 || (unit * yimg) % 16) unit *= 2;
-    per = (per + unit - 1) / unit * unit;
-    first = (first + unit - 1) / unit * unit;
+    int per, first;
+    piece_sizes(xh->n, pieces, ximg, yimg, &per, &first);
     for (int i = 0, n0 = 0, n = 0; n0 < xh->n && e == cudaSuccess; ++i, n0 += n) {
         n = std::min(i == 0 ? first : per, xh->n - n0);
         cudaEvent_t in = pipe->copied[i], done = pipe->computed[i];
@@ -266,7 +310,7 @@ gdws_status_t gdws_forward_host(gdws_plan_t *p, const gdws_tensor_t *xh, const v
     yd.ptr = p->stage_y;
     // Images are independent and contiguous: with both buffers pinned the batch goes through in pieces, so that a piece's
     // copy in, the forward of the one before and the copy out of an earlier one run at the same time (the link carries both
-    // directions at once; 8.4 MB each way: 354 us one after the other, the link's time for one direction is 150).
+    // directions at once; 8.4 MB each way: 350 us one after the other, the link's time for one direction is 150).
     const int pieces = host_pieces(p, xh, yh, xb, yb);
     if (HostPipe *pipe = pieces > 1 ? host_pipe_take(p->device) : nullptr) {
         st = check_pair(p, &xd, &yd);

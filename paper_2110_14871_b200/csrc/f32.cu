@@ -558,7 +558,7 @@ constexpr F32Config kF32Configs[] = {
 };
 
 // The tile whose busiest SM is done first: large tiles reuse more per load, small ones leave no SM idle.
-int f32_config(const gdws_plan_s *p, long long npix, int Wo)
+int f32_config(const gdws_plan_s *p, long long npix, int Wo, double *cycles = nullptr)
 {
     const int sms = sm_count_of(p);
     int best = 0;
@@ -576,10 +576,20 @@ int f32_config(const gdws_plan_s *p, long long npix, int Wo)
         const double cost = std::max(per_sm * per_block / f.rate, std::max(alone, per_block / (0.8 * f.rate)));
         if (cost < best_cost) { best_cost = cost; best = c; }
     }
+    if (cycles) *cycles = best_cost;
     return best_cost < 1e300 ? best : -1;
 }
 
 }  // namespace
+
+// Estimate of an fp32 forward of n images, for gdws_forward_host.
+double f32_forward_us(const gdws_plan_s *p, int n, int h, int w)
+{
+    const int Ho = gdws_out_dim(h, p->k, p->stride, p->pad), Wo = gdws_out_dim(w, p->k, p->stride, p->pad);
+    double cycles = 0;
+    f32_config(p, (long long)n * Ho * Wo, Wo, &cycles);
+    return 3.0 + cycles / 1850.0;
+}
 
 gdws_status_t f32_fused(gdws_plan_s *p, const gdws_tensor_t *x, const float *dw_w, const float *pw_w,
                         const float *bias, gdws_tensor_t *y, cudaStream_t st)

@@ -131,9 +131,9 @@ struct gdws_plan_s {
     void *stage_x = nullptr, *stage_y = nullptr;  // gdws_forward_host staging
     size_t stage_x_bytes = 0, stage_y_bytes = 0;
 
-    // Prepared launches of the three fused bf16 kernels and the choice between them (LaunchCache below; each file knows its
-    // own types).
-    std::shared_ptr<void> launch_cache[4];
+    // Prepared launches of the three fused bf16 kernels, the choice between them and the pieces of a host call (LaunchCache
+    // below; each file knows its own types).
+    std::shared_ptr<void> launch_cache[5];
 
     int64_t launches = 0;
 };
@@ -239,6 +239,7 @@ inline int sm_count_of(const gdws_plan_s *p) { return p->sm_count > 0 ? p->sm_co
 gdws_status_t f32_depthwise(gdws_plan_s *p, const gdws_tensor_t *x, const float *dw_w, float *z, cudaStream_t s);
 gdws_status_t f32_pointwise(gdws_plan_s *p, const float *z, const float *pw_w, const float *bias,
                             gdws_tensor_t *y, cudaStream_t s);
+double f32_forward_us(const gdws_plan_s *p, int n, int h, int w);
 gdws_status_t f32_fused(gdws_plan_s *p, const gdws_tensor_t *x, const float *dw_w, const float *pw_w,
                         const float *bias, gdws_tensor_t *y, cudaStream_t s);
 
@@ -258,6 +259,7 @@ gdws_status_t bf16_fused_tc(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_
 
 // fold.cu
 gdws_status_t bf16_folded(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t *y, cudaStream_t s);
+double bf16_forward_us(gdws_plan_s *p, int n, int h, int w, bool out_f32);
 int bf16_form_of(gdws_plan_s *p, int n, int h, int w, bool out_f32);   // 1 / 2: two stages, GDW on the ALUs / the tensor cores; 3: folded
 
 // Input row h = stride * ho + u - pad of filter row u (columns alike).  With stride 2 the input is read through four
