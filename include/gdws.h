@@ -117,7 +117,8 @@ typedef enum {
  * Host work: offsets off_c, the intermediate-channel -> input-channel table, the
  * padding of G to the tensor-core chunk, output-patch choice.  If a CUDA device is
  * current, the plan also allocates its device tables and packed-weight buffers
- * (O(G*(k*k+D)) bytes, and 4*C*k*k*D for the folded form where it is covered) on it; with no device the plan is still valid for the
+ * (O(G*(k*k+D)) bytes, and 4*C*k*k*D for the folded form where it is covered and they are free; ranges of 32 MB that plans of
+ * more than 512 KB and up to 16 MB share) on it; with no device the plan is still valid for the
  * host-side queries below and allocates at the first device call.
  * Errors: GDWS_ERR_INVALID_ARG, GDWS_ERR_ALLOC, GDWS_ERR_CUDA.
  */

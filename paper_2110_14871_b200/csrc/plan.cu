@@ -121,6 +121,14 @@ gdws_status_t ensure_device(gdws_plan_s *p)
         return fail(GDWS_ERR_ALLOC, "out of host memory");
     }
     e = plan_mem_alloc(dev, bytes, &p->d_arena);
+    if (e == cudaErrorMemoryAllocation && p->fold_ok) {      // no room for the folded filters (the last two places): the plan keeps to the two stages
+        cudaGetLastError();
+        places.pop_back();
+        bytes = places.back().second;
+        places.pop_back();
+        p->fold_ok = false;
+        e = plan_mem_alloc(dev, bytes, &p->d_arena);
+    }
     p->arena_bytes = bytes;
     if (e != cudaSuccess) {
         p->d_arena = nullptr;
