@@ -170,13 +170,14 @@ GDWS_API gdws_status_t gdws_plan_gdw_stage(const gdws_plan_t *plan, int *stage);
 /*
  * gdws_plan_form -- the kernel a fused bf16 forward of n x C x h x w takes with the plan's current options: *form = 1 or 2
  * (two stages, the GDW stage on the ALUs or on the tensor cores, as gdws_plan_gdw_stage) or 3 (one k x k convolution with
- * folded filters).  Host only; errors: GDWS_ERR_INVALID_ARG.
+ * folded filters).  (Weights given with a call are folded only if that call takes form 3; a later call that reuses them keeps
+ * to the two stages then.)  Host only; errors: GDWS_ERR_INVALID_ARG.
  */
 GDWS_API gdws_status_t gdws_plan_form(gdws_plan_t *plan, int n, int h, int w, int *form);
 
 /*
  * gdws_pack_weights -- convert one weight set to the kernels' internal form
- * (bf16 paths; Property 1 / 2 give the shapes).  Enqueues small kernels on `stream`.
+ * (bf16 paths; Property 1 / 2 give the shapes).  Enqueues one kernel on `stream`.
  *   dw_w   DEVICE, [G][k][k], dtype `dtype`, canonical order i = off_c + j
  *   pw_w   DEVICE, [D][G] row-major, dtype `dtype`
  *   bias   DEVICE float[D] or NULL (zero)
@@ -238,7 +239,8 @@ GDWS_API gdws_status_t gdws_pointwise(gdws_plan_t *plan, const void *z, const vo
  * gdws_forward_host -- the same forward with HOST activations: copies x_host to the
  * device, runs gdws_forward with the packed weights, copies y back, after what is on `stream`,
  * and waits for it all.  Large pinned batches go through in pieces of whole images whose copies
- * overlap with each other's forward (on two streams of the plan beside `stream`); the kernel
+ * overlap with each other's forward (on two streams beside `stream`, a set that the
+ * process's plans take turns with; as many pieces as the estimated time gains from); the kernel
  * is then the one that fits a piece (gdws_plan_form).  x_host / y_host: HOST, same dtype/layout rules as
  * gdws_forward (pinned memory makes the copies asynchronous with respect to the host).
  * The plan keeps device staging buffers that grow (cudaMalloc) when a call needs more

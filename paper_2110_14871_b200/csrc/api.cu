@@ -74,14 +74,14 @@ gdws_status_t prepare(gdws_plan_s *p)
 }
 
 gdws_status_t weights_ready(gdws_plan_s *p, const void *dw_w, const void *pw_w, const float *bias,
-                            gdws_dtype_t dtype, cudaStream_t st)
+                            gdws_dtype_t dtype, bool fold, cudaStream_t st)
 {
     if ((dw_w == nullptr) != (pw_w == nullptr))
         return fail(GDWS_ERR_INVALID_ARG, "dw_w and pw_w must both be given or both be NULL");
     if (dw_w) {
         if (!aligned16(dw_w) || !aligned16(pw_w) || (bias && ((uintptr_t)bias & 3)))
             return fail(GDWS_ERR_INVALID_ARG, "weight pointers must be 16-byte aligned");
-        return bf16_pack(p, dw_w, pw_w, bias, dtype, st);
+        return bf16_pack(p, dw_w, pw_w, bias, dtype, fold, st);
     }
     if (!p->packed) return fail(GDWS_ERR_INVALID_ARG, "no weights: pass dw_w/pw_w or call gdws_pack_weights first");
     return GDWS_OK;
@@ -198,7 +198,7 @@ gdws_status_t gdws_pack_weights(gdws_plan_t *p, const void *dw_w, const void *pw
     if (dtype != GDWS_F32 && dtype != GDWS_BF16) return fail(GDWS_ERR_INVALID_ARG, "gdws_pack_weights: bad dtype");
     gdws_status_t st = prepare(p);
     if (st != GDWS_OK) return st;
-    return weights_ready(p, dw_w, pw_w, bias, dtype, (cudaStream_t)stream);
+    return weights_ready(p, dw_w, pw_w, bias, dtype, true, (cudaStream_t)stream);
 }
 
 gdws_status_t gdws_forward(gdws_plan_t *p, const gdws_tensor_t *x, const void *dw_w, const void *pw_w,
@@ -222,7 +222,9 @@ gdws_status_t gdws_forward(gdws_plan_t *p, const gdws_tensor_t *x, const void *d
         if (st != GDWS_OK) return st;
         return f32_pointwise(p, (const float *)p->ws, (const float *)pw_w, bias, y, cs);
     }
-    st = weights_ready(p, dw_w, pw_w, bias, GDWS_BF16, cs);
+    // weights given with the call: their folded filters (up to half of the packing) are formed if this call reads them; a later
+    // call that would, with the weights left as they are, then keeps to the two stages
+    st = weights_ready(p, dw_w, pw_w, bias, GDWS_BF16, dw_w && fused && bf16_form_of(p, x->n, x->h, x->w, y->dtype == GDWS_F32) == 3, cs);
     if (st != GDWS_OK) return st;
     if (fused) {
         st = bf16_fused(p, x, y, cs);

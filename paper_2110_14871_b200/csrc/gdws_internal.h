@@ -94,7 +94,8 @@ struct gdws_plan_s {
     // Folded path (fold.cu): the layer as one k x k convolution.
     bool fold_ok = false;            // the layer is one the path covers
     int fold_nwin = 0, fold_dp = 0;  // windows of 64 input channels; output channels rounded up to 32
-    int fold_blocks = 0;             // packing blocks of the folded filters (windows x groups of kFoldPackD output channels)
+    int fold_per = 1;                // output channels per thread that packs them (1 or 4)
+    int fold_blocks = 0;             // packing blocks of the folded filters (windows x groups of 4 fold_per output channels)
     int fold_sum_step = 1, fold_nsums = 0;   // every fold_sum_step-th group of a window writes its sums, fold_nsums in all
 
     int opt_path = GDWS_PATH_AUTO;
@@ -123,7 +124,7 @@ struct gdws_plan_s {
     uint16_t *d_fold = nullptr;    // [2][fold_nwin][k*k][fold_dp][64] bf16: folded filters, then what their rounding left over
     float2 *d_fold_sums = nullptr; // [fold_nsums]: sums that decide whether a forward takes both terms
     int *d_status = nullptr;       // device status word
-    bool packed = false;
+    bool packed = false, fold_packed = false;      // the forms of the two stages; the folded filters
 
     void *ws = nullptr;
     size_t ws_bytes = 0;
@@ -244,9 +245,9 @@ gdws_status_t f32_fused(gdws_plan_s *p, const gdws_tensor_t *x, const float *dw_
                         const float *bias, gdws_tensor_t *y, cudaStream_t s);
 
 // pack.cu
-constexpr int kFoldPackD = 4;      // output channels x 64 input channels per packing block
+constexpr int kFoldPackWide = 256;   // packing blocks of 4 output channels from which on a thread takes four of them
 gdws_status_t bf16_pack(gdws_plan_s *p, const void *dw_w, const void *pw_w, const float *bias,
-                        gdws_dtype_t dtype, cudaStream_t s);
+                        gdws_dtype_t dtype, bool fold, cudaStream_t s);
 
 // bf16.cu
 gdws_status_t bf16_depthwise(gdws_plan_s *p, const gdws_tensor_t *x, void *z, cudaStream_t s);

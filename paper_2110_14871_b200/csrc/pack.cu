@@ -8,7 +8,7 @@
 namespace gdws {
 
 constexpr int kPackThreads = 256, kPackPiece = 2048;     // elements of a block where the output is a flat array
-constexpr int kFoldPackTaps = 9, kFoldPackBatch = 5;
+constexpr int kFoldPackTaps = 9;
 enum { kPackImg, kPackTaps, kPackBias, kPackFilt, kPackSlab, kPackFold, kPackParts };
 
 struct PackParams {
@@ -25,7 +25,7 @@ struct PackParams {
     const TcChunk *tc_chunks;
     int tc_nchunks, tc_nslabs, tc_dloc, tc_nparts, rec_hw;
     uint16_t *tc_filt, *tc_pw;
-    int fold_dblocks, fold_dp, fold_blocks, fold_sum_step;
+    int fold_per, fold_dblocks, fold_dp, fold_blocks, fold_sum_step;
     uint16_t *fold;
     float2 *fold_sums;
 };
@@ -115,51 +115,59 @@ __device__ void pack_slab(const PackParams &P, int idx)
 
 // Folded filters: W[d,c,tap] = sum_j P[d, off_c+j] K[off_c+j, tap] in fp32, as two bf16 terms: W rounded to nearest, and what
 // that leaves over rounded to nearest.  Rows are (term, window of 64 input channels, tap, output channel), 64 input channels
-// each; rows d >= D and channels >= C are zero.  A block takes one window and 4 output channels: thread = one channel x one
-// output channel, up to 9 taps of 5 filters at a time in registers, their loads in flight together.  (Four output channels per
-// thread read a tap once for all four, but left a 72 -> 120 layer 16 blocks: 5 us slower.)
+// each; rows d >= D and channels >= C are zero.  A block takes one window and 4 PER output channels: thread = one channel x PER
+// output channels, up to 9 taps of BATCH filters at a time in registers, their loads in flight together.  PER = 1 where blocks are
+// few (four output channels per thread left a 72 -> 120 layer 16 blocks: 5 us slower), 4 where the loads of the taps, which lie
+// far apart for neighbouring channels, take the time (kFoldPackWide).
 // Beside them, per block (or every n-th): the sum of the squared taps and of the filters' squared tap sums, from which the
 // forward decides whether it takes the second term.
-__device__ void pack_fold(const PackParams &P, int idx)
+template <int PER, int BATCH> __device__ __forceinline__ void pack_fold(const PackParams &P, int idx)
 {
     const int win = idx / P.fold_dblocks, group = idx - win * P.fold_dblocks, cl = threadIdx.x & 63, c = win * 64 + cl;
-    const int d = group * kFoldPackD + (threadIdx.x >> 6);
-    const int i0 = c < P.C ? P.off[c] : 0, i1 = c < P.C && d < P.D ? P.off[c + 1] : i0;
+    const int d0 = (group * 4 + (threadIdx.x >> 6)) * PER;
+    const int i0 = c < P.C ? P.off[c] : 0, i1 = c < P.C && d0 < P.D ? P.off[c + 1] : i0;
     auto weight = [&](const void *w, size_t i) {          // the two-stage kernels use the weights rounded to bf16 as well
         return P.is_bf16 ? bf16_bits_to_float(((const uint16_t *)w)[i]) : bf16_bits_to_float(float_to_bf16_bits(((const float *)w)[i]));
     };
     const size_t term = (size_t)P.fold_dp * (P.fold_blocks / P.fold_dblocks) * P.k2 * 64;
-    float energy = 0.f, sum = 0.f;
+    float energy = 0.f, sum[PER] = {};
     for (int t0 = 0; t0 < P.k2; t0 += kFoldPackTaps) {
-        float acc[kFoldPackTaps] = {};
+        float acc[PER][kFoldPackTaps] = {};
 #pragma unroll 1
-        for (int i = i0; i < i1; i += kFoldPackBatch) {
-            float p[kFoldPackBatch], v[kFoldPackBatch][kFoldPackTaps];
+        for (int i = i0; i < i1; i += BATCH) {
+            float p[BATCH][PER], v[BATCH][kFoldPackTaps];
 #pragma unroll
-            for (int j = 0; j < kFoldPackBatch; ++j) {
-                p[j] = i + j < i1 ? weight(P.pw, (size_t)d * P.G + i + j) : 0.f;
+            for (int j = 0; j < BATCH; ++j) {
+#pragma unroll
+                for (int e = 0; e < PER; ++e) p[j][e] = i + j < i1 && (PER == 1 || d0 + e < P.D) ? weight(P.pw, (size_t)(d0 + e) * P.G + i + j) : 0.f;
 #pragma unroll
                 for (int t = 0; t < kFoldPackTaps; ++t) v[j][t] = i + j < i1 && t0 + t < P.k2 ? weight(P.dw, (size_t)(i + j) * P.k2 + t0 + t) : 0.f;
             }
 #pragma unroll
-            for (int j = 0; j < kFoldPackBatch; ++j)
+            for (int j = 0; j < BATCH; ++j)
 #pragma unroll
-                for (int t = 0; t < kFoldPackTaps; ++t) acc[t] = fmaf(p[j], v[j][t], acc[t]);
+                for (int e = 0; e < PER; ++e)
+#pragma unroll
+                    for (int t = 0; t < kFoldPackTaps; ++t) acc[e][t] = fmaf(p[j][e], v[j][t], acc[e][t]);
         }
 #pragma unroll
         for (int t = 0; t < kFoldPackTaps; ++t)
-            if (t0 + t < P.k2) {
-                uint16_t *out = P.fold + (((size_t)win * P.k2 + t0 + t) * P.fold_dp + d) * 64 + cl;
-                const uint16_t hi = float_to_bf16_bits(acc[t]);
-                out[0] = hi;
-                out[term] = float_to_bf16_bits(acc[t] - bf16_bits_to_float(hi));
-                energy = fmaf(acc[t], acc[t], energy);
-                sum += acc[t];
-            }
+            if (t0 + t < P.k2)
+#pragma unroll
+                for (int e = 0; e < PER; ++e) {
+                    uint16_t *out = P.fold + (((size_t)win * P.k2 + t0 + t) * P.fold_dp + d0 + e) * 64 + cl;
+                    const uint16_t hi = float_to_bf16_bits(acc[e][t]);
+                    out[0] = hi;
+                    out[term] = float_to_bf16_bits(acc[e][t] - bf16_bits_to_float(hi));
+                    energy = fmaf(acc[e][t], acc[e][t], energy);
+                    sum[e] += acc[e][t];
+                }
     }
     if (group % P.fold_sum_step) return;
     __shared__ float2 part[kPackThreads / 32];
-    float2 v = make_float2(energy, sum * sum);
+    float2 v = make_float2(energy, 0.f);
+#pragma unroll
+    for (int e = 0; e < PER; ++e) v.y = fmaf(sum[e], sum[e], v.y);
 #pragma unroll
     for (int o = 16; o; o >>= 1) { v.x += __shfl_xor_sync(0xffffffffu, v.x, o); v.y += __shfl_xor_sync(0xffffffffu, v.y, o); }
     if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = v;
@@ -172,12 +180,15 @@ __device__ void pack_fold(const PackParams &P, int idx)
     }
 }
 
-__global__ void __launch_bounds__(kPackThreads) pack_kernel(const __grid_constant__ PackParams P)
+__global__ void __launch_bounds__(kPackThreads, 3) pack_kernel(const __grid_constant__ PackParams P)
 {
     grid_launch_dependents();
     grid_dependency_wait();      // the kernel before may still read what this one overwrites
     const int b = (int)blockIdx.x;
-    if (b >= P.first[kPackFold]) pack_fold(P, b - P.first[kPackFold]);
+    if (b >= P.first[kPackFold]) {
+        if (P.fold_per == 1) pack_fold<1, 5>(P, b - P.first[kPackFold]);
+        else pack_fold<4, 1>(P, b - P.first[kPackFold]);
+    }
     else if (b >= P.first[kPackSlab]) pack_slab(P, b - P.first[kPackSlab]);
     else if (b >= P.first[kPackFilt]) pack_filt(P, b - P.first[kPackFilt]);
     else if (b >= P.first[kPackBias]) {
@@ -188,8 +199,9 @@ __global__ void __launch_bounds__(kPackThreads) pack_kernel(const __grid_constan
     else pack_img(P, b);
 }
 
-gdws_status_t bf16_pack(gdws_plan_s *p, const void *dw_w, const void *pw_w, const float *bias, gdws_dtype_t dtype, cudaStream_t st)
+gdws_status_t bf16_pack(gdws_plan_s *p, const void *dw_w, const void *pw_w, const float *bias, gdws_dtype_t dtype, bool fold, cudaStream_t st)
 {
+    fold = p->fold_ok && (fold || p->opt_dw_math == 3 || p->Dpad > 512);      // beyond 512 output channels the two stages may have no kernel
     PackParams P;
     P.dw = dw_w; P.pw = pw_w; P.bias = bias; P.is_bf16 = dtype == GDWS_BF16;
     P.C = p->C; P.D = p->D; P.G = p->G; P.k2 = p->k * p->k; P.Dpad = p->Dpad; P.Gpad = p->Gpad; P.nchunks = p->nchunks; P.wstride = p->wstride;
@@ -197,7 +209,7 @@ gdws_status_t bf16_pack(gdws_plan_s *p, const void *dw_w, const void *pw_w, cons
     P.pw_img = p->d_pw_img; P.taps = p->d_dw; P.dwpack = p->d_dwpack; P.bias_out = p->d_bias;
     P.tc_chunks = p->d_tc_chunks; P.tc_nchunks = (int)p->tc_chunks.size(); P.tc_nslabs = p->tc_nslabs; P.tc_dloc = p->tc_dloc;
     P.tc_nparts = p->tc_nparts; P.rec_hw = p->tc_rec_hw; P.tc_filt = p->d_tc_filt; P.tc_pw = p->d_tc_pw;
-    P.fold_dblocks = p->fold_dp / kFoldPackD; P.fold_dp = p->fold_dp; P.fold_blocks = p->fold_blocks; P.fold = p->d_fold;
+    P.fold_per = p->fold_per; P.fold_dblocks = p->fold_dp / (4 * p->fold_per); P.fold_dp = p->fold_dp; P.fold_blocks = p->fold_blocks; P.fold = p->d_fold;
     P.fold_sum_step = p->fold_sum_step; P.fold_sums = p->d_fold_sums;
     const long long blocks[kPackParts] = {
         ((long long)p->nchunks * p->Dpad * kChunk + kPackPiece - 1) / kPackPiece,
@@ -205,7 +217,7 @@ gdws_status_t bf16_pack(gdws_plan_s *p, const void *dw_w, const void *pw_w, cons
         (p->Dpad + kPackThreads - 1) / kPackThreads,
         p->tc_ok ? (long long)p->tc_chunks.size() : 0,
         p->tc_ok ? (long long)p->tc_nslabs * p->tc_nparts : 0,
-        p->fold_ok ? (long long)p->fold_blocks : 0,
+        fold ? (long long)p->fold_blocks : 0,
     };
     long long total = 0;
     for (int i = 0; i < kPackParts; ++i) {
@@ -218,6 +230,7 @@ gdws_status_t bf16_pack(gdws_plan_s *p, const void *dw_w, const void *pw_w, cons
     if (e != cudaSuccess) { cudaGetLastError(); return cuda_fail(e, "weight pack launch"); }
     p->launches++;
     p->packed = true;
+    p->fold_packed = fold;
     return GDWS_OK;
 }
 

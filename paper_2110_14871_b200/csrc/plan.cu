@@ -71,7 +71,7 @@ static void free_device(gdws_plan_s *p)
     release(p->stage_y);
     p->stage_x_bytes = 0;
     p->stage_y_bytes = 0;
-    p->packed = false;
+    p->packed = p->fold_packed = false;
     plan_count(p->device, -1);
     cudaSetDevice(cur);
     p->device = -1;
@@ -406,7 +406,8 @@ gdws_status_t gdws_plan(int C, int D, int k, int stride, int pad, const int32_t 
         // Sums for the choice between one and two terms: from every window, and from as many of its output channels as keep them
         // at some 256, which a warp reads at once.  (What they look for is a matter of the depthwise filters, and those of a
         // window go into all output channels.)
-        const int groups = p->fold_dp / kFoldPackD, most = std::max(1, 256 / p->fold_nwin);
+        p->fold_per = p->fold_nwin * (p->fold_dp / 4) >= kFoldPackWide ? 4 : 1;
+        const int groups = p->fold_dp / (4 * p->fold_per), most = std::max(1, 256 / p->fold_nwin);
         p->fold_blocks = p->fold_nwin * groups;
         p->fold_sum_step = (groups + most - 1) / most;
         p->fold_nsums = p->fold_nwin * ((groups + p->fold_sum_step - 1) / p->fold_sum_step);

@@ -84,7 +84,7 @@ gdws_status_t gdws_forward_static(gdws_plan_t *p, const gdws_tensor_t *x, const 
         return fail(GDWS_ERR_INVALID_ARG, "dw_w and pw_w must both be given or both be NULL");
     if (dw_w) {   // re-pack into the plan's buffers (kernels only)
         if (!aligned16(dw_w) || !aligned16(pw_w)) return fail(GDWS_ERR_INVALID_ARG, "weight pointers must be 16-byte aligned");
-        st = bf16_pack(p, dw_w, pw_w, bias, GDWS_BF16, cs);
+        st = bf16_pack(p, dw_w, pw_w, bias, GDWS_BF16, false, cs);
         if (st != GDWS_OK) return st;
     } else if (!p->packed) {
         return fail(GDWS_ERR_INVALID_ARG, "no weights: pass dw_w/pw_w or call gdws_pack_weights first");

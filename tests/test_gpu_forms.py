@@ -66,3 +66,34 @@ def test_one_plan_serves_sizes_and_options_in_turn(dw_math):
         assert rel_err(yg.t.float().cpu().numpy(), want) <= 1e-2, (step, i, relu, f32)
     plan.status()
     plan.destroy()
+
+
+def test_weights_given_with_a_call_of_another_form():
+    """Weights that come with a call are folded only if it takes the folded form: a later call that reuses them computes with them
+    and not with folded filters of earlier ones, whichever form it would have taken."""
+    g = np.full(64, 2, dtype=np.int32)
+    layers = [gi.make_layer(small_spec("t", n, 64, 64, h, h, 3, 1, 1, ("const", 2), "bf16", "NHWC", seed=s)) for n, h, s in ((64, 28, 5), (2, 16, 6))]
+    plan = gdws.Plan(64, 64, 3, 1, 1, g)
+    assert plan.form(64, 28, 28) == 3 and plan.form(2, 16, 16) == 1
+    xs = [to_device(d.x, "bf16") for d in layers]
+    ys = [torch.empty((d.spec.N, d.spec.Ho, d.spec.Wo, 64), dtype=torch.bfloat16, device="cuda") for d in layers]
+    weights = [[to_device(d.dw_w, "bf16"), to_device(d.pw_w, "bf16"), torch.from_numpy(d.bias).cuda()] for d in layers]
+
+    def run(i, w=None):
+        ys[i].fill_(float("nan"))
+        plan.forward(xs[i], ys[i], "NHWC", *(weights[w] if w is not None else []))
+        torch.cuda.synchronize()
+        plan.status()
+        return ys[i].float().cpu().numpy()
+
+    def want(i, w):
+        d = gi.LayerData(layers[i].spec, layers[i].g, layers[i].x, layers[w].dw_w, layers[w].pw_w, layers[w].bias)
+        return run_oracle(d)[0]
+
+    plan.pack_weights(*weights[0])
+    assert rel_err(run(0), want(0, 0)) <= 1e-2
+    assert rel_err(run(1, 1), want(1, 1)) <= 1e-2          # two stages, other weights
+    assert rel_err(run(0), want(0, 1)) <= 1e-2             # would be folded
+    assert rel_err(run(0, 0), want(0, 0)) <= 1e-2          # folded, weights with the call
+    assert rel_err(run(1), want(1, 0)) <= 1e-2
+    plan.destroy()
