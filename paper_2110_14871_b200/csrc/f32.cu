@@ -98,13 +98,14 @@ __global__ void pw_f32_kernel(F32Shape s, const float *__restrict__ z, const flo
 // (transposed on the way to [channel][output channel]), the filters, and of each input channel the rows the tile's windows
 // read, zeros outside the image filled in.  NP producer threads start the copies and compute the next chunk's z from
 // shared memory while the other threads multiply this chunk; one barrier per chunk.  (In the multiplying threads' own
-// program order, copies and z cost their full latency on top: 105 us on the layer below, 39 of them for the products.)
+// program order, copies and z cost their full latency on top: 105 us for 16 x 128 -> 128 channels at 28 x 28,
+// G = 640, NCHW, 39 of them for the products; 84 now.)
 // KS groups of threads share a tile: each multiplies its share of a chunk's channels, and the sums meet in shared memory at
 // the end.  (One group of 8 x 8 thread tiles leaves 1.5 warps per scheduler, which cannot cover their own latencies.)
 // What bounds it: the FFMA pipe (G (k^2 + D) multiply-adds per pixel; nothing faster keeps fp32 products and sums).  The
 // packed form (two multiply-adds per instruction, same rate) leaves every other issue slot to loads and staging.  Large
 // thread tiles need fewer loads per multiply-add, small ones spread small layers over more SMs (f32_config chooses).  z straight from global memory, without the staging, took 870 cycles per
-// channel and thread: 139 us on the layer below.
+// channel and thread: 139 us on that layer.
 constexpr int kF32KC = 16;
 
 __device__ __forceinline__ void cp_async4(uint32_t dst, const void *src, bool valid)
@@ -551,7 +552,8 @@ gdws_status_t f32_launch_for(bool nhwc, const F32Shape &s, A... a)
     }
 }
 
-// Block tiles of fused_f32_kernel and the share of the multiply-add rate that a busy SM reaches with each (measured).
+// Block tiles of fused_f32_kernel and the share of the multiply-add rate that a busy SM reaches with each: measured in NCHW before
+// the z phase got its present form, which made the wide tiles some 8 % faster and left their order as it was.
 struct F32Config { int pt, dt; double rate; };
 constexpr F32Config kF32Configs[] = {
     {8, 16, 0.025}, {16, 32, 0.08}, {32, 32, 0.11}, {32, 64, 0.19}, {32, 128, 0.24}, {64, 128, 0.24}, {96, 128, 0.34}, {128, 128, 0.36},

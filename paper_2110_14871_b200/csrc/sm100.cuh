@@ -329,12 +329,6 @@ __device__ __forceinline__ void finish_store_row16_f32(const uint32_t (&acc)[16]
 }
 // Flags carried in the kernels' `relu` parameter.
 enum : int { kOutRelu = 1, kOutF32 = 2 };
-// One 32-byte sector per thread (dst 32-byte aligned).
-__device__ __forceinline__ void st_global_v8(void *dst, const uint32_t *v)
-{
-    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
-                 ::"l"(dst), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]) : "memory");
-}
 // Stores a row's 16 finished channels d0 .. d0+15 (those below D) to yrow.
 __device__ __forceinline__ void store_packed16(const uint32_t (&o)[8], int d0, int D, uint16_t *__restrict__ yrow)
 {
