@@ -602,7 +602,7 @@ bool fold_geometry(const gdws_plan_s *p, int n, int Ho, int Wo, bool out_f32, Fo
                 const double nblk = (np + 63) / 64;
                 const double mma = std::max(std::max(1.08 * fold_mma_cycles(np), issue), np * 16.0 / 60.0);
                 const double item = std::max(std::max(ksteps * mma, boxes), 1700.0 + 1100.0 * nblk) + 450.0;
-                g.us = 2.0 + (waves * item + 4000.0 + 900.0 * std::min(nblk, 2.0)) / 1850.0;
+                g.us = (2.0 + (waves * item + 4000.0 + 900.0 * std::min(nblk, 2.0)) / 1850.0) * (p->stride == 1 ? 1.0 : 1.15);      // the strided views' loads: 1.09 to 1.26
                 *out = g;
                 found = true;
             }
@@ -837,9 +837,9 @@ gdws_status_t fold_map_y(const gdws_plan_s *p, const gdws_tensor_t *y, FoldLaunc
 
 // ------------------------------------------------------------------------------------------
 // Which form a bf16 layer takes.  The folded form costs C k^2 D multiply-adds per pixel at full tensor-core rate, the
-// two-stage forms G (k^2 + D) at what their hand-overs allow.  The constants are fits to timings on B200 (60 random layers
-// and the 33 of the paper's networks): the cheaper estimate is the faster kernel except where the two are within a few per
-// cent of each other (mean loss 0.9 %).
+// two-stage forms G (k^2 + D) at what their hand-overs allow.  The constants are fits to timings on B200.  On 200 random layers
+// (k = 3 and 5, strides 1 and 2, half of them maps below 10 x 10) the chosen form is 2.9 % slower than the fastest in the mean,
+// mostly calls of 5 to 10 us where the three are close; against the two stages alone the choice loses on two of them, 4 and 6 %.
 // ------------------------------------------------------------------------------------------
 namespace {
 
@@ -850,7 +850,10 @@ double two_stage_us(const gdws_plan_s *p, int n, int h, int w, int Ho, int Wo, i
     if (stage == 1) {
         Tile t;
         if (p->D > 512 || !choose_tile(p, n, h, w, &t)) return 1e9;
-        const double chunk = (p->stride == 1 ? 0.95 : 1.25) * (p->k == 3 ? 1.0 : 2.1) * (p->D > 256 ? 1.3 : (p->D > 128 ? 1.12 : 1.0));
+        // with stride 2 a chunk's time follows the pixels that a tile has (0.6 to 0.85 us with a few, 1.3 with all; k = 5: 1.2 to 1.9)
+        const double fill = std::min(1.0, (double)n * Ho * Wo / (128.0 * (double)t.tiles()));
+        const double chunk = (p->stride == 1 ? 0.95 * (p->k == 3 ? 1.0 : 2.1) : 1.25 * (p->k == 3 ? 1.0 : 1.35) * (0.6 + 0.4 * fill)) *
+                             (p->D > 256 ? 1.3 : (p->D > 128 ? 1.12 : 1.0));
         return (p->stride == 1 ? 0.9 : 1.0) * (3.5 + waves((double)t.tiles()) * (p->nchunks * chunk + 0.5) + p->D / 128.0);
     }
     double tiles = 1e18;
