@@ -73,7 +73,7 @@ FORMS = {1: "ALUs", 2: "tensor cores", 3: "folded into one k x k convolution"}
 TRAFFIC_BYTES_PER_LAUNCH = {
     (1, 0, "fused", 2): 9180928,      # x + weights; y (8.39 MB) stays in L2 within the captured launch
     (1, 0, "fused", 3): 9633792,      # x + folded filters; y stays in L2
-    (3, 0, "fused", 3): 85866240,     # x (67.2 MB) + the part of y that left L2
+    (3, 0, "fused", 3): 84900352,     # x (67.2 MB) + the part of y that left L2
     (2, 0, "fused", 1): 25794304,     # x + weights; y (25.7 MB) stays in L2
     (3, 0, "fused", 2): 93909504,     # x (67.1 MB) + the part of y that left L2
 }
