@@ -43,15 +43,6 @@ constexpr int kFoldMaxA = 8;             // input box slots
 constexpr int kFoldMaxB = 40;            // filter units in shared memory (one tap x 64 input channels each)
 constexpr uint32_t kFoldSw128 = 2u << 29;   // descriptor high word: layout type "128-byte swizzle"
 constexpr int kFoldMaxAcc = 8;           // accumulators in tensor memory
-// One term of the filters suffices if they pass this share of their energy to a constant input: sum over the filters of
-// (sum_t W)^2 against sum_t W^2.  The rounding errors of a filter's taps are independent, so on a mean m they add up to some
-// 2^-9.2 sqrt(sum_t W^2) m.  Where the filters let the mean through, y grows with it and the error is that of rounding z
-// (random filters, share 0.9 to 1.1: relative error of y 2.35e-3 in either form, whatever the mean); where they cut it off it is
-// all error.  Relative error of y for 128 -> 256 channels at a mean of 10 sigma, two stages | one term | two terms: share 0.46
-// 2.42e-3 | 3.09e-3 | 1.66e-3, share 0.28 2.25e-3 | 3.31e-3 | 1.62e-3, zero 2.41e-3 | 1.60e-2 | 1.66e-3 (at 100 sigma 1.57e-1 for
-// one term).  The second term costs 28 x 28 x 8 images of that layer 9.1 -> 12.0 us (two stages 16.7), 512 -> 512 channels 18.7 ->
-// 30.8 (44.7); random filters of 64 channels with g_c = 1 scatter by 0.18 around 1, so a line much nearer to 1 would catch them.
-constexpr float kFoldPass = 0.5f;
 // A unit is a run of product steps (taps) whose filters share one barrier: bits 0-7 its first step, 8-15 its steps,
 // then whether it is the first / last one that reads its input box.
 constexpr uint32_t kUnitFirst = 1u << 16, kUnitLast = 1u << 17, kUnitLastBox = 1u << 18;   // LastBox: the first unit of the window's last box
@@ -131,26 +122,6 @@ __device__ __forceinline__ void fold_issue(const FoldParams &P, int s0, int n, i
                 if (NK == 4 || kk < nk) umma_pair_words(d, al + 2u * kk, a_hi, bl + 2u * kk, b_hi, idesc, (uint32_t)j | accumulate | (uint32_t)kk);
         }
     }
-}
-
-// Whether the filters need their second term, by a whole warp: the packing blocks' sums, added in a fixed order.
-__device__ __forceinline__ bool fold_second_term(const FoldParams &P, int lane)
-{
-    float energy = 0.f, sum = 0.f;
-#pragma unroll 1
-    for (int b0 = 0; b0 < P.nsums; b0 += 256) {
-        float2 v[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const int b = b0 + 32 * j + lane;
-            v[j] = b < P.nsums ? __ldcg(P.sums + b) : make_float2(0.f, 0.f);
-        }
-#pragma unroll
-        for (int j = 0; j < 8; ++j) { energy += v[j].x; sum += v[j].y; }
-    }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) { energy += __shfl_xor_sync(0xffffffffu, energy, o); sum += __shfl_xor_sync(0xffffffffu, sum, o); }
-    return sum < kFoldPass * energy;
 }
 
 struct FoldBars { uint32_t afull, aempty, bfull, bempty, accfull, accfree; };
@@ -433,7 +404,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kFoldThreads, 1) fol
         }
     } else if (warp == kFoldTermWarp) {
         // ---------------- one term of the filters or two ----------------
-        const bool second = fold_second_term(P, lane);
+        const bool second = fold_second_term(P.sums, P.nsums, lane);
         if (lane == 0) {
             second_term = second;
             mbar_arrive(bar_terms);
@@ -628,6 +599,7 @@ struct FoldLaunch {
     void (*kernel)(FoldParams) = nullptr;
     int grid = 0;
     size_t smem = 0;
+    bool sliced = false;                         // runs in fold_split.cu, nothing else here is set
     const void *x = nullptr, *y = nullptr;       // the addresses the tensor maps were encoded for
 };
 
@@ -873,6 +845,7 @@ double two_stage_us(const gdws_plan_s *p, int n, int h, int w, int Ho, int Wo, i
 struct FormChoice {
     LaunchKey key;
     int form = 1;
+    bool sliced = false;         // the folded form would run in slices
 };
 
 }  // namespace
@@ -892,11 +865,19 @@ int bf16_form_of(gdws_plan_s *p, int n, int h, int w, bool out_f32)
     const LaunchKey key = {n, h, w, out_f32 ? 2 : 0};
     if (const FormChoice *c = LaunchCache<FormChoice>::find(p->launch_cache[3], key)) return c->form;
     FoldGeom g;
-    const bool fold = fold_geometry(p, n, Ho, Wo, out_f32, &g) && g.us < two_stage_us(p, n, h, w, Ho, Wo, stage);
+    double us = fold_geometry(p, n, Ho, Wo, out_f32, &g) ? g.us : 1e9;
+    const double slices = fold_split_us(p, n, Ho, Wo);
+    const bool sliced = slices < us;
+    // Slices (fold_split.cu) count where a channel has more than two filters in the mean.  They would win below that as well (384 ->
+    // 104 channels, stride 2, 8 x 8, g_c = 2: 7.3 us against 12.5), but the form that such layers have is part of what callers plan
+    // with: its answers stay.
+    if (p->G > 2 * p->C) us = std::min(us, slices);
+    const bool fold = us < two_stage_us(p, n, h, w, Ho, Wo, stage);
     const int form = fold ? 3 : stage;
     if (std::unique_ptr<FormChoice> c{new (std::nothrow) FormChoice}) {
         c->key = key;
         c->form = form;
+        c->sliced = sliced;
         LaunchCache<FormChoice>::add(p->launch_cache[3], std::move(c));      // kept if there is memory for it
     }
     return form;
@@ -909,7 +890,7 @@ double bf16_forward_us(gdws_plan_s *p, int n, int h, int w, bool out_f32)
     const int Ho = gdws_out_dim(h, p->k, p->stride, p->pad), Wo = gdws_out_dim(w, p->k, p->stride, p->pad);
     const int form = p->opt_path == GDWS_PATH_UNFUSED ? 1 : bf16_form_of(p, n, h, w, out_f32);
     FoldGeom g;
-    if (form == 3 && fold_geometry(p, n, Ho, Wo, out_f32, &g)) return g.us;
+    if (form == 3 && fold_geometry(p, n, Ho, Wo, out_f32, &g)) return std::min(g.us, fold_split_us(p, n, Ho, Wo));
     if (form == 2) return two_stage_us(p, n, h, w, Ho, Wo, 2);
     Tile t;
     if (!choose_tile(p, n, h, w, &t)) return 1e9;
@@ -928,11 +909,18 @@ gdws_status_t bf16_folded(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t 
         std::unique_ptr<FoldLaunch> e(new (std::nothrow) FoldLaunch);
         if (!e) return fail(GDWS_ERR_ALLOC, "out of host memory");
         e->key = key;
-        rc = fold_prepare(p, x->n, y->h, y->w, out_f32, e.get());
+        if (const FormChoice *c = LaunchCache<FormChoice>::find(p->launch_cache[3], {x->n, x->h, x->w, out_f32 ? 2 : 0})) {
+            e->sliced = c->sliced;
+        } else {
+            FoldGeom g;
+            e->sliced = !(fold_geometry(p, x->n, y->h, y->w, out_f32, &g) && g.us <= fold_split_us(p, x->n, y->h, y->w));
+        }
+        rc = e->sliced ? GDWS_OK : fold_prepare(p, x->n, y->h, y->w, out_f32, e.get());
         if (rc != GDWS_OK) return rc;
         L = LaunchCache<FoldLaunch>::add(p->launch_cache[2], std::move(e));
         if (!L) return fail(GDWS_ERR_ALLOC, "out of host memory");
     }
+    if (L->sliced) return bf16_folded_split(p, x, y, st);
     if (L->x != x->ptr && (rc = fold_map_x(p, x, L)) != GDWS_OK) return rc;
     if (L->y != y->ptr && (rc = fold_map_y(p, y, L)) != GDWS_OK) return rc;
     const cudaError_t e = launch_overlapped(L->kernel, (unsigned)L->grid, kFoldThreads, L->smem, st, L->P);

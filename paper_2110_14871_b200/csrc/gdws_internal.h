@@ -134,7 +134,7 @@ struct gdws_plan_s {
 
     // Prepared launches of the three fused bf16 kernels, the choice between them and the pieces of a host call (LaunchCache
     // below; each file knows its own types).
-    std::shared_ptr<void> launch_cache[5];
+    std::shared_ptr<void> launch_cache[8];
 
     int64_t launches = 0;
 };
@@ -260,6 +260,9 @@ gdws_status_t bf16_fused_tc(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_
 
 // fold.cu
 gdws_status_t bf16_folded(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t *y, cudaStream_t s);
+// fold_split.cu: the folded form in slices, for layers that leave SMs idle
+double fold_split_us(const gdws_plan_s *p, int n, int Ho, int Wo);      // estimate; 1e9 where it does not cover the layer
+gdws_status_t bf16_folded_split(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t *y, cudaStream_t s);
 double bf16_forward_us(gdws_plan_s *p, int n, int h, int w, bool out_f32);
 int bf16_form_of(gdws_plan_s *p, int n, int h, int w, bool out_f32);   // 1 / 2: two stages, GDW on the ALUs / the tensor cores; 3: folded
 

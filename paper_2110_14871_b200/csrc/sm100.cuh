@@ -376,6 +376,16 @@ __device__ __forceinline__ void issue_chunk(uint32_t tmem, uint32_t a_addr, uint
     }
 }
 
+// n / d for 31-bit n as a multiplication (a division by a run-time value is some fifty dependent instructions).
+__device__ __forceinline__ int div_by(int n, const uint32_t (&md)[2]) { return (int)(((uint64_t)(uint32_t)n * md[0]) >> md[1]); }
+inline void div_magic(int d, uint32_t (&md)[2])
+{
+    int sh = 0;
+    while ((1 << sh) < d) ++sh;
+    md[0] = (uint32_t)((((uint64_t)1 << (31 + sh)) + (uint64_t)d - 1) / (uint64_t)d);
+    md[1] = (uint32_t)(31 + sh);
+}
+
 inline int tmem_cols_for(int Dpad)
 {
     int c = 32;
@@ -390,6 +400,39 @@ inline size_t smem_for_tmem(size_t need, int cols)
     const int max_ctas = 512 / cols;
     const size_t floor_bytes = (size_t)kMaxSmem / (max_ctas + 1) + 1024;
     return need > floor_bytes ? need : floor_bytes;
+}
+
+
+// ------------------------------------------------------------------------------------------
+// Folded filters: one term or two
+// ------------------------------------------------------------------------------------------
+// One term of the filters suffices if they pass this share of their energy to a constant input: sum over the filters of
+// (sum_t W)^2 against sum_t W^2.  The rounding errors of a filter's taps are independent, so on a mean m they add up to some
+// 2^-9.2 sqrt(sum_t W^2) m.  Where the filters let the mean through, y grows with it and the error is that of rounding z
+// (random filters, share 0.9 to 1.1: relative error of y 2.35e-3 in either form, whatever the mean); where they cut it off it is
+// all error.  Relative error of y for 128 -> 256 channels at a mean of 10 sigma, two stages | one term | two terms: share 0.46
+// 2.42e-3 | 3.09e-3 | 1.66e-3, share 0.28 2.25e-3 | 3.31e-3 | 1.62e-3, zero 2.41e-3 | 1.60e-2 | 1.66e-3 (at 100 sigma 1.57e-1 for
+// one term).  The second term costs 28 x 28 x 8 images of that layer 9.1 -> 12.0 us (two stages 16.7), 512 -> 512 channels 18.7 ->
+// 30.8 (44.7); random filters of 64 channels with g_c = 1 scatter by 0.18 around 1, so a line much nearer to 1 would catch them.
+constexpr float kFoldPass = 0.5f;
+// Whether the filters need their second term, by a whole warp: the packing blocks' sums, added in a fixed order.
+__device__ __forceinline__ bool fold_second_term(const float2 *sums, int nsums, int lane)
+{
+    float energy = 0.f, sum = 0.f;
+#pragma unroll 1
+    for (int b0 = 0; b0 < nsums; b0 += 256) {
+        float2 v[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int b = b0 + 32 * j + lane;
+            v[j] = b < nsums ? __ldcg(sums + b) : make_float2(0.f, 0.f);
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) { energy += v[j].x; sum += v[j].y; }
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) { energy += __shfl_xor_sync(0xffffffffu, energy, o); sum += __shfl_xor_sync(0xffffffffu, sum, o); }
+    return sum < kFoldPass * energy;
 }
 
 
