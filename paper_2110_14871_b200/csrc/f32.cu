@@ -1,5 +1,5 @@
-// fp32 kernels (NCHW or NHWC through explicit strides).  Plain FFMA on both stages:
-// the tensor cores have no full-fp32 mode and TF32 would miss the 1e-4 parity bound.
+// fp32 kernels (NCHW or NHWC through explicit strides).  Plain FFMA on both stages: the tensor cores have no full-fp32 mode and TF32
+// would miss the 1e-4 parity bound.  Larger layers of 3 x 3 and 5 x 5 filters run in f32_tc.cu (three bf16 pieces per value).
 #include <algorithm>
 
 #include "gdws_internal.h"
@@ -584,8 +584,8 @@ int f32_config(const gdws_plan_s *p, long long npix, int Wo, double *cycles = nu
 
 }  // namespace
 
-// Estimate of an fp32 forward of n images, for gdws_forward_host.
-double f32_forward_us(const gdws_plan_s *p, int n, int h, int w)
+// Estimate of fused_f32_kernel's time for n images.
+double f32_alu_us(const gdws_plan_s *p, int n, int h, int w)
 {
     const int Ho = gdws_out_dim(h, p->k, p->stride, p->pad), Wo = gdws_out_dim(w, p->k, p->stride, p->pad);
     double cycles = 0;
@@ -596,6 +596,7 @@ double f32_forward_us(const gdws_plan_s *p, int n, int h, int w)
 gdws_status_t f32_fused(gdws_plan_s *p, const gdws_tensor_t *x, const float *dw_w, const float *pw_w,
                         const float *bias, gdws_tensor_t *y, cudaStream_t st)
 {
+    if (f32_tc_takes(p, x->n, x->h, x->w)) return f32_fused_tc(p, x, dw_w, pw_w, bias, y, st);
     const F32Shape s = make_shape(p, x->layout, x->n, x->h, x->w);
     const bool nhwc = x->layout == GDWS_NHWC;
     const float *xp = (const float *)x->ptr;

@@ -240,9 +240,15 @@ inline int sm_count_of(const gdws_plan_s *p) { return p->sm_count > 0 ? p->sm_co
 gdws_status_t f32_depthwise(gdws_plan_s *p, const gdws_tensor_t *x, const float *dw_w, float *z, cudaStream_t s);
 gdws_status_t f32_pointwise(gdws_plan_s *p, const float *z, const float *pw_w, const float *bias,
                             gdws_tensor_t *y, cudaStream_t s);
-double f32_forward_us(const gdws_plan_s *p, int n, int h, int w);
+double f32_alu_us(const gdws_plan_s *p, int n, int h, int w);
 gdws_status_t f32_fused(gdws_plan_s *p, const gdws_tensor_t *x, const float *dw_w, const float *pw_w,
                         const float *bias, gdws_tensor_t *y, cudaStream_t s);
+
+// f32_tc.cu
+double f32_forward_us(gdws_plan_s *p, int n, int h, int w);
+bool f32_tc_takes(gdws_plan_s *p, int n, int h, int w);     // whether a forward of this size runs there
+gdws_status_t f32_fused_tc(gdws_plan_s *p, const gdws_tensor_t *x, const float *dw_w, const float *pw_w,
+                           const float *bias, gdws_tensor_t *y, cudaStream_t s);
 
 // pack.cu
 constexpr int kFoldPackWide = 256;   // packing blocks of 4 output channels from which on a thread takes four of them

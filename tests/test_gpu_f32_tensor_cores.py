@@ -1,0 +1,66 @@
+"""The fp32 forward with its pointwise products on the tensor cores: against the CPU oracle, no less exact than the ALU kernel, and
+with the same infinities and NaN.  Output channels around 16, 32, 64 and 128 and in two parts, chunks of 32 intermediate channels with
+remainders and one alone, clusters that share a tile's chunks, tiles of several images, both filter sizes, strides, channels without filters."""
+import numpy as np
+import pytest
+
+from paper_2110_14871_b200 import build as gbuild
+from paper_2110_14871_b200 import gdws
+from paper_2110_14871_b200 import inputs as gi
+
+from util import rel_err, run_gpu, run_oracle, small_spec
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    gbuild.build_library()
+
+
+SHAPES = [
+    # N, C, D, H, W, k, stride, g
+    (1, 1, 1, 5, 5, 3, 1, ("const", 1)),
+    (1, 16, 16, 32, 32, 3, 1, ("uniform", 1, 3)),
+    (9, 12, 33, 6, 7, 3, 1, ("uniform", 0, 9)),            # several images per tile, a channel without filters
+    (16, 64, 128, 28, 28, 3, 1, ("uniform", 1, 9)),
+    (2, 147, 117, 14, 10, 3, 1, ("uniform", 1, 9)),        # eight blocks per tile
+    (3, 40, 200, 17, 19, 3, 2, ("uniform", 1, 9)),         # two parts of the output channels
+    (5, 33, 65, 20, 22, 5, 1, ("uniform", 1, 25)),
+    (2, 64, 72, 31, 22, 5, 2, ("uniform", 1, 25)),
+    (400, 8, 31, 9, 9, 3, 1, ("const", 1)),                # many tiles of one chunk per block
+    (2, 20, 18, 40, 300, 3, 3, ("uniform", 1, 4)),         # stride 3, long rows
+]
+
+
+@pytest.mark.parametrize("layout", ["NCHW", "NHWC"])
+@pytest.mark.parametrize("shape", SHAPES)
+def test_matches_reference(shape, layout):
+    N, C, D, H, W, k, s, gd = shape
+    data = gi.make_layer(small_spec("t", N, C, D, H, W, k, s, k // 2, gd, "f32", layout, relu=D == 33, seed=3 + sum(shape[:7])))
+    ref, _ = run_oracle(data)
+    tc, alu = (run_gpu(data, path=gdws.PATH_FUSED, dw_math=m) for m in (2, 1))
+    # dropped pieces and the chunks' truncation: 2^-22 of sum |P||z|, some sqrt(G) times the largest output
+    assert rel_err(tc, ref) <= 1e-5
+    # one rounding per chunk instead of one per channel; both have z's own roundings (in the 2-norm, with a little room for few terms)
+    assert np.linalg.norm(tc - ref) <= 1.1 * np.linalg.norm(alu - ref) + 3e-8 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("layout", ["NCHW", "NHWC"])
+@pytest.mark.parametrize("N,C,D,H,W,k", [(2, 40, 40, 20, 20, 3), (1, 150, 130, 14, 10, 3), (3, 9, 20, 24, 24, 5)])
+def test_nonfinite_values_are_those_of_the_sums(N, C, D, H, W, k, layout):
+    data = gi.make_layer(small_spec("t", N, C, D, H, W, k, 1, k // 2, ("uniform", 1, 9), "f32", layout, seed=17 + C))
+    rng = np.random.default_rng(5)
+    flat = data.x.reshape(-1)
+    for v in (np.inf, -np.inf, np.nan, 3.4e38):
+        flat[rng.integers(0, flat.size, 3)] = v
+    data.pw_w[1, 2], data.pw_w[D - 1, 0] = np.inf, 0.0
+    got = []
+    for m in (2, 1):
+        got.append(run_gpu(data, path=gdws.PATH_FUSED, dw_math=m))
+    for test in (np.isnan, np.isposinf, np.isneginf):
+        assert np.array_equal(test(got[0]), test(got[1]))
+    fine = np.isfinite(got[1])
+    assert fine.any() and not fine.all()
+    scale = np.abs(got[1][fine]).max()
+    assert np.abs(got[0][fine] - got[1][fine]).max() <= 1e-5 * scale
