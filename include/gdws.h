@@ -92,7 +92,13 @@ typedef enum {
                               1 reads only channels with g_c > 0; 2 and 3 multiply the others (2:
                               those that share a group of 16 with used ones) by zeros, so that an
                               infinity or NaN in them reaches y.  0 takes 3 for layers with
-                              g_c = 0 only where no other kernel covers them (D > 512)      */
+                              g_c = 0 only where no other kernel covers them (D > 512).
+                              fp32 forwards: 1 = all arithmetic on the ALUs; 2 = pointwise products
+                              on the tensor cores (three bf16 pieces per value, fp32 sums, no less
+                              exact) for k = 3 and 5; 0 and 3 = whichever is estimated faster.
+                              gdws_depthwise, bf16: 1 = ALUs, 2 = tensor cores where they cover the
+                              layer, 0 and 3 = whichever is estimated faster: same z but for values
+                              next to a rounding boundary                                    */
     GDWS_OPT_OUT_DTYPE = 5 /* bf16 plans: 0 (default) = y has the dtype of x; 1 = y is fp32
                               (GDWS_F32, NHWC): bias and ReLU are applied to the fp32 sums of
                               the PW stage and stored without the rounding to bf16.  Every

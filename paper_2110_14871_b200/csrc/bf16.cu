@@ -59,6 +59,10 @@ __global__ void gdw_bf16_kernel(DwShape s, const uint16_t *__restrict__ x, const
 
 gdws_status_t bf16_depthwise(gdws_plan_s *p, const gdws_tensor_t *x, void *z, cudaStream_t st)
 {
+    if (p->opt_dw_math != 1 && !p->opt_tile && !p->opt_a_layout) {
+        const gdws_status_t rc = bf16_depthwise_tc(p, x, z, st);
+        if (rc != GDWS_ERR_UNSUPPORTED) return rc;
+    }
     if (p->C % 8 == 0) {   // tiled pipeline first; shapes it cannot tile fall through to the simple kernel
         const gdws_status_t rc = bf16_depthwise_tiled(p, x, z, st);
         if (rc != GDWS_ERR_UNSUPPORTED) return rc;

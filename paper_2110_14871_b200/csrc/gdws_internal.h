@@ -261,6 +261,9 @@ gdws_status_t bf16_pointwise(gdws_plan_s *p, const void *z, gdws_tensor_t *y, cu
 gdws_status_t bf16_fused(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t *y, cudaStream_t s);
 gdws_status_t bf16_depthwise_tiled(gdws_plan_s *p, const gdws_tensor_t *x, void *z, cudaStream_t s);
 
+// gdw_tc.cu
+gdws_status_t bf16_depthwise_tc(gdws_plan_s *p, const gdws_tensor_t *x, void *z, cudaStream_t s);
+
 // fused_tc.cu
 gdws_status_t bf16_fused_tc(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t *y, cudaStream_t s);
 
