@@ -100,7 +100,7 @@ static __device__ __noinline__ void fold_wait_cluster(uint32_t bar, uint32_t par
     atomicOr(status, code);
 }
 
-// The products of one unit: n steps of nk x (K = 16).  Straight-line code when both are constants.
+// The products of one unit: n steps of nk x (K = 16).  Straight-line code when both are constants (STEPS, NK not 0).
 template <int STEPS, int NK>
 __device__ __forceinline__ void fold_issue(const FoldParams &P, int s0, int n, int nk, uint32_t d, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
                                            uint32_t b_tap, uint32_t idesc, uint32_t accumulate)
@@ -110,8 +110,7 @@ __device__ __forceinline__ void fold_issue(const FoldParams &P, int s0, int n, i
         for (int j = 0; j < STEPS; ++j) {
             const uint32_t al = a_lo + (P.steps[s0 + j] & 0xFFFFu), bl = b_lo + (uint32_t)j * b_tap;
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk)
-                if (NK == 4 || kk < nk) umma_pair_words(d, al + 2u * kk, a_hi, bl + 2u * kk, b_hi, idesc, j | kk ? 1u : accumulate);
+            for (int kk = 0; kk < NK; ++kk) umma_pair_words(d, al + 2u * kk, a_hi, bl + 2u * kk, b_hi, idesc, j | kk ? 1u : accumulate);
         }
     } else {
 #pragma unroll 1
@@ -169,8 +168,10 @@ static __device__ __noinline__ void fold_second(const FoldParams *params, int my
     }
 }
 
-// UNITS x STEPS: the window's units when they are all alike (unrolled: 3 x 3 taps or 9 x 1), 0: table driven.
-template <int UNITS, int STEPS>
+// UNITS x STEPS: the window's units when they are all alike (unrolled: 3 x 3 taps or 9 x 1), 0: table driven.  NK: 1 to 3: the only
+// window has so many K steps of 16 channels (up to 48 channels: straight-line code as for whole windows, 16 x 32 -> 16 x 192 x 165 31.3 ->
+// 27.6 us); 4: whole windows, and a last one of any number.
+template <int UNITS, int STEPS, int NK = 4>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kFoldThreads, 1) fold_kernel(const __grid_constant__ FoldParams P)
 {
     extern __shared__ uint8_t smem_raw[];
@@ -283,7 +284,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kFoldThreads, 1) fol
                         if (two && w == P.nwin - 1 && (wait_b ? u == nunits - 1 : (un & kUnitLastBox) != 0)) mbar_arrive(bar_turn + 8 * (uint32_t)warp);
                         tc_fence_after();
                         const int s0 = STEPS ? u * STEPS : (int)(un & 0xFFu), n = (int)((un >> 8) & 0xFFu);
-                        if (nk == 4) fold_issue<STEPS, 4>(P, s0, n, 4, d, a_lo, a_hi, b_lo, b_hi, b_tap, idesc, (uint32_t)(w | u));
+                        if constexpr (NK != 4) fold_issue<STEPS, NK>(P, s0, n, NK, d, a_lo, a_hi, b_lo, b_hi, b_tap, idesc, (uint32_t)u);
+                        else if (nk == 4) fold_issue<STEPS, 4>(P, s0, n, 4, d, a_lo, a_hi, b_lo, b_hi, b_tap, idesc, (uint32_t)(w | u));
                         else fold_issue<0, 0>(P, s0, n, nk, d, a_lo, a_hi, b_lo, b_hi, b_tap, idesc, (uint32_t)(w | u));
                         if (!P.resident) umma_commit_pair(bar_bempty + 8 * bslot);
                         if (last) umma_commit_pair(bar_aempty + 8 * aslot);
@@ -744,11 +746,18 @@ gdws_status_t fold_prepare(gdws_plan_s *p, int n, int Ho, int Wo, bool out_f32, 
 
     void (*kernel)(FoldParams) = nullptr;
     int which = 0;
-    if (alike && unit_steps == 3 && P.nunits == 3) { kernel = fold_kernel<3, 3>; which = 0; }
-    else if (alike && unit_steps == 5 && P.nunits == 5) { kernel = fold_kernel<5, 5>; which = 1; }
+    const int nk = P.nwin == 1 ? P.nk_last : 4;
+    if (alike && unit_steps == 3 && P.nunits == 3) {
+        kernel = nk == 1 ? fold_kernel<3, 3, 1> : (nk == 2 ? fold_kernel<3, 3, 2> : (nk == 3 ? fold_kernel<3, 3, 3> : fold_kernel<3, 3>));
+        which = nk == 4 ? 0 : 3 + nk;
+    }
+    else if (alike && unit_steps == 5 && P.nunits == 5) {
+        kernel = nk == 1 ? fold_kernel<5, 5, 1> : (nk == 2 ? fold_kernel<5, 5, 2> : (nk == 3 ? fold_kernel<5, 5, 3> : fold_kernel<5, 5>));
+        which = nk == 4 ? 1 : 6 + nk;
+    }
     else if (alike && unit_steps == 1) { kernel = fold_kernel<0, 1>; which = 2; }
     else { kernel = fold_kernel<0, 0>; which = 3; }
-    static bool attr_set[64][4] = {};
+    static bool attr_set[64][10] = {};
     if (!attr_set[p->device & 63][which]) {
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kFoldMaxSmem);
         if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(fold_kernel)");
