@@ -584,6 +584,8 @@ int f32_config(const gdws_plan_s *p, long long npix, int Wo, double *cycles = nu
 
 }  // namespace
 
+int f32_alu_config(const gdws_plan_s *p, long long npix, int Wo) { return f32_config(p, npix, Wo); }
+
 // Estimate of fused_f32_kernel's time for n images.
 double f32_alu_us(const gdws_plan_s *p, int n, int h, int w)
 {
@@ -596,14 +598,15 @@ double f32_alu_us(const gdws_plan_s *p, int n, int h, int w)
 gdws_status_t f32_fused(gdws_plan_s *p, const gdws_tensor_t *x, const float *dw_w, const float *pw_w,
                         const float *bias, gdws_tensor_t *y, cudaStream_t st)
 {
-    if (f32_tc_takes(p, x->n, x->h, x->w)) return f32_fused_tc(p, x, dw_w, pw_w, bias, y, st);
+    int config = -2;
+    if (f32_tc_takes(p, x->n, x->h, x->w, &config)) return f32_fused_tc(p, x, dw_w, pw_w, bias, y, st);
     const F32Shape s = make_shape(p, x->layout, x->n, x->h, x->w);
     const bool nhwc = x->layout == GDWS_NHWC;
     const float *xp = (const float *)x->ptr;
     float *yp = (float *)y->ptr;
     gdws_status_t rc = GDWS_ERR_UNSUPPORTED;
     const gdws_plan_s *cp = p;
-    switch (f32_config(p, (long long)s.N * s.Ho * s.Wo, s.Wo)) {
+    switch (config == -2 ? f32_config(p, (long long)s.N * s.Ho * s.Wo, s.Wo) : config) {
     case 0: rc = f32_launch_for<8, 16, 1, 1, 1, 128>(nhwc, s, cp, xp, dw_w, pw_w, bias, yp, st); break;
     case 1: rc = f32_launch_for<16, 32, 2, 2, 1, 256>(nhwc, s, cp, xp, dw_w, pw_w, bias, yp, st); break;
     case 2: rc = f32_launch_for<32, 32, 4, 2, 1, 256>(nhwc, s, cp, xp, dw_w, pw_w, bias, yp, st); break;

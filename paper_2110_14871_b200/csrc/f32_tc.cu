@@ -669,6 +669,7 @@ struct F32TcLaunch {
     LaunchKey key;
     F32TcGeom g;
     bool taken = false;
+    int alu = -1;                // fused_f32_kernel's tile
 };
 
 size_t f32tc_smem(const gdws_plan_s *p, int slots, const F32TcGeom &g)
@@ -765,6 +766,7 @@ static const F32TcLaunch *f32tc_prepared(gdws_plan_s *p, int n, int h, int w)
     if (!e) return nullptr;
     const int Ho = gdws_out_dim(h, p->k, p->stride, p->pad), Wo = gdws_out_dim(w, p->k, p->stride, p->pad);
     e->key = key;
+    e->alu = f32_alu_config(p, (long long)n * Ho * Wo, Wo);
     e->taken = p->opt_dw_math != 1 && f32tc_geometry(p, n, Ho, Wo, (long long)p->C * h * w, &e->g);
     // The other kernel's estimate is 1.3 to 1.8 times too long for calls below 16 us and up to twice too short for large NHWC ones.
     const double alu = f32_alu_us(p, n, h, w);
@@ -772,9 +774,10 @@ static const F32TcLaunch *f32tc_prepared(gdws_plan_s *p, int n, int h, int w)
     return LaunchCache<F32TcLaunch>::add(p->launch_cache[5], std::move(e));
 }
 
-bool f32_tc_takes(gdws_plan_s *p, int n, int h, int w)
+bool f32_tc_takes(gdws_plan_s *p, int n, int h, int w, int *alu)
 {
     const F32TcLaunch *l = f32tc_prepared(p, n, h, w);
+    if (l) *alu = l->alu;
     return l && l->taken;
 }
 

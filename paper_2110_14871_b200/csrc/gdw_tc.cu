@@ -93,18 +93,20 @@ static __device__ __noinline__ float gdw_plain(const GdwParams *params, int n, i
     return z;
 }
 
-// The products of a box that holds the windows of all nine taps.
-template <int NK>
-__device__ __forceinline__ void gdw_issue9(const GdwParams &P, uint32_t d, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi, uint32_t tap, uint32_t idesc, uint32_t more)
+// The products of NS taps from s0 on, NK K steps each: straight-line code (a loop costs some 30 cycles per product).
+template <int NS, int NK>
+__device__ __forceinline__ void gdw_issue(const GdwParams &P, int s0, uint32_t d, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi, uint32_t tap, uint32_t idesc, uint32_t more)
 {
 #pragma unroll
-    for (int s = 0; s < 9; ++s) {
-        const uint32_t al = a_lo + (P.steps[s] & 0xFFFFu), bl = b_lo + (P.steps[s] >> 16) * tap;
+    for (int s = 0; s < NS; ++s) {
+        const uint32_t st = P.steps[s0 + s], al = a_lo + (st & 0xFFFFu), bl = b_lo + (st >> 16) * tap;
 #pragma unroll
         for (int kk = 0; kk < NK; ++kk) umma_pair_words(d, al + 2u * kk, a_hi, bl + 2u * kk, b_hi, idesc, s | kk ? 1u : more);
     }
 }
 
+// NINE: 3 x 3 taps from one box per tile.  (As one kernel with the other shapes' code it took 42 us instead of 40 for 64 -> 191 channels.)
+template <bool NINE>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGdwThreads, 1) gdw_tc_kernel(const __grid_constant__ GdwParams P)
 {
     extern __shared__ uint8_t smem_raw[];
@@ -199,21 +201,27 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGdwThreads, 1) gdw_
                     const int nk = min(steps, cb >> 4);
                     uint32_t at = slot, apar = par;      // boxes that several runs share: those of a tile stay until its last run has read them
 #pragma unroll 1
-                    for (int b = 0; b < P.nboxes; ++b) {
+                    for (int b = 0; b < (NINE ? 1 : P.nboxes); ++b) {
                         if (take) mbar_wait_call(bar_afull + 8 * at, apar, &abort_flag, P.status, kStatusWaitOperand);
                         tc_fence_after();
                         const uint32_t a_lo = ((((a_s + at * P.a_slot) & 0x3FFFFu) >> 4) | (1u << 16)) + k0;
-                        if (P.k2 == 9 && P.nboxes == 1) {        // straight-line code: a loop costs some 30 cycles per product
-                            if (nk == 1) gdw_issue9<1>(P, d, a_lo, a_hi, b_lo + k0, b_hi, tap, idesc, more);
-                            else if (nk == 2) gdw_issue9<2>(P, d, a_lo, a_hi, b_lo + k0, b_hi, tap, idesc, more);
-                            else if (nk == 3) gdw_issue9<3>(P, d, a_lo, a_hi, b_lo + k0, b_hi, tap, idesc, more);
-                            else gdw_issue9<4>(P, d, a_lo, a_hi, b_lo + k0, b_hi, tap, idesc, more);
+                        if constexpr (NINE) {
+                            if (nk == 1) gdw_issue<9, 1>(P, 0, d, a_lo, a_hi, b_lo + k0, b_hi, tap, idesc, more);
+                            else if (nk == 2) gdw_issue<9, 2>(P, 0, d, a_lo, a_hi, b_lo + k0, b_hi, tap, idesc, more);
+                            else if (nk == 3) gdw_issue<9, 3>(P, 0, d, a_lo, a_hi, b_lo + k0, b_hi, tap, idesc, more);
+                            else gdw_issue<9, 4>(P, 0, d, a_lo, a_hi, b_lo + k0, b_hi, tap, idesc, more);
                             more = 1;
                         } else {
                             const uint32_t box = P.boxes[b];
-                            const int s1 = (int)((box >> 16) & 0xFFu) + (int)(box >> 24);
+                            int s = (int)((box >> 16) & 0xFFu);
+                            const int s1 = s + (int)(box >> 24);
 #pragma unroll 1
-                            for (int s = (int)((box >> 16) & 0xFFu); s < s1; ++s) {
+                            for (; nk == 1 && s + 5 <= s1; s += 5) {        // 5 x 5 taps: few channels have many filters
+                                gdw_issue<5, 1>(P, s, d, a_lo, a_hi, b_lo + k0, b_hi, tap, idesc, more);
+                                more = 1;
+                            }
+#pragma unroll 1
+                            for (; s < s1; ++s) {
                                 const uint32_t st = P.steps[s], al = a_lo + (st & 0xFFFFu), bl = b_lo + k0 + (st >> 16) * tap;
                                 umma_pair_words(d, al, a_hi, bl, b_hi, idesc, more);
                                 more = 1;
@@ -605,13 +613,15 @@ gdws_status_t bf16_depthwise_tc(gdws_plan_s *p, const gdws_tensor_t *x, void *z,
     if (!L->taken) return fail(GDWS_ERR_UNSUPPORTED, "GDW stage on the tensor cores: layer not covered");
     const gdws_status_t rc = gdw_maps(p, x, z, L);
     if (rc != GDWS_OK) return rc;
-    static bool attr_set[64] = {};
-    if (!attr_set[p->device & 63]) {
-        const cudaError_t e = cudaFuncSetAttribute(gdw_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+    const int nine = L->P.k2 == 9 && L->P.nboxes == 1;
+    const auto kernel = nine ? gdw_tc_kernel<true> : gdw_tc_kernel<false>;
+    static bool attr_set[64][2] = {};
+    if (!attr_set[p->device & 63][nine]) {
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
         if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(gdw_tc_kernel)");
-        attr_set[p->device & 63] = true;
+        attr_set[p->device & 63][nine] = true;
     }
-    const cudaError_t e = launch_overlapped(gdw_tc_kernel, (unsigned)L->grid, kGdwThreads, L->smem, st, L->P);
+    const cudaError_t e = launch_overlapped(kernel, (unsigned)L->grid, kGdwThreads, L->smem, st, L->P);
     if (e != cudaSuccess) { cudaGetLastError(); return cuda_fail(e, "gdw_tc_kernel launch"); }
     p->launches++;
     return GDWS_OK;

@@ -240,13 +240,15 @@ inline int sm_count_of(const gdws_plan_s *p) { return p->sm_count > 0 ? p->sm_co
 gdws_status_t f32_depthwise(gdws_plan_s *p, const gdws_tensor_t *x, const float *dw_w, float *z, cudaStream_t s);
 gdws_status_t f32_pointwise(gdws_plan_s *p, const float *z, const float *pw_w, const float *bias,
                             gdws_tensor_t *y, cudaStream_t s);
+int f32_alu_config(const gdws_plan_s *p, long long npix, int Wo);     // tile of fused_f32_kernel, -1: none
 double f32_alu_us(const gdws_plan_s *p, int n, int h, int w);
 gdws_status_t f32_fused(gdws_plan_s *p, const gdws_tensor_t *x, const float *dw_w, const float *pw_w,
                         const float *bias, gdws_tensor_t *y, cudaStream_t s);
 
 // f32_tc.cu
 double f32_forward_us(gdws_plan_s *p, int n, int h, int w);
-bool f32_tc_takes(gdws_plan_s *p, int n, int h, int w);     // whether a forward of this size runs there
+// Whether a forward of this size runs there; if not *alu is the ALU kernel's tile (left as it is if there is no memory to keep the answer).
+bool f32_tc_takes(gdws_plan_s *p, int n, int h, int w, int *alu);
 gdws_status_t f32_fused_tc(gdws_plan_s *p, const gdws_tensor_t *x, const float *dw_w, const float *pw_w,
                            const float *bias, gdws_tensor_t *y, cudaStream_t s);
 
