@@ -701,14 +701,15 @@ bool f32tc_geometry(const gdws_plan_s *p, int n, int Ho, int Wo, long long xn, F
             if (f32tc_smem(p, slots, g) <= (size_t)kMaxSmem) break;
         if (g.ns < 2) return;
         const long long waves = (g.tiles * parts + sms - 1) / sms;
-        g.split = 1;
-        while (g.split < 8 && g.tiles * parts * g.split * 2 <= sms && nq >= g.split * 4) g.split *= 2;
         // Fitted to 40 layers: a chunk takes 1.5 us and more with more output channels and rounds of staged input (8 channels x 256
         // positions), a tile what its stores take, clusters the adding up.
-        const int rounds = (slots + 7) / 8 * ((g.np + 255) / 256), chunks = (nq + g.split - 1) / g.split;
+        const int rounds = (slots + 7) / 8 * ((g.np + 255) / 256);
         const double chunk = (p->k == 3 ? 1.5 : 1.9) + 0.006 * g.Nd + 0.35 * (rounds - 1);
-        g.us = 5.0 + (double)waves * (chunks * chunk + 0.01 * g.Nd) + (g.split > 1 ? 2.5 : 0.0) + 1e-4 * g.np;
-        if (!found || g.us < out->us) { *out = g; found = true; }
+        for (g.split = 1; g.split <= 8 && g.split <= nq; g.split *= 2) {
+            if (g.split > 1 && g.tiles * parts > cluster_capacity(p, g.split)) break;        // one wave
+            g.us = 5.0 + (double)waves * ((nq + g.split - 1) / g.split * chunk + 0.01 * g.Nd) + (g.split > 1 ? 2.5 : 0.0) + 1e-4 * g.np;
+            if (!found || g.us < out->us) { *out = g; found = true; }
+        }
     };
     for (int j = 1; j <= Wo; ++j) {
         const int PW = (Wo + j - 1) / j;
@@ -768,9 +769,10 @@ static const F32TcLaunch *f32tc_prepared(gdws_plan_s *p, int n, int h, int w)
     e->key = key;
     e->alu = f32_alu_config(p, (long long)n * Ho * Wo, Wo);
     e->taken = p->opt_dw_math != 1 && f32tc_geometry(p, n, Ho, Wo, (long long)p->C * h * w, &e->g);
-    // The other kernel's estimate is 1.3 to 1.8 times too long for calls below 16 us and up to twice too short for large NHWC ones.
+    // The other kernel's estimate is too long for short calls (5 x 32 -> 81 channels at 11 x 9, stride 2: 17.6 for 11.9 us, where this one
+    // takes 14.8) and up to twice too short for large NHWC ones.
     const double alu = f32_alu_us(p, n, h, w);
-    if (e->taken && p->opt_dw_math != 2) e->taken = e->g.us < (alu < 16.0 ? 0.8 : 1.1) * alu;
+    if (e->taken && p->opt_dw_math != 2) e->taken = e->g.us < (alu < 24.0 ? 3.0 + 0.65 * (alu - 3.0) : 1.1 * alu);
     return LaunchCache<F32TcLaunch>::add(p->launch_cache[5], std::move(e));
 }
 

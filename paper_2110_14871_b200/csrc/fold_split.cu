@@ -243,26 +243,9 @@ __global__ void __launch_bounds__(kSplitThreads, 1) fold_split_kernel(const __gr
 // ------------------------------------------------------------------------------------------
 // Host side
 // ------------------------------------------------------------------------------------------
-namespace {
-
-struct SplitGeom {
-    int layout = 0, TN = 0, PH = 0, PW = 0, IW = 0, nl = 0, tiles_n = 0, tiles_h = 0, tiles_w = 0, Npart = 0, nparts = 0, split = 0, na = 0;
-    uint32_t a_bytes = 0, a_load = 0, b_off = 0, slot = 0;
-    double us = 0;
-    int64_t tiles() const { return (int64_t)tiles_n * tiles_h * tiles_w; }
-};
-
-struct SplitLaunch {
-    LaunchKey key;
-    FoldSplitParams P;
-    SplitGeom g;
-    size_t smem = 0;
-    const void *x = nullptr;     // the address the tensor maps were encoded for
-};
-
 // Clusters of `split` blocks, one block per SM, that the plan's device runs at the same time: clusters do not cross the chip's groups of
 // SMs, so some are left over.  Asked once per device (without one, as for queries on a host without a GPU: what a B200 answered).
-int split_clusters(const gdws_plan_s *p, int split)
+int cluster_capacity(const gdws_plan_s *p, int split)
 {
     static int most[64][kSplitMost + 1] = {};
     int &n = most[p->device & 63][split];
@@ -281,6 +264,23 @@ int split_clusters(const gdws_plan_s *p, int split)
     }
     return n;
 }
+
+namespace {
+
+struct SplitGeom {
+    int layout = 0, TN = 0, PH = 0, PW = 0, IW = 0, nl = 0, tiles_n = 0, tiles_h = 0, tiles_w = 0, Npart = 0, nparts = 0, split = 0, na = 0;
+    uint32_t a_bytes = 0, a_load = 0, b_off = 0, slot = 0;
+    double us = 0;
+    int64_t tiles() const { return (int64_t)tiles_n * tiles_h * tiles_w; }
+};
+
+struct SplitLaunch {
+    LaunchKey key;
+    FoldSplitParams P;
+    SplitGeom g;
+    size_t smem = 0;
+    const void *x = nullptr;     // the address the tensor maps were encoded for
+};
 
 // Tile, output channels of a block and slices with the shortest estimated time, one wave of blocks; false where a layer does not fit that.
 bool split_geometry(const gdws_plan_s *p, int n, int Ho, int Wo, SplitGeom *out)
@@ -305,7 +305,7 @@ bool split_geometry(const gdws_plan_s *p, int n, int Ho, int Wo, SplitGeom *out)
             g.slot = g.b_off + (uint32_t)(k * g.Npart) * 128u;
             const size_t room = kMaxSmem - 1024;
             for (int split = 1; split <= std::min(kSplitMost, units); ++split) {
-                if (g.tiles() * g.nparts > split_clusters(p, split)) continue;
+                if (g.tiles() * g.nparts > cluster_capacity(p, split)) continue;
                 const int upc = (units + split - 1) / split;
                 g.split = split;
                 g.na = (int)std::min<size_t>(std::min(upc, kSplitMaxSlots), room / g.slot);

@@ -272,6 +272,7 @@ gdws_status_t bf16_fused_tc(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_
 // fold.cu
 gdws_status_t bf16_folded(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t *y, cudaStream_t s);
 // fold_split.cu: the folded form in slices, for layers that leave SMs idle
+int cluster_capacity(const gdws_plan_s *p, int split);     // clusters of `split` blocks, one per SM, that run at the same time
 double fold_split_us(const gdws_plan_s *p, int n, int Ho, int Wo);      // estimate; 1e9 where it does not cover the layer
 gdws_status_t bf16_folded_split(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t *y, cudaStream_t s);
 double bf16_forward_us(gdws_plan_s *p, int n, int h, int w, bool out_f32);
