@@ -92,24 +92,99 @@ __device__ __forceinline__ void split3(float a, float b, uint32_t &p1, uint32_t 
     p3 = pack_bf16x2(a, b);
 }
 
-// One output's sum over the intermediate channels, in fp32 on the ALUs: for outputs that are not finite.  Pieces of an infinity are
-// an infinity and NaN, so such outputs are computed again from the inputs.  (Once it is NaN a sum stays NaN.)
-template <int K> __device__ __forceinline__ float f32tc_plain(const F32TcParams &P, int n, int ho, int wo, int d)
+// Outputs that are not finite, once more in fp32 on the ALUs (pieces of an infinity are an infinity and NaN).  The warps that add
+// up the chunks leave NaN in their places in y; when a block's tiles are done, they look for them and work such a tile's columns c0
+// to c1 out from the inputs, 64 pixels and 32 intermediate channels at a time through shared memory, added in fused_f32_kernel's order.
+// Nobody waits for the block in a bounded wait meanwhile.  (Each such output summed up by its own thread took 89 ms where one tap of
+// 16 x 128 -> 128 channels at 28 x 28 is infinite, and its code beside the hot loops 2 us of every call; here 0.53 ms, an ordinary call 54 us.)
+constexpr int kF32TcRedoZ = 65, kF32TcRedoW = 129;       // pitches of z and of the weights: odd, for stores down a column
+template <int K, int NB, bool NHWC>
+__device__ __forceinline__ void f32tc_redo(const F32TcParams &P, uint8_t *base, const float *bias, volatile int *any, int tile0, int step, int c0, int c1)
 {
-    float acc = 0.f;
+    constexpr int K2 = K * K, CH = kF32TcChunk, T = 128, COLS = 4 * NB;
+    float *const zs = reinterpret_cast<float *>(base), *const ws = zs + CH * kF32TcRedoZ, *const taps = ws + CH * kF32TcRedoW;
+    int *const pn = reinterpret_cast<int *>(taps + CH * K2), *const ph0 = pn + 128, *const pw0 = ph0 + 128, *const py = pw0 + 128;      // py: pixel of the image
+    static_assert(4 * (CH * (kF32TcRedoZ + kF32TcRedoW + K2) + 4 * 128) <= 2 * (3 * kF32TcA + 3 * 16 * 64), "two stages of operands hold it");
+    const int tid = threadIdx.x, d0 = (int)blockIdx.y * 128 + c0, nd = c1 - c0, pg = tid & 15, dg = tid >> 4;
 #pragma unroll 1
-    for (int i = 0; i < P.G && acc == acc; ++i) {
-        const float *xc = P.x + n * P.xn + P.chan[i] * P.xc, *f = P.dw + (size_t)i * K * K;
-        float z = 0.f;
+    for (int tile = tile0; tile < P.ntiles; tile += step) {
+        const int hw = P.tiles_h * P.tiles_w, ppi = P.PH * P.PW, nl = tid / ppi, ph = (tid - nl * ppi) / P.PW, pw = tid - nl * ppi - ph * P.PW;
+        const int bn = tile / hw, bh = (tile - bn * hw) / P.tiles_w, bw = tile - bn * hw - bh * P.tiles_w;
+        const int n = bn * P.TN + nl, ho = bh * P.PH + ph, wo = bw * P.PW + pw;
+        const bool live = nl < P.TN && n < P.N && ho < P.Ho && wo < P.Wo;
+        pn[tid] = live ? n : -1; ph0[tid] = ho * P.stride - P.pad; pw0[tid] = wo * P.stride - P.pad; py[tid] = ho * P.Wo + wo;
+        if (tid == 0) *any = 0;
+        named_bar_sync(2, T);
+        const float *const yl = P.y + n * P.yn + ho * P.yh + wo * P.yw;
+        bool found = false;
+#pragma unroll 4
+        for (int d = 0; d < nd; ++d)
+            if (live) { const float v = yl[(d0 + d) * P.yc]; found = found || v != v; }
+        if (found) *any = 1;
+        named_bar_sync(2, T);
+        const bool go = *any != 0;
+        named_bar_sync(2, T);
 #pragma unroll 1
-        for (int t = 0; t < K * K; ++t) {
-            const int hi = ho * P.stride - P.pad + t / K, wi = wo * P.stride - P.pad + t % K;
-            const float v = hi >= 0 && hi < P.H && wi >= 0 && wi < P.W ? xc[hi * P.xh + wi * P.xw] : 0.f;
-            z = fmaf(f[t], v, z);
+        for (int half = 0; go && half < 128; half += 64) {
+            float acc[4][COLS] = {};             // pixels half + pg + 16 j, columns dg + 8 e
+#pragma unroll 1
+            for (int i0 = 0; i0 < P.G; i0 += CH) {
+                const int ni = min(CH, P.G - i0);
+#pragma unroll 4
+                for (int t = tid; t < ni * K2; t += T) taps[t % K2 * CH + t / K2] = __ldg(P.dw + (size_t)i0 * K2 + t);
+                if ((tid & (CH - 1)) < ni) {
+                    const float *const w = P.pw + (size_t)d0 * P.G + i0 + (tid & (CH - 1));
+#pragma unroll 8
+                    for (int d = tid / CH; d < nd; d += T / CH) ws[(tid & (CH - 1)) * kF32TcRedoW + d] = __ldg(w + (size_t)d * P.G);
+                }
+                named_bar_sync(2, T);
+#pragma unroll 2
+                for (int e = tid; e < CH * 64; e += T) {
+                    const int rh = NHWC ? e / CH : e & 63, r = half + rh, i = NHWC ? e & (CH - 1) : e >> 6;
+                    if (i < ni && pn[r] >= 0) {
+                        const float *const x = P.x + pn[r] * P.xn + __ldg(P.chan + i0 + i) * P.xc;
+                        const int h0 = ph0[r], w0 = pw0[r];
+                        float z = 0.f;
+#pragma unroll
+                        for (int t = 0; t < K2; ++t) {
+                            const int h = h0 + t / K, w = w0 + t % K;
+                            z = fmaf(taps[t * CH + i], h >= 0 && h < P.H && w >= 0 && w < P.W ? __ldg(x + h * P.xh + w * P.xw) : 0.f, z);
+                        }
+                        zs[i * kF32TcRedoZ + rh] = z;
+                    }
+                }
+                named_bar_sync(2, T);
+#pragma unroll 1
+                for (int i = 0; i < ni; ++i) {   // rows and columns outside: whatever is there, not stored below
+                    float z[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) z[j] = zs[i * kF32TcRedoZ + pg + 16 * j];
+#pragma unroll
+                    for (int e = 0; e < COLS; ++e) {
+                        const float w = ws[i * kF32TcRedoW + dg + 8 * e];
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) acc[j][e] = fmaf(z[j], w, acc[j][e]);
+                    }
+                }
+                named_bar_sync(2, T);
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int r = half + pg + 16 * j, px = py[r];
+                if (pn[r] < 0) continue;
+                float *const yr = P.y + pn[r] * P.yn + px * P.yw + d0 * P.yc;        // pixels of an image are yw apart in either layout
+#pragma unroll
+                for (int e = 0; e < COLS; ++e) {
+                    const int d = dg + 8 * e;
+                    float *const y = yr + d * P.yc;
+                    if (d >= nd || *y == *y) continue;
+                    const float v = acc[j][e] + bias[c0 + d];
+                    *y = P.relu ? fmaxf(v, 0.f) : v;
+                }
+            }
         }
-        acc = fmaf(z, P.pw[(size_t)d * P.G + i], acc);
+        named_bar_sync(2, T);                    // the table is written anew
     }
-    return acc;
 }
 
 // Floats per filter in shared memory: 3 x 3 taps twice each (the packed multiply-adds of two pixels take them as pairs).
@@ -201,7 +276,7 @@ __global__ void __launch_bounds__(kF32TcThreads, 1) f32_tc_kernel(const __grid_c
     // xfull[2] xfree[2] | full[3] free[3] | accfull[2] accfree[2] | drain
     __shared__ __align__(8) uint64_t bars[16];
     __shared__ uint32_t tmem_slot;
-    __shared__ int abort_flag;
+    __shared__ int abort_flag, redo, redo_any;           // redo: an output of this block is not finite
     constexpr int FP = f32tc_filt_pitch(K), K2 = K * K;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     uint8_t *const base = smem_raw + ((0u - smem_u32(smem_raw)) & 1023u);
@@ -211,7 +286,7 @@ __global__ void __launch_bounds__(kF32TcThreads, 1) f32_tc_kernel(const __grid_c
     const uint32_t bar_xfull = smem_u32(&bars[0]), bar_xfree = bar_xfull + 16, bar_full = bar_xfull + 32, bar_free = bar_full + 8 * kF32TcMaxStages;
     const uint32_t bar_accfull = bar_free + 8 * kF32TcMaxStages, bar_accfree = bar_accfull + 16, bar_drain = bar_accfree + 16;
     if (tid == 0) {
-        abort_flag = 0;
+        abort_flag = redo = 0;
 #pragma unroll 1
         for (int i = 0; i < 2; ++i) { mbar_init(bar_xfull + 8 * i, 8); mbar_init(bar_xfree + 8 * i, 8); mbar_init(bar_accfull + 8 * i, 1); mbar_init(bar_accfree + 8 * i, 4); }
 #pragma unroll 1
@@ -316,9 +391,8 @@ __global__ void __launch_bounds__(kF32TcThreads, 1) f32_tc_kernel(const __grid_c
                         for (odd = live ? odd : 0u; odd; odd &= odd - 1) {
                             const int d = c + __ffs(odd) - 1;
                             if (d >= dn) break;
-                            float v = f32tc_plain<K>(P, n, ho, wo, d0 + d) + bias_sm[d];
-                            if (P.relu) v = fmaxf(v, 0.f);
-                            yp[d * P.yc] = v;
+                            yp[d * P.yc] = __uint_as_float(0x7fffffffu);
+                            redo = 1;
                         }
                     }
                 }
@@ -328,6 +402,7 @@ __global__ void __launch_bounds__(kF32TcThreads, 1) f32_tc_kernel(const __grid_c
             }
             if (split > 1) break;
         }
+        int c0 = 0, c1 = dn;                     // columns that this block stores
         if (split > 1) {                         // all products are done: the operands' memory takes the sums, [column][pixel]
             float *part = reinterpret_cast<float *>(base);
             const uint32_t t = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(((q1 - q0 - 1) & 1) * 32 * NB);
@@ -339,7 +414,46 @@ __global__ void __launch_bounds__(kF32TcThreads, 1) f32_tc_kernel(const __grid_c
 #pragma unroll
                 for (int e = 0; e < 16; ++e) part[(c + e) * 128 + r] = __uint_as_float(a[e]);
             }
+            cluster_sync();                      // rank r of the cluster finishes its share of the output channels, at least 4
+            const int bn = cluster / hw, bh = (cluster - bn * hw) / P.tiles_w, bw = cluster - bn * hw - bh * P.tiles_w;
+            const int n = bn * P.TN + nl, ho = bh * P.PH + ph, wo = bw * P.PW + pw;
+            const bool live = nl < P.TN && n < P.N && ho < P.Ho && wo < P.Wo;
+            float *yp = P.y + n * P.yn + ho * P.yh + wo * P.yw + d0 * P.yc;
+            c0 = rank * (32 * NB / split); c1 = min(c0 + 32 * NB / split, dn);
+#pragma unroll 1
+            for (int c = c0; live && c < c1; c += 4) {
+                float v[4] = {};
+#pragma unroll 1
+                for (int o0 = 0; o0 < split; o0 += 4) {      // in the chunks' order, sixteen reads in flight
+                    float w[4][4];
+#pragma unroll
+                    for (int o = 0; o < 4; ++o) {
+                        if (o0 + o >= split) break;
+                        const uint32_t src = map_shared(ab_s + (uint32_t)(c * 128 + r) * 4u, (uint32_t)(o0 + o));
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(w[o][e]) : "r"(src + 512u * e));
+                    }
+#pragma unroll
+                    for (int o = 0; o < 4; ++o)
+#pragma unroll
+                        for (int e = 0; e < 4; ++e)
+                            if (o0 + o < split) v[e] += w[o][e];
+                }
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    if (c + e >= c1) break;
+                    const bool fine = fabsf(v[e]) <= FLT_MAX;
+                    if (!fine) redo = 1;
+                    v[e] += bias_sm[c + e];
+                    if (P.relu) v[e] = fmaxf(v[e], 0.f);
+                    yp[(c + e) * P.yc] = fine ? v[e] : __uint_as_float(0x7fffffffu);
+                }
+            }
+            __syncwarp();
+            cluster_sync();                      // every block's sums have been read
         }
+        named_bar_sync(2, 128);
+        if (*(volatile int *)&redo) f32tc_redo<K, NB, NHWC>(P, base, bias_sm, &redo_any, cluster, nclusters, c0, c1);
     } else if (warp < kF32TcLoadWarp) {
         // ---------------- z ----------------
         f32tc_regs_dec<kF32TcRegsZ>();
@@ -591,58 +705,13 @@ __global__ void __launch_bounds__(kF32TcThreads, 1) f32_tc_kernel(const __grid_c
         }
         __syncwarp();
     }
+    if (split > 1 && warp >= kF32TcZWarp) {      // the two of the warps that finish y
+        cluster_sync();
+        cluster_sync();
+    }
     tc_fence_before();
     __syncthreads();
     if (warp == kF32TcMmaWarp) tmem_dealloc(tmem, 64u * NB);
-    if (split > 1) {
-        cluster_sync();
-        if (warp < kF32TcZWarp) {                // rank r of the cluster finishes its share of the output channels
-            const int r = tid, ppi = P.PH * P.PW, per = 32 * NB / split;
-            const int nl = r / ppi, ph = (r - nl * ppi) / P.PW, pw = r - nl * ppi - ph * P.PW;
-            const int bn = cluster / hw, bh = (cluster - bn * hw) / P.tiles_w, bw = cluster - bn * hw - bh * P.tiles_w;
-            const int n = bn * P.TN + nl, ho = bh * P.PH + ph, wo = bw * P.PW + pw;
-            if (nl < P.TN && n < P.N && ho < P.Ho && wo < P.Wo) {
-                float *yp = P.y + n * P.yn + ho * P.yh + wo * P.yw + d0 * P.yc;
-#pragma unroll 1
-                for (int c = rank * per; c < (rank + 1) * per && c < dn; c += 4) {       // at least 4 columns each
-                    float v[4] = {};
-#pragma unroll 1
-                    for (int o0 = 0; o0 < split; o0 += 4) {  // in the chunks' order, sixteen reads in flight
-                        float w[4][4];
-#pragma unroll
-                        for (int o = 0; o < 4; ++o) {
-                            if (o0 + o >= split) break;
-                            const uint32_t src = map_shared(ab_s + (uint32_t)(c * 128 + r) * 4u, (uint32_t)(o0 + o));
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(w[o][e]) : "r"(src + 512u * e));
-                        }
-#pragma unroll
-                        for (int o = 0; o < 4; ++o)
-#pragma unroll
-                            for (int e = 0; e < 4; ++e)
-                                if (o0 + o < split) v[e] += w[o][e];
-                    }
-                    uint32_t odd = 0;
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        if (!(fabsf(v[e]) <= FLT_MAX)) odd |= 1u << e;
-                        v[e] += bias_sm[c + e];
-                        if (P.relu) v[e] = fmaxf(v[e], 0.f);
-                        if (c + e < dn) yp[(c + e) * P.yc] = v[e];
-                    }
-#pragma unroll 1
-                    for (; odd; odd &= odd - 1) {
-                        const int d = c + __ffs(odd) - 1;
-                        if (d >= dn) break;
-                        float t = f32tc_plain<K>(P, n, ho, wo, d0 + d) + bias_sm[d];
-                        if (P.relu) t = fmaxf(t, 0.f);
-                        yp[d * P.yc] = t;
-                    }
-                }
-            }
-        }
-        cluster_sync();                          // every block's sums have been read
-    }
 }
 
 namespace {
