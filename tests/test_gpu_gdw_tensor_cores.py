@@ -58,3 +58,41 @@ def test_matches_alu_kernel_and_reference(N, C, H, W, k, stride, g):
     fine = np.isfinite(alu)
     assert not fine.all() and np.abs(tc[fine] - alu[fine]).max() <= 2 ** -7 * np.abs(alu[fine]).max()
     plan.destroy()
+
+
+@pytest.mark.parametrize("v", [float("inf"), float("nan")])
+@pytest.mark.parametrize("N,C,H,W,k,stride", [(64, 64, 56, 56, 3, 1), (9, 48, 41, 39, 5, 2), (20, 64, 7, 4, 3, 1)])
+def test_values_that_are_not_finite_do_not_take_long(N, C, H, W, k, stride, v):
+    """x that is infinite or NaN everywhere: every z is worked out again on the ALUs, as the ALU kernel has it, within some 20 times
+    the time of ordinary values."""
+    data = gi.make_layer(small_spec("t", N, C, 16, H, W, k, stride, k // 2, ("uniform", 1, 4), "bf16", "NHWC", seed=C + H))
+    plan = make_plan(data)
+    plan.pack_weights(to_device(data.dw_w, "bf16"), to_device(data.pw_w, "bf16"))
+    G, Gp, _, _ = plan.info()
+    x = to_device(data.x, "bf16")
+    bad = torch.full_like(x, v)
+    zs = [torch.full((N * data.spec.Ho * data.spec.Wo, Gp), 7.0, dtype=torch.bfloat16, device="cuda") for _ in range(2)]
+
+    def least_ms(x):
+        ms = []
+        for _ in range(5):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for _ in range(4):
+                plan.depthwise(x, zs[0], "NHWC")
+            b.record()
+            torch.cuda.synchronize()
+            ms.append(a.elapsed_time(b))
+        return min(ms)
+
+    plan.set_option(gdws.OPT_DW_MATH, 2)
+    least_ms(x)
+    plain, slow = least_ms(x), least_ms(bad)
+    plan.set_option(gdws.OPT_DW_MATH, 1)
+    plan.depthwise(bad, zs[1], "NHWC")
+    torch.cuda.synchronize()
+    plan.status()
+    a, b = (z.float().cpu().numpy() for z in zs)
+    assert np.array_equal(a, b, equal_nan=True) and not np.isfinite(a[:, :G]).all()
+    assert slow <= 40 * plain
+    plan.destroy()
