@@ -98,3 +98,20 @@ def test_an_infinite_tap_does_not_take_long(N, C, D, H, W, k, layout):
     assert least_ms(dw) <= 100 * least_ms(plain)
     plan.status()
     plan.destroy()
+
+
+@pytest.mark.parametrize("N,C,D,H,W,k", [(2, 40, 48, 20, 21, 3), (1, 150, 130, 14, 10, 3), (2, 17, 64, 20, 20, 5)])
+def test_small_and_large_values_keep_their_bits(N, C, D, H, W, k):
+    """x, taps and weights around fp32's ends: as exact as the ALU kernel, whose sums round at 2^-149 too."""
+    data = gi.make_layer(small_spec("t", N, C, D, H, W, k, 1, k // 2, ("uniform", 1, 9), "f32", "NCHW", seed=31 + C))
+    data.bias[:] = 0
+    parts = [np.copy(a) for a in (data.x, data.dw_w, data.pw_w)]
+    for ends in [(0, 0, -60), (-60, 0, 0), (-60, -30, -20), (0, 0, -100), (0, 0, -110), (0, 0, -116), (0, 0, -123), (-100, 0, 0), (-110, 0, 0), (-116, 0, 0), (-123, 0, 0), (0, -123, 0), (-123, 100, 0), (60, 0, -123),
+                 (0, 0, 40), (40, 20, 30), (100, 0, 0), (0, 110, 0), (0, 0, 110), (0, 60, 50)]:
+        for a, p, e in zip((data.x, data.dw_w, data.pw_w), parts, ends):
+            a[...] = np.ldexp(p, e)
+        ref, _ = run_oracle(data)
+        tc, alu = (run_gpu(data, path=gdws.PATH_FUSED, dw_math=m) for m in (2, 1))
+        size = np.linalg.norm(np.ldexp(ref, -sum(ends)))         # in range for its squares
+        err = [np.linalg.norm(np.ldexp(y - ref, -sum(ends))) / size for y in (tc, alu)]
+        assert err[0] <= err[1] and err[0] <= 1e-5, (ends, err)
