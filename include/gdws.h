@@ -94,11 +94,12 @@ typedef enum {
                               infinity or NaN in them reaches y.  0 takes 3 for layers with
                               g_c = 0 only where no other kernel covers them (D > 512).
                               fp32 forwards: 1 = all arithmetic on the ALUs; 2 = pointwise products
-                              on the tensor cores (three bf16 pieces per value, fp32 sums, no less
-                              exact) for k = 3 and 5; 0 and 3 = whichever is estimated faster.
-                              gdws_depthwise, bf16: 1 = ALUs, 2 = tensor cores where they cover the
-                              layer, 0 and 3 = whichever is estimated faster: same z but for values
-                              next to a rounding boundary                                    */
+                              on the tensor cores (three bf16 pieces per value, fp32 sums) for
+                              k = 3 and 5; 0 and 3 = whichever is estimated faster.
+                              gdws_depthwise, bf16: 1 = ALUs, 2 = tensor cores, 0 and 3 = whichever
+                              is estimated faster: same z but for values next to a rounding boundary.
+                              In these two calls 2 is a preference: a layer that the tensor cores do
+                              not cover runs on the ALUs (gdws_plan_kernel tells)             */
     GDWS_OPT_OUT_DTYPE = 5 /* bf16 plans: 0 (default) = y has the dtype of x; 1 = y is fp32
                               (GDWS_F32, NHWC): bias and ReLU are applied to the fp32 sums of
                               the PW stage and stored without the rounding to bf16.  Every
@@ -180,6 +181,25 @@ GDWS_API gdws_status_t gdws_plan_gdw_stage(const gdws_plan_t *plan, int *stage);
  * to the two stages then.)  Host only; errors: GDWS_ERR_INVALID_ARG.
  */
 GDWS_API gdws_status_t gdws_plan_form(gdws_plan_t *plan, int n, int h, int w, int *form);
+
+/* The kernels among which the library chooses by estimated time. */
+typedef enum {
+    GDWS_KERNEL_TWO_STAGES_ALU = 1,  /* bf16 forward, form 1                                                */
+    GDWS_KERNEL_TWO_STAGES_TC = 2,   /* bf16 forward, form 2                                                */
+    GDWS_KERNEL_FOLDED_PAIRS = 3,    /* bf16 forward, form 3: pairs of SMs share a tile's products          */
+    GDWS_KERNEL_FOLDED_SLICES = 4,   /* bf16 forward, form 3, few tiles: clusters share a tile's sum        */
+    GDWS_KERNEL_F32_ALU = 5,         /* fp32 forward, all arithmetic on the ALUs                            */
+    GDWS_KERNEL_F32_PIECES = 6,      /* fp32 forward, pointwise products on the tensor cores in bf16 pieces */
+    GDWS_KERNEL_GDW_ALU = 7,         /* gdws_depthwise, bf16                                                */
+    GDWS_KERNEL_GDW_TC = 8
+} gdws_kernel_t;
+
+/*
+ * gdws_plan_kernel -- the kernel that a call of n x C x h x w takes with the plan's current options: gdws_depthwise
+ * (stage != 0; GDWS_BF16) or a fused gdws_forward with packed weights (stage = 0).  Diagnostic.  Host only; errors:
+ * GDWS_ERR_INVALID_ARG.
+ */
+GDWS_API gdws_status_t gdws_plan_kernel(gdws_plan_t *plan, int stage, gdws_dtype_t dtype, int n, int h, int w, int *kernel);
 
 /*
  * gdws_pack_weights -- convert one weight set to the kernels' internal form

@@ -59,7 +59,7 @@ __global__ void gdw_bf16_kernel(DwShape s, const uint16_t *__restrict__ x, const
 
 gdws_status_t bf16_depthwise(gdws_plan_s *p, const gdws_tensor_t *x, void *z, cudaStream_t st)
 {
-    if (p->opt_dw_math != 1 && !p->opt_tile && !p->opt_a_layout) {
+    if (bf16_depthwise_on_tc(p, x->n, x->h, x->w)) {
         const gdws_status_t rc = bf16_depthwise_tc(p, x, z, st);
         if (rc != GDWS_ERR_UNSUPPORTED) return rc;
     }

@@ -907,6 +907,14 @@ double bf16_forward_us(gdws_plan_s *p, int n, int h, int w, bool out_f32)
     return 4.0 + std::ceil((double)t.tiles() / sm_count_of(p)) * p->nchunks * 0.55 * p->k * p->k;
 }
 
+bool fold_in_slices(gdws_plan_s *p, int n, int h, int w, bool out_f32)
+{
+    if (const FormChoice *c = LaunchCache<FormChoice>::find(p->launch_cache[3], {n, h, w, out_f32 ? 2 : 0})) return c->sliced;
+    const int Ho = gdws_out_dim(h, p->k, p->stride, p->pad), Wo = gdws_out_dim(w, p->k, p->stride, p->pad);
+    FoldGeom g;
+    return !(fold_geometry(p, n, Ho, Wo, out_f32, &g) && g.us <= fold_split_us(p, n, Ho, Wo));
+}
+
 gdws_status_t bf16_folded(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t *y, cudaStream_t st)
 {
     if (!p->fold_ok) return fail(GDWS_ERR_UNSUPPORTED, "folded path: layer not covered (stride 1 or 2, k <= 5, C and D multiples of 8)");
@@ -918,12 +926,7 @@ gdws_status_t bf16_folded(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t 
         std::unique_ptr<FoldLaunch> e(new (std::nothrow) FoldLaunch);
         if (!e) return fail(GDWS_ERR_ALLOC, "out of host memory");
         e->key = key;
-        if (const FormChoice *c = LaunchCache<FormChoice>::find(p->launch_cache[3], {x->n, x->h, x->w, out_f32 ? 2 : 0})) {
-            e->sliced = c->sliced;
-        } else {
-            FoldGeom g;
-            e->sliced = !(fold_geometry(p, x->n, y->h, y->w, out_f32, &g) && g.us <= fold_split_us(p, x->n, y->h, y->w));
-        }
+        e->sliced = fold_in_slices(p, x->n, x->h, x->w, out_f32);
         rc = e->sliced ? GDWS_OK : fold_prepare(p, x->n, y->h, y->w, out_f32, e.get());
         if (rc != GDWS_OK) return rc;
         L = LaunchCache<FoldLaunch>::add(p->launch_cache[2], std::move(e));

@@ -613,23 +613,34 @@ gdws_status_t gdw_maps(const gdws_plan_s *p, const gdws_tensor_t *x, void *z, Gd
 
 }  // namespace
 
+// The prepared launch of a size; null without host memory for it.
+static GdwLaunch *gdw_prepared(gdws_plan_s *p, int n, int h, int w)
+{
+    const LaunchKey key = {n, h, w, p->opt_dw_math};
+    if (GdwLaunch *L = LaunchCache<GdwLaunch>::find(p->launch_cache[6], key)) return L;
+    std::unique_ptr<GdwLaunch> e(new (std::nothrow) GdwLaunch);
+    if (!e) return nullptr;
+    const int Ho = gdws_out_dim(h, p->k, p->stride, p->pad), Wo = gdws_out_dim(w, p->k, p->stride, p->pad);
+    e->key = key;
+    // one row or column and stride 2: the view of the odd ones is empty
+    e->taken = p->G > 0 && !(p->stride == 2 && (h < 2 || w < 2) && tc_taps(p->k, 2, p->pad).used[1]) && gdw_prepare(p, n, Ho, Wo, e.get());
+    e->P.H = h; e->P.W = w;
+    if (e->taken && p->opt_dw_math != 2) e->taken = e->us < gdw_alu_us(p, n, h, w);
+    return LaunchCache<GdwLaunch>::add(p->launch_cache[6], std::move(e));
+}
+
+bool bf16_depthwise_on_tc(gdws_plan_s *p, int n, int h, int w)
+{
+    if (p->opt_dw_math == 1 || p->opt_tile || p->opt_a_layout) return false;
+    const GdwLaunch *L = gdw_prepared(p, n, h, w);
+    return L && L->taken;
+}
+
 // GDWS_ERR_UNSUPPORTED: not covered, nothing was launched.
 gdws_status_t bf16_depthwise_tc(gdws_plan_s *p, const gdws_tensor_t *x, void *z, cudaStream_t st)
 {
-    const LaunchKey key = {x->n, x->h, x->w, p->opt_dw_math};
-    GdwLaunch *L = LaunchCache<GdwLaunch>::find(p->launch_cache[6], key);
-    if (!L) {
-        std::unique_ptr<GdwLaunch> e(new (std::nothrow) GdwLaunch);
-        if (!e) return fail(GDWS_ERR_ALLOC, "out of host memory");
-        const int Ho = gdws_out_dim(x->h, p->k, p->stride, p->pad), Wo = gdws_out_dim(x->w, p->k, p->stride, p->pad);
-        e->key = key;
-        // one row or column and stride 2: the view of the odd ones is empty
-        e->taken = p->G > 0 && !(p->stride == 2 && (x->h < 2 || x->w < 2) && tc_taps(p->k, 2, p->pad).used[1]) && gdw_prepare(p, x->n, Ho, Wo, e.get());
-        e->P.H = x->h; e->P.W = x->w;
-        if (e->taken && p->opt_dw_math != 2) e->taken = e->us < gdw_alu_us(p, x->n, x->h, x->w);
-        L = LaunchCache<GdwLaunch>::add(p->launch_cache[6], std::move(e));
-        if (!L) return fail(GDWS_ERR_ALLOC, "out of host memory");
-    }
+    GdwLaunch *L = gdw_prepared(p, x->n, x->h, x->w);
+    if (!L) return fail(GDWS_ERR_ALLOC, "out of host memory");
     if (!L->taken) return fail(GDWS_ERR_UNSUPPORTED, "GDW stage on the tensor cores: layer not covered");
     const gdws_status_t rc = gdw_maps(p, x, z, L);
     if (rc != GDWS_OK) return rc;

@@ -265,6 +265,7 @@ gdws_status_t bf16_depthwise_tiled(gdws_plan_s *p, const gdws_tensor_t *x, void 
 
 // gdw_tc.cu
 gdws_status_t bf16_depthwise_tc(gdws_plan_s *p, const gdws_tensor_t *x, void *z, cudaStream_t s);
+bool bf16_depthwise_on_tc(gdws_plan_s *p, int n, int h, int w);        // whether gdws_depthwise runs there
 
 // fused_tc.cu
 gdws_status_t bf16_fused_tc(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t *y, cudaStream_t s);
@@ -275,6 +276,7 @@ gdws_status_t bf16_folded(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t 
 int cluster_capacity(const gdws_plan_s *p, int split);     // clusters of `split` blocks, one per SM, that run at the same time
 double fold_split_us(const gdws_plan_s *p, int n, int Ho, int Wo);      // estimate; 1e9 where it does not cover the layer
 gdws_status_t bf16_folded_split(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t *y, cudaStream_t s);
+bool fold_in_slices(gdws_plan_s *p, int n, int h, int w, bool out_f32);      // whether a folded forward runs there
 double bf16_forward_us(gdws_plan_s *p, int n, int h, int w, bool out_f32);
 int bf16_form_of(gdws_plan_s *p, int n, int h, int w, bool out_f32);   // 1 / 2: two stages, GDW on the ALUs / the tensor cores; 3: folded
 

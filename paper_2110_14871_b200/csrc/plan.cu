@@ -527,6 +527,25 @@ gdws_status_t gdws_plan_form(gdws_plan_t *p, int n, int h, int w, int *form)
     return GDWS_OK;
 }
 
+gdws_status_t gdws_plan_kernel(gdws_plan_t *p, int stage, gdws_dtype_t dtype, int n, int h, int w, int *kernel)
+{
+    if (!p || !kernel) return fail(GDWS_ERR_INVALID_ARG, "gdws_plan_kernel: NULL argument");
+    if (n < 1 || gdws_out_dim(h, p->k, p->stride, p->pad) < 1 || gdws_out_dim(w, p->k, p->stride, p->pad) < 1)
+        return fail(GDWS_ERR_INVALID_ARG, "gdws_plan_kernel: no output for n=%d h=%d w=%d", n, h, w);
+    if ((dtype != GDWS_F32 && dtype != GDWS_BF16) || (stage && dtype != GDWS_BF16)) return fail(GDWS_ERR_INVALID_ARG, "gdws_plan_kernel: bad dtype");
+    if (stage) {
+        *kernel = bf16_depthwise_on_tc(p, n, h, w) ? GDWS_KERNEL_GDW_TC : GDWS_KERNEL_GDW_ALU;
+    } else if (dtype == GDWS_F32) {
+        int alu = 0;
+        *kernel = f32_tc_takes(p, n, h, w, &alu) ? GDWS_KERNEL_F32_PIECES : GDWS_KERNEL_F32_ALU;
+    } else {
+        const bool out_f32 = p->opt_out_f32 != 0;
+        const int form = bf16_form_of(p, n, h, w, out_f32);
+        *kernel = form == 3 && fold_in_slices(p, n, h, w, out_f32) ? GDWS_KERNEL_FOLDED_SLICES : form;
+    }
+    return GDWS_OK;
+}
+
 int64_t gdws_launch_count(const gdws_plan_t *p) { return p ? p->launches : 0; }
 
 const char *gdws_last_error(void) { return gdws::g_err; }

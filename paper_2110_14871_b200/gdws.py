@@ -23,6 +23,8 @@ F32, BF16 = 0, 1
 NCHW, NHWC = 0, 1
 OPT_PATH, OPT_RELU, OPT_TILE, OPT_A_LAYOUT, OPT_DW_MATH, OPT_OUT_DTYPE = range(6)
 PATH_AUTO, PATH_FUSED, PATH_UNFUSED = 0, 1, 2
+(KERNEL_TWO_STAGES_ALU, KERNEL_TWO_STAGES_TC, KERNEL_FOLDED_PAIRS, KERNEL_FOLDED_SLICES, KERNEL_F32_ALU, KERNEL_F32_PIECES,
+ KERNEL_GDW_ALU, KERNEL_GDW_TC) = range(1, 9)
 
 EXPORTS = [
     "gdws_plan", "gdws_plan_set_option", "gdws_plan_info", "gdws_plan_tables", "gdws_plan_tile",
@@ -30,6 +32,7 @@ EXPORTS = [
     "gdws_depthwise", "gdws_pointwise", "gdws_forward_host", "gdws_status", "gdws_launch_count",
     "gdws_last_error", "gdws_version", "gdws_destroy", "gdws_forward_static", "gdws_static_scratch_bytes",
     "gdws_measure_fma_rate", "gdws_measure_code_size", "gdws_selftest_wait", "gdws_plan_gdw_stage", "gdws_plan_form",
+    "gdws_plan_kernel",
 ]
 
 
@@ -79,6 +82,8 @@ def lib() -> ctypes.CDLL:
     L.gdws_plan_gdw_stage.restype = ci
     L.gdws_plan_form.argtypes = [vp, ci, ci, ci, pint]
     L.gdws_plan_form.restype = ci
+    L.gdws_plan_kernel.argtypes = [vp, ci, ci, ci, ci, ci, pint]
+    L.gdws_plan_kernel.restype = ci
     L.gdws_out_dim.argtypes = [ci, ci, ci, ci]
     L.gdws_out_dim.restype = ci
     L.gdws_pack_weights.argtypes = [vp, vp, vp, vp, ci, vp]
@@ -281,6 +286,12 @@ class Plan:
         form = ctypes.c_int()
         _check(lib().gdws_plan_form(self._h, n, h, w, ctypes.byref(form)))
         return form.value
+
+    def kernel(self, n: int, h: int, w: int, dtype: int = BF16, stage: bool = False) -> int:
+        """gdws_plan_kernel: KERNEL_* that a forward (stage: a depthwise call) of this size takes."""
+        kernel = ctypes.c_int()
+        _check(lib().gdws_plan_kernel(self._h, int(stage), dtype, n, h, w, ctypes.byref(kernel)))
+        return kernel.value
 
     def workspace_bytes(self, dtype: int, n: int, h: int, w: int) -> int:
         return int(lib().gdws_workspace_bytes(self._h, dtype, n, h, w))

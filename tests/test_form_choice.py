@@ -69,3 +69,20 @@ def test_small_maps_with_stride_2_keep_the_alu_kernel(C, D, k, g, n, h):
     plan = _plan(C, D, k, 2, g)
     assert plan.form(n, h, h) == 1
     plan.destroy()
+
+
+def test_kernel_agrees_with_form():
+    """gdws_plan_kernel: form 3 is the pairs' kernel or the slices', the others their own."""
+    for C, D, k, stride, g, n, h, kernel in [(64, 64, 3, 1, 5, 512, 32, gdws.KERNEL_FOLDED_PAIRS), (256, 256, 3, 1, 3, 1, 14, gdws.KERNEL_FOLDED_SLICES),
+                                             (512, 512, 3, 1, 2, 32, 28, gdws.KERNEL_TWO_STAGES_ALU)]:
+        plan = _plan(C, D, k, stride, g)
+        assert plan.kernel(n, h, h) == kernel and min(plan.kernel(n, h, h), 3) == plan.form(n, h, h)
+        plan.destroy()
+    plan = _plan(64, 64, 3, 1, 5)
+    assert plan.kernel(64, 28, 28, gdws.F32) == gdws.KERNEL_F32_PIECES and plan.kernel(64, 56, 56, stage=True) == gdws.KERNEL_GDW_TC
+    plan.set_option(gdws.OPT_DW_MATH, 1)
+    assert plan.kernel(64, 28, 28, gdws.F32) == gdws.KERNEL_F32_ALU and plan.kernel(64, 56, 56, stage=True) == gdws.KERNEL_GDW_ALU
+    for bad in [lambda: plan.kernel(0, 28, 28), lambda: plan.kernel(1, 28, 28, 7), lambda: plan.kernel(1, 28, 28, gdws.F32, stage=True)]:
+        with pytest.raises(gdws.GdwsError):
+            bad()
+    plan.destroy()

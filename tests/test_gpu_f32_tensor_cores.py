@@ -34,11 +34,19 @@ SHAPES = [
 ]
 
 
+def _on_tensor_cores(data):
+    """The option falls back to the ALUs where the tensor cores do not cover a layer."""
+    plan = make_plan(data, path=gdws.PATH_FUSED, dw_math=2)
+    assert plan.kernel(data.spec.N, data.spec.H, data.spec.W, gdws.F32) == gdws.KERNEL_F32_PIECES
+    plan.destroy()
+
+
 @pytest.mark.parametrize("layout", ["NCHW", "NHWC"])
 @pytest.mark.parametrize("shape", SHAPES)
 def test_matches_reference(shape, layout):
     N, C, D, H, W, k, s, gd = shape
     data = gi.make_layer(small_spec("t", N, C, D, H, W, k, s, k // 2, gd, "f32", layout, relu=D == 33, seed=3 + sum(shape[:7])))
+    _on_tensor_cores(data)
     ref, _ = run_oracle(data)
     tc, alu = (run_gpu(data, path=gdws.PATH_FUSED, dw_math=m) for m in (2, 1))
     # dropped pieces and the chunks' truncation: 2^-22 of sum |P||z|, some sqrt(G) times the largest output
@@ -56,6 +64,7 @@ def test_nonfinite_values_are_those_of_the_sums(N, C, D, H, W, k, layout):
     for v in (np.inf, -np.inf, np.nan, 3.4e38):
         flat[rng.integers(0, flat.size, 3)] = v
     data.pw_w[1, 2], data.pw_w[D - 1, 0] = np.inf, 0.0
+    _on_tensor_cores(data)
     got = []
     for m in (2, 1):
         got.append(run_gpu(data, path=gdws.PATH_FUSED, dw_math=m))
@@ -74,6 +83,7 @@ def test_an_infinite_tap_does_not_take_long(N, C, D, H, W, k, layout):
     a time that stays near an ordinary forward's (10 to 30 times it; 1000 and more with a sum per thread)."""
     data = gi.make_layer(small_spec("t", N, C, D, H, W, k, 1, k // 2, ("uniform", 1, 9), "f32", layout, seed=9 + C))
     data.dw_w[7, 1, 1], data.dw_w[9, 0, 0] = np.inf, 3e38
+    _on_tensor_cores(data)
     got = [run_gpu(data, path=gdws.PATH_FUSED, dw_math=m) for m in (2, 1)]
     for test in (np.isnan, np.isposinf, np.isneginf):
         assert np.array_equal(test(got[0]), test(got[1]))
@@ -105,6 +115,7 @@ def test_small_and_large_values_keep_their_bits(N, C, D, H, W, k):
     """x, taps and weights around fp32's ends: as exact as the ALU kernel, whose sums round at 2^-149 too."""
     data = gi.make_layer(small_spec("t", N, C, D, H, W, k, 1, k // 2, ("uniform", 1, 9), "f32", "NCHW", seed=31 + C))
     data.bias[:] = 0
+    _on_tensor_cores(data)
     parts = [np.copy(a) for a in (data.x, data.dw_w, data.pw_w)]
     for ends in [(0, 0, -60), (-60, 0, 0), (-60, -30, -20), (0, 0, -100), (0, 0, -110), (0, 0, -116), (0, 0, -123), (-100, 0, 0), (-110, 0, 0), (-116, 0, 0), (-123, 0, 0), (0, -123, 0), (-123, 100, 0), (60, 0, -123),
                  (0, 0, 40), (40, 20, 30), (100, 0, 0), (0, 110, 0), (0, 0, 110), (0, 60, 50)]:

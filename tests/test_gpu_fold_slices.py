@@ -31,7 +31,7 @@ def test_slices_match_reference(N, C, D, H, W, k, stride, zero_sum):
         data.dw_w[...] = torch.from_numpy(data.dw_w - data.dw_w.mean(axis=(1, 2), keepdims=True)).to(torch.bfloat16).float().numpy()
     plan = make_plan(data)
     plan.set_option(gdws.OPT_OUT_DTYPE, int(f32))
-    assert plan.form(N, H, W) == 3
+    assert plan.form(N, H, W) == 3 and plan.kernel(N, H, W) == gdws.KERNEL_FOLDED_SLICES
     plan.pack_weights(to_device(data.dw_w, "bf16"), to_device(data.pw_w, "bf16"), torch.from_numpy(data.bias).cuda())
     x = to_device(data.x, "bf16")
     yg = Guarded((N, s.Ho, s.Wo, D), torch.float32 if f32 else torch.bfloat16)

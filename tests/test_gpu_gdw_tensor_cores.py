@@ -36,6 +36,7 @@ def test_matches_alu_kernel_and_reference(N, C, H, W, k, stride, g):
 
     def run(dw_math):
         plan.set_option(gdws.OPT_DW_MATH, dw_math)
+        assert plan.kernel(N, H, W, stage=True) == (gdws.KERNEL_GDW_TC if dw_math == 2 else gdws.KERNEL_GDW_ALU)
         zg.t.fill_(7.0)
         plan.depthwise(x, zg.t, "NHWC")
         torch.cuda.synchronize()
@@ -86,6 +87,7 @@ def test_values_that_are_not_finite_do_not_take_long(N, C, H, W, k, stride, v):
         return min(ms)
 
     plan.set_option(gdws.OPT_DW_MATH, 2)
+    assert plan.kernel(N, H, W, stage=True) == gdws.KERNEL_GDW_TC
     least_ms(x)
     plain, slow = least_ms(x), least_ms(bad)
     plan.set_option(gdws.OPT_DW_MATH, 1)
