@@ -13,8 +13,9 @@
 // weights of 2^-110 the error was 5e-7 and at 2^-123 4e-3.)  At the other end outputs beyond 2^79 and z and weights beyond 2^103
 // overflow and are worked out again like those that are not finite.
 //
-// Measured against 64 bits over 60 layers (2-norm): 0.8e-7 to 1.4e-7, the ALU kernel 0.9e-7 to 6.8e-7, never less exact on the same
-// layer.
+// Error against 64 bits (2-norm), this kernel over the ALU kernel, G intermediate channels, 3 x 3 | 5 x 5 taps: 1.20 | 1.07 at G = 1, 1.04 |
+// 1.01 at 4, 0.98 | 0.96 at 8, 0.80 | 0.88 at 16, 0.71 | 0.78 at 32, 0.42 | 0.52 at 128, 0.22 | 0.18 at 648 | 1693 (positive values: 1.05 |
+// 1.09 at 8, 0.79 | 0.81 at 16).  With few terms the tensor cores' truncation outweighs the roundings saved: from kF32TcLeast on only.
 //
 // What bounds it: the serial instruction streams of the warps that load and cut (3900 cycles a chunk if nothing else runs) and that
 // compute z (3500), which share four schedulers at two instructions per cycle; the products (12 of 128 x N x 16, 768 cycles a chunk at
@@ -37,6 +38,7 @@
 namespace gdws {
 
 constexpr int kF32TcChunk = 32;          // intermediate channels per chunk: 64-byte rows of bf16
+constexpr int kF32TcLeast = 16;          // intermediate channels from which on it is as exact as the ALUs (above)
 constexpr int kF32TcThreads = 24 * 32;
 constexpr int kF32TcZWarp = 4, kF32TcLoadWarp = 12, kF32TcMmaWarp = 20;
 // Registers per thread after the split: setmaxnreg.inc can only claim what other warpgroups of the same block released, so the sum
@@ -855,7 +857,7 @@ static const F32TcLaunch *f32tc_prepared(gdws_plan_s *p, int n, int h, int w)
     // The other kernel's estimate is too long for short calls (5 x 32 -> 81 channels at 11 x 9, stride 2: 17.6 for 11.9 us, where this one
     // takes 14.8) and up to twice too short for large NHWC ones.
     const double alu = f32_alu_us(p, n, h, w);
-    if (e->taken && p->opt_dw_math != 2) e->taken = e->g.us < (alu < 24.0 ? 3.0 + 0.65 * (alu - 3.0) : 1.1 * alu);
+    if (e->taken && p->opt_dw_math != 2) e->taken = p->G >= kF32TcLeast && e->g.us < (alu < 24.0 ? 3.0 + 0.65 * (alu - 3.0) : 1.1 * alu);
     return LaunchCache<F32TcLaunch>::add(p->launch_cache[5], std::move(e));
 }
 

@@ -86,3 +86,12 @@ def test_kernel_agrees_with_form():
         with pytest.raises(gdws.GdwsError):
             bad()
     plan.destroy()
+
+
+@pytest.mark.parametrize("k", [3, 5])
+def test_fp32_with_few_intermediate_channels_stays_on_the_alus(k):
+    """Below 16 of them the products in pieces are less exact than fp32 sums."""
+    for G, kernel in [(1, gdws.KERNEL_F32_ALU), (8, gdws.KERNEL_F32_ALU), (15, gdws.KERNEL_F32_ALU), (16, gdws.KERNEL_F32_PIECES), (64, gdws.KERNEL_F32_PIECES)]:
+        plan = _plan(G, 64, k, 1, 1)
+        assert plan.kernel(39, 145, 145, gdws.F32) == kernel
+        plan.destroy()

@@ -51,8 +51,10 @@ def test_matches_reference(shape, layout):
     tc, alu = (run_gpu(data, path=gdws.PATH_FUSED, dw_math=m) for m in (2, 1))
     # dropped pieces and the chunks' truncation: 2^-22 of sum |P||z|, some sqrt(G) times the largest output
     assert rel_err(tc, ref) <= 1e-5
-    # one rounding per chunk instead of one per channel; both have z's own roundings (in the 2-norm, with a little room for few terms)
-    assert np.linalg.norm(tc - ref) <= 1.1 * np.linalg.norm(alu - ref) + 3e-8 * np.linalg.norm(ref)
+    # one rounding per chunk instead of one per channel; both have z's own roundings.  With fewer channels than the default takes here
+    # what the tensor cores truncate (2^-24 of the sum at most) can outweigh it.
+    few = data.g.sum() < 16
+    assert np.linalg.norm(tc - ref) <= np.linalg.norm(alu - ref) + (2 ** -24 * np.linalg.norm(ref) if few else 0.0)
 
 
 @pytest.mark.parametrize("layout", ["NCHW", "NHWC"])
