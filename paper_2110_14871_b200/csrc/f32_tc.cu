@@ -796,13 +796,14 @@ bool f32tc_geometry(const gdws_plan_s *p, int n, int Ho, int Wo, long long xn, F
             if (!found || g.us < out->us) { *out = g; found = true; }
         }
     };
-    for (int j = 1; j <= Wo; ++j) {
-        const int PW = (Wo + j - 1) / j;
-        if (PW > 128) continue;
+    // A row or column in so many equal parts: only those numbers are visited that change the parts' size (500 x 500 outputs: 700 us of a
+    // first call with all of them).
+    auto next = [](int total, int parts) { const int size = (total + parts - 1) / parts; return size > 1 ? (total + size - 2) / (size - 1) : total + 1; };
+    for (int j = (Wo + 127) / 128; j <= Wo; j = next(Wo, j)) {
+        const int PW = (Wo + j - 1) / j, most = 128 / PW;
         if (PW < 4 && PW < Wo) break;
-        for (int i = 1; i <= Ho; ++i) {
+        for (int i = (Ho + most - 1) / most; i <= Ho; i = next(Ho, i)) {
             const int PH = (Ho + i - 1) / i;
-            if (PH * PW > 128) continue;
             if (i == 1 && j == 1) {
                 for (int TN = std::min(n, 128 / (PH * PW)); TN >= 1; --TN) consider(TN, PH, PW);
             } else {

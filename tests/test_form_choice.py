@@ -1,4 +1,6 @@
 """gdws_plan_form: the library takes the folded form where its estimate is lower, and never against an option."""
+import time
+
 import numpy as np
 import pytest
 
@@ -95,3 +97,18 @@ def test_fp32_with_few_intermediate_channels_stays_on_the_alus(k):
         plan = _plan(G, 64, k, 1, 1)
         assert plan.kernel(39, 145, 145, gdws.F32) == kernel
         plan.destroy()
+
+
+def test_a_first_call_on_a_large_map_takes_no_longer_to_plan():
+    """The fp32 tile is looked for once per size: the search does not go through every height and width of a large map."""
+    def least_us(h):
+        us = []
+        for _ in range(30):
+            plan = _plan(64, 64, 3, 1, 5)
+            t0 = time.perf_counter()
+            plan.kernel(2, h, h, gdws.F32)
+            us.append(1e6 * (time.perf_counter() - t0))
+            plan.destroy()
+        return min(us)
+
+    assert least_us(500) <= 10 * least_us(28)        # it was 100 times
