@@ -755,6 +755,7 @@ struct F32TcLaunch {
     F32TcGeom g;
     bool taken = false;
     int alu = -1;                // fused_f32_kernel's tile
+    int slots = 0;               // most distinct input channels that a chunk reads
 };
 
 size_t f32tc_smem(const gdws_plan_s *p, int slots, const F32TcGeom &g)
@@ -764,10 +765,10 @@ size_t f32tc_smem(const gdws_plan_s *p, int slots, const F32TcGeom &g)
 }
 
 // Tile shape: the pixels of a tile are a patch of one image or whole small images, whatever fills 128 rows best.
-bool f32tc_geometry(const gdws_plan_s *p, int n, int Ho, int Wo, long long xn, F32TcGeom *out)
+bool f32tc_geometry(const gdws_plan_s *p, int n, int Ho, int Wo, long long xn, int slots, F32TcGeom *out)
 {
     if ((p->k != 3 && p->k != 5) || p->G < 1) return false;
-    const int sms = sm_count_of(p), slots = f32tc_slots(p), nq = (p->G + kF32TcChunk - 1) / kF32TcChunk;
+    const int sms = sm_count_of(p), nq = (p->G + kF32TcChunk - 1) / kF32TcChunk;
     const int parts = (p->D + 127) / 128;
     bool found = false;
     auto consider = [&](int TN, int PH, int PW) {
@@ -854,7 +855,10 @@ static const F32TcLaunch *f32tc_prepared(gdws_plan_s *p, int n, int h, int w)
     const int Ho = gdws_out_dim(h, p->k, p->stride, p->pad), Wo = gdws_out_dim(w, p->k, p->stride, p->pad);
     e->key = key;
     e->alu = f32_alu_config(p, (long long)n * Ho * Wo, Wo);
-    e->taken = p->opt_dw_math != 1 && f32tc_geometry(p, n, Ho, Wo, (long long)p->C * h * w, &e->g);
+    if (p->opt_dw_math != 1) {
+        e->slots = f32tc_slots(p);
+        e->taken = f32tc_geometry(p, n, Ho, Wo, (long long)p->C * h * w, e->slots, &e->g);
+    }
     // The other kernel's estimate is too long for short calls (5 x 32 -> 81 channels at 11 x 9, stride 2: 17.6 for 11.9 us, where this one
     // takes 14.8) and up to twice too short for large NHWC ones.
     const double alu = f32_alu_us(p, n, h, w);
@@ -892,7 +896,7 @@ gdws_status_t f32_fused_tc(gdws_plan_s *p, const gdws_tensor_t *x, const float *
     P.yc = nhwc ? 1 : (long long)y->h * y->w; P.yw = nhwc ? y->c : 1; P.yh = P.yw * y->w;
     P.TN = g.TN; P.PH = g.PH; P.PW = g.PW; P.IH = g.IH; P.IW = g.IW; P.np = g.np; P.pitch = g.pitch; P.tiles_h = g.tiles_h; P.tiles_w = g.tiles_w; P.ntiles = (int)g.tiles;
     P.nq = (p->G + kF32TcChunk - 1) / kF32TcChunk; P.Nd = g.Nd; P.ns = g.ns;
-    const int slots = f32tc_slots(p);
+    const int slots = l->slots;
     P.b_piece = (uint32_t)g.Nd * 64u; P.ab_bytes = 3u * kF32TcA + 3u * P.b_piece;
     P.x_bytes = (uint32_t)slots * (uint32_t)g.pitch * 4u;
     P.off_x = (uint32_t)g.ns * P.ab_bytes;

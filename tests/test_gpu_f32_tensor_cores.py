@@ -1,6 +1,8 @@
 """The fp32 forward with its pointwise products on the tensor cores: against the CPU oracle, no less exact than the ALU kernel, and
 with the same infinities and NaN.  Output channels around 16, 32, 64 and 128 and in two parts, chunks of 32 intermediate channels with
 remainders and one alone, clusters that share a tile's chunks, tiles of several images, both filter sizes, strides, channels without filters."""
+import time
+
 import numpy as np
 import pytest
 import torch
@@ -128,3 +130,21 @@ def test_small_and_large_values_keep_their_bits(N, C, D, H, W, k):
         size = np.linalg.norm(np.ldexp(ref, -sum(ends)))         # in range for its squares
         err = [np.linalg.norm(np.ldexp(y - ref, -sum(ends))) / size for y in (tc, alu)]
         assert err[0] <= err[1] and err[0] <= 1e-5, (ends, err)
+
+
+def test_a_repeated_call_does_no_work_per_filter_on_the_host():
+    """G = 262144: what a launch needs is worked out with the first call of a size (a pass over the filters takes 250 us)."""
+    data = gi.make_layer(small_spec("t", 1, 64, 8, 6, 6, 3, 1, 1, ("const", 4096), "f32", "NCHW", seed=5))
+    plan = make_plan(data, path=gdws.PATH_FUSED, dw_math=2)
+    assert plan.kernel(1, 6, 6, gdws.F32) == gdws.KERNEL_F32_PIECES
+    x, dw, pw = (to_device(a, "f32") for a in (data.x, data.dw_w, data.pw_w))
+    y = torch.empty((1, 8, 6, 6), device="cuda")
+    us = []
+    for _ in range(8):
+        torch.cuda.synchronize()
+        t0 = time.perf_counter()
+        plan.forward(x, y, "NCHW", dw, pw)
+        us.append(1e6 * (time.perf_counter() - t0))
+    plan.status()
+    plan.destroy()
+    assert min(us) <= 80, us
