@@ -14,6 +14,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <mutex>
 #include <new>
 
 #include "sm100.cuh"
@@ -21,7 +22,7 @@
 namespace gdws {
 
 constexpr int kSplitThreads = 8 * 32, kSplitMmaWarp = 0, kSplitAWarp = 1, kSplitBWarp = 2, kSplitTermWarp = 3;
-constexpr int kSplitMaxSlots = 8, kSplitMost = 8, kSplitMaxSteps = 25;
+constexpr int kSplitMaxSlots = 8, kSplitMaxSteps = 25;
 constexpr uint32_t kSplitSw128 = 2u << 29;   // descriptor high word: layout type "128-byte swizzle"
 
 struct alignas(64) FoldSplitParams {
@@ -243,26 +244,38 @@ __global__ void __launch_bounds__(kSplitThreads, 1) fold_split_kernel(const __gr
 // ------------------------------------------------------------------------------------------
 // Host side
 // ------------------------------------------------------------------------------------------
-// Clusters of `split` blocks, one block per SM, that the plan's device runs at the same time: clusters do not cross the chip's groups of
-// SMs, so some are left over.  Asked once per device (without one, as for queries on a host without a GPU: what a B200 answered).
+// Clusters of 1 to 8 blocks, one block per SM, that a device runs at the same time: clusters do not cross the chip's groups of SMs, so
+// some SMs are left over.  `device` is the current one; it is asked once.
+void cluster_capacities(int device, int sms, int (&most)[kMostSlices + 1])
+{
+    static std::mutex lock;
+    static struct { bool known; int most[kMostSlices + 1]; } kept[64];
+    std::lock_guard<std::mutex> hold(lock);
+    auto &k = kept[device & 63];
+    if (!k.known || device > 63) {
+        k.known = true;
+        k.most[1] = sms;
+        cudaFuncSetAttribute(fold_split_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+        for (int split = 2; split <= kMostSlices; ++split) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3((unsigned)(split * 64)); cfg.blockDim = dim3(kSplitThreads); cfg.dynamicSmemBytes = kMaxSmem / 2 + 2048;
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = (unsigned)split; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+            cfg.attrs = attr; cfg.numAttrs = 1;
+            int got = 0;
+            if (cudaOccupancyMaxActiveClusters(&got, fold_split_kernel, &cfg) != cudaSuccess) got = 0;      // no clusters: layers keep to the other kernels
+            k.most[split] = got;
+        }
+        cudaGetLastError();
+    }
+    std::copy(k.most, k.most + kMostSlices + 1, most);
+}
+
 int cluster_capacity(const gdws_plan_s *p, int split)
 {
-    static int most[64][kSplitMost + 1] = {};
-    int &n = most[p->device & 63][split];
-    if (p->device < 0 || split == 1) return sm_count_of(p) / split - (split > 4 ? 2 : 0);
-    if (n == 0) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)(split * 64)); cfg.blockDim = dim3(kSplitThreads); cfg.dynamicSmemBytes = kMaxSmem / 2 + 2048;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = (unsigned)split; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr; cfg.numAttrs = 1;
-        int got = 0;
-        cudaFuncSetAttribute(fold_split_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
-        if (cudaOccupancyMaxActiveClusters(&got, fold_split_kernel, &cfg) != cudaSuccess) { cudaGetLastError(); got = 0; }
-        n = got > 0 ? got : sm_count_of(p) / split - 2;
-    }
-    return n;
+    static constexpr int b200[kMostSlices + 1] = {0, kB200Sms, 74, 45, 33, 26, 22, 15, 15};      // as a B200 answers: for queries on a host without a GPU
+    return p->device >= 0 ? p->clusters[split] : b200[split];
 }
 
 namespace {
@@ -304,7 +317,7 @@ bool split_geometry(const gdws_plan_s *p, int n, int Ho, int Wo, SplitGeom *out)
             g.nparts = (p->D + g.Npart - 1) / g.Npart;
             g.slot = g.b_off + (uint32_t)(k * g.Npart) * 128u;
             const size_t room = kMaxSmem - 1024;
-            for (int split = 1; split <= std::min(kSplitMost, units); ++split) {
+            for (int split = 1; split <= std::min(kMostSlices, units); ++split) {
                 if (g.tiles() * g.nparts > cluster_capacity(p, split)) continue;
                 const int upc = (units + split - 1) / split;
                 g.split = split;

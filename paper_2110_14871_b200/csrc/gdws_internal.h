@@ -19,6 +19,7 @@ constexpr int kChunk = 64;          // intermediate channels per tensor-core K c
 constexpr int kTileRows = 128;      // output pixels per tensor-core tile (UMMA M)
 constexpr int kMaxK = 7;
 constexpr int kHostPieces = 5;      // pieces that gdws_forward_host overlaps
+constexpr int kMostSlices = 8;      // blocks of a cluster that share a tile's sum
 constexpr int kMaxSmem = 225 * 1024;      // dynamic shared memory a block may ask for (227 KB minus static use)
 
 // Bits of the device status word.
@@ -110,6 +111,7 @@ struct gdws_plan_s {
     size_t arena_bytes = 0;
     int device = -1;
     int sm_count = 0;              // SMs of the plan's device (grid size of the persistent kernel)
+    int clusters[gdws::kMostSlices + 1] = {};      // clusters of so many blocks, one per SM, that the device runs at the same time
     bool arch_ok = false;          // the plan's device was checked to be compute capability 10.x
     int32_t *d_off = nullptr;      // [C+1]
     int32_t *d_chan = nullptr;     // [Gpad], -1 for padding
@@ -273,6 +275,7 @@ gdws_status_t bf16_fused_tc(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_
 // fold.cu
 gdws_status_t bf16_folded(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t *y, cudaStream_t s);
 // fold_split.cu: the folded form in slices, for layers that leave SMs idle
+void cluster_capacities(int device, int sms, int (&most)[kMostSlices + 1]);
 int cluster_capacity(const gdws_plan_s *p, int split);     // clusters of `split` blocks, one per SM, that run at the same time
 double fold_split_us(const gdws_plan_s *p, int n, int Ho, int Wo);      // estimate; 1e9 where it does not cover the layer
 gdws_status_t bf16_folded_split(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t *y, cudaStream_t s);

@@ -139,6 +139,8 @@ gdws_status_t ensure_device(gdws_plan_s *p)
     p->device = dev;
     plan_count(dev, 1);
     if (cudaDeviceGetAttribute(&p->sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) p->sm_count = 0;
+    cluster_capacities(dev, sm_count_of(p), p->clusters);
+    for (auto &c : p->launch_cache) c.reset();     // what queries worked out for the device that was assumed
     e = cudaMemcpy(p->d_arena, tables.data(), tables.size(), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
         free_device(p);

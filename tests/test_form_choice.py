@@ -112,3 +112,23 @@ def test_a_first_call_on_a_large_map_takes_no_longer_to_plan():
         return min(us)
 
     assert least_us(500) <= 10 * least_us(28)        # it was 100 times
+
+
+def _clusters_decide():
+    """Layers that slices would take if more clusters ran at a time than do on a B200 (74, 45, 33, 26, 22, 15, 15 of 2 to 8 blocks)."""
+    for N, C, D, H, k, stride, G in [(5, 32, 32, 19, 5, 1, 72), (6, 136, 272, 12, 5, 1, 649), (2, 72, 216, 17, 5, 1, 175), (54, 88, 184, 5, 5, 1, 220)]:
+        g = np.full(C, G // C, dtype=np.int32)
+        g[:G % C] += 1
+        plan = gdws.Plan(C, D, k, stride, k // 2, g)
+        got = plan.kernel(N, H, H)
+        plan.destroy()
+        yield got
+
+
+def test_a_host_without_a_gpu_answers_as_a_b200():
+    assert list(_clusters_decide()) == [gdws.KERNEL_FOLDED_PAIRS] * 4
+
+
+@pytest.mark.gpu
+def test_a_b200_answers_as_a_host_without_a_gpu():
+    assert list(_clusters_decide()) == [gdws.KERNEL_FOLDED_PAIRS] * 4
