@@ -909,8 +909,11 @@ double bf16_forward_us(gdws_plan_s *p, int n, int h, int w, bool out_f32)
 {
     const int Ho = gdws_out_dim(h, p->k, p->stride, p->pad), Wo = gdws_out_dim(w, p->k, p->stride, p->pad);
     const int form = p->opt_path == GDWS_PATH_UNFUSED ? 1 : bf16_form_of(p, n, h, w, out_f32);
-    FoldGeom g;
-    if (form == 3 && fold_geometry(p, n, Ho, Wo, out_f32, &g)) return std::min(g.us, fold_split_us(p, n, Ho, Wo));
+    if (form == 3) {                     // either kernel may be the only one that covers the layer
+        FoldGeom g;
+        const double us = std::min(fold_geometry(p, n, Ho, Wo, out_f32, &g) ? g.us : 1e9, fold_split_us(p, n, Ho, Wo));
+        if (us < 1e9) return us;
+    }
     if (form == 2) return two_stage_us(p, n, h, w, Ho, Wo, 2);
     Tile t;
     if (!choose_tile(p, n, h, w, &t)) return 1e9;
