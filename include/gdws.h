@@ -177,9 +177,8 @@ GDWS_API gdws_status_t gdws_plan_gdw_stage(const gdws_plan_t *plan, int *stage);
 /*
  * gdws_plan_form -- the kernel a fused bf16 forward of n x C x h x w takes with the plan's current options: *form = 1 or 2
  * (two stages, the GDW stage on the ALUs or on the tensor cores, as gdws_plan_gdw_stage) or 3 (one k x k convolution with
- * folded filters), with weights packed beforehand.  (A call that is given its weights folds them first, which counts where only
- * the kernel for few tiles makes form 3 the faster one: it may keep to the two stages there.  Weights given with a call are
- * folded only if that call takes form 3; a later call that reuses them keeps to the two stages otherwise.)  Host only; errors: GDWS_ERR_INVALID_ARG.
+ * folded filters).  (Weights given with a call are folded only if that call takes form 3; a later call that reuses them keeps
+ * to the two stages then.)  Host only; errors: GDWS_ERR_INVALID_ARG.
  */
 GDWS_API gdws_status_t gdws_plan_form(gdws_plan_t *plan, int n, int h, int w, int *form);
 

@@ -224,7 +224,7 @@ gdws_status_t gdws_forward(gdws_plan_t *p, const gdws_tensor_t *x, const void *d
     }
     // weights given with the call: their folded filters (up to half of the packing) are formed if this call reads them; a later
     // call that would, with the weights left as they are, then keeps to the two stages
-    st = weights_ready(p, dw_w, pw_w, bias, GDWS_BF16, dw_w && fused && bf16_form_of(p, x->n, x->h, x->w, y->dtype == GDWS_F32, true) == 3, cs);
+    st = weights_ready(p, dw_w, pw_w, bias, GDWS_BF16, dw_w && fused && bf16_form_of(p, x->n, x->h, x->w, y->dtype == GDWS_F32) == 3, cs);
     if (st != GDWS_OK) return st;
     if (fused) {
         st = bf16_fused(p, x, y, cs);

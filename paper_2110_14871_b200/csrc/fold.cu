@@ -851,15 +851,6 @@ double two_stage_us(const gdws_plan_s *p, int n, int h, int w, int Ho, int Wo, i
     return (p->stride == 1 ? 0.93 : 1.25) * (4.0 + waves(tiles * p->tc_nparts) * chunks);
 }
 
-// What folding the filters adds to a call that is given its weights: a thread goes through its channel's filters, nine taps at a time.
-// Fitted to 160 layers, within 2 us of most: 3 x 3 taps nothing with 3 filters a channel, 2 us with 9; 5 x 5 taps 4 with 3, 8 with 9, 20 to
-// 60 with 25; and more for wide layers.
-double fold_pack_us(const gdws_plan_s *p)
-{
-    const double again = (p->k * p->k + 8) / 9 - 1, more = std::max(0, *std::max_element(p->g.begin(), p->g.end()) - 3);
-    return 1.9 * again + 0.33 * more + 0.04 * again * more * more + 4e-6 * p->C * p->D * p->k * p->k;
-}
-
 struct FormChoice {
     LaunchKey key;
     int form = 1;
@@ -868,7 +859,7 @@ struct FormChoice {
 
 }  // namespace
 
-int bf16_form_of(gdws_plan_s *p, int n, int h, int w, bool out_f32, bool given)
+int bf16_form_of(gdws_plan_s *p, int n, int h, int w, bool out_f32)
 {
     const int stage = gdw_stage_of(p);
     if (p->opt_dw_math) return p->opt_dw_math;
@@ -880,7 +871,7 @@ int bf16_form_of(gdws_plan_s *p, int n, int h, int w, bool out_f32, bool given)
     if (p->unused && !(stage == 1 && p->Dpad > 512)) return stage;
     const int Ho = gdws_out_dim(h, p->k, p->stride, p->pad), Wo = gdws_out_dim(w, p->k, p->stride, p->pad);
     if (n < 1 || Ho < 1 || Wo < 1) return stage;
-    const LaunchKey key = {n, h, w, (out_f32 ? 2 : 0) | (given ? 4 : 0)};
+    const LaunchKey key = {n, h, w, out_f32 ? 2 : 0};
     if (const FormChoice *c = LaunchCache<FormChoice>::find(p->launch_cache[3], key)) return c->form;
     FoldGeom g;
     double us = fold_geometry(p, n, Ho, Wo, out_f32, &g) ? g.us : 1e9;
@@ -889,9 +880,7 @@ int bf16_form_of(gdws_plan_s *p, int n, int h, int w, bool out_f32, bool given)
     // Slices (fold_split.cu) count where a channel has more than two filters in the mean.  They would win below that as well (384 ->
     // 104 channels, stride 2, 8 x 8, g_c = 2: 7.3 us against 12.5), but the form that such layers have is part of what callers plan
     // with: its answers stay.
-    // Given its weights a call folds them first: small layers that only the slices make faster would lose by it (4 x 56 -> 40 channels at
-    // 6 x 6, 5 x 5 taps, stride 2: 13.0 us in two stages, 18.5).
-    if (p->G > 2 * p->C) us = std::min(us, slices + (given ? fold_pack_us(p) : 0.0));
+    if (p->G > 2 * p->C) us = std::min(us, slices);
     const bool fold = us < two_stage_us(p, n, h, w, Ho, Wo, stage);
     const int form = fold ? 3 : stage;
     if (std::unique_ptr<FormChoice> c{new (std::nothrow) FormChoice}) {

@@ -281,8 +281,7 @@ double fold_split_us(const gdws_plan_s *p, int n, int Ho, int Wo);      // estim
 gdws_status_t bf16_folded_split(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t *y, cudaStream_t s);
 bool fold_in_slices(gdws_plan_s *p, int n, int h, int w, bool out_f32);      // whether a folded forward runs there
 double bf16_forward_us(gdws_plan_s *p, int n, int h, int w, bool out_f32);
-// 1 / 2: two stages, GDW on the ALUs / the tensor cores; 3: folded.  given: the weights come with the call.
-int bf16_form_of(gdws_plan_s *p, int n, int h, int w, bool out_f32, bool given = false);
+int bf16_form_of(gdws_plan_s *p, int n, int h, int w, bool out_f32);   // 1 / 2: two stages, GDW on the ALUs / the tensor cores; 3: folded
 
 // Input row h = stride * ho + u - pad of filter row u (columns alike).  With stride 2 the input is read through four
 // dense views, one per parity of row and column (every other row, every other column): in the view of parity par

@@ -97,32 +97,3 @@ def test_weights_given_with_a_call_of_another_form():
     assert rel_err(run(0, 0), want(0, 0)) <= 1e-2          # folded, weights with the call
     assert rel_err(run(1), want(1, 0)) <= 1e-2
     plan.destroy()
-
-
-@pytest.mark.parametrize("N,C,D,H,k,stride,gd,folds", [
-    (4, 56, 40, 6, 5, 2, ("heavy",), False),               # 6.5 us instead of 8.3 once folded, but folding takes 7 more
-    (1, 16, 160, 11, 5, 2, ("uniform", 1, 9), False),      # 5.4 instead of 6.5, folding 8
-    (1, 424, 200, 7, 3, 2, ("uniform", 2, 3), True),       # 7.8 us instead of 15.7, folding 3
-    (64, 64, 64, 28, 3, 1, ("uniform", 3, 7), True),       # folded on pairs
-])
-def test_a_call_given_its_weights_folds_them_where_that_pays(N, C, D, H, k, stride, gd, folds):
-    """All of these run folded with weights packed beforehand.  A forced folded call without weights is refused after one that was
-    given weights and kept to the two stages."""
-    data = gi.make_layer(small_spec("t", N, C, D, H, H, k, stride, k // 2, gd, "bf16", "NHWC", seed=2))
-    plan = make_plan(data, path=gdws.PATH_FUSED)
-    assert plan.form(N, H, H) == 3
-    x, dw, pw, b = to_device(data.x, "bf16"), to_device(data.dw_w, "bf16"), to_device(data.pw_w, "bf16"), torch.from_numpy(data.bias).cuda()
-    y = torch.full((N, data.spec.Ho, data.spec.Wo, D), float("nan"), dtype=torch.bfloat16, device="cuda")
-    plan.forward(x, y, "NHWC", dw, pw, b)
-    torch.cuda.synchronize()
-    plan.status()
-    assert rel_err(y.float().cpu().numpy(), run_oracle(data)[0]) <= 1e-2
-    plan.set_option(gdws.OPT_DW_MATH, 3)
-    try:
-        plan.forward(x, y, "NHWC")
-        folded = True
-    except gdws.GdwsError as e:
-        assert e.status == gdws.ERR_INVALID_ARG
-        folded = False
-    assert folded == folds
-    plan.destroy()
