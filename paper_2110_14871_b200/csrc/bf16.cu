@@ -59,10 +59,8 @@ __global__ void gdw_bf16_kernel(DwShape s, const uint16_t *__restrict__ x, const
 
 gdws_status_t bf16_depthwise(gdws_plan_s *p, const gdws_tensor_t *x, void *z, cudaStream_t st)
 {
-    if (bf16_depthwise_on_tc(p, x->n, x->h, x->w)) {
-        const gdws_status_t rc = bf16_depthwise_tc(p, x, z, st);
-        if (rc != GDWS_ERR_UNSUPPORTED) return rc;
-    }
+    // a launch that is refused leaves the layer to the ALUs, which cover it as well
+    if (bf16_depthwise_on_tc(p, x->n, x->h, x->w) && bf16_depthwise_tc(p, x, z, st) == GDWS_OK) return GDWS_OK;
     if (p->C % 8 == 0) {   // tiled pipeline first; shapes it cannot tile fall through to the simple kernel
         const gdws_status_t rc = bf16_depthwise_tiled(p, x, z, st);
         if (rc != GDWS_ERR_UNSUPPORTED) return rc;

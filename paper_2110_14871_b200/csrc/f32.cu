@@ -599,7 +599,8 @@ gdws_status_t f32_fused(gdws_plan_s *p, const gdws_tensor_t *x, const float *dw_
                         const float *bias, gdws_tensor_t *y, cudaStream_t st)
 {
     int config = -2;
-    if (f32_tc_takes(p, x->n, x->h, x->w, &config)) return f32_fused_tc(p, x, dw_w, pw_w, bias, y, st);
+    // a launch that is refused leaves the layer to the kernel below, which covers it as well
+    if (f32_tc_takes(p, x->n, x->h, x->w, &config) && f32_fused_tc(p, x, dw_w, pw_w, bias, y, st) == GDWS_OK) return GDWS_OK;
     const F32Shape s = make_shape(p, x->layout, x->n, x->h, x->w);
     const bool nhwc = x->layout == GDWS_NHWC;
     const float *xp = (const float *)x->ptr;

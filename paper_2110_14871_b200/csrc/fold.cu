@@ -781,6 +781,7 @@ gdws_status_t fold_map_x(const gdws_plan_s *p, const gdws_tensor_t *x, FoldLaunc
 {
     tensor_map_encode_fn encode = encode_fn();
     const int sd = p->stride;
+    L->x = nullptr;              // until all of them are of this address
     for (int m = 0; m < 4; ++m) {
         if (!((L->P.maps_used >> m) & 1)) continue;
         const int hp = m >> 1, wp = m & 1;
@@ -935,7 +936,13 @@ gdws_status_t bf16_folded(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t 
         L = LaunchCache<FoldLaunch>::add(p->launch_cache[2], std::move(e));
         if (!L) return fail(GDWS_ERR_ALLOC, "out of host memory");
     }
-    if (L->sliced) return bf16_folded_split(p, x, y, st);
+    if (L->sliced) {
+        rc = bf16_folded_split(p, x, y, st);
+        if (rc == GDWS_OK) return rc;
+        // refused: pairs cover all but layers of very many output channels
+        if (fold_prepare(p, x->n, y->h, y->w, out_f32, L) != GDWS_OK) return rc;
+        L->sliced = false;
+    }
     if (L->x != x->ptr && (rc = fold_map_x(p, x, L)) != GDWS_OK) return rc;
     if (L->y != y->ptr && (rc = fold_map_y(p, y, L)) != GDWS_OK) return rc;
     const cudaError_t e = launch_overlapped(L->kernel, (unsigned)L->grid, kFoldThreads, L->smem, st, L->P);

@@ -392,6 +392,7 @@ gdws_status_t split_prepare(gdws_plan_s *p, int n, int Ho, int Wo, bool out_f32,
 gdws_status_t split_map_x(const gdws_plan_s *p, const gdws_tensor_t *x, SplitLaunch *L)
 {
     const int sd = p->stride;
+    L->x = nullptr;              // until all of them are of this address
     for (int m = 0; m < 4; ++m) {
         if (!((L->P.maps_used >> m) & 1)) continue;
         const int hp = m >> 1, wp = m & 1, Wp = (x->w - wp + sd - 1) / sd, Hp = (x->h - hp + sd - 1) / sd;

@@ -586,7 +586,9 @@ gdws_status_t gdw_maps(const gdws_plan_s *p, const gdws_tensor_t *x, void *z, Gd
     const int sd = p->stride;
     const CUtensorMapSwizzle sw = P.rb == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : (P.rb == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B);
     const cuuint32_t estr[4] = {1, 1, 1, 1};
-    for (int m = 0; m < 4 && L->x != x->ptr; ++m) {
+    const bool anew = L->x != x->ptr;
+    if (anew) L->x = nullptr;    // until all of them are of this address
+    for (int m = 0; m < 4 && anew; ++m) {
         if (!((P.maps_used >> m) & 1)) continue;
         const int hp = m >> 1, wp = m & 1, Wp = (x->w - wp + sd - 1) / sd, Hp = (x->h - hp + sd - 1) / sd;
         const cuuint64_t dims[4] = {(cuuint64_t)p->C, (cuuint64_t)Wp, (cuuint64_t)Hp, (cuuint64_t)x->n};
