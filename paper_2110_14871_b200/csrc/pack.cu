@@ -8,7 +8,7 @@
 namespace gdws {
 
 constexpr int kPackThreads = 256, kPackPiece = 2048;     // elements of a block where the output is a flat array
-constexpr int kFoldPackTaps = 9;
+constexpr int kFoldPackStage = 12288;     // bf16 values of filters and weights that a block holds at a time
 enum { kPackImg, kPackTaps, kPackBias, kPackFilt, kPackSlab, kPackFold, kPackParts };
 
 struct PackParams {
@@ -25,7 +25,7 @@ struct PackParams {
     const TcChunk *tc_chunks;
     int tc_nchunks, tc_nslabs, tc_dloc, tc_nparts, rec_hw;
     uint16_t *tc_filt, *tc_pw;
-    int fold_per, fold_dblocks, fold_dp, fold_blocks, fold_sum_step;
+    int fold_dblocks, fold_dp, fold_blocks, fold_sum_step;
     uint16_t *fold;
     float2 *fold_sums;
 };
@@ -116,53 +116,33 @@ __device__ void pack_slab(const PackParams &P, int idx)
 // Folded filters: W[d,c,tap] = sum_j P[d, off_c+j] K[off_c+j, tap] in fp32, as two bf16 terms: W rounded to nearest, and what
 // that leaves over rounded to nearest.  Rows are (term, window of 64 input channels, tap, output channel), 64 input channels
 // each; rows d >= D and channels >= C are zero.  A block takes one window and 4 PER output channels: thread = one channel x PER
-// output channels, up to 9 taps of BATCH filters at a time in registers, their loads in flight together.  PER = 1 where blocks are
-// few (four output channels per thread left a 72 -> 120 layer 16 blocks: 5 us slower), 4 where the loads of the taps, which lie
-// far apart for neighbouring channels, take the time (kFoldPackWide).
+// output channels.  PER = 1 where blocks are few (four output channels per thread left a 72 -> 120 layer 16 blocks: 5 us slower), 4
+// where the loads of the taps, which lie far apart for neighbouring channels, take the time (kFoldPackWide).
 // Beside them, per block (or every n-th): the sum of the squared taps and of the filters' squared tap sums, from which the
 // forward decides whether it takes the second term.
-template <int PER, int BATCH> __device__ __forceinline__ void pack_fold(const PackParams &P, int idx)
+
+// A weight rounded to bf16: the two-stage kernels use them so as well.
+__device__ __forceinline__ float fold_weight(const PackParams &P, const void *w, size_t i)
 {
-    const int win = idx / P.fold_dblocks, group = idx - win * P.fold_dblocks, cl = threadIdx.x & 63, c = win * 64 + cl;
-    const int d0 = (group * 4 + (threadIdx.x >> 6)) * PER;
-    const int i0 = c < P.C ? P.off[c] : 0, i1 = c < P.C && d0 < P.D ? P.off[c + 1] : i0;
-    auto weight = [&](const void *w, size_t i) {          // the two-stage kernels use the weights rounded to bf16 as well
-        return P.is_bf16 ? bf16_bits_to_float(((const uint16_t *)w)[i]) : bf16_bits_to_float(float_to_bf16_bits(((const float *)w)[i]));
-    };
-    const size_t term = (size_t)P.fold_dp * (P.fold_blocks / P.fold_dblocks) * P.k2 * 64;
-    float energy = 0.f, sum[PER] = {};
-    for (int t0 = 0; t0 < P.k2; t0 += kFoldPackTaps) {
-        float acc[PER][kFoldPackTaps] = {};
-#pragma unroll 1
-        for (int i = i0; i < i1; i += BATCH) {
-            float p[BATCH][PER], v[BATCH][kFoldPackTaps];
+    return P.is_bf16 ? bf16_bits_to_float(((const uint16_t *)w)[i]) : bf16_bits_to_float(float_to_bf16_bits(((const float *)w)[i]));
+}
+
+// One tap of a thread's channel and PER output channels.
+template <int PER> __device__ __forceinline__ void pack_fold_store(const PackParams &P, int win, int cl, int t, int d0, size_t term, const float (&w)[PER], float &energy, float (&sum)[PER])
+{
 #pragma unroll
-            for (int j = 0; j < BATCH; ++j) {
-#pragma unroll
-                for (int e = 0; e < PER; ++e) p[j][e] = i + j < i1 && (PER == 1 || d0 + e < P.D) ? weight(P.pw, (size_t)(d0 + e) * P.G + i + j) : 0.f;
-#pragma unroll
-                for (int t = 0; t < kFoldPackTaps; ++t) v[j][t] = i + j < i1 && t0 + t < P.k2 ? weight(P.dw, (size_t)(i + j) * P.k2 + t0 + t) : 0.f;
-            }
-#pragma unroll
-            for (int j = 0; j < BATCH; ++j)
-#pragma unroll
-                for (int e = 0; e < PER; ++e)
-#pragma unroll
-                    for (int t = 0; t < kFoldPackTaps; ++t) acc[e][t] = fmaf(p[j][e], v[j][t], acc[e][t]);
-        }
-#pragma unroll
-        for (int t = 0; t < kFoldPackTaps; ++t)
-            if (t0 + t < P.k2)
-#pragma unroll
-                for (int e = 0; e < PER; ++e) {
-                    uint16_t *out = P.fold + (((size_t)win * P.k2 + t0 + t) * P.fold_dp + d0 + e) * 64 + cl;
-                    const uint16_t hi = float_to_bf16_bits(acc[e][t]);
-                    out[0] = hi;
-                    out[term] = float_to_bf16_bits(acc[e][t] - bf16_bits_to_float(hi));
-                    energy = fmaf(acc[e][t], acc[e][t], energy);
-                    sum[e] += acc[e][t];
-                }
+    for (int e = 0; e < PER; ++e) {
+        uint16_t *out = P.fold + (((size_t)win * P.k2 + t) * P.fold_dp + d0 + e) * 64 + cl;
+        const uint16_t hi = float_to_bf16_bits(w[e]);
+        out[0] = hi;
+        out[term] = float_to_bf16_bits(w[e] - bf16_bits_to_float(hi));
+        energy = fmaf(w[e], w[e], energy);
+        sum[e] += w[e];
     }
+}
+
+template <int PER> __device__ __forceinline__ void pack_fold_sums(const PackParams &P, int win, int group, float energy, const float (&sum)[PER])
+{
     if (group % P.fold_sum_step) return;
     __shared__ float2 part[kPackThreads / 32];
     float2 v = make_float2(energy, 0.f);
@@ -180,14 +160,107 @@ template <int PER, int BATCH> __device__ __forceinline__ void pack_fold(const Pa
     }
 }
 
-__global__ void __launch_bounds__(kPackThreads, 3) pack_kernel(const __grid_constant__ PackParams P)
+// PER = 4: up to 9 taps of a filter in registers, their loads in flight together.  (Through shared memory as below: 6.3 -> 8.5 us for 352 ->
+// 336 channels.)
+__device__ __forceinline__ void pack_fold_wide(const PackParams &P, int idx)
+{
+    constexpr int PER = 4, TAPS = 9;
+    const int win = idx / P.fold_dblocks, group = idx - win * P.fold_dblocks, cl = threadIdx.x & 63, c = win * 64 + cl;
+    const int d0 = (group * 4 + (threadIdx.x >> 6)) * PER;
+    const int i0 = c < P.C ? P.off[c] : 0, i1 = c < P.C && d0 < P.D ? P.off[c + 1] : i0;
+    const size_t term = (size_t)P.fold_dp * (P.fold_blocks / P.fold_dblocks) * P.k2 * 64;
+    float energy = 0.f, sum[PER] = {};
+    for (int t0 = 0; t0 < P.k2; t0 += TAPS) {
+        float acc[TAPS][PER] = {};
+#pragma unroll 1
+        for (int i = i0; i < i1; ++i) {
+            float p[PER], v[TAPS];
+#pragma unroll
+            for (int e = 0; e < PER; ++e) p[e] = d0 + e < P.D ? fold_weight(P, P.pw, (size_t)(d0 + e) * P.G + i) : 0.f;
+#pragma unroll
+            for (int t = 0; t < TAPS; ++t) v[t] = t0 + t < P.k2 ? fold_weight(P, P.dw, (size_t)i * P.k2 + t0 + t) : 0.f;
+#pragma unroll
+            for (int e = 0; e < PER; ++e)
+#pragma unroll
+                for (int t = 0; t < TAPS; ++t) acc[t][e] = fmaf(p[e], v[t], acc[t][e]);
+        }
+#pragma unroll
+        for (int t = 0; t < TAPS; ++t)
+            if (t0 + t < P.k2) pack_fold_store<PER>(P, win, cl, t0 + t, d0, term, acc[t], energy, sum);
+    }
+    pack_fold_sums<PER>(P, win, group, energy, sum);
+}
+
+// PER = 1.  A window's filters lie in a row: the block fetches them and their weights to shared memory in wide loads, all in flight
+// together, as many filters at a time as fit.  (Each thread fetching its own, 9 taps of 5 filters at a time, left a call that is given
+// its weights waiting for load after load: packing alone 80 -> 176 channels,
+// 5 x 5 taps 11.6 -> 6.6 us.)
+template <int TAPS> __device__ __forceinline__ void pack_fold(const PackParams &P, int idx)
+{
+    extern __shared__ __align__(16) uint16_t stage[];        // kFoldPackStage
+    constexpr int ROWS = 4;
+    const int win = idx / P.fold_dblocks, group = idx - win * P.fold_dblocks, cl = threadIdx.x & 63, c = win * 64 + cl;
+    const int row = threadIdx.x >> 6, r0 = group * ROWS, d0 = r0 + row;
+    const int i0 = c < P.C ? P.off[c] : 0, i1 = c < P.C && d0 < P.D ? P.off[c + 1] : i0;
+    const int f0 = P.off[win * 64], f1 = P.off[min(P.C, win * 64 + 64)];        // the window's filters
+    const int most = (kFoldPackStage - 32) / (P.k2 + ROWS);
+    uint16_t *const pws = stage + (most * P.k2 + 23) / 8 * 8;
+    float acc[TAPS][1] = {};
+#pragma unroll 1
+    for (int f = f0; f < f1; f += most) {
+        const int n = min(most, f1 - f);
+        const size_t e0 = (size_t)f * P.k2 & ~(size_t)7, e1 = (size_t)(f + n) * P.k2, all = (size_t)P.G * P.k2;
+        if (f > f0) __syncthreads();             // what was there has been read
+#pragma unroll 4
+        for (size_t e = e0 + 8 * threadIdx.x; e < e1; e += 8 * kPackThreads) {
+            uint4 v;
+            if (P.is_bf16 && e + 8 <= all) {
+                v = *reinterpret_cast<const uint4 *>((const uint16_t *)P.dw + e);
+            } else {
+                uint32_t h[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) h[j] = e + j < all ? float_to_bf16_bits(fold_weight(P, P.dw, e + j)) : 0u;
+                v = make_uint4(h[0] | h[1] << 16, h[2] | h[3] << 16, h[4] | h[5] << 16, h[6] | h[7] << 16);
+            }
+            *reinterpret_cast<uint4 *>(stage + (e - e0)) = v;
+        }
+#pragma unroll 2
+        for (int i = threadIdx.x; i < n; i += kPackThreads) {
+            uint16_t v[ROWS];
+#pragma unroll
+            for (int r = 0; r < ROWS; ++r) v[r] = r0 + r < P.D ? float_to_bf16_bits(fold_weight(P, P.pw, (size_t)(r0 + r) * P.G + f + i)) : 0;
+#pragma unroll
+            for (int r = 0; r < ROWS; ++r) pws[r * most + i] = v[r];
+        }
+        __syncthreads();
+        const uint16_t *const taps = stage + ((size_t)f * P.k2 - e0);
+#pragma unroll 1
+        for (int i = max(i0, f); i < min(i1, f + n); ++i) {
+            const float p = bf16_bits_to_float(pws[row * most + i - f]);
+#pragma unroll
+            for (int t = 0; t < TAPS; ++t)
+                if (t < P.k2) acc[t][0] = fmaf(p, bf16_bits_to_float(taps[(i - f) * P.k2 + t]), acc[t][0]);
+        }
+    }
+    const size_t term = (size_t)P.fold_dp * (P.fold_blocks / P.fold_dblocks) * P.k2 * 64;
+    float energy = 0.f, sum[1] = {};
+#pragma unroll
+    for (int t = 0; t < TAPS; ++t)
+        if (t < P.k2) pack_fold_store<1>(P, win, cl, t, d0, term, acc[t], energy, sum);
+    pack_fold_sums<1>(P, win, group, energy, sum);
+}
+
+// One kernel per way to fold: with the code of all of them in one, calls that fold nothing took up to 0.8 us longer.
+enum { kFoldNot, kFoldWide, kFoldNine, kFoldMore };
+template <int FOLD> __global__ void __launch_bounds__(kPackThreads, 3) pack_kernel(const __grid_constant__ PackParams P)
 {
     grid_launch_dependents();
     grid_dependency_wait();      // the kernel before may still read what this one overwrites
     const int b = (int)blockIdx.x;
-    if (b >= P.first[kPackFold]) {
-        if (P.fold_per == 1) pack_fold<1, 5>(P, b - P.first[kPackFold]);
-        else pack_fold<4, 1>(P, b - P.first[kPackFold]);
+    if (FOLD != kFoldNot && b >= P.first[kPackFold]) {
+        const int idx = b - P.first[kPackFold];
+        if constexpr (FOLD == kFoldWide) pack_fold_wide(P, idx);
+        else pack_fold<FOLD == kFoldNine ? 9 : 25>(P, idx);
     }
     else if (b >= P.first[kPackSlab]) pack_slab(P, b - P.first[kPackSlab]);
     else if (b >= P.first[kPackFilt]) pack_filt(P, b - P.first[kPackFilt]);
@@ -209,7 +282,7 @@ gdws_status_t bf16_pack(gdws_plan_s *p, const void *dw_w, const void *pw_w, cons
     P.pw_img = p->d_pw_img; P.taps = p->d_dw; P.dwpack = p->d_dwpack; P.bias_out = p->d_bias;
     P.tc_chunks = p->d_tc_chunks; P.tc_nchunks = (int)p->tc_chunks.size(); P.tc_nslabs = p->tc_nslabs; P.tc_dloc = p->tc_dloc;
     P.tc_nparts = p->tc_nparts; P.rec_hw = p->tc_rec_hw; P.tc_filt = p->d_tc_filt; P.tc_pw = p->d_tc_pw;
-    P.fold_per = p->fold_per; P.fold_dblocks = p->fold_dp / (4 * p->fold_per); P.fold_dp = p->fold_dp; P.fold_blocks = p->fold_blocks; P.fold = p->d_fold;
+    P.fold_dblocks = p->fold_dp / (4 * p->fold_per); P.fold_dp = p->fold_dp; P.fold_blocks = p->fold_blocks; P.fold = p->d_fold;
     P.fold_sum_step = p->fold_sum_step; P.fold_sums = p->d_fold_sums;
     const long long blocks[kPackParts] = {
         ((long long)p->nchunks * p->Dpad * kChunk + kPackPiece - 1) / kPackPiece,
@@ -226,7 +299,9 @@ gdws_status_t bf16_pack(gdws_plan_s *p, const void *dw_w, const void *pw_w, cons
         if (total > 0x7fffffffLL) return fail(GDWS_ERR_UNSUPPORTED, "weights too large to pack");
     }
     P.first[kPackParts] = (int)total;
-    const cudaError_t e = launch_overlapped(pack_kernel, (unsigned)total, kPackThreads, 0, st, P);
+    const bool staged = fold && p->fold_per == 1;
+    const auto kernel = !fold ? pack_kernel<kFoldNot> : (!staged ? pack_kernel<kFoldWide> : (P.k2 <= 9 ? pack_kernel<kFoldNine> : pack_kernel<kFoldMore>));
+    const cudaError_t e = launch_overlapped(kernel, (unsigned)total, kPackThreads, staged ? kFoldPackStage * sizeof(uint16_t) : 0, st, P);
     if (e != cudaSuccess) { cudaGetLastError(); return cuda_fail(e, "weight pack launch"); }
     p->launches++;
     p->packed = true;
