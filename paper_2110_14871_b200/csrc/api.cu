@@ -227,7 +227,7 @@ gdws_status_t gdws_forward(gdws_plan_t *p, const gdws_tensor_t *x, const void *d
     st = weights_ready(p, dw_w, pw_w, bias, GDWS_BF16, dw_w && fused && bf16_form_of(p, x->n, x->h, x->w, y->dtype == GDWS_F32) == 3, cs);
     if (st != GDWS_OK) return st;
     if (fused) {
-        st = bf16_fused(p, x, y, cs);
+        st = bf16_fused(p, x, y, dw_w != nullptr, cs);
         if (st != GDWS_ERR_UNSUPPORTED || p->opt_path == GDWS_PATH_FUSED) return st;
         // GDWS_PATH_AUTO and no fused kernel for this shape: take the unfused pair
     }

@@ -919,7 +919,7 @@ bool fold_in_slices(gdws_plan_s *p, int n, int h, int w, bool out_f32)
     return !(fold_geometry(p, n, Ho, Wo, out_f32, &g) && g.us <= fold_split_us(p, n, Ho, Wo));
 }
 
-gdws_status_t bf16_folded(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t *y, cudaStream_t st)
+gdws_status_t bf16_folded(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t *y, bool given, cudaStream_t st)
 {
     if (!p->fold_ok) return fail(GDWS_ERR_UNSUPPORTED, "folded path: layer not covered (stride 1 or 2, k <= 5, C and D multiples of 8)");
     const bool out_f32 = y->dtype == GDWS_F32;
@@ -937,7 +937,7 @@ gdws_status_t bf16_folded(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t 
         if (!L) return fail(GDWS_ERR_ALLOC, "out of host memory");
     }
     if (L->sliced) {
-        rc = bf16_folded_split(p, x, y, st);
+        rc = bf16_folded_split(p, x, y, given, st);
         if (rc == GDWS_OK) return rc;
         // refused: pairs cover all but layers of very many output channels
         if (fold_prepare(p, x->n, y->h, y->w, out_f32, L) != GDWS_OK) return rc;

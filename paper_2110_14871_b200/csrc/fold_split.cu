@@ -416,7 +416,7 @@ double fold_split_us(const gdws_plan_s *p, int n, int Ho, int Wo)
     return split_geometry(p, n, Ho, Wo, &g) ? g.us : 1e9;
 }
 
-gdws_status_t bf16_folded_split(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t *y, cudaStream_t st)
+gdws_status_t bf16_folded_split(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t *y, bool given, cudaStream_t st)
 {
     const bool out_f32 = y->dtype == GDWS_F32;
     const LaunchKey key = {x->n, x->h, x->w, (p->opt_relu ? 1 : 0) | (out_f32 ? 2 : 0)};
@@ -444,7 +444,11 @@ gdws_status_t bf16_folded_split(gdws_plan_s *p, const gdws_tensor_t *x, gdws_ten
     cfg.blockDim = dim3(kSplitThreads); cfg.dynamicSmemBytes = L->smem; cfg.stream = st;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    // All 45 clusters of three fit an idle chip, but not one that the packing kernel leaves SM by SM: with overlapped launches a call that is
+    // given its weights waited 3 to 8 us for the last ones (448 -> 264 channels at 4 x 20 x 20: 27 us, 23 without; overlap gains 1 elsewhere;
+    // other cluster sizes and forwards before it showed nothing of the kind on 250 layers).
+    const bool full = L->g.split == 3 && L->g.tiles() * L->g.nparts == cluster_capacity(p, 3);
+    attr[0].val.programmaticStreamSerializationAllowed = given && full ? 0 : 1;
     attr[1].id = cudaLaunchAttributeClusterDimension;
     attr[1].val.clusterDim.x = (unsigned)L->g.split; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr; cfg.numAttrs = L->g.split > 1 ? 2 : 1;

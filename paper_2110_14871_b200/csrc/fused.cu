@@ -1037,14 +1037,14 @@ static gdws_status_t run_tiled(gdws_plan_s *p, const gdws_tensor_t *x, void *out
     return GDWS_OK;
 }
 
-gdws_status_t bf16_fused(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t *y, cudaStream_t st)
+gdws_status_t bf16_fused(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t *y, bool given, cudaStream_t st)
 {
     // GDWS_OPT_DW_MATH: 1 = GDW stage on the ALUs, 2 = on the tensor cores, 3 = folded, 0 = whichever measured faster for this kind of layer
     const int form = bf16_form_of(p, x->n, x->h, x->w, y->dtype == GDWS_F32);
     if (form == 3 && !p->fold_packed && p->opt_dw_math == 3 && p->fold_ok)
         return fail(GDWS_ERR_INVALID_ARG, "the last weights came with a call that took another form: call gdws_pack_weights");
     if (form == 3 && (p->fold_packed || p->opt_dw_math == 3)) {
-        const gdws_status_t rc = bf16_folded(p, x, y, st);
+        const gdws_status_t rc = bf16_folded(p, x, y, given, st);
         if (rc != GDWS_ERR_UNSUPPORTED || p->opt_dw_math == 3) return rc;
     }
     if (form == 2 || (form == 3 && gdw_stage_of(p) == 2)) {

@@ -262,7 +262,8 @@ gdws_status_t bf16_pack(gdws_plan_s *p, const void *dw_w, const void *pw_w, cons
 // bf16.cu
 gdws_status_t bf16_depthwise(gdws_plan_s *p, const gdws_tensor_t *x, void *z, cudaStream_t s);
 gdws_status_t bf16_pointwise(gdws_plan_s *p, const void *z, gdws_tensor_t *y, cudaStream_t s);
-gdws_status_t bf16_fused(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t *y, cudaStream_t s);
+// given: the weights came with the call, the kernel before is the one that packs them
+gdws_status_t bf16_fused(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t *y, bool given, cudaStream_t s);
 gdws_status_t bf16_depthwise_tiled(gdws_plan_s *p, const gdws_tensor_t *x, void *z, cudaStream_t s);
 
 // gdw_tc.cu
@@ -273,12 +274,12 @@ bool bf16_depthwise_on_tc(gdws_plan_s *p, int n, int h, int w);        // whethe
 gdws_status_t bf16_fused_tc(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t *y, cudaStream_t s);
 
 // fold.cu
-gdws_status_t bf16_folded(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t *y, cudaStream_t s);
+gdws_status_t bf16_folded(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t *y, bool given, cudaStream_t s);
 // fold_split.cu: the folded form in slices, for layers that leave SMs idle
 void cluster_capacities(int device, int sms, int (&most)[kMostSlices + 1]);
 int cluster_capacity(const gdws_plan_s *p, int split);     // clusters of `split` blocks, one per SM, that run at the same time
 double fold_split_us(const gdws_plan_s *p, int n, int Ho, int Wo);      // estimate; 1e9 where it does not cover the layer
-gdws_status_t bf16_folded_split(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t *y, cudaStream_t s);
+gdws_status_t bf16_folded_split(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t *y, bool given, cudaStream_t s);
 bool fold_in_slices(gdws_plan_s *p, int n, int h, int w, bool out_f32);      // whether a folded forward runs there
 double bf16_forward_us(gdws_plan_s *p, int n, int h, int w, bool out_f32);
 int bf16_form_of(gdws_plan_s *p, int n, int h, int w, bool out_f32);   // 1 / 2: two stages, GDW on the ALUs / the tensor cores; 3: folded
