@@ -125,7 +125,7 @@ int host_pieces(gdws_plan_s *p, const gdws_tensor_t *xh, const gdws_tensor_t *yh
     if ((p->opt_path == GDWS_PATH_UNFUSED || (p->opt_path == GDWS_PATH_AUTO && p->ws)) && p->ws_bytes < gdws_workspace_bytes(p, xh->dtype, xh->n, xh->h, xh->w)) return 1;
     const bool f32 = xh->dtype == GDWS_F32;
     const LaunchKey key = {xh->n, xh->h, xh->w, (f32 ? 1 : 0) | (p->opt_out_f32 ? 2 : 0) | p->opt_path << 2 | p->opt_dw_math << 4};
-    if (const PieceChoice *c = LaunchCache<PieceChoice>::find(p->launch_cache[4], key)) return c->pieces;
+    if (const PieceChoice *c = LaunchCache<PieceChoice>::find(p->launch_cache[kCachePieces], key)) return c->pieces;
     auto forward_us = [&](int n) { return f32 ? f32_forward_us(p, n, xh->h, xh->w) : bf16_forward_us(p, n, xh->h, xh->w, p->opt_out_f32 != 0); };
     const double ximg = (double)xb / xh->n, yimg = (double)yb / xh->n;
     const double link = 18e-6, link_both = link + 4e-6 * std::min(ximg, yimg) / std::max(ximg, yimg);      // us per byte, one direction alone and with the other one busy
@@ -150,7 +150,7 @@ int host_pieces(gdws_plan_s *p, const gdws_tensor_t *xh, const gdws_tensor_t *yh
     if (std::unique_ptr<PieceChoice> c{new (std::nothrow) PieceChoice}) {
         c->key = key;
         c->pieces = best;
-        LaunchCache<PieceChoice>::add(p->launch_cache[4], std::move(c));
+        LaunchCache<PieceChoice>::add(p->launch_cache[kCachePieces], std::move(c));
     }
     return best;
 }

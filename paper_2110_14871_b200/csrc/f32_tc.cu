@@ -3,7 +3,8 @@
 // z is computed on the ALUs in fp32, tap by tap as in fused_f32_kernel.  The pointwise stage is a contraction, and bf16 products
 // with fp32 sums can carry it at full fp32 precision: an fp32 value is the exact sum of three bf16 values (its 24 significant
 // bits in pieces of 8), z = z1 + z2 + z3 and P = p1 + p2 + p3 with every piece at most 2^-8 of the one before, and
-//     z P = z1 p1 + (z1 p2 + z2 p1) + (z1 p3 + z2 p2 + z3 p1) + what is below 2^-25 of the product.
+//     z P = z1 p1 + (z1 p2 + z2 p1) + (z1 p3 + z2 p2 + z3 p1) + what is below 2^-24 of the product
+// (2^-27.5 in the root mean square).
 // The tensor cores add to their accumulators without rounding to nearest, which would cost a long sum more than fp32 arithmetic
 // does.  An accumulator therefore holds one chunk of kF32TcChunk intermediate channels only, smallest products first, and the chunks'
 // sums are added in fp32 registers: fewer roundings than one multiply-add per channel.
@@ -849,7 +850,7 @@ template <int K, int NB, bool NHWC> gdws_status_t f32tc_launch(gdws_plan_s *p, c
 static const F32TcLaunch *f32tc_prepared(gdws_plan_s *p, int n, int h, int w)
 {
     const LaunchKey key = {n, h, w, p->opt_dw_math};
-    if (const F32TcLaunch *l = LaunchCache<F32TcLaunch>::find(p->launch_cache[5], key)) return l;
+    if (const F32TcLaunch *l = LaunchCache<F32TcLaunch>::find(p->launch_cache[kCacheF32], key)) return l;
     std::unique_ptr<F32TcLaunch> e(new (std::nothrow) F32TcLaunch);
     if (!e) return nullptr;
     const int Ho = gdws_out_dim(h, p->k, p->stride, p->pad), Wo = gdws_out_dim(w, p->k, p->stride, p->pad);
@@ -863,7 +864,7 @@ static const F32TcLaunch *f32tc_prepared(gdws_plan_s *p, int n, int h, int w)
     // takes 14.8) and up to twice too short for large NHWC ones.
     const double alu = f32_alu_us(p, n, h, w);
     if (e->taken && p->opt_dw_math != 2) e->taken = p->G >= kF32TcLeast && e->g.us < (alu < 24.0 ? 3.0 + 0.65 * (alu - 3.0) : 1.1 * alu);
-    return LaunchCache<F32TcLaunch>::add(p->launch_cache[5], std::move(e));
+    return LaunchCache<F32TcLaunch>::add(p->launch_cache[kCacheF32], std::move(e));
 }
 
 bool f32_tc_takes(gdws_plan_s *p, int n, int h, int w, int *alu)

@@ -170,7 +170,7 @@ static __device__ __noinline__ void fold_second(const FoldParams *params, int my
 
 // UNITS x STEPS: the window's units when they are all alike (unrolled: 3 x 3 taps or 9 x 1), 0: table driven.  NK: 1 to 3: the only
 // window has so many K steps of 16 channels (up to 48 channels: straight-line code as for whole windows, 16 x 32 -> 16 x 192 x 165 31.3 ->
-// 27.6 us); 4: whole windows, and a last one of any number.
+// 26.6 us); 4: whole windows, and a last one of any number.
 template <int UNITS, int STEPS, int NK = 4>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kFoldThreads, 1) fold_kernel(const __grid_constant__ FoldParams P)
 {
@@ -735,14 +735,7 @@ gdws_status_t fold_prepare(gdws_plan_s *p, int n, int Ho, int Wo, bool out_f32, 
     size_t smem = 1024 + (size_t)P.off_bias + bias_bytes;
     if (smem < (size_t)kFoldMaxSmem / 2 + 4096) smem = (size_t)kFoldMaxSmem / 2 + 4096;     // one block per SM: tensor memory is never oversubscribed
 
-
-    auto magic = [](int d, uint32_t (&md)[2]) {
-        int sh = 0;
-        while ((1 << sh) < d) ++sh;
-        md[0] = (uint32_t)((((uint64_t)1 << (31 + sh)) + (uint64_t)d - 1) / (uint64_t)d);
-        md[1] = (uint32_t)(31 + sh);
-    };
-    magic(g.nparts, P.dv_parts); magic(g.tiles_h * g.tiles_w, P.dv_thw); magic(g.tiles_w, P.dv_tw);
+    div_magic(g.nparts, P.dv_parts); div_magic(g.tiles_h * g.tiles_w, P.dv_thw); div_magic(g.tiles_w, P.dv_tw);
 
     void (*kernel)(FoldParams) = nullptr;
     int which = 0;
@@ -873,14 +866,14 @@ int bf16_form_of(gdws_plan_s *p, int n, int h, int w, bool out_f32)
     const int Ho = gdws_out_dim(h, p->k, p->stride, p->pad), Wo = gdws_out_dim(w, p->k, p->stride, p->pad);
     if (n < 1 || Ho < 1 || Wo < 1) return stage;
     const LaunchKey key = {n, h, w, out_f32 ? 2 : 0};
-    if (const FormChoice *c = LaunchCache<FormChoice>::find(p->launch_cache[3], key)) return c->form;
+    if (const FormChoice *c = LaunchCache<FormChoice>::find(p->launch_cache[kCacheForm], key)) return c->form;
     FoldGeom g;
     double us = fold_geometry(p, n, Ho, Wo, out_f32, &g) ? g.us : 1e9;
     const double slices = fold_split_us(p, n, Ho, Wo);
     const bool sliced = slices < us;
-    // Slices (fold_split.cu) count where a channel has more than two filters in the mean.  They would win below that as well (384 ->
-    // 104 channels, stride 2, 8 x 8, g_c = 2: 7.3 us against 12.5), but the form that such layers have is part of what callers plan
-    // with: its answers stay.
+    // Slices (fold_split.cu) count where a channel has more than two filters in the mean: the estimates were compared with timings there.
+    // Below it the choice is the one without them, and a layer that they would win keeps the two stages (384 -> 104 channels, stride 2,
+    // 8 x 8, g_c = 2: 12.5 us, in slices 7.3).
     if (p->G > 2 * p->C) us = std::min(us, slices);
     const bool fold = us < two_stage_us(p, n, h, w, Ho, Wo, stage);
     const int form = fold ? 3 : stage;
@@ -888,7 +881,7 @@ int bf16_form_of(gdws_plan_s *p, int n, int h, int w, bool out_f32)
         c->key = key;
         c->form = form;
         c->sliced = sliced;
-        LaunchCache<FormChoice>::add(p->launch_cache[3], std::move(c));      // kept if there is memory for it
+        LaunchCache<FormChoice>::add(p->launch_cache[kCacheForm], std::move(c));      // kept if there is memory for it
     }
     return form;
 }
@@ -913,7 +906,7 @@ double bf16_forward_us(gdws_plan_s *p, int n, int h, int w, bool out_f32)
 
 bool fold_in_slices(gdws_plan_s *p, int n, int h, int w, bool out_f32)
 {
-    if (const FormChoice *c = LaunchCache<FormChoice>::find(p->launch_cache[3], {n, h, w, out_f32 ? 2 : 0})) return c->sliced;
+    if (const FormChoice *c = LaunchCache<FormChoice>::find(p->launch_cache[kCacheForm], {n, h, w, out_f32 ? 2 : 0})) return c->sliced;
     const int Ho = gdws_out_dim(h, p->k, p->stride, p->pad), Wo = gdws_out_dim(w, p->k, p->stride, p->pad);
     FoldGeom g;
     return !(fold_geometry(p, n, Ho, Wo, out_f32, &g) && g.us <= fold_split_us(p, n, Ho, Wo));
@@ -925,7 +918,7 @@ gdws_status_t bf16_folded(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t 
     const bool out_f32 = y->dtype == GDWS_F32;
     const LaunchKey key = {x->n, x->h, x->w, (p->opt_relu ? 1 : 0) | (out_f32 ? 2 : 0)};
     gdws_status_t rc;
-    FoldLaunch *L = LaunchCache<FoldLaunch>::find(p->launch_cache[2], key);
+    FoldLaunch *L = LaunchCache<FoldLaunch>::find(p->launch_cache[kCacheFold], key);
     if (!L) {
         std::unique_ptr<FoldLaunch> e(new (std::nothrow) FoldLaunch);
         if (!e) return fail(GDWS_ERR_ALLOC, "out of host memory");
@@ -933,7 +926,7 @@ gdws_status_t bf16_folded(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_t 
         e->sliced = fold_in_slices(p, x->n, x->h, x->w, out_f32);
         rc = e->sliced ? GDWS_OK : fold_prepare(p, x->n, y->h, y->w, out_f32, e.get());
         if (rc != GDWS_OK) return rc;
-        L = LaunchCache<FoldLaunch>::add(p->launch_cache[2], std::move(e));
+        L = LaunchCache<FoldLaunch>::add(p->launch_cache[kCacheFold], std::move(e));
         if (!L) return fail(GDWS_ERR_ALLOC, "out of host memory");
     }
     if (L->sliced) {

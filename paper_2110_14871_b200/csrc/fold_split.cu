@@ -421,14 +421,14 @@ gdws_status_t bf16_folded_split(gdws_plan_s *p, const gdws_tensor_t *x, gdws_ten
     const bool out_f32 = y->dtype == GDWS_F32;
     const LaunchKey key = {x->n, x->h, x->w, (p->opt_relu ? 1 : 0) | (out_f32 ? 2 : 0)};
     gdws_status_t rc;
-    SplitLaunch *L = LaunchCache<SplitLaunch>::find(p->launch_cache[7], key);
+    SplitLaunch *L = LaunchCache<SplitLaunch>::find(p->launch_cache[kCacheSplit], key);
     if (!L) {
         std::unique_ptr<SplitLaunch> e(new (std::nothrow) SplitLaunch);
         if (!e) return fail(GDWS_ERR_ALLOC, "out of host memory");
         e->key = key;
         rc = split_prepare(p, x->n, y->h, y->w, out_f32, e.get());
         if (rc != GDWS_OK) return rc;
-        L = LaunchCache<SplitLaunch>::add(p->launch_cache[7], std::move(e));
+        L = LaunchCache<SplitLaunch>::add(p->launch_cache[kCacheSplit], std::move(e));
         if (!L) return fail(GDWS_ERR_ALLOC, "out of host memory");
     }
     if (L->x != x->ptr && (rc = split_map_x(p, x, L)) != GDWS_OK) return rc;

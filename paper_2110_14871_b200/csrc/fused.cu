@@ -1019,14 +1019,14 @@ static gdws_status_t run_tiled(gdws_plan_s *p, const gdws_tensor_t *x, void *out
 {
     const LaunchKey key = {x->n, x->h, x->w, (p->opt_relu ? 1 : 0) | (out_f32 ? 2 : 0) | (zout ? 4 : 0) | (p->opt_a_layout ? 8 : 0) | (p->opt_tile << 4)};
     gdws_status_t rc;
-    AluLaunch *L = LaunchCache<AluLaunch>::find(p->launch_cache[0], key);
+    AluLaunch *L = LaunchCache<AluLaunch>::find(p->launch_cache[kCacheAlu], key);
     if (!L) {
         std::unique_ptr<AluLaunch> e(new (std::nothrow) AluLaunch);
         if (!e) return fail(GDWS_ERR_ALLOC, "out of host memory");
         e->key = key;
         rc = alu_prepare(p, x->n, x->h, x->w, Ho, Wo, zout, out_f32, e.get());
         if (rc != GDWS_OK) return rc;
-        L = LaunchCache<AluLaunch>::add(p->launch_cache[0], std::move(e));
+        L = LaunchCache<AluLaunch>::add(p->launch_cache[kCacheAlu], std::move(e));
         if (!L) return fail(GDWS_ERR_ALLOC, "out of host memory");
     }
     if (L->x != x->ptr && (rc = alu_map_x(p, x, L)) != GDWS_OK) return rc;

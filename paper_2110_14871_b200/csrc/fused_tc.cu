@@ -979,14 +979,14 @@ gdws_status_t bf16_fused_tc(gdws_plan_s *p, const gdws_tensor_t *x, gdws_tensor_
     const bool out_f32 = y->dtype == GDWS_F32;
     const LaunchKey key = {x->n, x->h, x->w, (p->opt_relu ? 1 : 0) | (out_f32 ? 2 : 0)};
     gdws_status_t rc;
-    TcLaunch *L = LaunchCache<TcLaunch>::find(p->launch_cache[1], key);
+    TcLaunch *L = LaunchCache<TcLaunch>::find(p->launch_cache[kCacheTc], key);
     if (!L) {
         std::unique_ptr<TcLaunch> e(new (std::nothrow) TcLaunch);
         if (!e) return fail(GDWS_ERR_ALLOC, "out of host memory");
         e->key = key;
         rc = tc_prepare(p, x->n, y->h, y->w, out_f32, e.get());
         if (rc != GDWS_OK) return rc;
-        L = LaunchCache<TcLaunch>::add(p->launch_cache[1], std::move(e));
+        L = LaunchCache<TcLaunch>::add(p->launch_cache[kCacheTc], std::move(e));
         if (!L) return fail(GDWS_ERR_ALLOC, "out of host memory");
     }
     if (L->x != x->ptr && (rc = tc_map_x(p, x, L)) != GDWS_OK) return rc;

@@ -7,7 +7,7 @@
 // cycles of multiply-adds and loads (2900 in the kernel that does so), here 64 channels at a mean multiplier of 2.7 some 500.
 //
 // Measured, ALUs | here: 64 -> 191 channels at 64 x 56 x 56 47.6 | 40.3 us, 424 -> 1181 at 38 x 19 x 25, stride 2 57.7 | 21.2, 512 -> 1415
-// at 9 x 9 x 9 35.6 | 10.2, 176 -> 2203 at 28 x 28 x 28, 5 x 5 taps 146 | 97; nothing in it, 6.7 us against 4.5.
+// at 9 x 9 x 9 35.6 | 10.2, 176 -> 2203 at 28 x 28 x 28, 5 x 5 taps 146 | 80.5; nothing in it, 6.7 us against 4.5.
 // What bounds it: an item (a pair of tiles x 64 channels) takes some 1.05 us, of which its 18 products at a mean multiplier of 2.7 are
 // 0.4; without its stores the first layer takes 33 us, without its products 38.  The layout that follows:
 //   * A operand: the input box of a tile, all taps from one box, as in the folded kernel (csrc/fold.cu); 16, 32 or 64
@@ -461,7 +461,7 @@ bool gdw_prepare(const gdws_plan_s *p, int n, int Ho, int Wo, GdwLaunch *L)
         g.IW = layout == 3 ? 4 : PW + t.ext;
         g.IH = layout == 1 ? PH + t.ext : PH;
         g.nloads = layout == 1 ? t.npar * t.npar : (layout == 2 ? k * t.npar : k * k);
-        const double boxes = (double)g.nloads * TN * g.IH * g.IW * cb * 2 * nw / 45.0;       // one thread's loads: 49 bytes per clock
+        const double boxes = (double)g.nloads * TN * g.IH * g.IW * cb * 2 * nw / 45.0;       // one thread's loads: some 45 bytes per clock
         const double item = std::max(std::max(ksteps / p->nchunks * 46.0 + 300.0, boxes), 700.0);
         g.cycles = std::ceil((double)g.pairs * p->nchunks / nclusters) * item;
         if (!best.layout || g.cycles < best.cycles) best = g;
@@ -619,7 +619,7 @@ gdws_status_t gdw_maps(const gdws_plan_s *p, const gdws_tensor_t *x, void *z, Gd
 static GdwLaunch *gdw_prepared(gdws_plan_s *p, int n, int h, int w)
 {
     const LaunchKey key = {n, h, w, p->opt_dw_math};
-    if (GdwLaunch *L = LaunchCache<GdwLaunch>::find(p->launch_cache[6], key)) return L;
+    if (GdwLaunch *L = LaunchCache<GdwLaunch>::find(p->launch_cache[kCacheGdw], key)) return L;
     std::unique_ptr<GdwLaunch> e(new (std::nothrow) GdwLaunch);
     if (!e) return nullptr;
     const int Ho = gdws_out_dim(h, p->k, p->stride, p->pad), Wo = gdws_out_dim(w, p->k, p->stride, p->pad);
@@ -628,7 +628,7 @@ static GdwLaunch *gdw_prepared(gdws_plan_s *p, int n, int h, int w)
     e->taken = p->G > 0 && !(p->stride == 2 && (h < 2 || w < 2) && tc_taps(p->k, 2, p->pad).used[1]) && gdw_prepare(p, n, Ho, Wo, e.get());
     e->P.H = h; e->P.W = w;
     if (e->taken && p->opt_dw_math != 2) e->taken = e->us < gdw_alu_us(p, n, h, w);
-    return LaunchCache<GdwLaunch>::add(p->launch_cache[6], std::move(e));
+    return LaunchCache<GdwLaunch>::add(p->launch_cache[kCacheGdw], std::move(e));
 }
 
 bool bf16_depthwise_on_tc(gdws_plan_s *p, int n, int h, int w)

@@ -22,6 +22,10 @@ constexpr int kHostPieces = 5;      // pieces that gdws_forward_host overlaps
 constexpr int kMostSlices = 8;      // blocks of a cluster that share a tile's sum
 constexpr int kMaxSmem = 225 * 1024;      // dynamic shared memory a block may ask for (227 KB minus static use)
 
+// What a plan keeps per input size: launches of fused_bf16_kernel, fused_tc_kernel and fold_kernel, the form of a bf16 forward, the pieces
+// of a host call, launches of f32_tc_kernel, gdw_tc_kernel and fold_split_kernel.
+enum { kCacheAlu, kCacheTc, kCacheFold, kCacheForm, kCachePieces, kCacheF32, kCacheGdw, kCacheSplit, kCaches };
+
 // Bits of the device status word.
 enum : int {
     kStatusWaitStage = 1,   // wait for a free shared-memory stage ran out
@@ -134,9 +138,8 @@ struct gdws_plan_s {
     void *stage_x = nullptr, *stage_y = nullptr;  // gdws_forward_host staging
     size_t stage_x_bytes = 0, stage_y_bytes = 0;
 
-    // Prepared launches of the three fused bf16 kernels, the choice between them and the pieces of a host call (LaunchCache
-    // below; each file knows its own types).
-    std::shared_ptr<void> launch_cache[8];
+    // Prepared launches and choices (LaunchCache below; each file knows its own types).
+    std::shared_ptr<void> launch_cache[gdws::kCaches];
 
     int64_t launches = 0;
 };

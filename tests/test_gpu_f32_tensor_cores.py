@@ -1,5 +1,5 @@
-"""The fp32 forward with its pointwise products on the tensor cores: against the CPU oracle, no less exact than the ALU kernel, and
-with the same infinities and NaN.  Output channels around 16, 32, 64 and 128 and in two parts, chunks of 32 intermediate channels with
+"""The fp32 forward with its pointwise products on the tensor cores: against the CPU oracle, no less exact than the ALU kernel from 16
+intermediate channels on, for values of all sizes, and with the same infinities and NaN.  Output channels around 16, 32, 64 and 128 and in two parts, chunks of 32 intermediate channels with
 remainders and one alone, clusters that share a tile's chunks, tiles of several images, both filter sizes, strides, channels without filters."""
 import time
 
@@ -51,7 +51,7 @@ def test_matches_reference(shape, layout):
     _on_tensor_cores(data)
     ref, _ = run_oracle(data)
     tc, alu = (run_gpu(data, path=gdws.PATH_FUSED, dw_math=m) for m in (2, 1))
-    # dropped pieces and the chunks' truncation: 2^-22 of sum |P||z|, some sqrt(G) times the largest output
+    # dropped products (2^-24 each) and the chunks' truncation: 2^-22 of sum |P||z|, some sqrt(G) times the largest output
     assert rel_err(tc, ref) <= 1e-5
     # one rounding per chunk instead of one per channel; both have z's own roundings.  With fewer channels than the default takes here
     # what the tensor cores truncate (2^-24 of the sum at most) can outweigh it.

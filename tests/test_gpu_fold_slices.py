@@ -46,3 +46,38 @@ def test_slices_match_reference(N, C, D, H, W, k, stride, zero_sum):
     assert np.array_equal(got[0], got[1])
     assert rel_err(got[0], run_oracle(data)[0]) <= 1e-2        # folded filters and y rounded once each: 2^-8 and 2^-9, and sums
     plan.destroy()
+
+
+@pytest.mark.parametrize("N,D", [(2, 264), (4, 264)])
+def test_every_cluster_of_three_right_after_packing(N, D):
+    """A layer that takes all of the clusters of three that fit, given its weights: no more than packing, then the forward, and a launch
+    between them (its last clusters came in a second round when the launches overlapped: 5 to 8 us more)."""
+    data = gi.make_layer(small_spec("t", N, 448, D, 20, 20, 3, 1, 1, ("uniform", 1, 5), "bf16", "NHWC", seed=3))
+    plan = make_plan(data)
+    assert plan.kernel(N, 20, 20) == gdws.KERNEL_FOLDED_SLICES
+    x, dw, pw, b = to_device(data.x, "bf16"), to_device(data.dw_w, "bf16"), to_device(data.pw_w, "bf16"), torch.from_numpy(data.bias).cuda()
+    y = torch.empty((N, 20, 20, D), dtype=torch.bfloat16, device="cuda")
+
+    def least_us(call):
+        call()
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            for _ in range(20):
+                call()
+        us = []
+        for _ in range(6):
+            a, e = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            graph.replay()
+            e.record()
+            torch.cuda.synchronize()
+            us.append(a.elapsed_time(e) * 50)
+        return min(us)
+
+    given = least_us(lambda: plan.forward(x, y, "NHWC", dw, pw, b))
+    pack = least_us(lambda: plan.pack_weights(dw, pw, b))
+    packed = least_us(lambda: plan.forward(x, y, "NHWC"))
+    plan.status()
+    plan.destroy()
+    assert given <= pack + packed + 3.0, (given, pack, packed)
