@@ -94,8 +94,9 @@ typedef enum {
                               infinity or NaN in them reaches y.  0 takes 3 for layers with
                               g_c = 0 only where no other kernel covers them (D > 512).
                               fp32 forwards: 1 = all arithmetic on the ALUs; 2 = pointwise products
-                              on the tensor cores (three bf16 pieces per value, fp32 sums) for
-                              k = 3 and 5; 0 and 3 = whichever is estimated faster.
+                              on the tensor cores (three bf16 pieces per value, fp32 sums; no less
+                              exact than 1 from G = 16 on) for k = 3 and 5; 0 and 3 = whichever is
+                              estimated faster, 1 for G < 16.
                               gdws_depthwise, bf16: 1 = ALUs, 2 = tensor cores, 0 and 3 = whichever
                               is estimated faster: same z but for values next to a rounding boundary.
                               In these two calls 2 is a preference: a layer that the tensor cores do

@@ -46,10 +46,10 @@ def test_folded_filters_match_reference(N, C, D, H, W, k, gd):
     plan.destroy()
 
 
-@pytest.mark.parametrize("N,C,D,H,k,gd,most", [(4, 56, 40, 6, 5, ("heavy",), 2.3), (8, 48, 64, 34, 5, ("uniform", 1, 25), 5.0), (2, 72, 120, 13, 3, ("uniform", 1, 9), 2.3)])
+@pytest.mark.parametrize("N,C,D,H,k,gd,most", [(4, 56, 40, 6, 5, ("heavy",), 2.5), (8, 48, 64, 34, 5, ("uniform", 1, 25), 5.0), (2, 72, 120, 13, 3, ("uniform", 1, 9), 2.5)])
 def test_folding_adds_little_to_a_call_given_its_weights(N, C, D, H, k, gd, most):
     """What packing takes in front of a folded forward against what it takes in front of the two stages, which is part of the same launch:
-    1.5 to 2 times, 3.4 with up to 25 filters a channel (2.7 and 7.6 when each thread fetched its own filters)."""
+    2.3 times at most, 3.4 with up to 25 filters a channel (2.7 and 7.6 when each thread fetched its own filters)."""
     data = gi.make_layer(small_spec("t", N, C, D, H, H, k, 1, k // 2, gd, "bf16", "NHWC", seed=3))
     plan = make_plan(data, path=gdws.PATH_FUSED)
     x, dw, pw, b = to_device(data.x, "bf16"), to_device(data.dw_w, "bf16"), to_device(data.pw_w, "bf16"), torch.from_numpy(data.bias).cuda()
